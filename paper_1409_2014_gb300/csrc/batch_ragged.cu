@@ -306,8 +306,7 @@ dsnu_status ragged_create(const RaggedGroupIn* groups, int n, Ragged** out) {
     a.ay = AxisTabs<float>{static_cast<const cpx<float>*>(t.stw_y), static_cast<const cpx<float>*>(t.twm_lo_y),
                            static_cast<const cpx<float>*>(t.twm_hi_y), g.log2lo_y,
                            static_cast<const float*>(t.decon_y), nullptr};
-    a.mt = MultTabs<float>{static_cast<const float*>(t.m_wx2), static_cast<const float*>(t.m_gx), g.n_gy,
-                           float(1.0 / (g.sigma * g.sigma)),
+    a.mt = MultTabs<float>{static_cast<const float*>(t.m_wx2), static_cast<const float*>(t.m_gx),
                            float(-g.dky2 / (g.sigma * g.sigma) * 1.4426950408889634), float(g.dky2), g.ny, g.sharp,
                            float(g.cut_radius * g.cut_radius), 0, 0, 0.f, 0.f, 0.f, float(std::sqrt(g.dky2)),
                            static_cast<const float*>(t.m_kx), static_cast<const float*>(t.m1tab), g.ny + 4};

@@ -571,13 +571,6 @@ __device__ __forceinline__ float f32_of_f64_int(double d, bool& odd) {
 }
 static __device__ __noinline__ float f32_of_f64_hw(double d) { return __double2float_rn(d); }
 
-// expm1 in the working precision (library function).
-template <typename R>
-__device__ __forceinline__ R expm1_r(R x) {
-  if constexpr (sizeof(R) == 4) return expm1f(x);
-  else return expm1(x);
-}
-
 // 1/b in FP64 by Newton-Raphson: the hardware's approximate reciprocal
 // (rcp.approx.ftz.f64, about 2^-20 relative) refined twice by
 // r <- r + r (1 - b r), which squares the relative error each step, so the

@@ -1,0 +1,314 @@
+// fx.cuh -- the FP64 transforms in 64-bit block fixed point.
+//
+// GB300 issues FP64 instructions at 1/64 of its FP32 rate: one warp-wide FP64
+// addition occupies an SM's FP64 pipe for 20 cycles (measured), a 64-bit
+// integer addition the integer pipes for 0.76, and a 32 x 32 + 64 bit
+// multiply-add for about one.  The FFTs of the FP64 plans, which are additions
+// for the most part, therefore run on 64-bit integers: one complex
+// multiplication by a table factor costs 16 cycles instead of 75, one addition
+// 0.76 instead of 20, a radix-16 butterfly with its twiddles about 460 instead
+// of 4200 cycles per warp.
+//
+// Block fixed point: the values of one transform share one exponent E, value =
+// v 2^E.  Before each radix-16 stage the values are shifted left as far as the
+// largest component allows (|component| < 2^61), and the stage's twiddle
+// multiplication carries the factor 1/16: complex magnitudes enter a butterfly
+// below 2^57.5 and leave it below 2^61.5, with no overflow in any partial sum
+// (a partial sum of a DFT is a DFT of fewer terms).  The quantum is then at
+// most 2^-56 of the largest component at every stage, whatever the data: a
+// fixed 1/16 per stage would cost localised data, which do not grow in the
+// first stages, four bits each (measured: 5 times the FP64 transforms' error).
+// As in floating point, errors are relative to the norm of a transform's
+// input, not to single elements.
+//
+// Multiplication: x = xh 2^32 + xl with both halves signed (xl in [-2^31,
+// 2^31)), the constant as w 2^k = h + l 2^-32 in two signed 32-bit halves;
+//   x w 2^(k-32) = xh h + 2^-32 (xh l + xl h) + 2^-64 xl l,
+// the last term (at most 1/4 of the quantum) dropped, the middle one rounded.
+#pragma once
+
+#include "common.cuh"
+
+namespace dsnu {
+
+using i64 = long long;
+
+struct alignas(16) fxc {  // fixed-point complex value
+  i64 x, y;
+};
+struct alignas(16) fxw {  // constant w 2^k: re = rh + rl 2^-32, im = ih + il 2^-32 (|rl|, |il| < 2^31)
+  int rh, rl, ih, il;
+};
+struct alignas(8) fxr {  // real constant in the same form
+  int h, l;
+};
+
+// k of the tables: the twiddles carry 1/16, the multiplier 1/32, the
+// deconvolution factors 1/2
+constexpr int kFxTwBits = 28, kFxMultBits = 27, kFxDeconBits = 31;
+
+// Exponents of all-zero transforms, and of ones with an infinity or a NaN.
+constexpr int kFxZero = -(1 << 20), kFxBad = 1 << 20;
+
+__device__ __forceinline__ fxc fx_mk(i64 x, i64 y) { fxc c; c.x = x; c.y = y; return c; }
+__device__ __forceinline__ fxc operator+(fxc a, fxc b) { return fx_mk(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ fxc operator-(fxc a, fxc b) { return fx_mk(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ fxc fx_swap(fxc a) { return fx_mk(a.y, a.x); }
+
+__device__ __forceinline__ i64 fx_mad(int a, int b, i64 c) {
+  i64 d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ i64 fx_mulw(int a, int b) {
+  i64 d;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+  return d;
+}
+__device__ __forceinline__ void fx_split(i64 x, int& h, int& l) {
+  l = int(x);
+  h = int(x >> 32) + int(unsigned(l) >> 31);
+}
+__device__ __forceinline__ i64 fx_hi(i64 q) { return i64(int(q >> 32)); }
+constexpr i64 kFxHalf = i64(1) << 31;
+
+// x c 2^(k-32)
+__device__ __forceinline__ i64 fx_mulr(i64 x, int h, int l) {
+  int xh, xl;
+  fx_split(x, xh, xl);
+  return fx_mad(xh, h, fx_hi(fx_mad(xl, h, fx_mad(xh, l, kFxHalf))));
+}
+__device__ __forceinline__ i64 fx_mulr(i64 x, fxr c) { return fx_mulr(x, c.h, c.l); }
+// a w 2^(k-32) and a conj(w) 2^(k-32)
+__device__ __forceinline__ fxc fx_mul(fxc a, fxw w) {
+  int xh, xl, yh, yl;
+  fx_split(a.x, xh, xl);
+  fx_split(a.y, yh, yl);
+  const int nh = -w.ih, nl = -w.il;
+  const i64 q = fx_mad(yl, nh, fx_mad(yh, nl, fx_mad(xl, w.rh, fx_mad(xh, w.rl, kFxHalf))));
+  const i64 r = fx_mad(yl, w.rh, fx_mad(yh, w.rl, fx_mad(xl, w.ih, fx_mad(xh, w.il, kFxHalf))));
+  return fx_mk(fx_mad(yh, nh, fx_mad(xh, w.rh, fx_hi(q))), fx_mad(yh, w.rh, fx_mad(xh, w.ih, fx_hi(r))));
+}
+__device__ __forceinline__ fxw fx_conj(fxw w) {
+  w.ih = -w.ih;
+  w.il = -w.il;
+  return w;
+}
+// v 2^-s rounded (s > 0 a constant)
+template <int S>
+__device__ __forceinline__ i64 fx_shr(i64 v) { return (v + (i64(1) << (S - 1))) >> S; }
+template <int S>
+__device__ __forceinline__ fxc fx_shr(fxc a) { return fx_mk(fx_shr<S>(a.x), fx_shr<S>(a.y)); }
+__device__ __forceinline__ fxc fx_shl(fxc a, int s) { return fx_mk(a.x << s, a.y << s); }
+
+// a e^{-2 pi i m/16} / 2 (m = 1, 2, 3, 5, 6, 7): cos(pi/8), sin(pi/8) and
+// sqrt(1/2) times 2^31 as h + l 2^-32
+constexpr int kFxC1h = 1984016189, kFxC1l = -902489949;
+constexpr int kFxS1h = 821806413, kFxS1l = 1565705635;
+constexpr int kFxR2h = 1518500250, kFxR2l = -51432894;
+template <int M16>
+__device__ __forceinline__ fxc fx_rot16h(fxc a) {
+  if constexpr (M16 == 2) {
+    return fx_mk(fx_mulr(a.x + a.y, kFxR2h, kFxR2l), fx_mulr(a.y - a.x, kFxR2h, kFxR2l));
+  } else if constexpr (M16 == 6) {
+    return fx_mk(fx_mulr(a.y - a.x, kFxR2h, kFxR2l), fx_mulr(a.x + a.y, -kFxR2h, -kFxR2l));
+  } else {
+    constexpr int ch = (M16 == 1) ? kFxC1h : (M16 == 3) ? kFxS1h : (M16 == 5) ? -kFxS1h : -kFxC1h;
+    constexpr int cl = (M16 == 1) ? kFxC1l : (M16 == 3) ? kFxS1l : (M16 == 5) ? -kFxS1l : -kFxC1l;
+    constexpr int sh = (M16 == 1 || M16 == 7) ? kFxS1h : kFxC1h;
+    constexpr int sl = (M16 == 1 || M16 == 7) ? kFxS1l : kFxC1l;
+    fxw w;  // cos - i sin
+    w.rh = ch;
+    w.rl = cl;
+    w.ih = -sh;
+    w.il = -sl;
+    return fx_mul(a, w);
+  }
+}
+
+// In-place forward DFT of v[0..RAD) (natural order in and out), as dft_rec.
+template <int RAD>
+__device__ __forceinline__ void fx_dft(fxc (&v)[RAD]) {
+  if constexpr (RAD == 2) {
+    const fxc a = v[0], b = v[1];
+    v[0] = a + b;
+    v[1] = a - b;
+  } else if constexpr (RAD > 2) {
+    constexpr int H = RAD / 2, step = 16 / RAD;
+    fxc e[H], o[H];
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      e[i] = v[2 * i];
+      o[i] = v[2 * i + 1];
+    }
+    fx_dft<H>(e);
+    fx_dft<H>(o);
+#define DSNU_FXTW(K)                                                             \
+  if constexpr ((K) < H) {                                                       \
+    constexpr int RK = ((K) * step) & 15;                                        \
+    if constexpr (RK == 0) {                                                     \
+      v[(K)] = e[(K)] + o[(K)];                                                  \
+      v[(K) + H] = e[(K)] - o[(K)];                                              \
+    } else if constexpr (RK == 4) {                                              \
+      v[(K)] = fx_mk(e[(K)].x + o[(K)].y, e[(K)].y - o[(K)].x);                  \
+      v[(K) + H] = fx_mk(e[(K)].x - o[(K)].y, e[(K)].y + o[(K)].x);              \
+    } else {                                                                     \
+      const fxc h = fx_rot16h<RK>(o[(K)]); /* half of the rotated value */       \
+      v[(K)] = fx_mk(e[(K)].x + h.x + h.x, e[(K)].y + h.y + h.y);                \
+      v[(K) + H] = fx_mk(e[(K)].x - h.x - h.x, e[(K)].y - h.y - h.y);            \
+    }                                                                            \
+  }
+    DSNU_FXTW(0) DSNU_FXTW(1) DSNU_FXTW(2) DSNU_FXTW(3) DSNU_FXTW(4) DSNU_FXTW(5) DSNU_FXTW(6) DSNU_FXTW(7)
+#undef DSNU_FXTW
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Scaling.  fx_mag collects (by OR) the magnitudes' high words of a thread's
+// values; after the OR over the transform's group, every |v| < 2^(64 - clz).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned fx_mag(unsigned m, i64 v) {
+  const int h = int(v >> 32);
+  return m | unsigned(h ^ (h >> 31));
+}
+__device__ __forceinline__ unsigned fx_mag(unsigned m, fxc a) { return fx_mag(fx_mag(m, a.x), a.y); }
+__device__ __forceinline__ unsigned fx_mag(const fxc (&a)[16]) {
+  unsigned m = 0;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) m = fx_mag(m, a[i]);
+  return m;
+}
+
+// OR (or maximum) over the P threads of a pair of groups (the even and the odd
+// chain of one row or column), in two halves around a barrier of the CTA:
+// fx_post gives the warp's part, fx_read collects the pair's.  P <= 32: the
+// pair lies in one warp and fx_read needs no barrier.  `red`: one word per warp.
+template <int P, bool MAX = false>
+__device__ __forceinline__ unsigned fx_post(unsigned m, unsigned* red) {
+  if constexpr (P <= 32) {
+#pragma unroll
+    for (int s = 1; s < P; s <<= 1) {
+      const unsigned o = __shfl_xor_sync(0xffffffffu, m, s);
+      m = MAX ? max(m, o) : (m | o);
+    }
+  } else {
+    m = MAX ? __reduce_max_sync(0xffffffffu, m) : __reduce_or_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  }
+  return m;
+}
+template <int P, bool MAX = false>
+__device__ __forceinline__ unsigned fx_read(unsigned m, const unsigned* red) {
+  if constexpr (P > 32) {
+    constexpr int W = P / 32;
+    const unsigned* r = red + (threadIdx.x / P) * W;
+    m = r[0];
+#pragma unroll
+    for (int i = 1; i < W; ++i) m = MAX ? max(m, r[i]) : (m | r[i]);
+  }
+  return m;
+}
+// Left shift that brings magnitudes OR-ed to m just below 2^T (0 where one is
+// above: a component of a complex value whose magnitude is below 2^(T + 1/2)).
+template <int T>
+__device__ __forceinline__ int fx_norm_shift(unsigned m) { return max(__clz(int(m)) - (64 - T), 0); }
+
+// ---------------------------------------------------------------------------
+// Length-N DFT by a group of G = N/16 threads, 16 values per thread (the index
+// order and buffer layout of block_fft_regs); a pair of groups (P = 2 G
+// threads) runs the even and the odd chain of one row or column, with one
+// scale for both.  One transform per thread keeps it at 128 registers and one
+// copy of the radix-16 code for all stages (the loop below): two transforms per
+// thread at 8 warps per SM, the stages unrolled, came to 200 KB of code and ran
+// twice as long (column pass at 4096^2 1405 us).
+// Returns the exponent that the result gained.  red: 2 words per warp.
+template <int LOG2N>
+__device__ __forceinline__ int fx_fft(fxc (&v)[16], fxc* buf, int t, const fxw* __restrict__ stw, unsigned* red) {
+  constexpr int N = 1 << LOG2N, G = N / 16, P = 2 * G, FULL = LOG2N / 4, LR = LOG2N - 4 * FULL;
+  int ex = 0;
+  // leave stage s (radix 16, NS = 16^s): exchange, and scale for the next one
+  auto exchange = [&](int s) {
+    const int ns = 1 << (4 * s), k = t & (ns - 1);
+    const int base = pad16((t - k) * 16 + k), st = (s == 0) ? 1 : ns + (ns >> 4);
+    unsigned* rd = red + (s & 1) * (blockDim.x >> 5);
+    const unsigned m0 = fx_post<P>(fx_mag(v), rd);
+    __syncthreads();  // every load of this buffer done (in place)
+#pragma unroll
+    for (int r = 0; r < 16; ++r) buf[base + r * st] = v[r];
+    __syncthreads();
+    const int sh = fx_norm_shift<61>(fx_read<P>(m0, rd));
+    ex += 4 - sh;
+    return sh;
+  };
+#pragma unroll 1
+  for (int s = 0;; ++s) {
+    fx_dft<16>(v);
+    if (s == FULL - 1) break;
+    const int sh = exchange(s);
+    const int ns = 16 << (4 * s);
+    const fxw* tw = stw + (ns - 16) + (t & (ns - 1));  // 15 (16 + .. + ns/16) = ns - 16 entries before
+    v[0] = fx_shr<4>(fx_shl(buf[pad16(t)], sh));
+#pragma unroll
+    for (int r = 1; r < 16; ++r) v[r] = fx_mul(fx_shl(buf[pad16(t + r * G)], sh), tw[(r - 1) * ns]);
+  }
+  if constexpr (LR > 0) {
+    constexpr int RAD = 1 << LR, NS = 1 << (4 * FULL), PER = 16 / RAD, NB = N / RAD;
+    const int sh = exchange(FULL - 1);
+    fxc o[16];
+#pragma unroll
+    for (int b = 0; b < PER; ++b) {
+      const int j = t + b * G;
+      const fxw* tw = stw + (NS - 16) + (j & (NS - 1));
+      fxc u[RAD];
+      u[0] = fx_shr<4>(fx_shl(buf[pad16(j)], sh));
+#pragma unroll
+      for (int r = 1; r < RAD; ++r) u[r] = fx_mul(fx_shl(buf[pad16(j + r * NB)], sh), tw[(r - 1) * NS]);
+      fx_dft<RAD>(u);
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) o[b + r * PER] = u[r];
+    }
+#pragma unroll
+    for (int m = 0; m < 16; ++m) v[m] = o[m];
+  }
+  return ex;
+}
+// The unnormalised inverse e^{+2 pi i nk/N}: real and imaginary parts
+// exchanged before and after (register renaming).
+template <int LOG2N>
+__device__ __forceinline__ int fx_ifft(fxc (&v)[16], fxc* buf, int t, const fxw* __restrict__ stw, unsigned* red) {
+#pragma unroll
+  for (int m = 0; m < 16; ++m) v[m] = fx_swap(v[m]);
+  const int ex = fx_fft<LOG2N>(v, buf, t, stw, red);
+#pragma unroll
+  for (int m = 0; m < 16; ++m) v[m] = fx_swap(v[m]);
+  return ex;
+}
+
+// FP64 -> fixed, |v| <= 2^62, relative to the exponent field efm >= 1 of the
+// transform's largest component: d = v 2^(efm - kFxBias), rounded to nearest.
+constexpr int kFxBias = 1084;
+__device__ __forceinline__ i64 fx_from_f64(double d, int efm) {
+  const int hi = __double2hiint(d);
+  const int ef = (hi >> 20) & 0x7FF;
+  const unsigned mh = (unsigned(hi) & 0xFFFFFu) | (ef ? 0x100000u : 0u);
+  const i64 m = i64(((unsigned long long)mh << 32) | unsigned(__double2loint(d))) << 10;
+  const int r = min(efm - max(ef, 1), 62);
+  const i64 v = ((m >> r) + 1) >> 1;
+  return hi < 0 ? -v : v;
+}
+
+// v 2^e as FP64 (round to nearest).  The conversion runs on the FP64 pipe,
+// which is otherwise idle here; the exponent is added to its bit pattern.
+static __device__ __noinline__ double fx_scale_slow(double d, int e) { return scalbn(d, e); }
+__device__ __forceinline__ double fx_scale(double d, int e) {
+  const int hi = __double2hiint(d);
+  const int ne = ((hi >> 20) & 0x7FF) + e;
+  const bool slow = unsigned(ne - 1) >= 0x7FEu || e != max(min(e, 4000), -4000);
+  double r = __hiloint2double(int(unsigned(hi) + unsigned(e) * 0x100000u), __double2loint(d));
+  if (d == 0.0) r = d;
+  else if (slow) r = fx_scale_slow(d, e);
+  return r;
+}
+__device__ __forceinline__ double fx_to_f64(i64 v, int e) { return fx_scale(__ll2double_rn(v), e); }
+
+}  // namespace dsnu

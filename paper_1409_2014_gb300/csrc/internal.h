@@ -13,6 +13,8 @@ namespace dsnu {
 
 // Device tables of a plan.  Real-valued tables are in the plan's working
 // precision (float for DSNU_MIXED, double for DSNU_FP64); node_D is FP64.
+// The split solver's tables down to m_kx belong to mixed plans, the fx_ ones
+// to FP64 plans.
 // The standard solver uses stw_x, stwc_x, stw_y, m_wx2 ((q_x dk_x)^2,
 // q_x <= nx/2), m_kx and status only.
 struct PlanTables {
@@ -27,7 +29,6 @@ struct PlanTables {
   void* decon_y;
   void* m_wx2;    // real, nx + 1  (q_x dk_x)^2
   void* m_gx;     // real, nx + 1  1 - exp(-(q_x dk_x)^2/sigma^2)
-  void* m_gy;     // real, n_gy    1 - exp(-(a dk_y)^2/sigma^2), a < n_gy
   void* m_kx;     // real, k_x per column for the sin 2theta term (0 at the Nyquist column); generic only
   int2* node_q0;  // n_nodes
   int* itile_ptr;   // n_itiles + 1: interpolation item -> range of itile_nodes
@@ -44,6 +45,11 @@ struct PlanTables {
   int* status;    // one int
   void* m1tab;    // split plans with the DS multiplier: m1(q_x, |qbar_y|) in the plan's precision,
                   // (nx + 1) rows of ny + 4 entries, each row's even |qbar_y| first (MultTabs::m1); else NULL
+                  // FP64 plans: fxr entries for every multiplier (FxMult)
+  // FP64 plans: the fixed-point tables of both axes (fx.cuh, FxAxis) and the
+  // multiplier's exponent per column (generic multipliers, else NULL)
+  void *fx_stw_x, *fx_wm_x, *fx_dec_x, *fx_stw_y, *fx_wm_y, *fx_dec_y;
+  int* fx_mexp;
 };
 
 
@@ -67,18 +73,20 @@ struct Members {
 struct WsLayout {
   // off_sched: the column pass's work counter (one int, reset by the forward row pass)
   size_t off_A, off_B, off_Bband, off_Sband, off_c, off_partial, off_sched, total;
+  size_t off_rexp, off_rexpb, off_cexp, off_bexp;  // FP64 plans: exponents of the rows of A and B, the columns of A and B (ints)
   int ldqA, ldqB, ldq;  // q columns of the row-tiled A and B; band column length
 };
 
 struct PlanGeom {
   int nx, ny, mx, my, log2nx, log2ny;
   int log2lo_x, log2lo_y;  // two-level e^{-2 pi i n/M} tables
-  int n_gy;                // entries of the short partition table
   double dky2;             // dk_y^2
   int cap_rowf, cap_col, cap_bandf, cap_bandi, cap_rowi;  // resident CTAs (SMs x occupancy)
   int rowi_bpf;            // inverse row pass prefetches the band values too (FP32)
   int row_pf;              // bit 0 forward row prefetch, bit 1 inverse, bit 2 rowi_bpf
   size_t smem_rowi;        // its dynamic shared memory per CTA
+  int kdx, kdy;            // FP64 plans: 2^kd > the axis' largest deconvolution factor
+  int m1_full, m1_ld;      // FP64 plans: the multiplier rows hold all M_y frequencies (else |qbar_y| <= N_y); entries per row
   int w, Q, n_nodes, n_tiles, tiles_x, tiles_y, max_tile_nodes, n_items;
   int n_itiles;            // interpolation items (at most kItileNodes nodes of one kItile x kItile tile)
   int spread_cfg;          // index into kSpreadCfgs (chosen by the autotuner)

@@ -1,4 +1,6 @@
-// kernels.cuh -- the split-solver pipeline for one density (Sec. 2.1).
+// kernels.cuh -- the split-solver pipeline for one density (Sec. 2.1).  The FFT
+// passes here are those of the mixed (FP32) plans; FP64 plans run the fixed-point
+// passes of kernels_fx.cuh around the interpolation and spreading kernels below.
 //
 // Notation: N x N physical grid (nx, ny), padded/fine grid M = 2N per axis,
 // natural frequency index q in [0, M) with signed value q - M for q >= N.
@@ -106,8 +108,6 @@ template <typename R>
 struct MultTabs {
   const R* wx2;       // (q_x dk_x)^2, q_x in [0, nx]
   const R* gx;        // 1 - exp(-(q_x dk_x)^2 / sigma^2)
-  int n_gy;           // 1 - exp(-(a dk_y)^2 / sigma^2) rounds to 1 for a = |qbar_y| >= n_gy
-  R inv_sigma2;       // 1 / sigma^2
   R neg_dky2_s2_log2e;  // -dk_y^2 / (sigma^2 ln 2)
   R dky2;             // dk_y^2
   int half_my;        // N_y (= M_y / 2)
@@ -120,9 +120,8 @@ struct MultTabs {
   R dky;              // dk_y
   const R* kx;        // k_x of column q_x for the sin 2theta term (0 at the Nyquist column)
   // plans with the DS multiplier: m1(q_x, a) for a = |qbar_y| <= N_y,
-  // computed in FP64 at plan creation (stored in the plan's precision), one
-  // row of ldm entries per column with the even a first (a = 2 j at j) and the
-  // odd a after them (a = 2 j' + 1 at N_y/2 + 1 + j')
+  // computed in FP64 at plan creation (one rounding to FP32), one row of ldm
+  // entries per column with the even a first (a = 2 j at j) and the odd a after them (a = 2 j' + 1 at N_y/2 + 1 + j')
   const R* m1;
   int ldm;
 };
@@ -155,15 +154,11 @@ __device__ __forceinline__ R mult_high(const MultTabs<R>& mt, R wx2, R kx, R gx,
   R part;
   if (mt.sharp) {
     part = (s > mt.cut2) ? R(1) : R(0);
-  } else if constexpr (sizeof(R) == 4) {
+  } else {
     // 1 - e^{-kx^2/s^2} e^{-ky^2/s^2} with e^{-ky^2/s^2} = 2^{-a^2 dk^2 / (s^2 ln 2)}
     // (hardware exp2): absolute error ~1e-7, at the level of FP32 rounding of m1
     const R ey = exp2f(R(a * a) * mt.neg_dky2_s2_log2e);
     part = R(1) - (R(1) - gx) * ey;
-  } else {
-    // 1 - exp(-ky^2/s^2): below working precision of 1 only for a < n_gy
-    const R gy = (a < mt.n_gy) ? -expm1_r(-wy2 * mt.inv_sigma2) : R(1);
-    part = gx + gy * (R(1) - gx);
   }
   if constexpr (GEN)
     return mult_generic(mt, wx2, wy2, kx, (q < mt.half_my) ? q : (q == mt.half_my ? 0 : q - 2 * mt.half_my), s) *
@@ -571,18 +566,6 @@ __device__ __forceinline__ void col_main_body(int vb, int vg, Members mem, WsOff
           const int qq = q + h;
           const int a = (qq < N) ? qq : 2 * N - qq;
           const R mv = valid ? mr[(h ? MH : 0) + (a >> 1)] : R(0);
-          if (h == 0) e[m] = e[m] * mv;
-          else o[m] = o[m] * mv;
-        }
-      } else if constexpr (!GEN) {
-        // FP64: m1 read from the plan's table in global memory (the pass is
-        // bound by FP64 arithmetic, which the table saves; the loads overlap it)
-        const R* mg = mt.m1 + size_t(valid ? col : 0) * mt.ldm;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int qq = q + h;
-          const int a = (qq < N) ? qq : 2 * N - qq;
-          const R mv = valid ? mg[(h ? MH : 0) + (a >> 1)] : R(0);
           if (h == 0) e[m] = e[m] * mv;
           else o[m] = o[m] * mv;
         }
@@ -1008,16 +991,13 @@ __device__ __forceinline__ void row_inv_body(int vb, int vg, Members mem, WsOff 
   const int tid = threadIdx.x;
   const int rr = GG::ILV_I ? (tid & 1) : tid / G;
   const int t = GG::ILV_I ? (tid >> 1) : tid - rr * G;
-  // FP32: the deconvolution factors of the outputs n = 2 (t + G m) + {0, 1}
+  // the deconvolution factors of the outputs n = 2 (t + G m) + {0, 1}
   // this thread writes, the same for every row: kept in registers for the
   // whole launch (loaded per item, at the end of each transform, they came
   // from L2 and stalled the stores)
-  constexpr int ND = sizeof(R) == 4 ? 8 : 1;
-  float2 dec[ND];
-  if constexpr (sizeof(R) == 4) {
+  float2 dec[8];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) dec[m] = *reinterpret_cast<const float2*>(ax.decon + 2 * (t + G * m));
-  }
+  for (int m = 0; m < 8; ++m) dec[m] = *reinterpret_cast<const float2*>(ax.decon + 2 * (t + G * m));
   __syncthreads();
   grid_dep_wait();
   const int si = cj ? -1 : 1;
@@ -1139,7 +1119,7 @@ __device__ __forceinline__ void row_inv_body(int vb, int vg, Members mem, WsOff 
     double* __restrict__ phi = mb.phi;
     if (valid) {
       // slot m holds T(2 (t + G m)) in a and T(2 (t + G m) + 1) in b; n < N for m < 8
-      if (sizeof(R) == 4 && acc64) {
+      if (acc64) {
         const R dys = dy * scale;
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
@@ -1158,10 +1138,8 @@ __device__ __forceinline__ void row_inv_body(int vb, int vg, Members mem, WsOff 
           const R ia = cj ? -a[m].y : a[m].y;
           const R ib = cj ? -b[m].y : b[m].y;
           double2 out;
-          const R d0 = (sizeof(R) == 4) ? R(dec[m & (ND - 1)].x) : ax.decon[n];
-          const R d1 = (sizeof(R) == 4) ? R(dec[m & (ND - 1)].y) : ax.decon[n + 1];
-          out.x = to_f64<R>((a[m].x + ia * d0 * dy) * scale);
-          out.y = to_f64<R>((b[m].x + ib * d1 * dy) * scale);
+          out.x = to_f64<R>((a[m].x + ia * R(dec[m].x) * dy) * scale);
+          out.y = to_f64<R>((b[m].x + ib * R(dec[m].y) * dy) * scale);
           *reinterpret_cast<double2*>(phi + size_t(row) * N + n) = out;
         }
       }

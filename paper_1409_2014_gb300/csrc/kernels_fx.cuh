@@ -1,0 +1,536 @@
+// kernels_fx.cuh -- the FFT passes of the FP64 plans, in 64-bit block fixed
+// point (fx.cuh).
+//
+// The passes, their order and the row-tiled buffers A and B are those of
+// kernels.cuh; here
+//   * A and B hold fixed-point values.  The row pass scales each row by its
+//     own exponent (rexp[iy]); the column passes align a column's rows to the
+//     largest of them, scale the column to its own largest component, and write
+//     it with its own exponent (cexp, bexp); the inverse row pass aligns the
+//     columns and scales each row again.
+//   * the deconvolution factor d_y of a row is a factor of the whole row, so
+//     it multiplies the band columns (forward and inverse), not the rows;
+//     z = rho + i rho d_x / 2^k, k per row so that both parts fill the format
+//     (B's rows then have exponents of their own, rexpb).
+//   * an infinity or a NaN in a row makes its exponent kFxBad, which travels
+//     with the maxima: every result is then NaN.
+//   * for real input the transposed pipeline (every complex constant
+//     conjugated) computes the complex conjugate of each intermediate and the
+//     same real result, so dsnu_solve_adjoint runs these same kernels.
+// A pair of groups of G = N/16 threads works on one row or column: group h = 0
+// runs the even, h = 1 the odd chain (even and odd frequencies, or output
+// points).  Inputs are loaded, converted and aligned once, each thread taking
+// N/(2 G) of them, and handed to both chains through shared memory.  A CTA
+// holds one pair, or as many as fill a warp, so that a small grid spreads over
+// as many SMs as it has rows.
+#pragma once
+
+#include "fx.cuh"
+#include "kernels.cuh"
+
+namespace dsnu {
+
+template <int LOG2N>
+struct FxGeo {
+  static constexpr int N = 1 << LOG2N, M = 2 * N;
+  static constexpr int G = N / 16, P = 2 * G;         // threads per chain, per pair
+  static constexpr int PER = (P >= 32) ? 1 : 32 / P;  // pairs per CTA
+  static constexpr int T = PER * P;
+  static constexpr int MINB = 512 / T;                // 16 warps per SM
+  static constexpr int FB = fft_buf_elems(N);
+  static constexpr int STW = fft_stage_tw_elems(LOG2N) > 0 ? fft_stage_tw_elems(LOG2N) : 1;
+  static constexpr int W = T / 32, RED = 5 * W;       // words of the reductions: two for the FFT, three more
+  static constexpr size_t smem = size_t(STW + PER * 2 * FB) * 16 + ((RED * 4 + 15) & ~15);
+  // inverse rows: a byte of alignment shift per column of A, and one of B
+  static constexpr size_t smem_row_inv(int Q) { return smem + ((N + 1 + 15) & ~15) + ((Q + 1 + 15) & ~15); }
+};
+
+// Plan tables of one axis.
+struct FxAxis {
+  const fxw* stw;    // stage twiddles e^{-2 pi i rk/(NS RAD)} 2^kFxTwBits
+  const fxw* wm;     // e^{-2 pi i n/M} 2^kFxTwBits, n < N/2
+  const fxr* dec;    // d / 2^kd 2^kFxDeconBits
+};
+
+struct FxOff {
+  size_t A, B, Bband, Sband, rexp, rexpb, cexp, bexp;
+};
+
+struct FxMult {
+  const fxr* m1;     // m1 2^-mexp[q] 2^kFxMultBits, row of ldm entries per column
+  const int* mexp;   // NULL: 0
+  int ldm;
+};
+
+// e^{-2 pi i n/M} at n = t + G m
+__device__ __forceinline__ fxw fx_wm(const fxw* __restrict__ wm, int t, int m, int G) {
+  const int4 v = __ldg(reinterpret_cast<const int4*>(wm + t + G * (m & 7)));
+  fxw w;
+  if (m < 8) {
+    w.rh = v.x;
+    w.rl = v.y;
+    w.ih = v.z;
+    w.il = v.w;
+  } else {  // e^{-2 pi i (n' + N/2)/M} = -i e^{-2 pi i n'/M}
+    w.rh = v.z;
+    w.rl = v.w;
+    w.ih = -v.x;
+    w.il = -v.y;
+  }
+  return w;
+}
+__device__ __forceinline__ fxr fx_ldr(const fxr* __restrict__ p) {
+  const int2 v = __ldg(reinterpret_cast<const int2*>(p));
+  fxr r;
+  r.h = v.x;
+  r.l = v.y;
+  return r;
+}
+
+__device__ __forceinline__ void fx_copy(fxw* __restrict__ dst, const fxw* __restrict__ src, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x)
+    *reinterpret_cast<int4*>(dst + i) = __ldg(reinterpret_cast<const int4*>(src + i));
+}
+
+// Maximum of n exponents over the CTA (every thread calls it; contains barriers).
+__device__ __forceinline__ int fx_cta_max(const int* e, int n, unsigned* red) {
+  int m = kFxZero;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) m = max(m, e[i]);
+  m = __reduce_max_sync(0xffffffffu, m);
+  __syncthreads();  // earlier reads of `red`
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = unsigned(m);
+  __syncthreads();
+  int r = int(red[0]);
+  for (int w = 1; w < int(blockDim.x >> 5); ++w) r = max(r, int(red[w]));
+  return r;
+}
+
+// a 2^-s rounded to nearest, s >= 1 (a shift alone rounds down: its mean error
+// of half a quantum adds up over a transform to a spike at index 0).
+__device__ __forceinline__ i64 fx_sra(i64 v, int s) { return ((v >> (s - 1)) + 1) >> 1; }
+__device__ __forceinline__ fxc fx_sra(fxc a, int s) { return fx_mk(fx_sra(a.x, s), fx_sra(a.y, s)); }
+// Right shift that aligns a value of exponent e to exponent emax + HEAD (values
+// are stored below 2^63 and become smaller than 2^(63 - HEAD)).
+template <int HEAD>
+__device__ __forceinline__ int fx_align(int emax, int e) { return min(emax - e + HEAD, 63); }
+
+// The chains' inputs from the staged values z (|component| < 2^61 after the
+// shift s): z/16 for the even one, z e^{-2 pi i n/M}/16 for the odd one.
+template <int G>
+__device__ __forceinline__ void fx_chain_in(fxc (&v)[16], const fxc* st, int s, int h, int t, const fxw* wm) {
+  if (h == 0) {
+#pragma unroll
+    for (int m = 0; m < 16; ++m) v[m] = fx_shr<4>(fx_shl(st[pad16(t + G * m)], s));
+  } else {
+#pragma unroll
+    for (int m = 0; m < 16; ++m) v[m] = fx_mul(fx_shl(st[pad16(t + G * m)], s), fx_wm(wm, t, m, G));
+  }
+}
+// The column sum e(n)/16 + e^{+2 pi i n/M} o(n)/16 of the two chains' results at
+// n = t + G (m + 8 h), m < 8: each chain hands the other half of its values over
+// (in its own buffer) and multiplies half of the odd ones.
+template <int G>
+__device__ __forceinline__ void fx_chain_out(fxc (&v)[16], fxc* buf_e, fxc* buf_o, int s, int h, int t,
+                                             const fxw* wm) {
+  __syncthreads();  // the last stage's loads of the buffers are done
+  if (h == 0) {
+#pragma unroll
+    for (int m = 8; m < 16; ++m) buf_e[pad16(t + G * m)] = v[m];
+  } else {
+#pragma unroll
+    for (int m = 0; m < 8; ++m) buf_o[pad16(t + G * m)] = v[m];
+  }
+  __syncthreads();
+  if (h == 0) {
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+      v[m] = fx_shr<4>(fx_shl(v[m], s)) + fx_mul(fx_shl(buf_o[pad16(t + G * m)], s), fx_conj(fx_wm(wm, t, m, G)));
+  } else {
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+      v[m] = fx_shr<4>(fx_shl(buf_e[pad16(t + G * (m + 8))], s)) +
+             fx_mul(fx_shl(v[m + 8], s), fx_conj(fx_wm(wm, t, m + 8, G)));
+  }
+}
+
+// Common prologue of the passes: the CTA's tables, buffers and thread roles.
+#define DSNU_FX_SETUP(AX)                                                  \
+  using GG = FxGeo<LOG2N>;                                                 \
+  using TL = Tile<double>;                                                 \
+  constexpr int N = GG::N, G = GG::G, P = GG::P, PER = GG::PER, W = GG::W; \
+  extern __shared__ __align__(16) unsigned char smem_raw[];                \
+  fxw* stw = reinterpret_cast<fxw*>(smem_raw);                             \
+  fxc* sm = reinterpret_cast<fxc*>(stw + GG::STW);                         \
+  unsigned* red = reinterpret_cast<unsigned*>(sm + PER * 2 * GG::FB);      \
+  fx_copy(stw, (AX).stw, fft_stage_tw_elems(LOG2N));                       \
+  const int pr = threadIdx.x / P, tp = threadIdx.x - pr * P;               \
+  const int h = tp / G, t = tp - h * G;                                    \
+  fxc* buf_e = sm + (2 * pr) * GG::FB;                                     \
+  fxc* buf_o = buf_e + GG::FB;                                             \
+  fxc* buf = h ? buf_o : buf_e;                                            \
+  __syncthreads();                                                         \
+  grid_dep_wait();
+
+// ---------------------------------------------------------------------------
+// Forward row pass (k_row_fwd in fixed point).
+template <int LOG2N>
+__global__ void __launch_bounds__(FxGeo<LOG2N>::T, FxGeo<LOG2N>::MINB)
+k_fx_row_fwd(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis ax, int kd) {
+  DSNU_FX_SETUP(ax)
+  const int items = (ny + PER - 1) / PER;
+#pragma unroll 1
+  for (int it = blockIdx.x; it < items * mem.count; it += gridDim.x) {
+    if (it + int(gridDim.x) >= items * mem.count) grid_dep_trigger();  // last item of this CTA
+    const int mi = it / items, row = (it - mi * items) * PER + pr;
+    const Member mb = member_at(mem, mi);
+    const bool valid = row < ny;
+    double x[8];
+    fxr d[8];
+    unsigned mx = 0, md = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      x[i] = valid ? __ldg(mb.rho + size_t(row) * N + tp + P * i) : 0.0;
+      d[i] = fx_ldr(ax.dec + tp + P * i);
+      const unsigned a = unsigned(__double2hiint(x[i])) & 0x7FFFFFFFu;
+      mx = max(mx, a);
+      md = max(md, (a >> 20) + 32u - unsigned(__clz(d[i].h)));
+      if (__double2loint(x[i]) != 0) mx |= 1u;  // (a subnormal below 2^-1042)
+    }
+    mx = fx_post<P, true>(mx, red + 2 * W);
+    md = fx_post<P, true>(md, red + 3 * W);
+    __syncthreads();
+    mx = fx_read<P, true>(mx, red + 2 * W);
+    md = fx_read<P, true>(md, red + 3 * W);
+    const int efm = max(int(mx >> 20), 1);
+    // the smallest k with |rho d_x| <= 2^k max |rho| by the exponents (|rho| <
+    // 2^(ef + 1), d_x/2^kd < 2^(1 - clz h)): z = rho + i rho d_x/2^k
+    const int kr = min(max(int(md) - 32 + kd + 1 - efm, 0), kd);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const i64 v = fx_from_f64(x[i], efm);
+      buf_e[pad16(tp + P * i)] = fx_mk(fx_shr<1>(v), fx_mulr(v, d[i]) << (kd - kr));  // <= 2^61
+    }
+    __syncthreads();
+    fxc v[16];
+    fx_chain_in<G>(v, buf_e, 0, h, t, ax.wm);
+    const int ef = fx_fft<LOG2N>(v, buf, t, stw, red);
+    const unsigned mag = fx_post<P>(fx_mag(v), red + 4 * W);
+    __syncthreads();  // (and the last stage's loads are done)
+    const int s1 = fx_norm_shift<62>(fx_read<P>(mag, red + 4 * W));  // sums of two: below 2^63
+#pragma unroll
+    for (int m = 0; m < 16; ++m) buf[pad16(t + G * m)] = v[m];
+    __syncthreads();
+    // exponent of Z: from_f64 (efm - kFxBias), the five bits, the stages;
+    // A = (Z(q) + conj Z(M - q))/2 and B = (Z(q) - conj Z(M - q))/2i as sums, times 2^s1
+    if (tp == 0 && valid) {
+      const int ea = (mx >= 0x7FF00000u) ? kFxBad : (mx == 0u) ? kFxZero : efm - kFxBias + 5 + ef - 1 - s1;
+      ws_ptr<int>(mb, off.rexp)[row] = ea;
+      ws_ptr<int>(mb, off.rexpb)[row] = (mx == 0u || mx >= 0x7FF00000u) ? ea : ea + kr;
+    }
+    if (valid) {
+      fxc* Ar = ws_ptr<fxc>(mb, off.A) + TL::at(row, 0, ldqA);
+      fxc* Br = ws_ptr<fxc>(mb, off.B) + TL::at(row, 0, ldqB);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        const int q = tp + P * i;
+        if (i == 8 && q > N) break;
+        const int k = q >> 1;
+        const fxc zq = (q & 1) ? buf_o[pad16(k)] : buf_e[pad16(k & (N - 1))];
+        const fxc zm = (q & 1) ? buf_o[pad16(N - 1 - k)] : buf_e[pad16((N - k) & (N - 1))];
+        Ar[q * TL::TR] = fx_shl(fx_mk(zq.x + zm.x, zq.y - zm.y), s1);
+        if (q <= Q) Br[q * TL::TR] = fx_shl(fx_mk(zq.y + zm.y, zm.x - zq.x), s1);
+      }
+    }
+  }
+}
+
+// Alignment shifts, a byte each, of the rows tp + P i that a thread stages.
+// Returns the rows' largest exponent.
+template <int P>
+__device__ __forceinline__ int fx_row_shifts(const int* rexp, int ny, int tp, unsigned* red, unsigned (&pk)[2]) {
+  const int emax = fx_cta_max(rexp, ny, red);
+  pk[0] = pk[1] = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) pk[i >> 2] |= unsigned(fx_align<2>(emax, rexp[tp + P * i])) << (8 * (i & 3));
+  return emax;
+}
+__device__ __forceinline__ int fx_byte(const unsigned (&pk)[2], int i) { return int((pk[i >> 2] >> (8 * (i & 3))) & 0xFFu); }
+
+// ---------------------------------------------------------------------------
+// Column pass of I1 (k_col_main in fixed point).  FULL: the multiplier row has
+// an entry for each of the M natural frequencies (multipliers with a sin 2theta
+// term), else for a = |qbar| <= N only; both parity-split.
+template <int LOG2N, bool FULL>
+__global__ void __launch_bounds__(FxGeo<LOG2N>::T, FxGeo<LOG2N>::MINB)
+k_fx_col_main(Members mem, FxOff off, int ldqA, int ncols, FxAxis ay, FxMult mt) {
+  DSNU_FX_SETUP(ay)
+  constexpr int MH = FULL ? N : N / 2 + 1;  // even entries
+  const int items = (ncols + PER - 1) / PER;
+  int cur = -1, emax = 0;
+  unsigned pk[2] = {0, 0};
+#pragma unroll 1
+  for (int it = blockIdx.x; it < items * mem.count; it += gridDim.x) {
+    if (it + int(gridDim.x) >= items * mem.count) grid_dep_trigger();  // last item of this CTA
+    const int mi = it / items, col = (it - mi * items) * PER + pr;
+    const Member mb = member_at(mem, mi);
+    if (mi != cur) {
+      emax = fx_row_shifts<P>(ws_ptr<int>(mb, off.rexp), N, tp, red + 4 * W, pk);
+      cur = mi;
+    }
+    fxc* __restrict__ A = ws_ptr<fxc>(mb, off.A);
+    const bool valid = col < ncols;
+    fxc v[16];
+    unsigned mag = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = valid ? A[TL::at(tp + P * i, col, ldqA)] : fx_mk(0, 0);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      v[i] = fx_sra(v[i], fx_byte(pk, i));
+      mag = fx_mag(mag, v[i]);
+    }
+    mag = fx_post<P>(mag, red + 2 * W);
+    __syncthreads();  // (and the previous item's reads of the buffers are done)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) buf_e[pad16(tp + P * i)] = v[i];
+    __syncthreads();
+    const int s0 = fx_norm_shift<61>(fx_read<P>(mag, red + 2 * W));
+    fx_chain_in<G>(v, buf_e, s0, h, t, ay.wm);
+    // exponent: the rows', s0, /16, stages, s1, multiplier (its own and /32), stages, s2, /16, the last 3 bits
+    int ex = emax + 2 - s0 + 4 + (mt.mexp && valid ? mt.mexp[col] : 0) + 5 + 4 - 3;
+#pragma unroll 1
+    for (int inv = 0;; ++inv) {  // forward, then inverse (one copy of the transform's code)
+      ex += fx_fft<LOG2N>(v, buf, t, stw, red);
+      mag = fx_post<P>(fx_mag(v), red + (2 + inv) * W);
+      __syncthreads();
+      const int s = fx_norm_shift<62>(fx_read<P>(mag, red + (2 + inv) * W));
+      ex -= s;
+      if (inv) {
+#pragma unroll
+        for (int m = 0; m < 16; ++m) v[m] = fx_swap(v[m]);
+        fx_chain_out<G>(v, buf_e, buf_o, s, h, t, ay.wm);
+        break;
+      }
+      const fxr* mg = mt.m1 + size_t(valid ? col : 0) * mt.ldm + (h ? MH : 0);
+#pragma unroll
+      for (int m = 0; m < 16; ++m) {
+        const int k = t + G * m;  // row q = 2 k + h: |qbar| / 2 rounded down
+        const fxr c = fx_ldr(mg + (FULL ? k : (m < 8 ? k : N - h - k)));
+        const fxc x = fx_shl(v[m], s);
+        v[m] = fx_mk(fx_mulr(x.y, c), fx_mulr(x.x, c));  // (components exchanged: the inverse transform)
+      }
+    }
+    if (valid) {
+#pragma unroll
+      for (int m = 0; m < 8; ++m) A[TL::at(t + G * (m + 8 * h), col, ldqA)] = fx_shl(v[m], 3);  // < 2^59.5 before
+      if (tp == 0) ws_ptr<int>(mb, off.cexp)[col] = (emax >= kFxBad) ? kFxBad : (emax <= kFxZero) ? kFxZero : ex;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Band columns of the type-2 spectrum (k_band_fwd in fixed point), written in
+// FP64; kdy: the deconvolution factors' scale.
+template <int LOG2N>
+__global__ void __launch_bounds__(FxGeo<LOG2N>::T, FxGeo<LOG2N>::MINB)
+k_fx_band_fwd(Members mem, FxOff off, int ldqB, int ncols, int ldq, int Q, FxAxis ay, int kdy) {
+  DSNU_FX_SETUP(ay)
+  constexpr int M = GG::M;
+  const int items = (ncols + PER - 1) / PER;
+  int cur = -1, emax = 0;
+  unsigned pk[2] = {0, 0};
+#pragma unroll 1
+  for (int it = blockIdx.x; it < items * mem.count; it += gridDim.x) {
+    if (it + int(gridDim.x) >= items * mem.count) grid_dep_trigger();  // last item of this CTA
+    const int mi = it / items, col = (it - mi * items) * PER + pr;
+    const Member mb = member_at(mem, mi);
+    if (mi != cur) {
+      emax = fx_row_shifts<P>(ws_ptr<int>(mb, off.rexpb), N, tp, red + 4 * W, pk);
+      cur = mi;
+    }
+    const fxc* __restrict__ B = ws_ptr<fxc>(mb, off.B);
+    double2* __restrict__ Bband = ws_ptr<double2>(mb, off.Bband);
+    const bool valid = col < ncols;
+    fxc v[16];
+    unsigned mag = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = valid ? B[TL::at(tp + P * i, col, ldqB)] : fx_mk(0, 0);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      v[i] = fx_sra(v[i], fx_byte(pk, i));
+      mag = fx_mag(mag, v[i]);
+    }
+    mag = fx_post<P>(mag, red + 2 * W);
+    __syncthreads();
+    const int s0 = fx_norm_shift<61>(fx_read<P>(mag, red + 2 * W));
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const fxr d = fx_ldr(ay.dec + tp + P * i);  // d_y/2^kdy, and /2
+      const fxc x = fx_shl(v[i], s0);
+      buf_e[pad16(tp + P * i)] = fx_mk(fx_mulr(x.x, d), fx_mulr(x.y, d));
+    }
+    __syncthreads();
+    fx_chain_in<G>(v, buf_e, 1, h, t, ay.wm);
+    const int ex = emax + 2 - s0 + kdy + 4 + fx_fft<LOG2N>(v, buf, t, stw, red);
+    if (valid) {
+      const bool bad = emax >= kFxBad;
+      const double nan = __longlong_as_double(0x7FF8000000000000ll);
+#pragma unroll
+      for (int m = 0; m < 16; ++m) {
+        const int q = 2 * (t + G * m) + h, sq = q < N ? q : q - M;
+        if (sq >= -Q && sq <= Q)
+          Bband[size_t(col) * ldq + sq + Q] =
+              bad ? make_double2(nan, nan) : make_double2(fx_to_f64(v[m].x, ex), fx_to_f64(v[m].y, ex));
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Inverse band columns (k_band_inv in fixed point) of the FP64 S, times d_y.
+template <int LOG2N>
+__global__ void __launch_bounds__(FxGeo<LOG2N>::T, FxGeo<LOG2N>::MINB)
+k_fx_band_inv(Members mem, FxOff off, int ldq, int Q, int ncols, int ldqB, FxAxis ay, int kdy) {
+  DSNU_FX_SETUP(ay)
+  constexpr int M = GG::M;
+  const int items = (ncols + PER - 1) / PER;
+#pragma unroll 1
+  for (int it = blockIdx.x; it < items * mem.count; it += gridDim.x) {
+    if (it + int(gridDim.x) >= items * mem.count) grid_dep_trigger();  // last item of this CTA
+    const int mi = it / items, col = (it - mi * items) * PER + pr;
+    const Member mb = member_at(mem, mi);
+    const double2* __restrict__ Sband = ws_ptr<double2>(mb, off.Sband);
+    fxc* __restrict__ St = ws_ptr<fxc>(mb, off.B);
+    const bool valid = col < ncols;
+    fxc v[16];
+    unsigned mx = 0;
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      const int q = 2 * (t + G * m) + h, sq = q < N ? q : q - M;
+      double2 a = make_double2(0.0, 0.0);
+      if (valid && sq >= -Q && sq <= Q) a = Sband[size_t(col) * ldq + sq + Q];
+      mx = max(mx, unsigned(__double2hiint(a.x)) & 0x7FFFFFFFu);
+      mx = max(mx, unsigned(__double2hiint(a.y)) & 0x7FFFFFFFu);
+      if ((__double2loint(a.x) | __double2loint(a.y)) != 0) mx |= 1u;
+      v[m] = fx_mk(__double_as_longlong(a.x), __double_as_longlong(a.y));
+    }
+    mx = fx_post<P, true>(mx, red + 2 * W);
+    __syncthreads();
+    mx = fx_read<P, true>(mx, red + 2 * W);
+    const int efm = max(int(mx >> 20), 1);
+#pragma unroll
+    for (int m = 0; m < 16; ++m)
+      v[m] = fx_shr<5>(fx_mk(fx_from_f64(__longlong_as_double(v[m].x), efm), fx_from_f64(__longlong_as_double(v[m].y), efm)));
+    const int ef = fx_ifft<LOG2N>(v, buf, t, stw, red);
+    const unsigned mag = fx_post<P>(fx_mag(v), red + 3 * W);
+    __syncthreads();
+    const int s1 = fx_norm_shift<62>(fx_read<P>(mag, red + 3 * W));
+    fx_chain_out<G>(v, buf_e, buf_o, s1, h, t, ay.wm);
+    if (valid) {
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        const int n = t + G * (m + 8 * h);
+        const fxr d = fx_ldr(ay.dec + n);
+        St[TL::at(n, col, ldqB)] = fx_shl(fx_mk(fx_mulr(v[m].x, d), fx_mulr(v[m].y, d)), 4);  // < 2^58.5 before
+      }
+      if (tp == 0)
+        ws_ptr<int>(mb, off.bexp)[col] = (mx >= 0x7FF00000u) ? kFxBad
+                                         : (mx == 0u)        ? kFxZero
+                                                             : efm - kFxBias + 5 + ef - s1 + 4 + kdy + 1 - 4;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Inverse row pass (k_row_inv in fixed point): with X = Y + i S and R = Y - i S,
+//   T(2j) = IDFT_N[X(q) + conj R(N - q)](j),
+//   T(2j+1) = IDFT_N[(X(q) - conj R(N - q)) e^{+2 pi i q/M}](j)
+// (at q = 0 the second term is X(N)); Phi = (Re T + d_x Im T) 2^lscale.
+template <int LOG2N>
+__global__ void __launch_bounds__(FxGeo<LOG2N>::T, FxGeo<LOG2N>::MINB)
+k_fx_row_inv(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis ax, int kd, int lscale) {
+  DSNU_FX_SETUP(ax)
+  unsigned char* sh_a = smem_raw + GG::smem;            // alignment shifts of the columns of A
+  unsigned char* sh_b = sh_a + ((N + 1 + 15) & ~15);    // and of B
+  const int items = (ny + PER - 1) / PER;
+  int cur = -1, emax = 0;
+#pragma unroll 1
+  for (int it = blockIdx.x; it < items * mem.count; it += gridDim.x) {
+    if (it + int(gridDim.x) >= items * mem.count) grid_dep_trigger();  // last item of this CTA
+    const int mi = it / items, row = (it - mi * items) * PER + pr;
+    const Member mb = member_at(mem, mi);
+    if (mi != cur) {
+      const int* ce = ws_ptr<int>(mb, off.cexp);
+      const int* be = ws_ptr<int>(mb, off.bexp);
+      emax = max(fx_cta_max(ce, N + 1, red + 4 * W), fx_cta_max(be, Q + 1, red + 4 * W));
+      for (int q = threadIdx.x; q <= N; q += GG::T) sh_a[q] = (unsigned char)fx_align<4>(emax, ce[q]);
+      for (int q = threadIdx.x; q <= Q; q += GG::T) sh_b[q] = (unsigned char)fx_align<4>(emax, be[q]);
+      cur = mi;
+      __syncthreads();
+    }
+    const bool valid = row < ny;
+    const fxc* __restrict__ Ar = ws_ptr<fxc>(mb, off.A) + TL::at(valid ? row : 0, 0, ldqA);
+    const fxc* __restrict__ Br = ws_ptr<fxc>(mb, off.B) + TL::at(valid ? row : 0, 0, ldqB);
+    const fxc z = fx_mk(0, 0);
+    fxc v[16];  // X in the first, R in the second half
+    unsigned mag = 0;
+    fxc yn = z;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = valid ? Ar[(tp + P * i) * TL::TR] : z;
+    if (valid && tp == 0) yn = Ar[N * TL::TR];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int q = tp + P * i;
+      const fxc y = fx_sra(v[i], sh_a[q]);
+      const fxc s = (valid && q <= Q) ? fx_sra(Br[q * TL::TR], sh_b[q]) : z;
+      v[i] = fx_mk(y.x - s.y, y.y + s.x);
+      v[i + 8] = fx_mk(y.x + s.y, y.y - s.x);
+    }
+    mag = fx_mag(v);
+    if (tp == 0) {  // conj X(N) (Q < N: no band value) in the place of conj R(N - 0)
+      yn = fx_sra(yn, sh_a[N]);
+      yn.y = -yn.y;
+      mag = fx_mag(mag, yn);
+    }
+    mag = fx_post<P>(mag, red + 2 * W);
+    __syncthreads();  // (and the previous item's reads of the buffers are done)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int q = tp + P * i;
+      buf_e[pad16(q)] = v[i];
+      if (q != 0) buf_o[pad16(N - q)] = v[i + 8];  // R(N - q) at q
+    }
+    if (tp == 0) buf_o[0] = yn;
+    __syncthreads();
+    const int s0 = fx_norm_shift<60>(fx_read<P>(mag, red + 2 * W));
+    if (h == 0) {
+#pragma unroll
+      for (int m = 0; m < 16; ++m) {
+        const fxc x = buf_e[pad16(t + G * m)], r = buf_o[pad16(t + G * m)];
+        v[m] = fx_shr<4>(fx_shl(fx_mk(x.x + r.x, x.y - r.y), s0));
+      }
+    } else {
+#pragma unroll
+      for (int m = 0; m < 16; ++m) {
+        const fxc x = buf_e[pad16(t + G * m)], r = buf_o[pad16(t + G * m)];
+        v[m] = fx_mul(fx_shl(fx_mk(x.x - r.x, x.y + r.y), s0), fx_conj(fx_wm(ax.wm, t, m, G)));
+      }
+    }
+    const int ex = emax + 4 - s0 + 4 + kd + 1 + lscale + fx_ifft<LOG2N>(v, buf, t, stw, red);
+    if (valid) {
+      double* __restrict__ phi = mb.phi + size_t(row) * N + h;
+      const bool bad = emax >= kFxBad;
+      const i64 half = i64(1) << kd;
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        const int n = 2 * (t + G * m);
+        // Re T 2^-(kd + 1) + Im T d_x/2^kd /2
+        const i64 f = ((v[m].x + half) >> (kd + 1)) + fx_mulr(v[m].y, fx_ldr(ax.dec + n + h));
+        phi[n] = bad ? __longlong_as_double(0x7FF8000000000000ll) : fx_to_f64(f, ex);
+      }
+    }
+  }
+}
+
+#undef DSNU_FX_SETUP
+
+}  // namespace dsnu

@@ -99,24 +99,28 @@ cudaError_t prepare_std_cols(PlanGeom& g) {
 }
 
 template <typename R>
-cudaError_t prepare_kernels(PlanGeom& g) {
+cudaError_t prepare_standard(PlanGeom& g) {
   cudaError_t e = cudaSuccess;
-  if (g.standard) {
 #define DSNU_PREP_SR(L2) e = prepare_std_rows<R, L2>(g)
 #define DSNU_PREP_SC(L2) e = prepare_std_cols<R, L2>(g)
-    switch (g.log2nx) {
-      DSNU_LOG2_CASES(DSNU_PREP_SR)
-      default: return cudaErrorInvalidValue;
-    }
-    if (e != cudaSuccess) return e;
-    switch (g.log2ny) {
-      DSNU_LOG2_CASES(DSNU_PREP_SC)
-      default: return cudaErrorInvalidValue;
-    }
+  switch (g.log2nx) {
+    DSNU_LOG2_CASES(DSNU_PREP_SR)
+    default: return cudaErrorInvalidValue;
+  }
+  if (e != cudaSuccess) return e;
+  switch (g.log2ny) {
+    DSNU_LOG2_CASES(DSNU_PREP_SC)
+    default: return cudaErrorInvalidValue;
+  }
 #undef DSNU_PREP_SR
 #undef DSNU_PREP_SC
-    return e;
-  }
+  return e;
+}
+
+template <typename R>
+cudaError_t prepare_kernels(PlanGeom& g) {
+  if (g.standard) return prepare_standard<R>(g);
+  cudaError_t e = cudaSuccess;
 #define DSNU_PREP_R(L2) e = prepare_rows<R, L2>(g)
 #define DSNU_PREP_C(L2) e = prepare_cols<R, L2>(g)
   switch (g.log2nx) {
@@ -213,7 +217,6 @@ dsnu_status run_pipeline(const PlanGeom& g, const PlanTables& t, const WsLayout&
                        static_cast<const cpx<R>*>(t.twm_hi_y), g.log2lo_y, static_cast<const R*>(t.decon_y),
                        nullptr};
   const MultTabs<R> mt{static_cast<const R*>(t.m_wx2), static_cast<const R*>(t.m_gx),
-                       g.n_gy, R(1.0 / (g.sigma * g.sigma)),
                        R(-g.dky2 / (g.sigma * g.sigma) * 1.4426950408889634), R(g.dky2), g.ny, g.sharp,
                        R(g.cut_radius * g.cut_radius), g.m_generic, g.m_alpha, R(g.m_a0), R(g.m_ac),
                        R(2.0 * g.m_as), R(std::sqrt(g.dky2)), static_cast<const R*>(t.m_kx),

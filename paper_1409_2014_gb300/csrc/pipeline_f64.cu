@@ -1,14 +1,141 @@
-// FP64 (DSNU_FP64) instantiation of the pipeline.
+// FP64 (DSNU_FP64) plans: the FFT passes in 64-bit block fixed point
+// (kernels_fx.cuh), interpolation, weighting and spreading in FP64.
+#include "kernels_fx.cuh"
 #include "pipeline.cuh"
 
 namespace dsnu {
-dsnu_status run_pipeline_f64(const PlanGeom& g, const PlanTables& t, const WsLayout& L,
-                             const Members& mem, cudaStream_t st, int cj, cudaEvent_t* ev, const Overlap* ov) {
-  return run_pipeline<double>(g, t, L, mem, st, cj, ev, ov);
+
+namespace {
+
+template <int L2>
+cudaError_t prepare_fx_rows(PlanGeom& g) {
+  using GG = FxGeo<L2>;
+  const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e;
+  g.smem_rowi = GG::smem_row_inv(g.Q);
+  if ((e = cudaFuncSetAttribute(k_fx_row_fwd<L2>, A, int(GG::smem)))) return e;
+  if ((e = cudaFuncSetAttribute(k_fx_row_inv<L2>, A, int(GG::smem_row_inv(GG::N))))) return e;
+  if ((e = resident_ctas(k_fx_row_fwd<L2>, GG::T, GG::smem, &g.cap_rowf))) return e;
+  return resident_ctas(k_fx_row_inv<L2>, GG::T, g.smem_rowi, &g.cap_rowi);
 }
-cudaError_t prepare_kernels_f64(PlanGeom& g) { return prepare_kernels<double>(g); }
+
+template <int L2>
+cudaError_t prepare_fx_cols(PlanGeom& g) {
+  using GG = FxGeo<L2>;
+  const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(k_fx_col_main<L2, false>, A, int(GG::smem)))) return e;
+  if ((e = cudaFuncSetAttribute(k_fx_col_main<L2, true>, A, int(GG::smem)))) return e;
+  if ((e = cudaFuncSetAttribute(k_fx_band_fwd<L2>, A, int(GG::smem)))) return e;
+  if ((e = cudaFuncSetAttribute(k_fx_band_inv<L2>, A, int(GG::smem)))) return e;
+  if ((e = g.m1_full ? resident_ctas(k_fx_col_main<L2, true>, GG::T, GG::smem, &g.cap_col)
+                     : resident_ctas(k_fx_col_main<L2, false>, GG::T, GG::smem, &g.cap_col)))
+    return e;
+  if ((e = resident_ctas(k_fx_band_fwd<L2>, GG::T, GG::smem, &g.cap_bandf))) return e;
+  return resident_ctas(k_fx_band_inv<L2>, GG::T, GG::smem, &g.cap_bandi);
+}
+
+}  // namespace
+
+cudaError_t prepare_kernels_f64(PlanGeom& g) {
+  if (g.standard) return prepare_standard<double>(g);
+  cudaError_t e = cudaSuccess;
+#define DSNU_PREP_R(L2) e = prepare_fx_rows<L2>(g)
+#define DSNU_PREP_C(L2) e = prepare_fx_cols<L2>(g)
+  switch (g.log2nx) {
+    DSNU_LOG2_CASES(DSNU_PREP_R)
+    default: return cudaErrorInvalidValue;
+  }
+  if (e != cudaSuccess) return e;
+  switch (g.log2ny) {
+    DSNU_LOG2_CASES(DSNU_PREP_C)
+    default: return cudaErrorInvalidValue;
+  }
+#undef DSNU_PREP_R
+#undef DSNU_PREP_C
+  return e;
+}
+
+dsnu_status run_pipeline_f64(const PlanGeom& g, const PlanTables& t, const WsLayout& L, const Members& mem,
+                             cudaStream_t st, int cj, cudaEvent_t* ev, const Overlap* ov) {
+  if (g.standard) return run_standard<double>(g, t, L, mem, st, cj, ev);
+  (void)ov;
+  // the conjugated pipeline of a real input is the conjugate of this one: the
+  // same result (kernels_fx.cuh), so `cj` selects nothing
+  const WsOff off{L.off_A, L.off_B, L.off_Bband, L.off_Sband, L.off_c, L.off_partial, L.off_sched};
+  const FxOff fo{L.off_A, L.off_B, L.off_Bband, L.off_Sband, L.off_rexp, L.off_rexpb, L.off_cexp, L.off_bexp};
+  const FxAxis ax{static_cast<const fxw*>(t.fx_stw_x), static_cast<const fxw*>(t.fx_wm_x),
+                  static_cast<const fxr*>(t.fx_dec_x)};
+  const FxAxis ay{static_cast<const fxw*>(t.fx_stw_y), static_cast<const fxw*>(t.fx_wm_y),
+                  static_cast<const fxr*>(t.fx_dec_y)};
+  const FxMult mt{static_cast<const fxr*>(t.m1tab), t.fx_mexp, g.m1_ld};
+  const bool pdl = g.pdl != 0;
+  const long nm = mem.count;
+  const double* wts = static_cast<const double*>(t.node_w);
+  auto grid = [&](long n, int per, int cap) { return dim3(persistent_grid(nm * ((n + per - 1) / per), cap)); };
+#define DSNU_ROWF(L2)                                                                                       \
+  launch_k(pdl, k_fx_row_fwd<L2>, grid(g.ny, FxGeo<L2>::PER, g.cap_rowf), dim3(FxGeo<L2>::T), FxGeo<L2>::smem, st, \
+           mem, fo, L.ldqA, L.ldqB, g.Q, g.ny, ax, g.kdx)
+#define DSNU_BANDF(L2)                                                                                      \
+  launch_k(pdl, k_fx_band_fwd<L2>, grid(g.Q + 1, FxGeo<L2>::PER, g.cap_bandf), dim3(FxGeo<L2>::T), FxGeo<L2>::smem, \
+           st, mem, fo, L.ldqB, g.Q + 1, L.ldq, g.Q, ay, g.kdy)
+#define DSNU_BANDI(L2)                                                                                      \
+  launch_k(pdl, k_fx_band_inv<L2>, grid(g.Q + 1, FxGeo<L2>::PER, g.cap_bandi), dim3(FxGeo<L2>::T), FxGeo<L2>::smem, \
+           st, mem, fo, L.ldq, g.Q, g.Q + 1, L.ldqB, ay, g.kdy)
+#define DSNU_COLM(L2)                                                                                       \
+  if (g.m1_full)                                                                                            \
+    launch_k(pdl, k_fx_col_main<L2, true>, grid(g.nx + 1, FxGeo<L2>::PER, g.cap_col), dim3(FxGeo<L2>::T),   \
+             FxGeo<L2>::smem, st, mem, fo, L.ldqA, g.nx + 1, ay, mt);                                       \
+  else                                                                                                      \
+    launch_k(pdl, k_fx_col_main<L2, false>, grid(g.nx + 1, FxGeo<L2>::PER, g.cap_col), dim3(FxGeo<L2>::T),  \
+             FxGeo<L2>::smem, st, mem, fo, L.ldqA, g.nx + 1, ay, mt)
+#define DSNU_ROWI(L2)                                                                                       \
+  launch_k(pdl, k_fx_row_inv<L2>, grid(g.ny, FxGeo<L2>::PER, g.cap_rowi), dim3(FxGeo<L2>::T), g.smem_rowi, st, \
+           mem, fo, L.ldqA, L.ldqB, g.Q, g.ny, ax, g.kdx, -(ilogb(double(g.mx)) + ilogb(double(g.my))))
+#define DSNU_STEP(SIZE, CALL)              \
+  switch (SIZE) {                          \
+    DSNU_LOG2_CASES(CALL)                  \
+    default: return DSNU_EUNSUPPORTED;     \
+  }
+#define DSNU_MARK(I) \
+  if (ev) cudaEventRecord(ev[I], st)
+  DSNU_MARK(0);
+  DSNU_STEP(g.log2nx, DSNU_ROWF)
+  DSNU_MARK(1);
+  DSNU_STEP(g.log2ny, DSNU_BANDF)
+  DSNU_MARK(2);
+  launch_k(pdl, k_interp_tile<double>, dim3(g.n_itiles, mem.count), dim3(256),
+           interp_tile_smem(g.w, sizeof(cpx<double>)), st, mem, off, L.ldq, g.Q, t.node_q0, wts, t.node_D, t.itile_ptr,
+           t.itile_org, t.itile_nodes, g.w, 0);
+  DSNU_MARK(3);
+  launch_spread<double>(g.spread_cfg, mem, off, t, g, L.ldq, 0, st, 0, pdl);
+  DSNU_MARK(4);
+  launch_spread<double>(g.spread_cfg, mem, off, t, g, L.ldq, 0, st, 1, pdl);
+  DSNU_MARK(5);
+  DSNU_STEP(g.log2ny, DSNU_BANDI)
+  DSNU_MARK(6);
+  DSNU_STEP(g.log2ny, DSNU_COLM)
+  DSNU_MARK(7);
+  DSNU_STEP(g.log2nx, DSNU_ROWI)
+  DSNU_MARK(8);
+#undef DSNU_ROWF
+#undef DSNU_COLM
+#undef DSNU_BANDF
+#undef DSNU_BANDI
+#undef DSNU_ROWI
+#undef DSNU_STEP
+#undef DSNU_MARK
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    set_last_error(std::string("kernel launch failed: ") + cudaGetErrorString(e));
+    return DSNU_ECUDA;
+  }
+  return DSNU_OK;
+}
+
 cudaError_t time_spread_f64(const PlanGeom& g, const PlanTables& t, const WsLayout& L, void* ws, int reps,
                             float* ms) {
   return time_spread<double>(g, t, L, ws, reps, ms);
 }
+
 }  // namespace dsnu

@@ -29,6 +29,7 @@
 
 #include "internal.h"
 #include "kernels.cuh"
+#include "kernels_fx.cuh"
 
 namespace dsnu {
 
@@ -197,13 +198,35 @@ template <typename R>
 struct HostTables {
   // complex tables interleaved (re, im)
   std::vector<R> stw_x, stwc_x, twm_lo_x, twm_hi_x, decon_x, stw_y, twm_lo_y, twm_hi_y, decon_y;
-  std::vector<R> m_wx2, m_gx, m_gy, m_kx;
+  std::vector<R> m_wx2, m_gx, m_kx;
   std::vector<int2> node_q0;
   std::vector<int> itile_ptr, itile_nodes;
   std::vector<int2> itile_org;
   std::vector<R> node_w;
   std::vector<double> node_D;
+  // FP64 plans: fixed-point tables (fx.cuh), four or two ints per entry
+  std::vector<int> fx_stw_x, fx_wm_x, fx_dec_x, fx_stw_y, fx_wm_y, fx_dec_y, fx_mexp;
 };
+
+// A constant |v| <= 1 as v 2^bits = h + l 2^-32, h and l signed 32-bit (|l| < 2^31).
+static void fx_put(std::vector<int>& out, double v, int bits) {
+  const double s = std::ldexp(v, bits), h = std::nearbyint(s);
+  const double l = std::nearbyint((s - h) * 4294967296.0);
+  out.push_back(int(h));
+  out.push_back(int(std::min(std::max(l, -2147483647.0), 2147483647.0)));
+}
+static std::vector<int> fx_table(const std::vector<double>& v, int bits) {
+  std::vector<int> out;
+  out.reserve(2 * v.size());
+  for (double x : v) fx_put(out, x, bits);
+  return out;
+}
+// The deconvolution factors d / 2^kd with 2^kd > max d; returns kd.
+static int fx_decon(const std::vector<double>& d, std::vector<int>& out) {
+  const int kd = int(std::floor(std::log2(*std::max_element(d.begin(), d.end()) * (1.0 + 1e-6)))) + 1;
+  for (double x : d) fx_put(out, std::ldexp(x, -kd), kFxDeconBits);
+  return kd;
+}
 
 // Spreading tables for one tile configuration (see k_spread).
 template <typename R>
@@ -468,24 +491,59 @@ static dsnu_status setup_spread(dsnu_plan_s* P, const std::vector<int2>& q0, con
 // The column multiplier of I1 (eq. SubInt1) on the padded grid,
 //   m1(q_x, a) = -(q_x dk_x)^2 / s * (1 - p),  s = (q_x dk_x)^2 + (a dk_y)^2,
 // with p = e^{-s/sigma^2} (Gaussian partition) or the indicator of s <= P^2
-// (sharp), m1 = 0 at s = 0; computed in FP64 and stored in the plan's
-// precision (one rounding for FP32).  Row q_x holds a = 2 j at j <= ny/2 and
+// (sharp), m1 = 0 at s = 0; computed in FP64 with one rounding to FP32 (mixed
+// plans).  Row q_x holds a = 2 j at j <= ny/2 and
 // a = 2 j' + 1 at ny/2 + 1 + j', then zeros up to its ldm = ny + 4 entries.
-template <typename T>
-__global__ void k_fill_m1(T* tab, int nx1, int ny, int ldm, double dkx, double dky, double inv_sigma2, int sharp,
+__global__ void k_fill_m1(float* tab, int nx1, int ny, int ldm, double dkx, double dky, double inv_sigma2, int sharp,
                           double cut2) {
   const long long n = (long long)nx1 * ldm;
   const int mh = ny / 2 + 1;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const int col = int(i / ldm), j = int(i - (long long)col * ldm);
-    T v = T(0);
+    float v = 0.f;
     if (j <= ny) {
       const int a = (j < mh) ? 2 * j : 2 * (j - mh) + 1;
       const double wx = col * dkx, wy = a * dky;
       const double wx2 = wx * wx, s = wx2 + wy * wy;
       if (s > 0.0) {
         const double part = sharp ? (s > cut2 ? 1.0 : 0.0) : -expm1(-s * inv_sigma2);
-        v = T(-wx2 / s * part);
+        v = float(-wx2 / s * part);
+      }
+    }
+    tab[i] = v;
+  }
+}
+
+// The multiplier table of the FP64 plans (FxMult): m1 2^-mexp[q_x] in
+// fixed-point halves, for any multiplier of the family.  Row q_x holds the
+// even frequencies first: |qbar| = 2 j at j, 2 j' + 1 at ny/2 + 1 + j' (full:
+// the natural frequency q = 2 j at j, 2 j' + 1 at ny + j').
+__global__ void k_fill_m1_fx(int2* tab, int nx, int ny, int ld, int full, double dkx, double dky, double inv_sigma2,
+                             int sharp, double cut2, int generic, int alpha, double a0, double ac, double as,
+                             const int* mexp) {
+  const long long n = (long long)(nx + 1) * ld;
+  const int mh = full ? ny : ny / 2 + 1, last = full ? 2 * ny : ny + 1;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const int col = int(i / ld), j = int(i - (long long)col * ld);
+    int2 v = make_int2(0, 0);
+    if (j < last) {
+      const int q = (j < mh) ? 2 * j : 2 * (j - mh) + 1;
+      const int qs = (q < ny) ? q : (q == ny ? 0 : q - 2 * ny);  // signed, 0 at the Nyquist row (sin 2theta term)
+      const int a = (q <= ny) ? q : 2 * ny - q;
+      const double wx = col * dkx, wy = a * dky;
+      const double wx2 = wx * wx, wy2 = wy * wy, s = wx2 + wy2;
+      if (s > 0.0) {
+        double m = -wx2 / s;
+        if (generic) {
+          const double kx = col < nx ? wx : 0.0;  // (and at the Nyquist column)
+          m = a0 + (ac * (wx2 - wy2) + 2.0 * as * kx * (qs * dky)) / s;
+          if (alpha == 1) m *= sqrt(s);
+          if (alpha == -1) m /= sqrt(s);
+        }
+        m *= sharp ? (s > cut2 ? 1.0 : 0.0) : -expm1(-s * inv_sigma2);
+        const long long w = __double2ll_rn(ldexp(m, kFxMultBits + 32 - (mexp ? mexp[col] : 0)));
+        v.y = int(w);
+        v.x = int((w - v.y) >> 32);
       }
     }
     tab[i] = v;
@@ -495,13 +553,18 @@ __global__ void k_fill_m1(T* tab, int nx1, int ny, int ldm, double dkx, double d
 template <typename R>
 static dsnu_status build_m1_table(dsnu_plan_s* P, double dkx, double dky, cudaStream_t st) {
   const PlanGeom& g = P->geom;
-  const int ldm = g.ny + 4;
+  const int ldm = (sizeof(R) == 8) ? g.m1_ld : g.ny + 4;
   const size_t bytes = size_t(g.nx + 1) * ldm * sizeof(R);
   void* m = nullptr;
   cudaError_t e = cudaMalloc(&m, bytes);
   if (e != cudaSuccess) return fail(DSNU_ENOMEM, std::string("cudaMalloc(multiplier table): ") + cudaGetErrorString(e));
-  k_fill_m1<R><<<1024, 256, 0, st>>>(static_cast<R*>(m), g.nx + 1, g.ny, ldm, dkx, dky, 1.0 / (g.sigma * g.sigma),
-                                     g.sharp, g.cut_radius * g.cut_radius);
+  if constexpr (sizeof(R) == 8)
+    k_fill_m1_fx<<<1024, 256, 0, st>>>(static_cast<int2*>(m), g.nx, g.ny, ldm, g.m1_full, dkx, dky,
+                                       1.0 / (g.sigma * g.sigma), g.sharp, g.cut_radius * g.cut_radius, g.m_generic,
+                                       g.m_alpha, g.m_a0, g.m_ac, g.m_as, P->tab.fx_mexp);
+  else
+    k_fill_m1<<<1024, 256, 0, st>>>(static_cast<float*>(m), g.nx + 1, g.ny, ldm, dkx, dky, 1.0 / (g.sigma * g.sigma),
+                                       g.sharp, g.cut_radius * g.cut_radius);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
@@ -549,43 +612,53 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   const double ph0 = fh(0.0);
   HostTables<R> T;
   std::vector<double> tmp, tmp2;
-  fft_stage_twiddles(g.log2nx, tmp); T.stw_x = cast<R>(tmp);
-  fft_stage_twiddles(g.log2ny, tmp); T.stw_y = cast<R>(tmp);
-  fft_stage_twiddles_ct(g.log2nx, tmp); T.stwc_x = cast<R>(tmp);
-  if (int(T.stw_x.size()) != 2 * std::max(1, fft_stage_tw_elems(g.log2nx)) ||
-      int(T.stw_y.size()) != 2 * std::max(1, fft_stage_tw_elems(g.log2ny)) ||
-      int(T.stwc_x.size()) != 2 * std::max(1, fft_stage_tw_elems_ct(g.log2nx)))
-    return fail(DSNU_EINVAL, "internal: stage twiddle table size mismatch");
-  g.log2lo_x = half_angle_tables(nx, tmp, tmp2); T.twm_lo_x = cast<R>(tmp); T.twm_hi_x = cast<R>(tmp2);
-  g.log2lo_y = half_angle_tables(ny, tmp, tmp2); T.twm_lo_y = cast<R>(tmp); T.twm_hi_y = cast<R>(tmp2);
-  T.decon_x.resize(nx);
-  for (int n = 0; n < nx; ++n) T.decon_x[n] = R(ph0 / fh(2.0 * M_PI * (n - nx / 2) / Mx));
-  T.decon_y.resize(ny);
-  for (int n = 0; n < ny; ++n) T.decon_y[n] = R(ph0 / fh(2.0 * M_PI * (n - ny / 2) / My));
-
-  // multiplier axis tables: per column q_x; along y only the partition factor
-  // 1 - exp(-(a dk_y)^2/sigma^2) up to the first |qbar_y| = a where it is 1 in
-  // working precision ((a dk_y)^2 itself is formed in the kernel)
-  T.m_wx2.resize(nx + 1);
-  T.m_gx.resize(nx + 1);
-  T.m_kx.resize(nx + 1);
-  for (int q = 0; q <= nx; ++q) {
-    const double a = q * dkx;
-    T.m_wx2[q] = R(a * a);
-    T.m_gx[q] = R(-std::expm1(-(a * a) / (sigma * sigma)));
-    T.m_kx[q] = R(q < nx ? a : 0.0);  // Nyquist column: +-K averaged, the sin 2theta term vanishes
-  }
-  g.dky2 = dky * dky;
-  T.m_gy.clear();
-  if (!g.sharp) {
-    for (int a = 0; a <= ny; ++a) {
-      const double v = -std::expm1(-(a * dky) * (a * dky) / (sigma * sigma));
-      if (R(v) == R(1)) break;
-      T.m_gy.push_back(R(v));
+  std::vector<double> dcx(nx), dcy(ny);
+  for (int n = 0; n < nx; ++n) dcx[n] = ph0 / fh(2.0 * M_PI * (n - nx / 2) / Mx);
+  for (int n = 0; n < ny; ++n) dcy[n] = ph0 / fh(2.0 * M_PI * (n - ny / 2) / My);
+  if constexpr (sizeof(R) == 8) {
+    fft_stage_twiddles(g.log2nx, tmp); T.fx_stw_x = fx_table(tmp, kFxTwBits);
+    fft_stage_twiddles(g.log2ny, tmp); T.fx_stw_y = fx_table(tmp, kFxTwBits);
+    twiddles(nx / 2, Mx, tmp); T.fx_wm_x = fx_table(tmp, kFxTwBits);
+    twiddles(ny / 2, My, tmp); T.fx_wm_y = fx_table(tmp, kFxTwBits);
+    g.kdx = fx_decon(dcx, T.fx_dec_x);
+    g.kdy = fx_decon(dcy, T.fx_dec_y);
+    g.m1_full = (g.m_generic && g.m_as != 0.0) ? 1 : 0;
+    g.m1_ld = g.m1_full ? My : ny + 4;
+    if (g.m_generic) {
+      // |m| <= (|a0| + |a_cos| + |a_sin|) |k|^alpha on a column
+      const double amp = std::fabs(g.m_a0) + std::fabs(g.m_ac) + std::fabs(g.m_as), kmax = ny * dky;
+      for (int q = 0; q <= nx; ++q) {
+        const double k1 = q * dkx;
+        const double b = (g.m_alpha == 1) ? amp * std::sqrt(k1 * k1 + kmax * kmax)
+                         : (g.m_alpha == -1) ? amp / (q == 0 ? dky : k1) : amp;
+        T.fx_mexp.push_back(b > 0.0 ? std::min(std::max(std::ilogb(b) + 2, -1200), 1100) : 0);
+      }
+    }
+  } else {
+    fft_stage_twiddles(g.log2nx, tmp); T.stw_x = cast<R>(tmp);
+    fft_stage_twiddles(g.log2ny, tmp); T.stw_y = cast<R>(tmp);
+    fft_stage_twiddles_ct(g.log2nx, tmp); T.stwc_x = cast<R>(tmp);
+    if (int(T.stw_x.size()) != 2 * std::max(1, fft_stage_tw_elems(g.log2nx)) ||
+        int(T.stw_y.size()) != 2 * std::max(1, fft_stage_tw_elems(g.log2ny)) ||
+        int(T.stwc_x.size()) != 2 * std::max(1, fft_stage_tw_elems_ct(g.log2nx)))
+      return fail(DSNU_EINVAL, "internal: stage twiddle table size mismatch");
+    g.log2lo_x = half_angle_tables(nx, tmp, tmp2); T.twm_lo_x = cast<R>(tmp); T.twm_hi_x = cast<R>(tmp2);
+    g.log2lo_y = half_angle_tables(ny, tmp, tmp2); T.twm_lo_y = cast<R>(tmp); T.twm_hi_y = cast<R>(tmp2);
+    T.decon_x = cast<R>(dcx);
+    T.decon_y = cast<R>(dcy);
+    // multiplier axis tables: per column q_x
+    T.m_wx2.resize(nx + 1);
+    T.m_gx.resize(nx + 1);
+    T.m_kx.resize(nx + 1);
+    for (int q = 0; q <= nx; ++q) {
+      const double a = q * dkx;
+      T.m_wx2[q] = R(a * a);
+      T.m_gx[q] = R(-std::expm1(-(a * a) / (sigma * sigma)));
+      T.m_kx[q] = R(q < nx ? a : 0.0);  // Nyquist column: +-K averaged, the sin 2theta term vanishes
     }
   }
-  g.n_gy = int(T.m_gy.size());
-  if (T.m_gy.empty()) T.m_gy.push_back(R(0));
+
+  g.dky2 = dky * dky;
 
   // per-node stencils
   T.node_q0.resize(nn);
@@ -647,8 +720,11 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   const size_t o_dx = b.add(T.decon_x), o_scx = b.add(T.stwc_x);
   const size_t o_sty = b.add(T.stw_y), o_tly = b.add(T.twm_lo_y), o_thy = b.add(T.twm_hi_y);
   const size_t o_dy = b.add(T.decon_y);
-  const size_t o_wx2 = b.add(T.m_wx2), o_gx = b.add(T.m_gx), o_gy = b.add(T.m_gy), o_kx = b.add(T.m_kx);
+  const size_t o_wx2 = b.add(T.m_wx2), o_gx = b.add(T.m_gx), o_kx = b.add(T.m_kx);
   const size_t o_q0 = b.add(T.node_q0), o_w = b.add(T.node_w), o_D = b.add(T.node_D);
+  const size_t o_fsx = b.add(T.fx_stw_x), o_fwx = b.add(T.fx_wm_x), o_fdx = b.add(T.fx_dec_x);
+  const size_t o_fsy = b.add(T.fx_stw_y), o_fwy = b.add(T.fx_wm_y), o_fdy = b.add(T.fx_dec_y);
+  const size_t o_fme = b.add(T.fx_mexp);
   const size_t o_itp = b.add(T.itile_ptr), o_ito = b.add(T.itile_org), o_itn = b.add(T.itile_nodes);
   const int zero = 0;
   const size_t o_st = b.add(&zero, sizeof(int));
@@ -666,7 +742,7 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   t.stw_x = d + o_stx; t.twm_lo_x = d + o_tlx; t.twm_hi_x = d + o_thx; t.decon_x = d + o_dx;
   t.stwc_x = d + o_scx;
   t.stw_y = d + o_sty; t.twm_lo_y = d + o_tly; t.twm_hi_y = d + o_thy; t.decon_y = d + o_dy;
-  t.m_wx2 = d + o_wx2; t.m_gx = d + o_gx; t.m_gy = d + o_gy; t.m_kx = d + o_kx;
+  t.m_wx2 = d + o_wx2; t.m_gx = d + o_gx; t.m_kx = d + o_kx;
   t.node_q0 = reinterpret_cast<int2*>(d + o_q0);
   t.itile_ptr = reinterpret_cast<int*>(d + o_itp);
   t.itile_org = reinterpret_cast<int2*>(d + o_ito);
@@ -674,9 +750,12 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   t.node_w = d + o_w;
   t.node_D = reinterpret_cast<double*>(d + o_D);
   t.status = reinterpret_cast<int*>(d + o_st);
+  t.fx_stw_x = d + o_fsx; t.fx_wm_x = d + o_fwx; t.fx_dec_x = d + o_fdx;
+  t.fx_stw_y = d + o_fsy; t.fx_wm_y = d + o_fwy; t.fx_dec_y = d + o_fdy;
+  t.fx_mexp = (sizeof(R) == 8 && g.m_generic) ? reinterpret_cast<int*>(d + o_fme) : nullptr;
   P->table_block = dev;
   P->table_bytes = b.bytes.size();
-  if (!g.m_generic) {
+  if (sizeof(R) == 8 || !g.m_generic) {
     const dsnu_status sm = build_m1_table<R>(P, dkx, dky, st);
     if (sm != DSNU_OK) return sm;
   }
@@ -756,6 +835,12 @@ static void layout_workspace(dsnu_plan_s* P) {  // defined after the autotuner, 
   L.off_c = take(size_t(g.n_nodes) * csz);
   L.off_partial = take(size_t(std::max(g.n_items, 1)) * g.spread_tile * g.spread_tile * csz);
   L.off_sched = take(sizeof(int));
+  if (g.precision == DSNU_FP64) {
+    L.off_rexp = take(size_t(g.ny) * sizeof(int));
+    L.off_rexpb = take(size_t(g.ny) * sizeof(int));
+    L.off_cexp = take(size_t(g.nx + 1) * sizeof(int));
+    L.off_bexp = take(size_t(g.Q + 1) * sizeof(int));
+  }
   L.total = off;
 }
 
