@@ -12,6 +12,7 @@
 // plan, complex128 for DSNU_FP64.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -19,7 +20,7 @@
 #include <vector>
 
 #include "internal.h"
-#include "kernels.cuh"
+#include "kernels_fx.cuh"
 
 namespace dsnu {
 
@@ -107,6 +108,135 @@ k_c2c_cols_phase(cpx<R>* __restrict__ u, int nx, const cpx<R>* __restrict__ stw_
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same two passes for complex128 fields, in 64-bit block fixed point
+// (fx.cuh): each row and each pair of columns is scaled to its own largest
+// component on loading and written back in FP64, so the passes keep no state
+// between them (the field is the caller's, and several fields may be under way).
+// An infinity or a NaN makes its whole row, then every column, NaN.
+
+// u[row][t + G m] of group threads t: the values' bits, and their largest
+// exponent (fx_top).
+template <int G, int P>
+__device__ __forceinline__ unsigned fx_load(fxc (&v)[16], const double2* __restrict__ u, size_t stride, bool valid,
+                                            unsigned* red) {
+  unsigned mx = 0;
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const double2 a = valid ? u[stride * m] : make_double2(0.0, 0.0);
+    mx = fx_top(fx_top(mx, a.x), a.y);
+    v[m] = fx_mk(__double_as_longlong(a.x), __double_as_longlong(a.y));
+  }
+  mx = fx_post<P, true>(mx, red);
+  __syncthreads();
+  mx = fx_read<P, true>(mx, red);
+  const int efm = fx_efm(mx);
+#pragma unroll
+  for (int m = 0; m < 16; ++m)
+    v[m] = fx_shr<5>(fx_mk(fx_from_f64(__longlong_as_double(v[m].x), efm), fx_from_f64(__longlong_as_double(v[m].y), efm)));
+  return mx;
+}
+__device__ __forceinline__ double2 fx_store(fxc v, int ex, unsigned mx) {
+  const double nan = __longlong_as_double(0x7FF8000000000000ll);
+  return mx >= kFxInf ? make_double2(nan, nan) : make_double2(fx_to_f64(v.x, ex), fx_to_f64(v.y, ex));
+}
+
+template <int LOG2N>
+__global__ void __launch_bounds__(FxOne<LOG2N>::T, FxOne<LOG2N>::MINB)
+k_fx_c2c_rows(double2* __restrict__ u, int ny, const fxw* __restrict__ stw_g, int inv) {
+  using GG = FxOne<LOG2N>;
+  constexpr int N = GG::N, G = GG::G, PER = GG::PER, W = GG::W;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  fxw* stw = reinterpret_cast<fxw*>(smem_raw);
+  fxc* sm = reinterpret_cast<fxc*>(stw + GG::STW);
+  unsigned* red = reinterpret_cast<unsigned*>(sm + PER * GG::FB);
+  fx_copy(stw, stw_g, fft_stage_tw_elems(LOG2N));
+  const int pr = threadIdx.x / G, t = threadIdx.x - pr * G;
+  fxc* buf = sm + pr * GG::FB;
+  __syncthreads();
+  const int items = (ny + PER - 1) / PER;
+#pragma unroll 1
+  for (int item = blockIdx.x; item < items; item += gridDim.x) {
+    const int row = item * PER + pr;
+    const bool valid = row < ny;
+    double2* ur = u + size_t(valid ? row : 0) * N + t;
+    fxc v[16];
+    const unsigned mx = fx_load<G, G>(v, ur, G, valid, red + 2 * W);
+    if (inv) {
+#pragma unroll
+      for (int m = 0; m < 16; ++m) v[m] = fx_swap(v[m]);
+    }
+    const int ex = fx_efm(mx) - kFxBias + 5 + fx_fft<LOG2N, G>(v, buf, t, stw, red);
+    if (valid) {
+#pragma unroll
+      for (int m = 0; m < 16; ++m) ur[G * m] = fx_store(inv ? fx_swap(v[m]) : v[m], ex, mx);
+    }
+  }
+}
+
+// Two adjacent columns per pair of groups, their threads interleaved (whole
+// 32-byte sectors), with one scale; buffers 4 elements apart modulo 8, so that
+// the two columns' lanes of a quarter warp fall in different banks.
+template <int LOG2N>
+struct FxCols : FxGeo<LOG2N> {
+  using B = FxGeo<LOG2N>;
+  static constexpr int FBS = B::FB + 4 + ((8 - (B::FB & 7)) & 7);
+  static constexpr size_t smem = size_t(B::STW + B::PER * 2 * FBS) * 16 + ((B::RED * 4 + 15) & ~15);
+  static_assert(smem <= 232448, "shared memory per CTA");
+};
+
+// px, py: the phases in fixed point (k_phase_tables_fx); the result carries
+// 2^lscale = 1/(nx ny).
+template <int LOG2N>
+__global__ void __launch_bounds__(FxCols<LOG2N>::T, FxCols<LOG2N>::MINB)
+k_fx_c2c_cols_phase(double2* __restrict__ u, int nx, const fxw* __restrict__ stw_g, const fxw* __restrict__ px,
+                    const fxw* __restrict__ py, int lscale, int adj) {
+  using GG = FxCols<LOG2N>;
+  constexpr int G = GG::G, P = GG::P, PER = GG::PER, W = GG::W;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  fxw* stw = reinterpret_cast<fxw*>(smem_raw);
+  fxc* sm = reinterpret_cast<fxc*>(stw + GG::STW);
+  unsigned* red = reinterpret_cast<unsigned*>(sm + PER * 2 * GG::FBS);
+  fx_copy(stw, stw_g, fft_stage_tw_elems(LOG2N));
+  const int pr = threadIdx.x / P, tp = threadIdx.x - pr * P;
+  const int h = tp & 1, t = tp >> 1;
+  fxc* buf = sm + (2 * pr + h) * GG::FBS;
+  __syncthreads();
+  const int items = (nx / 2 + PER - 1) / PER;
+#pragma unroll 1
+  for (int item = blockIdx.x; item < items; item += gridDim.x) {
+    const int col = 2 * (item * PER + pr) + h;
+    const bool valid = col < nx;
+    double2* uc = u + size_t(t) * nx + (valid ? col : h);
+    fxc v[16];
+    const unsigned mx = fx_load<G, P>(v, uc, size_t(G) * nx, valid, red + 2 * W);
+    int ex = fx_efm(mx) - kFxBias + 5 + lscale;
+#pragma unroll 1
+    for (int inv = 0;; ++inv) {  // forward, then inverse (one copy of the transform's code)
+      ex += fx_fft<LOG2N, P>(v, buf, t, stw, red);
+      if (inv) break;
+      const unsigned mag = fx_post<P>(fx_mag(v), red + 2 * W);
+      __syncthreads();
+      const int s = fx_norm_shift<62>(fx_read<P>(mag, red + 2 * W));
+      ex += 4 - 3 + 4 - s;
+      fxw wx = fx_ldw(px + (valid ? col : 0));
+      if (adj) wx = fx_conj(wx);
+#pragma unroll
+      for (int m = 0; m < 16; ++m) {
+        fxw wy = fx_ldw(py + t + G * m);
+        if (adj) wy = fx_conj(wy);
+        // /16 by each phase (magnitudes < 2^62.5), 2^3 between them; components
+        // exchanged for the inverse transform
+        v[m] = fx_swap(fx_mul(fx_shl(fx_mul(fx_shl(v[m], s), wy), 3), wx));
+      }
+    }
+    if (valid) {
+#pragma unroll
+      for (int m = 0; m < 16; ++m) uc[size_t(G) * m * nx] = fx_store(fx_swap(v[m]), ex, mx);
+    }
+  }
+}
+
 // rho = |u|^2 (FP64 out).
 template <typename R>
 __global__ void k_abs2(const cpx<R>* __restrict__ u, double* __restrict__ rho, size_t n) {
@@ -187,8 +317,8 @@ __global__ void k_nonlinear_vjp_finish(const cpx<R>* __restrict__ u, const doubl
 
 // Linear-flow phase tables in FFT order: px[q] = e^{-i tau k_x^2} and
 // py[q] = e^{+i tau alpha k_y^2}, k = qs dk with qs the signed index.  The
-// angles and their sine/cosine are formed in FP64 and rounded to the plan's
-// precision; launched on the caller's stream, so a change of step size needs
+// angles and their sine/cosine are formed in FP64 and rounded to FP32 (or put
+// in fixed point, below); launched on the caller's stream, so a change of step size needs
 // no host round trip.
 template <typename R>
 __global__ void k_phase_tables(cpx<R>* __restrict__ px, cpx<R>* __restrict__ py, int nx, int ny, double dkx,
@@ -205,6 +335,34 @@ __global__ void k_phase_tables(cpx<R>* __restrict__ px, cpx<R>* __restrict__ py,
     double s, c;
     sincos(tau * alpha * k * k, &s, &c);
     py[i] = mk<R>(R(c), R(s));
+  }
+}
+
+// The same in fixed point (fxw, 2^kFxTwBits), for complex128 plans.
+__device__ __forceinline__ fxw fx_unit(double c, double s) {
+  auto half = [](double v, int& h, int& l) {
+    const double x = v * double(1 << kFxTwBits), r = rint(x);
+    h = int(r);
+    l = int(fmax(fmin(rint((x - r) * 4294967296.0), 2147483647.0), -2147483647.0));
+  };
+  fxw w;
+  half(c, w.rh, w.rl);
+  half(s, w.ih, w.il);
+  return w;
+}
+__global__ void k_phase_tables_fx(fxw* __restrict__ px, fxw* __restrict__ py, int nx, int ny, double dkx, double dky,
+                                  double tau, double alpha) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  double s, c;
+  if (i < nx) {
+    const double k = double(i < nx / 2 ? i : i - nx) * dkx;
+    sincos(-tau * k * k, &s, &c);
+    px[i] = fx_unit(c, s);
+  }
+  if (i < ny) {
+    const double k = double(i < ny / 2 ? i : i - ny) * dky;
+    sincos(tau * alpha * k * k, &s, &c);
+    py[i] = fx_unit(c, s);
   }
 }
 
@@ -249,14 +407,14 @@ void stage_twiddles(int log2n, std::vector<double>& out) {
   if (out.empty()) out.assign(2, 0.0);
 }
 
-template <typename R>
-void upload(void* dst, const std::vector<double>& v, cudaStream_t st, cudaError_t* e) {
+template <typename R, typename V>
+void upload(void* dst, const V& v, cudaStream_t st, cudaError_t* e) {
   std::vector<R> tmp(v.begin(), v.end());
   if (*e == cudaSuccess) *e = cudaMemcpyAsync(dst, tmp.data(), tmp.size() * sizeof(R), cudaMemcpyHostToDevice, st);
   if (*e == cudaSuccess) *e = cudaStreamSynchronize(st);
 }
 
-template <typename R, typename K>
+template <typename K>
 int grid_for(K kernel, int threads, size_t smem, int items) {
   int dev = 0, sms = 1, per = 1;
   cudaGetDevice(&dev);
@@ -278,19 +436,19 @@ int grid_for(K kernel, int threads, size_t smem, int items) {
   case 11: CALL(11); break;  \
   case 12: CALL(12); break;
 
-template <typename R>
-cudaError_t prepare(dsnu_ds_plan_s* P) {
+cudaError_t prepare_f32(dsnu_ds_plan_s* P) {
+  using R = float;
   cudaError_t e = cudaSuccess;
   const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
 #define DSNU_PR(L2)                                                                                 \
   e = cudaFuncSetAttribute(k_c2c_rows<R, L2>, A, int(GeoC2C<R, L2>::smem));                        \
   if (e == cudaSuccess)                                                                             \
-    P->grid_rows = grid_for<R>(k_c2c_rows<R, L2>, GeoC2C<R, L2>::T, GeoC2C<R, L2>::smem,            \
+    P->grid_rows = grid_for(k_c2c_rows<R, L2>, GeoC2C<R, L2>::T, GeoC2C<R, L2>::smem,            \
                                (P->prm.ny + GeoC2C<R, L2>::PER - 1) / GeoC2C<R, L2>::PER)
 #define DSNU_PC(L2)                                                                                 \
   e = cudaFuncSetAttribute(k_c2c_cols_phase<R, L2>, A, int(GeoC2C<R, L2>::smem));                  \
   if (e == cudaSuccess)                                                                             \
-    P->grid_cols = grid_for<R>(k_c2c_cols_phase<R, L2>, GeoC2C<R, L2>::T, GeoC2C<R, L2>::smem,      \
+    P->grid_cols = grid_for(k_c2c_cols_phase<R, L2>, GeoC2C<R, L2>::T, GeoC2C<R, L2>::smem,      \
                                (P->prm.nx + GeoC2C<R, L2>::PER - 1) / GeoC2C<R, L2>::PER)
   switch (P->log2nx) {
     DSNU_C2C_CASES(DSNU_PR)
@@ -306,8 +464,35 @@ cudaError_t prepare(dsnu_ds_plan_s* P) {
   return e;
 }
 
-template <typename R>
-dsnu_status linear(dsnu_ds_plan_s* P, void* uv, int adjoint, cudaStream_t st) {
+cudaError_t prepare_f64(dsnu_ds_plan_s* P) {
+  cudaError_t e = cudaSuccess;
+  const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+#define DSNU_PR(L2)                                                                                 \
+  e = cudaFuncSetAttribute(k_fx_c2c_rows<L2>, A, int(FxOne<L2>::smem));                             \
+  if (e == cudaSuccess)                                                                             \
+    P->grid_rows = grid_for(k_fx_c2c_rows<L2>, FxOne<L2>::T, FxOne<L2>::smem,                       \
+                            (P->prm.ny + FxOne<L2>::PER - 1) / FxOne<L2>::PER)
+#define DSNU_PC(L2)                                                                                 \
+  e = cudaFuncSetAttribute(k_fx_c2c_cols_phase<L2>, A, int(FxCols<L2>::smem));                      \
+  if (e == cudaSuccess)                                                                             \
+    P->grid_cols = grid_for(k_fx_c2c_cols_phase<L2>, FxCols<L2>::T, FxCols<L2>::smem,               \
+                            (P->prm.nx / 2 + FxCols<L2>::PER - 1) / FxCols<L2>::PER)
+  switch (P->log2nx) {
+    DSNU_C2C_CASES(DSNU_PR)
+    default: return cudaErrorInvalidValue;
+  }
+  if (e != cudaSuccess) return e;
+  switch (P->log2ny) {
+    DSNU_C2C_CASES(DSNU_PC)
+    default: return cudaErrorInvalidValue;
+  }
+#undef DSNU_PR
+#undef DSNU_PC
+  return e;
+}
+
+dsnu_status linear_f32(dsnu_ds_plan_s* P, void* uv, int adjoint, cudaStream_t st) {
+  using R = float;
   cpx<R>* u = static_cast<cpx<R>*>(uv);
   const R scale = R(1.0 / (double(P->prm.nx) * double(P->prm.ny)));
   const cpx<R>* sx = static_cast<const cpx<R>*>(P->stw_x);
@@ -321,6 +506,40 @@ dsnu_status linear(dsnu_ds_plan_s* P, void* uv, int adjoint, cudaStream_t st) {
 #define DSNU_CP(L2)                                                                          \
   k_c2c_cols_phase<R, L2><<<P->grid_cols, GeoC2C<R, L2>::T, GeoC2C<R, L2>::smem, st>>>(     \
       u, P->prm.nx, sy, px, py, scale, adjoint)
+  switch (P->log2nx) {
+    DSNU_C2C_CASES(DSNU_RF)
+    default: return DSNU_EUNSUPPORTED;
+  }
+  switch (P->log2ny) {
+    DSNU_C2C_CASES(DSNU_CP)
+    default: return DSNU_EUNSUPPORTED;
+  }
+  switch (P->log2nx) {
+    DSNU_C2C_CASES(DSNU_RI)
+    default: return DSNU_EUNSUPPORTED;
+  }
+#undef DSNU_ROWS
+#undef DSNU_RF
+#undef DSNU_RI
+#undef DSNU_CP
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? DSNU_OK : ds_fail(DSNU_ECUDA, std::string("launch: ") + cudaGetErrorString(e));
+}
+
+dsnu_status linear_f64(dsnu_ds_plan_s* P, void* uv, int adjoint, cudaStream_t st) {
+  double2* u = static_cast<double2*>(uv);
+  const int lscale = -(P->log2nx + P->log2ny);
+  const fxw* sx = static_cast<const fxw*>(P->stw_x);
+  const fxw* sy = static_cast<const fxw*>(P->stw_y);
+  const fxw* px = static_cast<const fxw*>(P->px);
+  const fxw* py = static_cast<const fxw*>(P->py);
+#define DSNU_ROWS(L2, INV) \
+  k_fx_c2c_rows<L2><<<P->grid_rows, FxOne<L2>::T, FxOne<L2>::smem, st>>>(u, P->prm.ny, sx, INV)
+#define DSNU_RF(L2) DSNU_ROWS(L2, 0)
+#define DSNU_RI(L2) DSNU_ROWS(L2, 1)
+#define DSNU_CP(L2)                                                                               \
+  k_fx_c2c_cols_phase<L2><<<P->grid_cols, FxCols<L2>::T, FxCols<L2>::smem, st>>>(u, P->prm.nx, sy, px, py, lscale, \
+                                                                                adjoint)
   switch (P->log2nx) {
     DSNU_C2C_CASES(DSNU_RF)
     default: return DSNU_EUNSUPPORTED;
@@ -395,11 +614,21 @@ dsnu_status dsnu_ds_plan_create(const dsnu_ds_params* params, void* stream, dsnu
   if (p.precision == DSNU_MIXED) {
     upload<float>(P->stw_x, sx, st, &e);
     upload<float>(P->stw_y, sy, st, &e);
-    if (e == cudaSuccess) e = prepare<float>(P);
+    if (e == cudaSuccess) e = prepare_f32(P);
   } else {
-    upload<double>(P->stw_x, sx, st, &e);
-    upload<double>(P->stw_y, sy, st, &e);
-    if (e == cudaSuccess) e = prepare<double>(P);
+    auto fixed = [](const std::vector<double>& v) {  // fxw entries
+      std::vector<int> out;
+      for (double c : v) {
+        const double x = std::ldexp(c, kFxTwBits), h = std::nearbyint(x);
+        const double l = std::nearbyint((x - h) * 4294967296.0);
+        out.push_back(int(h));
+        out.push_back(int(std::min(std::max(l, -2147483647.0), 2147483647.0)));
+      }
+      return out;
+    };
+    upload<int>(P->stw_x, fixed(sx), st, &e);
+    upload<int>(P->stw_y, fixed(sy), st, &e);
+    if (e == cudaSuccess) e = prepare_f64(P);
   }
   if (e != cudaSuccess) {
     cudaFree(P->block);
@@ -424,9 +653,8 @@ dsnu_status dsnu_ds_set_linear_step(dsnu_ds_plan plan, double tau, double alpha,
                                                            static_cast<cpx<float>*>(plan->py), p.nx, p.ny,
                                                            dkx, dky, tau, alpha);
   else
-    k_phase_tables<double><<<(n + 255) / 256, 256, 0, st>>>(static_cast<cpx<double>*>(plan->px),
-                                                            static_cast<cpx<double>*>(plan->py), p.nx, p.ny,
-                                                            dkx, dky, tau, alpha);
+    k_phase_tables_fx<<<(n + 255) / 256, 256, 0, st>>>(static_cast<fxw*>(plan->px), static_cast<fxw*>(plan->py), p.nx,
+                                                       p.ny, dkx, dky, tau, alpha);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return ds_fail(DSNU_ECUDA, std::string("phase tables: ") + cudaGetErrorString(e));
   plan->tau = tau;
@@ -439,8 +667,8 @@ dsnu_status dsnu_ds_linear(dsnu_ds_plan plan, void* u_dev, int32_t adjoint, void
   if (!plan || !u_dev) return ds_fail(DSNU_EINVAL, "NULL plan or field");
   if (!plan->has_phase) return ds_fail(DSNU_EINVAL, "no linear step set (dsnu_ds_set_linear_step)");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  return plan->prm.precision == DSNU_MIXED ? linear<float>(plan, u_dev, adjoint, st)
-                                           : linear<double>(plan, u_dev, adjoint, st);
+  return plan->prm.precision == DSNU_MIXED ? linear_f32(plan, u_dev, adjoint, st)
+                                           : linear_f64(plan, u_dev, adjoint, st);
 }
 
 dsnu_status dsnu_ds_abs2(dsnu_ds_plan plan, const void* u_dev, double* rho_dev, void* stream) {

@@ -215,16 +215,16 @@ __device__ __forceinline__ int fx_norm_shift(unsigned m) { return max(__clz(int(
 
 // ---------------------------------------------------------------------------
 // Length-N DFT by a group of G = N/16 threads, 16 values per thread (the index
-// order and buffer layout of block_fft_regs); a pair of groups (P = 2 G
-// threads) runs the even and the odd chain of one row or column, with one
-// scale for both.  One transform per thread keeps it at 128 registers and one
+// order and buffer layout of block_fft_regs).  P threads share one scale: G, or
+// 2 G where two groups work together (the even and the odd chain of one row or
+// column, two adjacent columns).  One transform per thread keeps it at 128 registers and one
 // copy of the radix-16 code for all stages (the loop below): two transforms per
 // thread at 8 warps per SM, the stages unrolled, came to 200 KB of code and ran
 // twice as long (column pass at 4096^2 1405 us).
 // Returns the exponent that the result gained.  red: 2 words per warp.
-template <int LOG2N>
+template <int LOG2N, int P>
 __device__ __forceinline__ int fx_fft(fxc (&v)[16], fxc* buf, int t, const fxw* __restrict__ stw, unsigned* red) {
-  constexpr int N = 1 << LOG2N, G = N / 16, P = 2 * G, FULL = LOG2N / 4, LR = LOG2N - 4 * FULL;
+  constexpr int N = 1 << LOG2N, G = N / 16, FULL = LOG2N / 4, LR = LOG2N - 4 * FULL;
   int ex = 0;
   // leave stage s (radix 16, NS = 16^s): exchange, and scale for the next one
   auto exchange = [&](int s) {
@@ -274,11 +274,11 @@ __device__ __forceinline__ int fx_fft(fxc (&v)[16], fxc* buf, int t, const fxw* 
 }
 // The unnormalised inverse e^{+2 pi i nk/N}: real and imaginary parts
 // exchanged before and after (register renaming).
-template <int LOG2N>
+template <int LOG2N, int P>
 __device__ __forceinline__ int fx_ifft(fxc (&v)[16], fxc* buf, int t, const fxw* __restrict__ stw, unsigned* red) {
 #pragma unroll
   for (int m = 0; m < 16; ++m) v[m] = fx_swap(v[m]);
-  const int ex = fx_fft<LOG2N>(v, buf, t, stw, red);
+  const int ex = fx_fft<LOG2N, P>(v, buf, t, stw, red);
 #pragma unroll
   for (int m = 0; m < 16; ++m) v[m] = fx_swap(v[m]);
   return ex;
@@ -310,5 +310,77 @@ __device__ __forceinline__ double fx_scale(double d, int e) {
   return r;
 }
 __device__ __forceinline__ double fx_to_f64(i64 v, int e) { return fx_scale(__ll2double_rn(v), e); }
+
+// ---------------------------------------------------------------------------
+// Launch geometry of the passes with one transform per group (standard solver,
+// linear flow): two groups per CTA for the long transforms (16 warps per SM),
+// one warp's worth for the short ones (a small grid spreads over the SMs).
+template <int LOG2N>
+struct FxOne {
+  static constexpr int N = 1 << LOG2N;
+  static constexpr int G = N / 16;
+  static constexpr int PER = (G >= 64) ? 2 : (G >= 32) ? 1 : 32 / G;
+  static constexpr int T = PER * G;
+  static constexpr int MINB = 512 / T;
+  static constexpr int FB = fft_buf_elems(N);
+  static constexpr int STW = fft_stage_tw_elems(LOG2N) > 0 ? fft_stage_tw_elems(LOG2N) : 1;
+  static constexpr int W = T / 32, RED = 5 * W;
+  static constexpr size_t smem = size_t(STW + PER * FB) * 16 + ((RED * 4 + 15) & ~15);
+};
+
+__device__ __forceinline__ fxr fx_ldr(const fxr* __restrict__ p) {
+  const int2 v = __ldg(reinterpret_cast<const int2*>(p));
+  fxr r;
+  r.h = v.x;
+  r.l = v.y;
+  return r;
+}
+__device__ __forceinline__ fxw fx_ldw(const fxw* __restrict__ p) {
+  const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+  fxw w;
+  w.rh = v.x;
+  w.rl = v.y;
+  w.ih = v.z;
+  w.il = v.w;
+  return w;
+}
+__device__ __forceinline__ void fx_copy(fxw* __restrict__ dst, const fxw* __restrict__ src, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x)
+    *reinterpret_cast<int4*>(dst + i) = __ldg(reinterpret_cast<const int4*>(src + i));
+}
+
+// Collects into mx the largest high word of FP64 values (bit 0 set too for a
+// subnormal below 2^-1042): its exponent field for fx_from_f64, 0 only when all
+// are zero, >= 0x7FF00000 when one is infinite or a NaN.
+__device__ __forceinline__ unsigned fx_top(unsigned mx, double d) {
+  mx = max(mx, unsigned(__double2hiint(d)) & 0x7FFFFFFFu);
+  return __double2loint(d) != 0 ? (mx | 1u) : mx;
+}
+constexpr unsigned kFxInf = 0x7FF00000u;
+__device__ __forceinline__ int fx_efm(unsigned mx) { return max(int(mx >> 20), 1); }
+// Exponent to store for a transform whose inputs had fx_top mx.
+__device__ __forceinline__ int fx_exp(unsigned mx, int e) { return mx >= kFxInf ? kFxBad : mx == 0u ? kFxZero : e; }
+
+// Maximum of n exponents over the CTA (every thread calls it; contains barriers).
+__device__ __forceinline__ int fx_cta_max(const int* e, int n, unsigned* red) {
+  int m = kFxZero;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) m = max(m, e[i]);
+  m = __reduce_max_sync(0xffffffffu, m);
+  __syncthreads();  // earlier reads of `red`
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = unsigned(m);
+  __syncthreads();
+  int r = int(red[0]);
+  for (int w = 1; w < int(blockDim.x >> 5); ++w) r = max(r, int(red[w]));
+  return r;
+}
+
+// a 2^-s rounded to nearest, s >= 1 (a shift alone rounds down: its mean error
+// of half a quantum adds up over a transform to a spike at index 0).
+__device__ __forceinline__ i64 fx_sra(i64 v, int s) { return ((v >> (s - 1)) + 1) >> 1; }
+__device__ __forceinline__ fxc fx_sra(fxc a, int s) { return fx_mk(fx_sra(a.x, s), fx_sra(a.y, s)); }
+// Right shift that aligns a value of exponent e to exponent emax + HEAD (values
+// are stored below 2^63 and become smaller than 2^(63 - HEAD)).
+template <int HEAD>
+__device__ __forceinline__ int fx_align(int emax, int e) { return min(emax - e + HEAD, 63); }
 
 }  // namespace dsnu

@@ -64,56 +64,16 @@ struct FxMult {
 
 // e^{-2 pi i n/M} at n = t + G m
 __device__ __forceinline__ fxw fx_wm(const fxw* __restrict__ wm, int t, int m, int G) {
-  const int4 v = __ldg(reinterpret_cast<const int4*>(wm + t + G * (m & 7)));
-  fxw w;
-  if (m < 8) {
-    w.rh = v.x;
-    w.rl = v.y;
-    w.ih = v.z;
-    w.il = v.w;
-  } else {  // e^{-2 pi i (n' + N/2)/M} = -i e^{-2 pi i n'/M}
-    w.rh = v.z;
-    w.rl = v.w;
-    w.ih = -v.x;
-    w.il = -v.y;
+  fxw w = fx_ldw(wm + t + G * (m & 7));
+  if (m >= 8) {  // e^{-2 pi i (n' + N/2)/M} = -i e^{-2 pi i n'/M}
+    const fxw v = w;
+    w.rh = v.ih;
+    w.rl = v.il;
+    w.ih = -v.rh;
+    w.il = -v.rl;
   }
   return w;
 }
-__device__ __forceinline__ fxr fx_ldr(const fxr* __restrict__ p) {
-  const int2 v = __ldg(reinterpret_cast<const int2*>(p));
-  fxr r;
-  r.h = v.x;
-  r.l = v.y;
-  return r;
-}
-
-__device__ __forceinline__ void fx_copy(fxw* __restrict__ dst, const fxw* __restrict__ src, int n) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x)
-    *reinterpret_cast<int4*>(dst + i) = __ldg(reinterpret_cast<const int4*>(src + i));
-}
-
-// Maximum of n exponents over the CTA (every thread calls it; contains barriers).
-__device__ __forceinline__ int fx_cta_max(const int* e, int n, unsigned* red) {
-  int m = kFxZero;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) m = max(m, e[i]);
-  m = __reduce_max_sync(0xffffffffu, m);
-  __syncthreads();  // earlier reads of `red`
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = unsigned(m);
-  __syncthreads();
-  int r = int(red[0]);
-  for (int w = 1; w < int(blockDim.x >> 5); ++w) r = max(r, int(red[w]));
-  return r;
-}
-
-// a 2^-s rounded to nearest, s >= 1 (a shift alone rounds down: its mean error
-// of half a quantum adds up over a transform to a spike at index 0).
-__device__ __forceinline__ i64 fx_sra(i64 v, int s) { return ((v >> (s - 1)) + 1) >> 1; }
-__device__ __forceinline__ fxc fx_sra(fxc a, int s) { return fx_mk(fx_sra(a.x, s), fx_sra(a.y, s)); }
-// Right shift that aligns a value of exponent e to exponent emax + HEAD (values
-// are stored below 2^63 and become smaller than 2^(63 - HEAD)).
-template <int HEAD>
-__device__ __forceinline__ int fx_align(int emax, int e) { return min(emax - e + HEAD, 63); }
-
 // The chains' inputs from the staged values z (|component| < 2^61 after the
 // shift s): z/16 for the even one, z e^{-2 pi i n/M}/16 for the odd one.
 template <int G>
@@ -191,17 +151,15 @@ k_fx_row_fwd(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
     for (int i = 0; i < 8; ++i) {
       x[i] = valid ? __ldg(mb.rho + size_t(row) * N + tp + P * i) : 0.0;
       d[i] = fx_ldr(ax.dec + tp + P * i);
-      const unsigned a = unsigned(__double2hiint(x[i])) & 0x7FFFFFFFu;
-      mx = max(mx, a);
-      md = max(md, (a >> 20) + 32u - unsigned(__clz(d[i].h)));
-      if (__double2loint(x[i]) != 0) mx |= 1u;  // (a subnormal below 2^-1042)
+      mx = fx_top(mx, x[i]);
+      md = max(md, ((unsigned(__double2hiint(x[i])) >> 20) & 0x7FFu) + 32u - unsigned(__clz(d[i].h)));
     }
     mx = fx_post<P, true>(mx, red + 2 * W);
     md = fx_post<P, true>(md, red + 3 * W);
     __syncthreads();
     mx = fx_read<P, true>(mx, red + 2 * W);
     md = fx_read<P, true>(md, red + 3 * W);
-    const int efm = max(int(mx >> 20), 1);
+    const int efm = fx_efm(mx);
     // the smallest k with |rho d_x| <= 2^k max |rho| by the exponents (|rho| <
     // 2^(ef + 1), d_x/2^kd < 2^(1 - clz h)): z = rho + i rho d_x/2^k
     const int kr = min(max(int(md) - 32 + kd + 1 - efm, 0), kd);
@@ -213,7 +171,7 @@ k_fx_row_fwd(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
     __syncthreads();
     fxc v[16];
     fx_chain_in<G>(v, buf_e, 0, h, t, ax.wm);
-    const int ef = fx_fft<LOG2N>(v, buf, t, stw, red);
+    const int ef = fx_fft<LOG2N, P>(v, buf, t, stw, red);
     const unsigned mag = fx_post<P>(fx_mag(v), red + 4 * W);
     __syncthreads();  // (and the last stage's loads are done)
     const int s1 = fx_norm_shift<62>(fx_read<P>(mag, red + 4 * W));  // sums of two: below 2^63
@@ -223,9 +181,9 @@ k_fx_row_fwd(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
     // exponent of Z: from_f64 (efm - kFxBias), the five bits, the stages;
     // A = (Z(q) + conj Z(M - q))/2 and B = (Z(q) - conj Z(M - q))/2i as sums, times 2^s1
     if (tp == 0 && valid) {
-      const int ea = (mx >= 0x7FF00000u) ? kFxBad : (mx == 0u) ? kFxZero : efm - kFxBias + 5 + ef - 1 - s1;
-      ws_ptr<int>(mb, off.rexp)[row] = ea;
-      ws_ptr<int>(mb, off.rexpb)[row] = (mx == 0u || mx >= 0x7FF00000u) ? ea : ea + kr;
+      const int ea = efm - kFxBias + 5 + ef - 1 - s1;
+      ws_ptr<int>(mb, off.rexp)[row] = fx_exp(mx, ea);
+      ws_ptr<int>(mb, off.rexpb)[row] = fx_exp(mx, ea + kr);
     }
     if (valid) {
       fxc* Ar = ws_ptr<fxc>(mb, off.A) + TL::at(row, 0, ldqA);
@@ -299,7 +257,7 @@ k_fx_col_main(Members mem, FxOff off, int ldqA, int ncols, FxAxis ay, FxMult mt)
     int ex = emax + 2 - s0 + 4 + (mt.mexp && valid ? mt.mexp[col] : 0) + 5 + 4 - 3;
 #pragma unroll 1
     for (int inv = 0;; ++inv) {  // forward, then inverse (one copy of the transform's code)
-      ex += fx_fft<LOG2N>(v, buf, t, stw, red);
+      ex += fx_fft<LOG2N, P>(v, buf, t, stw, red);
       mag = fx_post<P>(fx_mag(v), red + (2 + inv) * W);
       __syncthreads();
       const int s = fx_norm_shift<62>(fx_read<P>(mag, red + (2 + inv) * W));
@@ -370,7 +328,7 @@ k_fx_band_fwd(Members mem, FxOff off, int ldqB, int ncols, int ldq, int Q, FxAxi
     }
     __syncthreads();
     fx_chain_in<G>(v, buf_e, 1, h, t, ay.wm);
-    const int ex = emax + 2 - s0 + kdy + 4 + fx_fft<LOG2N>(v, buf, t, stw, red);
+    const int ex = emax + 2 - s0 + kdy + 4 + fx_fft<LOG2N, P>(v, buf, t, stw, red);
     if (valid) {
       const bool bad = emax >= kFxBad;
       const double nan = __longlong_as_double(0x7FF8000000000000ll);
@@ -408,19 +366,17 @@ k_fx_band_inv(Members mem, FxOff off, int ldq, int Q, int ncols, int ldqB, FxAxi
       const int q = 2 * (t + G * m) + h, sq = q < N ? q : q - M;
       double2 a = make_double2(0.0, 0.0);
       if (valid && sq >= -Q && sq <= Q) a = Sband[size_t(col) * ldq + sq + Q];
-      mx = max(mx, unsigned(__double2hiint(a.x)) & 0x7FFFFFFFu);
-      mx = max(mx, unsigned(__double2hiint(a.y)) & 0x7FFFFFFFu);
-      if ((__double2loint(a.x) | __double2loint(a.y)) != 0) mx |= 1u;
+      mx = fx_top(fx_top(mx, a.x), a.y);
       v[m] = fx_mk(__double_as_longlong(a.x), __double_as_longlong(a.y));
     }
     mx = fx_post<P, true>(mx, red + 2 * W);
     __syncthreads();
     mx = fx_read<P, true>(mx, red + 2 * W);
-    const int efm = max(int(mx >> 20), 1);
+    const int efm = fx_efm(mx);
 #pragma unroll
     for (int m = 0; m < 16; ++m)
       v[m] = fx_shr<5>(fx_mk(fx_from_f64(__longlong_as_double(v[m].x), efm), fx_from_f64(__longlong_as_double(v[m].y), efm)));
-    const int ef = fx_ifft<LOG2N>(v, buf, t, stw, red);
+    const int ef = fx_ifft<LOG2N, P>(v, buf, t, stw, red);
     const unsigned mag = fx_post<P>(fx_mag(v), red + 3 * W);
     __syncthreads();
     const int s1 = fx_norm_shift<62>(fx_read<P>(mag, red + 3 * W));
@@ -433,9 +389,7 @@ k_fx_band_inv(Members mem, FxOff off, int ldq, int Q, int ncols, int ldqB, FxAxi
         St[TL::at(n, col, ldqB)] = fx_shl(fx_mk(fx_mulr(v[m].x, d), fx_mulr(v[m].y, d)), 4);  // < 2^58.5 before
       }
       if (tp == 0)
-        ws_ptr<int>(mb, off.bexp)[col] = (mx >= 0x7FF00000u) ? kFxBad
-                                         : (mx == 0u)        ? kFxZero
-                                                             : efm - kFxBias + 5 + ef - s1 + 4 + kdy + 1 - 4;
+        ws_ptr<int>(mb, off.bexp)[col] = fx_exp(mx, efm - kFxBias + 5 + ef - s1 + 4 + kdy + 1 - 4);
     }
   }
 }
@@ -515,7 +469,7 @@ k_fx_row_inv(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
         v[m] = fx_mul(fx_shl(fx_mk(x.x - r.x, x.y + r.y), s0), fx_conj(fx_wm(ax.wm, t, m, G)));
       }
     }
-    const int ex = emax + 4 - s0 + 4 + kd + 1 + lscale + fx_ifft<LOG2N>(v, buf, t, stw, red);
+    const int ex = emax + 4 - s0 + 4 + kd + 1 + lscale + fx_ifft<LOG2N, P>(v, buf, t, stw, red);
     if (valid) {
       double* __restrict__ phi = mb.phi + size_t(row) * N + h;
       const bool bad = emax >= kFxBad;

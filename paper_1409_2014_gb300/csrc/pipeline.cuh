@@ -148,8 +148,8 @@ cudaError_t prepare_kernels(PlanGeom& g) {
 template <typename R>
 dsnu_status run_standard(const PlanGeom& g, const PlanTables& t, const WsLayout& L, const Members& mem,
                          cudaStream_t st, int cj, cudaEvent_t* ev) {
-  // FP32 row passes read the compact stage table (GeoStd::PF)
-  const cpx<R>* sx = static_cast<const cpx<R>*>(sizeof(R) == 4 ? t.stwc_x : t.stw_x);
+  // the row passes read the compact stage table
+  const cpx<R>* sx = static_cast<const cpx<R>*>(t.stwc_x);
   const cpx<R>* sy = static_cast<const cpx<R>*>(t.stw_y);
   MultTabs<R> mt{};
   mt.wx2 = static_cast<const R*>(t.m_wx2);

@@ -1,7 +1,9 @@
 // FP64 (DSNU_FP64) plans: the FFT passes in 64-bit block fixed point
-// (kernels_fx.cuh), interpolation, weighting and spreading in FP64.
+// (kernels_fx.cuh, standard_fx.cuh), interpolation, weighting and spreading in
+// FP64.
 #include "kernels_fx.cuh"
 #include "pipeline.cuh"
+#include "standard_fx.cuh"
 
 namespace dsnu {
 
@@ -35,13 +37,84 @@ cudaError_t prepare_fx_cols(PlanGeom& g) {
   return resident_ctas(k_fx_band_inv<L2>, GG::T, GG::smem, &g.cap_bandi);
 }
 
+template <int L2>
+cudaError_t prepare_fx_std_rows(PlanGeom& g) {
+  using GG = FxOne<L2>;
+  const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(k_fx_std_row_fwd<L2>, A, int(GG::smem)))) return e;
+  if ((e = cudaFuncSetAttribute(k_fx_std_row_inv<L2>, A, int(GG::smem)))) return e;
+  if ((e = resident_ctas(k_fx_std_row_fwd<L2>, GG::T, GG::smem, &g.cap_rowf))) return e;
+  return resident_ctas(k_fx_std_row_inv<L2>, GG::T, GG::smem, &g.cap_rowi);
+}
+
+template <int L2>
+cudaError_t prepare_fx_std_cols(PlanGeom& g) {
+  using GG = FxOne<L2>;
+  const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(k_fx_std_col<L2, false>, A, int(GG::smem)))) return e;
+  if ((e = cudaFuncSetAttribute(k_fx_std_col<L2, true>, A, int(GG::smem)))) return e;
+  return g.m1_full ? resident_ctas(k_fx_std_col<L2, true>, GG::T, GG::smem, &g.cap_col)
+                   : resident_ctas(k_fx_std_col<L2, false>, GG::T, GG::smem, &g.cap_col);
+}
+
+// The standard solver's three passes (run_standard in fixed point).
+dsnu_status run_standard_fx(const PlanGeom& g, const PlanTables& t, const WsLayout& L, const Members& mem,
+                            cudaStream_t st, cudaEvent_t* ev) {
+  const fxw* sx = static_cast<const fxw*>(t.fx_stw_x);
+  const fxw* sy = static_cast<const fxw*>(t.fx_stw_y);
+  const FxMult mt{static_cast<const fxr*>(t.m1tab), t.fx_mexp, g.m1_ld};
+  const bool pdl = g.pdl != 0;
+  const int ldq = L.ldqA;
+  auto grid = [&](long n, int per, int cap) { return dim3(persistent_grid(mem.count * ((n + per - 1) / per), cap)); };
+#define DSNU_SROWF(L2)                                                                                         \
+  launch_k(pdl, k_fx_std_row_fwd<L2>, grid(g.ny / 2, FxOne<L2>::PER, g.cap_rowf), dim3(FxOne<L2>::T),          \
+           FxOne<L2>::smem, st, mem, L.off_A, L.off_rexp, ldq, g.ny, sx)
+#define DSNU_SCOL(L2)                                                                                          \
+  if (g.m1_full)                                                                                               \
+    launch_k(pdl, k_fx_std_col<L2, true>, grid(ldq, FxOne<L2>::PER, g.cap_col), dim3(FxOne<L2>::T),            \
+             FxOne<L2>::smem, st, mem, L.off_A, L.off_rexp, L.off_cexp, ldq, ldq, sy, mt);                     \
+  else                                                                                                         \
+    launch_k(pdl, k_fx_std_col<L2, false>, grid(ldq, FxOne<L2>::PER, g.cap_col), dim3(FxOne<L2>::T),           \
+             FxOne<L2>::smem, st, mem, L.off_A, L.off_rexp, L.off_cexp, ldq, ldq, sy, mt)
+#define DSNU_SROWI(L2)                                                                                         \
+  launch_k(pdl, k_fx_std_row_inv<L2>, grid(g.ny / 2, FxOne<L2>::PER, g.cap_rowi), dim3(FxOne<L2>::T),          \
+           FxOne<L2>::smem, st, mem, L.off_A, L.off_cexp, ldq, g.ny, sx, -(ilogb(double(g.nx)) + ilogb(double(g.ny))))
+  if (ev) cudaEventRecord(ev[0], st);
+  switch (g.log2nx) {
+    DSNU_LOG2_CASES(DSNU_SROWF)
+    default: return DSNU_EUNSUPPORTED;
+  }
+  if (ev)
+    for (int i = 1; i <= 6; ++i) cudaEventRecord(ev[i], st);
+  switch (g.log2ny) {
+    DSNU_LOG2_CASES(DSNU_SCOL)
+    default: return DSNU_EUNSUPPORTED;
+  }
+  if (ev) cudaEventRecord(ev[7], st);
+  switch (g.log2nx) {
+    DSNU_LOG2_CASES(DSNU_SROWI)
+    default: return DSNU_EUNSUPPORTED;
+  }
+  if (ev) cudaEventRecord(ev[8], st);
+#undef DSNU_SROWF
+#undef DSNU_SCOL
+#undef DSNU_SROWI
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    set_last_error(std::string("kernel launch failed: ") + cudaGetErrorString(e));
+    return DSNU_ECUDA;
+  }
+  return DSNU_OK;
+}
+
 }  // namespace
 
 cudaError_t prepare_kernels_f64(PlanGeom& g) {
-  if (g.standard) return prepare_standard<double>(g);
   cudaError_t e = cudaSuccess;
-#define DSNU_PREP_R(L2) e = prepare_fx_rows<L2>(g)
-#define DSNU_PREP_C(L2) e = prepare_fx_cols<L2>(g)
+#define DSNU_PREP_R(L2) e = g.standard ? prepare_fx_std_rows<L2>(g) : prepare_fx_rows<L2>(g)
+#define DSNU_PREP_C(L2) e = g.standard ? prepare_fx_std_cols<L2>(g) : prepare_fx_cols<L2>(g)
   switch (g.log2nx) {
     DSNU_LOG2_CASES(DSNU_PREP_R)
     default: return cudaErrorInvalidValue;
@@ -58,10 +131,11 @@ cudaError_t prepare_kernels_f64(PlanGeom& g) {
 
 dsnu_status run_pipeline_f64(const PlanGeom& g, const PlanTables& t, const WsLayout& L, const Members& mem,
                              cudaStream_t st, int cj, cudaEvent_t* ev, const Overlap* ov) {
-  if (g.standard) return run_standard<double>(g, t, L, mem, st, cj, ev);
-  (void)ov;
   // the conjugated pipeline of a real input is the conjugate of this one: the
   // same result (kernels_fx.cuh), so `cj` selects nothing
+  (void)cj;
+  (void)ov;
+  if (g.standard) return run_standard_fx(g, t, L, mem, st, ev);
   const WsOff off{L.off_A, L.off_B, L.off_Bband, L.off_Sband, L.off_c, L.off_partial, L.off_sched};
   const FxOff fo{L.off_A, L.off_B, L.off_Bband, L.off_Sband, L.off_rexp, L.off_rexpb, L.off_cexp, L.off_bexp};
   const FxAxis ax{static_cast<const fxw*>(t.fx_stw_x), static_cast<const fxw*>(t.fx_wm_x),

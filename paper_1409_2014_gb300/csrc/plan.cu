@@ -372,6 +372,22 @@ struct Builder {
 };
 
 
+// Upload the plan's tables as one device block.
+static dsnu_status upload_block(dsnu_plan_s* P, const Builder& b, cudaStream_t st) {
+  void* dev = nullptr;
+  cudaError_t e = cudaMalloc(&dev, b.bytes.size());
+  if (e != cudaSuccess) return fail(DSNU_ENOMEM, std::string("cudaMalloc(plan tables): ") + cudaGetErrorString(e));
+  e = cudaMemcpyAsync(dev, b.bytes.data(), b.bytes.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) {
+    cudaFree(dev);
+    return fail(DSNU_ECUDA, std::string("plan table upload: ") + cudaGetErrorString(e));
+  }
+  P->table_block = dev;
+  P->table_bytes = b.bytes.size();
+  return DSNU_OK;
+}
+
 template <typename R>
 static dsnu_status upload_spread(const HostSpread<R>& H, cudaStream_t st, void** block, PlanTables& t) {
   Builder b;
@@ -550,6 +566,48 @@ __global__ void k_fill_m1_fx(int2* tab, int nx, int ny, int ld, int full, double
   }
 }
 
+// The same for the standard solver (no partition): columns q_x <= nx/2, entry j
+// at |qbar_y| = j <= ny/2 (full: at the natural frequency q_y = j).
+__global__ void k_fill_std_fx(int2* tab, int nx, int ny, int ld, int full, double dkx, double dky, int generic,
+                              int alpha, double a0, double ac, double as, const int* mexp) {
+  const long long n = (long long)(nx / 2 + 1) * ld;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const int col = int(i / ld), q = int(i - (long long)col * ld);
+    const int a = (q <= ny / 2) ? q : ny - q;
+    const int qs = (q < ny / 2) ? q : (q == ny / 2 ? 0 : q - ny);  // signed, 0 at the Nyquist row (sin 2theta term)
+    int2 v = make_int2(0, 0);
+    const double wx = col * dkx, wy = a * dky;
+    const double wx2 = wx * wx, wy2 = wy * wy, s = wx2 + wy2;
+    if (s > 0.0) {
+      double m = -wx2 / s;
+      if (generic) {
+        const double kx = col < nx / 2 ? wx : 0.0;  // (and at the Nyquist column)
+        m = a0 + (ac * (wx2 - wy2) + 2.0 * as * kx * (qs * dky)) / s;
+        if (alpha == 1) m *= sqrt(s);
+        if (alpha == -1) m /= sqrt(s);
+      }
+      const long long w = __double2ll_rn(ldexp(m, kFxMultBits + 32 - (mexp ? mexp[col] : 0)));
+      v.y = int(w);
+      v.x = int((w - v.y) >> 32);
+    }
+    tab[i] = v;
+  }
+}
+
+// Exponents of the columns of a generic multiplier's fixed-point table:
+// |m| <= (|a0| + |a_cos| + |a_sin|) |k|^alpha < 2^(mexp - 1) on column q.
+static std::vector<int> fx_mult_exponents(const PlanGeom& g, int ncols, double dkx, double dky, double kymax) {
+  std::vector<int> out;
+  const double amp = std::fabs(g.m_a0) + std::fabs(g.m_ac) + std::fabs(g.m_as);
+  for (int q = 0; q < ncols; ++q) {
+    const double k1 = q * dkx;
+    const double b = (g.m_alpha == 1) ? amp * std::sqrt(k1 * k1 + kymax * kymax)
+                     : (g.m_alpha == -1) ? amp / (q == 0 ? dky : k1) : amp;
+    out.push_back(b > 0.0 ? std::min(std::max(std::ilogb(b) + 2, -1200), 1100) : 0);
+  }
+  return out;
+}
+
 template <typename R>
 static dsnu_status build_m1_table(dsnu_plan_s* P, double dkx, double dky, cudaStream_t st) {
   const PlanGeom& g = P->geom;
@@ -624,16 +682,7 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
     g.kdy = fx_decon(dcy, T.fx_dec_y);
     g.m1_full = (g.m_generic && g.m_as != 0.0) ? 1 : 0;
     g.m1_ld = g.m1_full ? My : ny + 4;
-    if (g.m_generic) {
-      // |m| <= (|a0| + |a_cos| + |a_sin|) |k|^alpha on a column
-      const double amp = std::fabs(g.m_a0) + std::fabs(g.m_ac) + std::fabs(g.m_as), kmax = ny * dky;
-      for (int q = 0; q <= nx; ++q) {
-        const double k1 = q * dkx;
-        const double b = (g.m_alpha == 1) ? amp * std::sqrt(k1 * k1 + kmax * kmax)
-                         : (g.m_alpha == -1) ? amp / (q == 0 ? dky : k1) : amp;
-        T.fx_mexp.push_back(b > 0.0 ? std::min(std::max(std::ilogb(b) + 2, -1200), 1100) : 0);
-      }
-    }
+    if (g.m_generic) T.fx_mexp = fx_mult_exponents(g, nx + 1, dkx, dky, ny * dky);
   } else {
     fft_stage_twiddles(g.log2nx, tmp); T.stw_x = cast<R>(tmp);
     fft_stage_twiddles(g.log2ny, tmp); T.stw_y = cast<R>(tmp);
@@ -728,16 +777,9 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   const size_t o_itp = b.add(T.itile_ptr), o_ito = b.add(T.itile_org), o_itn = b.add(T.itile_nodes);
   const int zero = 0;
   const size_t o_st = b.add(&zero, sizeof(int));
-  void* dev = nullptr;
-  cudaError_t e = cudaMalloc(&dev, b.bytes.size());
-  if (e != cudaSuccess) return fail(DSNU_ENOMEM, std::string("cudaMalloc(plan tables): ") + cudaGetErrorString(e));
-  e = cudaMemcpyAsync(dev, b.bytes.data(), b.bytes.size(), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) {
-    cudaFree(dev);
-    return fail(DSNU_ECUDA, std::string("plan table upload: ") + cudaGetErrorString(e));
-  }
-  char* d = static_cast<char*>(dev);
+  const dsnu_status su = upload_block(P, b, st);
+  if (su != DSNU_OK) return su;
+  char* d = static_cast<char*>(P->table_block);
   PlanTables& t = P->tab;
   t.stw_x = d + o_stx; t.twm_lo_x = d + o_tlx; t.twm_hi_x = d + o_thx; t.decon_x = d + o_dx;
   t.stwc_x = d + o_scx;
@@ -753,8 +795,6 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   t.fx_stw_x = d + o_fsx; t.fx_wm_x = d + o_fwx; t.fx_dec_x = d + o_fdx;
   t.fx_stw_y = d + o_fsy; t.fx_wm_y = d + o_fwy; t.fx_dec_y = d + o_fdy;
   t.fx_mexp = (sizeof(R) == 8 && g.m_generic) ? reinterpret_cast<int*>(d + o_fme) : nullptr;
-  P->table_block = dev;
-  P->table_bytes = b.bytes.size();
   if (sizeof(R) == 8 || !g.m_generic) {
     const dsnu_status sm = build_m1_table<R>(P, dkx, dky, st);
     if (sm != DSNU_OK) return sm;
@@ -762,24 +802,23 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   return setup_spread<R>(P, T.node_q0, T.node_w, st);
 }
 
-// Tables of the standard periodic FFT solver: the stage twiddles of both
-// axes and (q_x dk_x)^2 for q_x in [0, nx/2], dk = 2 pi/(2 l) (no padding).
-template <typename R>
-static dsnu_status build_tables_standard(dsnu_plan_s* P, cudaStream_t st) {
+// Tables of the standard periodic FFT solver (mixed plans): the stage twiddles
+// of both axes and (q_x dk_x)^2 for q_x in [0, nx/2], dk = 2 pi/(2 l) (no padding).
+static dsnu_status build_tables_standard_f32(dsnu_plan_s* P, cudaStream_t st) {
   const dsnu_params& p = P->prm;
   PlanGeom& g = P->geom;
   std::vector<double> tmp;
   fft_stage_twiddles(g.log2nx, tmp);
-  const std::vector<R> stw_x = cast<R>(tmp);
+  const std::vector<float> stw_x = cast<float>(tmp);
   fft_stage_twiddles(g.log2ny, tmp);
-  const std::vector<R> stw_y = cast<R>(tmp);
+  const std::vector<float> stw_y = cast<float>(tmp);
   fft_stage_twiddles_ct(g.log2nx, tmp);
-  const std::vector<R> stwc_x = cast<R>(tmp);
+  const std::vector<float> stwc_x = cast<float>(tmp);
   const double dkx = M_PI / p.lx, dky = M_PI / p.ly;
-  std::vector<R> wx2(g.nx / 2 + 1), kx(g.nx / 2 + 1);
+  std::vector<float> wx2(g.nx / 2 + 1), kx(g.nx / 2 + 1);
   for (int q = 0; q <= g.nx / 2; ++q) {
-    wx2[q] = R((q * dkx) * (q * dkx));
-    kx[q] = R(q < g.nx / 2 ? q * dkx : 0.0);  // Nyquist column: +-K averaged (no sin 2theta term)
+    wx2[q] = float((q * dkx) * (q * dkx));
+    kx[q] = float(q < g.nx / 2 ? q * dkx : 0.0);  // Nyquist column: +-K averaged (no sin 2theta term)
   }
   g.dky2 = dky * dky;
   Builder b;
@@ -787,16 +826,9 @@ static dsnu_status build_tables_standard(dsnu_plan_s* P, cudaStream_t st) {
   const size_t o_scx = b.add(stwc_x);
   const int zero = 0;
   const size_t o_st = b.add(&zero, sizeof(int));
-  void* dev = nullptr;
-  cudaError_t e = cudaMalloc(&dev, b.bytes.size());
-  if (e != cudaSuccess) return fail(DSNU_ENOMEM, std::string("cudaMalloc(plan tables): ") + cudaGetErrorString(e));
-  e = cudaMemcpyAsync(dev, b.bytes.data(), b.bytes.size(), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) {
-    cudaFree(dev);
-    return fail(DSNU_ECUDA, std::string("plan table upload: ") + cudaGetErrorString(e));
-  }
-  char* d = static_cast<char*>(dev);
+  const dsnu_status s = upload_block(P, b, st);
+  if (s != DSNU_OK) return s;
+  char* d = static_cast<char*>(P->table_block);
   PlanTables& t = P->tab;
   t.stw_x = d + o_stx;
   t.stwc_x = d + o_scx;
@@ -804,8 +836,47 @@ static dsnu_status build_tables_standard(dsnu_plan_s* P, cudaStream_t st) {
   t.m_wx2 = d + o_wx2;
   t.m_kx = d + o_kx;
   t.status = reinterpret_cast<int*>(d + o_st);
-  P->table_block = dev;
-  P->table_bytes = b.bytes.size();
+  return DSNU_OK;
+}
+
+// The FP64 standard plan: fixed-point stage twiddles and the multiplier table.
+static dsnu_status build_tables_standard_fx(dsnu_plan_s* P, cudaStream_t st) {
+  const dsnu_params& p = P->prm;
+  PlanGeom& g = P->geom;
+  std::vector<double> tmp;
+  fft_stage_twiddles(g.log2nx, tmp);
+  const std::vector<int> stw_x = fx_table(tmp, kFxTwBits);
+  fft_stage_twiddles(g.log2ny, tmp);
+  const std::vector<int> stw_y = fx_table(tmp, kFxTwBits);
+  const double dkx = M_PI / p.lx, dky = M_PI / p.ly;
+  std::vector<int> mexp;
+  if (g.m_generic) mexp = fx_mult_exponents(g, g.nx / 2 + 1, dkx, dky, 0.5 * g.ny * dky);
+  g.m1_full = (g.m_generic && g.m_as != 0.0) ? 1 : 0;
+  g.m1_ld = g.m1_full ? g.ny : g.ny / 2 + 1;
+  Builder b;
+  const size_t o_stx = b.add(stw_x), o_sty = b.add(stw_y), o_me = b.add(mexp);
+  const int zero = 0;
+  const size_t o_st = b.add(&zero, sizeof(int));
+  const dsnu_status s = upload_block(P, b, st);
+  if (s != DSNU_OK) return s;
+  char* d = static_cast<char*>(P->table_block);
+  PlanTables& t = P->tab;
+  t.fx_stw_x = d + o_stx;
+  t.fx_stw_y = d + o_sty;
+  t.fx_mexp = g.m_generic ? reinterpret_cast<int*>(d + o_me) : nullptr;
+  t.status = reinterpret_cast<int*>(d + o_st);
+  const size_t bytes = size_t(g.nx / 2 + 1) * g.m1_ld * sizeof(int2);
+  cudaError_t e = cudaMalloc(&P->m1_block, bytes);
+  if (e != cudaSuccess) {
+    P->m1_block = nullptr;
+    return fail(DSNU_ENOMEM, std::string("cudaMalloc(multiplier table): ") + cudaGetErrorString(e));
+  }
+  k_fill_std_fx<<<1024, 256, 0, st>>>(static_cast<int2*>(P->m1_block), g.nx, g.ny, g.m1_ld, g.m1_full, dkx, dky,
+                                      g.m_generic, g.m_alpha, g.m_a0, g.m_ac, g.m_as, t.fx_mexp);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return fail(DSNU_ECUDA, std::string("multiplier table: ") + cudaGetErrorString(e));
+  t.m1tab = P->m1_block;
   return DSNU_OK;
 }
 
@@ -817,6 +888,11 @@ static void layout_workspace(dsnu_plan_s* P) {  // defined after the autotuner, 
     L = WsLayout{};
     L.ldqA = g.nx / 2 + 1;
     L.total = (size_t(g.ny) * L.ldqA * csz + 255) & ~size_t(255);
+    if (g.precision == DSNU_FP64) {  // exponents of the row pairs and of the columns
+      L.off_rexp = L.total;
+      L.off_cexp = (L.off_rexp + size_t(g.ny / 2) * sizeof(int) + 255) & ~size_t(255);
+      L.total = (L.off_cexp + size_t(L.ldqA) * sizeof(int) + 255) & ~size_t(255);
+    }
     return;
   }
   L.ldqA = g.nx + 1;
@@ -934,7 +1010,7 @@ dsnu_status dsnu_plan_create_multiplier(const dsnu_params* params, const dsnu_mu
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   dsnu_status s;
   if (standard)
-    s = (p.precision == DSNU_MIXED) ? build_tables_standard<float>(P, st) : build_tables_standard<double>(P, st);
+    s = (p.precision == DSNU_MIXED) ? build_tables_standard_f32(P, st) : build_tables_standard_fx(P, st);
   else
     s = (p.precision == DSNU_MIXED) ? build_tables<float>(P, st) : build_tables<double>(P, st);
   if (s != DSNU_OK) {

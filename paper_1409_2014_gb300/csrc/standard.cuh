@@ -18,7 +18,8 @@
 // `cj` = 1 conjugates every transform (the transposed operator, equal to the
 // operator itself since m is real and even).
 //
-// FP32 plans (PF): the row passes read their inputs from shared-memory
+// The kernels here are the mixed (FP32) plans'; FP64 plans run standard_fx.cuh.
+// The row passes read their inputs from shared-memory
 // landing buffers filled while the previous item is transformed (a bulk copy
 // of the item's rows of rho; cp.async of the row pairs' 16-byte segments of the
 // half spectrum), with the compact stage table making room; the column pass
@@ -53,21 +54,19 @@ struct GeoStd {
 };
 
 template <typename R, int LOG2N>
-__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, min_blocks<R>(2))
+__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, 2)
 k_std_row_fwd(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restrict__ stw_g, int cj, int* status) {
   using GG = GeoStd<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, PER = GG::PER;
-  constexpr bool PF = GG::PF;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* stw = reinterpret_cast<cpx<R>*>(smem_raw);
-  copy_to_smem(stw, stw_g, PF ? GG::STWC : GG::STW);
+  copy_to_smem(stw, stw_g, GG::STWC);
   const int tid = threadIdx.x;
   const int rr = tid / G, t = tid - rr * G;
-  cpx<R>* buf = stw + (PF ? GG::STWCP : GG::STWP) + rr * GG::FB;
-  double* land = reinterpret_cast<double*>(stw + (PF ? GG::STWCP : GG::STWP) + PER * GG::FB);  // PF: 2 PER rows
+  cpx<R>* buf = stw + GG::STWCP + rr * GG::FB;
+  double* land = reinterpret_cast<double*>(stw + GG::STWCP + PER * GG::FB);  // 2 PER rows
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(land + 2 * PER * N);
-  if constexpr (PF)
-    if (tid == 0) mbar_init(bar, 1);
+  if (tid == 0) mbar_init(bar, 1);
   __syncthreads();
   grid_dep_wait();
   const int pairs = ny / 2;
@@ -81,8 +80,7 @@ k_std_row_fwd(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restric
     mbar_expect_tx(bar, bytes);
     bulk_load(land, member_at(mem, mi2).rho + size_t(r0) * N, bytes, bar, l2_evict_first());
   };
-  if constexpr (PF)
-    if (tid == 0 && int(blockIdx.x) < total) prefetch(blockIdx.x);
+  if (tid == 0 && int(blockIdx.x) < total) prefetch(blockIdx.x);
   unsigned phase = 0;
 #pragma unroll 1
   for (int it = blockIdx.x; it < total; it += gridDim.x) {
@@ -93,34 +91,24 @@ k_std_row_fwd(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restric
     const int pr = item * PER + rr;
     const bool valid = pr < pairs;
     const int row = 2 * pr;
-    bool landed = true;
-    if constexpr (PF) {
-      // bounded wait (1 s); on expiry the CTA stops after the reads below
-      landed = mbar_wait(bar, phase, 1000000000ull);
-      phase ^= 1u;
-    }
+    // bounded wait (1 s); on expiry the CTA stops after the reads below
+    const bool landed = mbar_wait(bar, phase, 1000000000ull);
+    phase ^= 1u;
     cpx<R> v[16];
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
       const int n = t + G * m;
       R a = R(0), b = R(0);
       if (valid) {
-        if constexpr (PF) {
-          a = from_f64<R>(land[(2 * rr) * N + n]);
-          b = from_f64<R>(land[(2 * rr + 1) * N + n]);
-        } else {
-          a = from_f64<R>(mb.rho[size_t(row) * N + n]);
-          b = from_f64<R>(mb.rho[size_t(row + 1) * N + n]);
-        }
+        a = from_f64<R>(land[(2 * rr) * N + n]);
+        b = from_f64<R>(land[(2 * rr + 1) * N + n]);
       }
       v[m] = mk<R>(a, b);
     }
-    if constexpr (PF) {
-      // every thread has read the landing buffer (a barrier); stop if a wait expired
-      if (cta_timed_out(landed, bar, phase ^ 1u, status)) return;
-      if (tid == 0 && it + int(gridDim.x) < total) prefetch(it + gridDim.x);
-    }
-    block_fft_regs<R, LOG2N, PF>(v, buf, t, stw, cj != 0);
+    // every thread has read the landing buffer (a barrier); stop if a wait expired
+    if (cta_timed_out(landed, bar, phase ^ 1u, status)) return;
+    if (tid == 0 && it + int(gridDim.x) < total) prefetch(it + gridDim.x);
+    block_fft_regs<R, LOG2N, true>(v, buf, t, stw, cj != 0);
     __syncthreads();  // the last stage's loads of buf are done
 #pragma unroll
     for (int m = 0; m < 16; ++m) buf[pad16(t + G * m)] = v[m];
@@ -133,24 +121,19 @@ k_std_row_fwd(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restric
         const cpx<R> xa = mk<R>(R(0.5) * (zq.x + zm.x), R(0.5) * (zq.y - zm.y));
         const cpx<R> xb = mk<R>(R(0.5) * (zq.y + zm.y), R(-0.5) * (zq.x - zm.x));
         cpx<R>* dst = H + Tile<R>::at(row, q, ldq);  // row + 1 is the next element
-        if constexpr (sizeof(R) == 4) {              // (16-byte aligned: row is even)
-          *reinterpret_cast<float4*>(dst) = make_float4(xa.x, xa.y, xb.x, xb.y);
-        } else {
-          dst[0] = xa;
-          dst[1] = xb;
-        }
+        *reinterpret_cast<float4*>(dst) = make_float4(xa.x, xa.y, xb.x, xb.y);  // (16-byte aligned: row is even)
       }
     }
   }
 }
 
 template <typename R, int LOG2N>
-__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, min_blocks<R>(2))
+__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, 2)
 k_std_col(Members mem, size_t offH, int ldq, int ncols, const cpx<R>* __restrict__ stw_g,
           MultTabs<R> mt, R scale, int cj) {
   using GG = GeoStd<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, PER = GG::PER;
-  constexpr bool PF = GG::PF && LOG2N >= 9;  // (below, the registers for it are not there)
+  constexpr bool PF = LOG2N >= 9;  // (below, the registers for it are not there)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* stw = reinterpret_cast<cpx<R>*>(smem_raw);
   copy_to_smem(stw, stw_g, GG::STW);
@@ -214,20 +197,19 @@ k_std_col(Members mem, size_t offH, int ldq, int ncols, const cpx<R>* __restrict
 }
 
 template <typename R, int LOG2N>
-__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, min_blocks<R>(2))
+__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, 2)
 k_std_row_inv(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restrict__ stw_g, int cj) {
   using GG = GeoStd<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, PER = GG::PER, T = GG::T;
-  constexpr bool PF = GG::PF;
   constexpr int HS = N / 2 + 1;  // segments per row pair
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* stw = reinterpret_cast<cpx<R>*>(smem_raw);
-  copy_to_smem(stw, stw_g, PF ? GG::STWC : GG::STW);
+  copy_to_smem(stw, stw_g, GG::STWC);
   const int tid = threadIdx.x;
   const int rr = tid / G, t = tid - rr * G;
-  cpx<R>* buf = stw + (PF ? GG::STWCP : GG::STWP) + rr * GG::FB;
-  // PF: Y_a(q), Y_b(q) of each row pair of the item at [2 (pair HS + q) + row]
-  cpx<R>* land = stw + (PF ? GG::STWCP : GG::STWP) + PER * GG::FB;
+  cpx<R>* buf = stw + GG::STWCP + rr * GG::FB;
+  // Y_a(q), Y_b(q) of each row pair of the item at [2 (pair HS + q) + row]
+  cpx<R>* land = stw + GG::STWCP + PER * GG::FB;
   __syncthreads();
   grid_dep_wait();
   const int pairs = ny / 2;
@@ -244,21 +226,17 @@ k_std_row_inv(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restric
     }
     cp_async_commit();
   };
-  if constexpr (PF)
-    if (int(blockIdx.x) < total) prefetch(blockIdx.x);
+  if (int(blockIdx.x) < total) prefetch(blockIdx.x);
 #pragma unroll 1
   for (int it = blockIdx.x; it < total; it += gridDim.x) {
     if (it + int(gridDim.x) >= total) grid_dep_trigger();  // last item of this CTA
     const int mi = it / items, item = it - mi * items;
     const Member mb = member_at(mem, mi);
-    const cpx<R>* __restrict__ H = ws_ptr<cpx<R>>(mb, offH);
     const int pr = item * PER + rr;
     const bool valid = pr < pairs;
     const int row = 2 * pr;
-    if constexpr (PF) {
-      cp_async_wait_all();
-      __syncthreads();  // the item's segments have landed
-    }
+    cp_async_wait_all();
+    __syncthreads();  // the item's segments have landed
     cpx<R> v[16];
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
@@ -267,7 +245,7 @@ k_std_row_inv(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restric
       const int qq = hi ? N - q : q;
       cpx<R> ya = mk<R>(R(0), R(0)), yb = ya;
       if (valid) {
-        const cpx<R>* src = PF ? land + 2 * (rr * HS + qq) : H + Tile<R>::at(row, qq, ldq);
+        const cpx<R>* src = land + 2 * (rr * HS + qq);
         ya = src[0];
         yb = src[1];
       }
@@ -277,11 +255,9 @@ k_std_row_inv(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restric
       }
       v[m] = mk<R>(ya.x - yb.y, ya.y + yb.x);  // Y_a + i Y_b
     }
-    if constexpr (PF) {
-      __syncthreads();  // every thread has read the landing buffer
-      if (it + int(gridDim.x) < total) prefetch(it + gridDim.x);
-    }
-    block_fft_regs<R, LOG2N, PF>(v, buf, t, stw, cj == 0);
+    __syncthreads();  // every thread has read the landing buffer
+    if (it + int(gridDim.x) < total) prefetch(it + gridDim.x);
+    block_fft_regs<R, LOG2N, true>(v, buf, t, stw, cj == 0);
     if (valid) {
 #pragma unroll
       for (int m = 0; m < 16; ++m) {

@@ -116,3 +116,42 @@ def test_batch_members_keep_their_own_scale():
     b.close()
     for p in plans:
         p.close()
+
+
+@pytest.mark.parametrize("mult", [DS, (0, -0.5, -0.3, 0.4), (1, 1.0, 0.2, -0.5), (-1, 2 * np.pi, 0.0, 0.0)])
+@pytest.mark.parametrize("nx,ny,kind", [(n, m, k) for n, m in GRIDS for k in ("noise", "rows")] + [(64, 512, "points")])
+def test_standard_solver_matches_the_oracle(nx, ny, kind, mult):
+    rho = _field(kind, nx, ny)
+    ref = oracle.standard_fft_solve(rho, 4.0, 5.0, multiplier=mult)
+    phi, adj = _solve(rho, multiplier=mult, nx=nx, ny=ny, lx=4.0, ly=5.0, partition="none")
+    assert _rel(phi, ref) <= TOL
+    assert _rel(adj, ref) <= TOL
+
+
+@pytest.mark.parametrize("nx,ny", GRIDS)
+def test_linear_flow_matches_numpy(nx, ny):
+    """u -> F^-1[e^{-i tau (kx^2 - alpha ky^2)} F u] and its inverse.  Tolerance: FP64 rounding of two 2D
+    transforms (about 1e-15) plus the phase's own, eps times its largest angle."""
+    from paper_1409_2014_gb300.ds import DSPlan
+
+    tau, alpha = 0.7e-3, 1.3
+    ds = DSPlan(nx, ny, 4.0, 5.0, precision="fp64")
+    for kind in ("noise", "rows", "points"):
+        im = synth.normal_field(nx, ny, seed=7) * (1e-3 if kind == "points" else 1.0)
+        u = _field(kind, nx, ny) + 1j * im
+        kx = 2 * np.pi * np.fft.fftfreq(nx, 8.0 / nx)[None]
+        ky = 2 * np.pi * np.fft.fftfreq(ny, 10.0 / ny)[:, None]
+        ang = tau * (kx ** 2 - alpha * ky ** 2)
+        ref = np.fft.ifft2(np.fft.fft2(u) * np.exp(-1j * ang))
+        tol = 1e-14 + 4 * np.finfo(float).eps * np.abs(ang).max()
+        ds.set_linear_step(tau, alpha)
+        v = ds.linear_(torch.from_numpy(u).cuda())
+        assert np.linalg.norm(v.cpu().numpy() - ref) <= tol * np.linalg.norm(ref)
+        back = ds.linear_(v, adjoint=True).cpu().numpy()
+        assert np.linalg.norm(back - u) <= 2 * tol * np.linalg.norm(u)
+    for z in (0.0, np.nan, np.inf):
+        w = torch.zeros((ny, nx), dtype=torch.complex128, device="cuda")
+        w[1, 2] = z
+        w = ds.linear_(w)
+        assert bool(torch.isnan(w.real).all()) if z != 0.0 else not bool(w.abs().any())
+    ds.close()
