@@ -128,10 +128,10 @@ typedef struct {
  * The spreading tile configuration is chosen by timing the candidates on the
  * device (temporary scratch, cached per device and parameters for the
  * process); DSNU_AUTOTUNE=0 in the environment keeps the default one.
- * Plans with the DS multiplier also tabulate the column multiplier
- * m1(q_x, |qbar_y|) of I1 on the device in FP64, stored in the plan's
- * precision ((nx + 1) (ny + 4) entries: 67 MB mixed, 134 MB FP64 at
- * 4096 x 4096).
+ * The column multiplier m1(q_x, |qbar_y|) of I1 is tabulated on the device in
+ * FP64 and stored in FP32 or, for FP64 plans, in 64-bit fixed point ((nx + 1)
+ * (ny + 4) entries: 67 MB mixed, 134 MB FP64 at 4096 x 4096; twice that for
+ * multipliers with a_sin != 0; FP64 standard plans (nx/2 + 1)(ny/2 + 1) entries).
  * Ownership: the plan owns its tables (device memory, freed by
  * dsnu_plan_destroy); it does not own the workspace.
  * Errors: DSNU_EINVAL (bad params, *out untouched), DSNU_ENOMEM, DSNU_ECUDA. */
@@ -159,13 +159,13 @@ size_t dsnu_workspace_bytes(dsnu_plan plan);
 dsnu_status dsnu_set_workspace(dsnu_plan plan, void* workspace_dev, size_t bytes);
 
 /* Phi = I1 + I2 (Sec. 2.1, eq. PotSplitWhoSpace) for one density.
- * For mixed plans on grids of at least 2048 x 2048 the band chain (the NUFFT
- * part) runs on a low-priority stream owned by the plan, concurrently with the
- * column pass of I1, which then leaves 12 of every 152 SMs free
- * (DSNU_BAND_SMS=<n> in the environment at plan creation sets the number of
- * SMs, 0 runs everything on `stream`); the plan orders that stream after
- * `stream`'s earlier work and `stream` after it, so the call behaves as if
- * everything ran on `stream`.
+ * The band chain (the NUFFT part) and the column pass of I1 run side by side,
+ * one of them on a low-priority stream owned by the plan (the band chain on
+ * grids of at least 2048 x 2048, the column pass on smaller ones), the column
+ * pass leaving a number of SMs free (DSNU_BAND_SMS=<n> in the environment at
+ * plan creation sets it, 0 runs everything on `stream`); the plan orders that
+ * stream after `stream`'s earlier work and `stream` after it, so the call
+ * behaves as if everything ran on `stream`.
  * rho_dev: [ny][nx] FP64 density (device, read only).
  * phi_dev: [ny][nx] FP64 potential (device, written); must not alias rho_dev.
  * Both 16-byte aligned (every cudaMalloc'd or torch-allocated buffer is).

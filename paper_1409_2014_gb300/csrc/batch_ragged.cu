@@ -52,7 +52,7 @@ struct RagGroup {
   Members mem;
   WsOff off;
   AxisTabs<float> ax, ay;
-  MultTabs<float> mt;
+  MultRows<float> mt;
   const float* decon_y;
   float scale;
   int* status;
@@ -63,7 +63,7 @@ struct RagGroup {
   const int* itile_ptr;    // the plan's interpolation items (k_interp_tile)
   const int2* itile_org;
   const int* itile_nodes;
-  int n_nodes, w;
+  int n_nodes, w, n_half;
   const int2* item_range;
   const int* ent_node;
   const int2* ent_q0;
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(256) k_rag_interp(const __grid_constant__ RagT
   rag_numbered(T, RS_INTERP, &g, &bx, &mi);
   const RagGroup& a = T.g[g];
   interp_tile_body<float>(bx, mi, a.mem, a.off, a.ldq, a.Q, a.node_q0, a.node_w, a.node_D, a.itile_ptr, a.itile_org,
-                          a.itile_nodes, a.w, 0);
+                          a.itile_nodes, a.w, a.n_half, 0);
 }
 
 template <int TILE, int SPLIT, int CHUNK>
@@ -306,10 +306,7 @@ dsnu_status ragged_create(const RaggedGroupIn* groups, int n, Ragged** out) {
     a.ay = AxisTabs<float>{static_cast<const cpx<float>*>(t.stw_y), static_cast<const cpx<float>*>(t.twm_lo_y),
                            static_cast<const cpx<float>*>(t.twm_hi_y), g.log2lo_y,
                            static_cast<const float*>(t.decon_y), nullptr};
-    a.mt = MultTabs<float>{static_cast<const float*>(t.m_wx2), static_cast<const float*>(t.m_gx),
-                           float(-g.dky2 / (g.sigma * g.sigma) * 1.4426950408889634), float(g.dky2), g.ny, g.sharp,
-                           float(g.cut_radius * g.cut_radius), 0, 0, 0.f, 0.f, 0.f, float(std::sqrt(g.dky2)),
-                           static_cast<const float*>(t.m_kx), static_cast<const float*>(t.m1tab), g.ny + 4};
+    a.mt = MultRows<float>{static_cast<const float*>(t.m1tab), g.m1_ld};
     a.decon_y = static_cast<const float*>(t.decon_y);
     a.scale = float(g.scale);
     a.status = t.status;
@@ -331,6 +328,7 @@ dsnu_status ragged_create(const RaggedGroupIn* groups, int n, Ragged** out) {
     a.itile_nodes = t.itile_nodes;
     a.n_nodes = g.n_nodes;
     a.w = g.w;
+    a.n_half = g.n_half;
     a.item_range = t.item_range;
     a.ent_node = t.ent_node;
     a.ent_q0 = t.ent_q0;

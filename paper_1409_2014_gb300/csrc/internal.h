@@ -27,25 +27,22 @@ struct PlanTables {
   void* twm_lo_y;
   void* twm_hi_y;
   void* decon_y;
-  void* m_wx2;    // real, nx + 1  (q_x dk_x)^2
-  void* m_gx;     // real, nx + 1  1 - exp(-(q_x dk_x)^2/sigma^2)
-  void* m_kx;     // real, k_x per column for the sin 2theta term (0 at the Nyquist column); generic only
+  void* m_wx2;    // standard solver, real, nx/2 + 1: (q_x dk_x)^2
+  void* m_kx;     // standard solver, real: k_x per column for the sin 2theta term (0 at the Nyquist column)
   int2* node_q0;  // n_nodes
   int* itile_ptr;   // n_itiles + 1: interpolation item -> range of itile_nodes
   int2* itile_org;  // n_itiles: the item's tile's first (q_x, q_y) (its nodes' stencil origins from there)
-  int* itile_nodes; // n_nodes: node indices grouped by the tile of their stencil origin
-  void* node_w;   // real, n_nodes * 2w (x weights then y weights)
+  int* itile_nodes; // n_nodes/2: indices of the nodes with theta < pi, grouped by the tile of their stencil origin
+  void* node_w;   // real, n_nodes * 2w (x weights then y weights); FP64 plans: {wh, wl} (spread_fx.cuh)
   double* node_D; // n_nodes
   int* tile_items;  // n_tiles + 1: spreading tile -> range of work items
   int2* item_range; // per work item: [first, end) entry
   int* item_tile;   // per work item: its tile
   int* ent_node;  // per entry: node index
   int2* ent_q0;   // per entry: stencil origin of the node
-  void* ent_w;    // real, per entry: the node's 2w ES weights
+  void* ent_w;    // per entry: the node's 2w ES weights, as in node_w
   int* status;    // one int
-  void* m1tab;    // split plans with the DS multiplier: m1(q_x, |qbar_y|) in the plan's precision,
-                  // (nx + 1) rows of ny + 4 entries, each row's even |qbar_y| first (MultTabs::m1); else NULL
-                  // FP64 plans: fxr entries for every multiplier (FxMult)
+  void* m1tab;    // split plans: the multiplier rows (MultRows), in fixed point in FP64 plans (FxMult, both solvers)
   // FP64 plans: the fixed-point tables of both axes (fx.cuh, FxAxis) and the
   // multiplier's exponent per column (generic multipliers, else NULL)
   void *fx_stw_x, *fx_wm_x, *fx_dec_x, *fx_stw_y, *fx_wm_y, *fx_dec_y;
@@ -84,10 +81,12 @@ struct PlanGeom {
   int cap_rowf, cap_col, cap_bandf, cap_bandi, cap_rowi;  // resident CTAs (SMs x occupancy)
   int rowi_bpf;            // inverse row pass prefetches the band values too (FP32)
   int row_pf;              // bit 0 forward row prefetch, bit 1 inverse, bit 2 rowi_bpf
+  int sms;                 // multiprocessors of the plan's device
   size_t smem_rowi;        // its dynamic shared memory per CTA
   int kdx, kdy;            // FP64 plans: 2^kd > the axis' largest deconvolution factor
-  int m1_full, m1_ld;      // FP64 plans: the multiplier rows hold all M_y frequencies (else |qbar_y| <= N_y); entries per row
+  int m1_full, m1_ld;      // the multiplier rows hold all frequencies (else |qbar_y| only); entries per row
   int w, Q, n_nodes, n_tiles, tiles_x, tiles_y, max_tile_nodes, n_items;
+  int n_half;              // n_theta/2: the distance of the nodes k and -k in a ring
   int n_itiles;            // interpolation items (at most kItileNodes nodes of one kItile x kItile tile)
   int spread_cfg;          // index into kSpreadCfgs (chosen by the autotuner)
   int spread_tile;         // its tile edge (cells)
@@ -105,13 +104,15 @@ struct PlanGeom {
 constexpr int kStages = 8;       // kernels per solve
 constexpr int kProfEvents = kStages + 1;  // events per profiled solve (see run_pipeline)
 
-// Concurrency of the band chain with the column pass: the band kernels run
-// on `side` (a low-priority stream owned by the plan) while the column pass's
-// persistent grid leaves `reserve` SMs free for them.
+// Concurrency of the band chain with the column pass: one of the two runs on
+// `side` (a low-priority stream owned by the plan): the band chain, or with
+// col_side the column pass, whose persistent grid leaves `reserve` SMs free.
 struct Overlap {
   cudaStream_t side;
   cudaEvent_t fork, join;
   int reserve;
+  int col_side;
+  bool on;
 };
 
 // Launchers (one translation unit per precision).  `ev`, when not NULL,

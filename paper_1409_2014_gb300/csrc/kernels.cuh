@@ -104,26 +104,29 @@ __device__ __forceinline__ cpx<R> twm(const AxisTabs<R>& a, int n) {
   return cmul(a.twm_hi[n >> a.log2lo], a.twm_lo[n & ((1 << a.log2lo) - 1)]);
 }
 
+// The split solver's multiplier: m1 = m (1 - p) tabulated in FP64 at plan
+// creation (one rounding to FP32), one row of ldm entries per column.  The rows
+// are parity-split: with a = |qbar_y| the even a first (a = 2 j at j) and the odd
+// a after them (a = 2 j' + 1 at N_y/2 + 1 + j'); FULL rows (multipliers with a
+// sin 2theta term) hold the M_y natural frequencies instead (q = 2 j at j, q =
+// 2 j' + 1 at N_y + j').
+template <typename R>
+struct MultRows {
+  const R* m1;
+  int ldm;
+};
+
+// The standard solver's multiplier, evaluated in its column pass.
 template <typename R>
 struct MultTabs {
-  const R* wx2;       // (q_x dk_x)^2, q_x in [0, nx]
-  const R* gx;        // 1 - exp(-(q_x dk_x)^2 / sigma^2)
-  R neg_dky2_s2_log2e;  // -dk_y^2 / (sigma^2 ln 2)
+  const R* wx2;       // (q_x dk_x)^2, q_x in [0, nx/2]
   R dky2;             // dk_y^2
-  int half_my;        // N_y (= M_y / 2)
-  int sharp;          // 1: p = indicator of |k| <= P
-  R cut2;             // P^2
   // another multiplier |k|^alpha (a0 + ac cos 2theta + as sin 2theta) when
   // `generic` (the DS one, -k_x^2/|k|^2, otherwise)
   int generic, alpha;
   R a0, ac, as2;      // as2 = 2 as
   R dky;              // dk_y
   const R* kx;        // k_x of column q_x for the sin 2theta term (0 at the Nyquist column)
-  // plans with the DS multiplier: m1(q_x, a) for a = |qbar_y| <= N_y,
-  // computed in FP64 at plan creation (one rounding to FP32), one row of ldm
-  // entries per column with the even a first (a = 2 j at j) and the odd a after them (a = 2 j' + 1 at N_y/2 + 1 + j')
-  const R* m1;
-  int ldm;
 };
 
 // The angular and radial factor of the generic multiplier at (k_x, qbar_y):
@@ -139,32 +142,6 @@ __device__ __forceinline__ R mult_generic(const MultTabs<R>& mt, R wx2, R wy2, R
   if (mt.alpha == 1) rad = sqrt(s);
   else if (mt.alpha == -1) rad = R(1) / sqrt(s);
   return rad * ang;
-}
-
-// m1 = -(k_x^2/|k|^2) (1 - p(k)), m1(0) = 0, at column q_x and natural row
-// frequency q (signed qbar = q or q - M_y).  With the Gaussian partition
-// 1 - p = 1 - e^{-kx^2/s^2} e^{-ky^2/s^2} = gx + gy (1 - gx), a sum of
-// non-negative terms (no cancellation near k = 0).
-template <bool GEN, typename R>
-__device__ __forceinline__ R mult_high(const MultTabs<R>& mt, R wx2, R kx, R gx, int q) {
-  const int a = (q < mt.half_my) ? q : 2 * mt.half_my - q;
-  const R wy2 = R(a * a) * mt.dky2;
-  const R s = wx2 + wy2;
-  if (s == R(0)) return R(0);
-  R part;
-  if (mt.sharp) {
-    part = (s > mt.cut2) ? R(1) : R(0);
-  } else {
-    // 1 - e^{-kx^2/s^2} e^{-ky^2/s^2} with e^{-ky^2/s^2} = 2^{-a^2 dk^2 / (s^2 ln 2)}
-    // (hardware exp2): absolute error ~1e-7, at the level of FP32 rounding of m1
-    const R ey = exp2f(R(a * a) * mt.neg_dky2_s2_log2e);
-    part = R(1) - (R(1) - gx) * ey;
-  }
-  if constexpr (GEN)
-    return mult_generic(mt, wx2, wy2, kx, (q < mt.half_my) ? q : (q == mt.half_my ? 0 : q - 2 * mt.half_my), s) *
-           part;
-  else
-    return -fdiv(wx2, s) * part;
 }
 
 // Workspace offsets (bytes) of one member's buffers, and member access.
@@ -256,13 +233,13 @@ struct Geo {
   static constexpr int MINB_F = (T_RF >= 512) ? 1 : DSNU_ROW_MINB;
   static constexpr int MINB_I = (T_RI >= 512) ? 1 : DSNU_ROW_MINB;
   static constexpr size_t smem_col = size_t(STWP + 2 * CC * FB) * sizeof(cpx<R>);  // two chains
-  // FP32 column pass of I1 with the DS multiplier: two shared tables on top,
-  // e^{-2 pi i n/M} (n < N) and {(a dk_y)^2, e^{-(a dk_y)^2/sigma^2}} (a <= N)
+  // FP32 column pass of I1: on top the table e^{-2 pi i n/M} (n < N)
   static constexpr bool COL_TAB = sizeof(R) == 4;
-  // and two buffers of CC multiplier rows (N + 4 floats each), the current
-  // item's and the next one's
+  // and two buffers of CC multiplier rows (N + 4 floats each, M for FULL ones),
+  // the current item's and the next one's
   static constexpr int LDM = N + 4;
   static constexpr size_t smem_col_main = smem_col + (COL_TAB ? size_t(N) * 8 + size_t(2 * CC * LDM) * 4 : 0);
+  static constexpr size_t smem_col_full = smem_col + (COL_TAB ? size_t(N) * 8 + size_t(2 * CC * M) * 4 : 0);
   static_assert(LOG2N >= 4 && LOG2N <= 12, "grid size 16..4096");
 };
 
@@ -452,17 +429,17 @@ k_row_fwd(Members mem, WsOff off, int ldqA, int ldqB, int Q, int ny, AxisTabs<R>
 // padded column DFT) go forward together, are multiplied by m1 and come back
 // together; their sum is the column of I1's inverse.  All loads of a column
 // precede the first barrier, so the in-place update is safe.
-template <typename R, int LOG2N, bool GEN>
+template <typename R, int LOG2N, bool FULL>
 __device__ __forceinline__ void col_main_body(int vb, int vg, Members mem, WsOff off, int ldqA, int ncols,
-                                              AxisTabs<R> ay, MultTabs<R> mt, int cj, int* ctr) {
+                                              AxisTabs<R> ay, MultRows<R> mt, int cj, int* ctr) {
   using GG = Geo<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, CC = GG::CC, FB = GG::FB;
-  // FP32 with the DS multiplier: the e^{-2 pi i n/M} factors of the odd chain
-  // come from a shared table filled once per CTA with the arithmetic of twm(),
-  // and m1 of the item's columns from the plan's FP64-computed table, copied
-  // row by row into shared memory (cp.async) one item ahead
-  constexpr bool TAB = GG::COL_TAB && !GEN;
-  constexpr int LDM = GG::LDM;
+  // the e^{-2 pi i n/M} factors of the odd chain come from a shared table filled
+  // once per CTA with the arithmetic of twm(), and m1 of the item's columns from
+  // the plan's FP64-computed table, copied row by row into shared memory
+  // (cp.async) one item ahead (coulomb 2 pi/|k| on 2048 x 512: evaluated per
+  // element the pass took 33 us, from the table 19)
+  constexpr int LDM = FULL ? GG::M : GG::LDM;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* stw = reinterpret_cast<cpx<R>*>(smem_raw);
   cpx<R>* sm = stw + GG::STWP;
@@ -472,12 +449,11 @@ __device__ __forceinline__ void col_main_body(int vb, int vg, Members mem, WsOff
   const R isg = cj ? R(-1) : R(1);
   cpx<R>* buf_e = sm + (2 * cl) * FB;
   cpx<R>* buf_o = buf_e + FB;
-  cpx<R>* wtab = sm + 2 * CC * FB;                       // N entries (TAB only)
-  // TAB: buffer b holds the m1 rows of an item's CC columns; a warp reads a's
-  // of one parity (a = |qbar| of the rows 2 (t + G m) + h), so consecutive
-  // entries of the parity-split rows
+  cpx<R>* wtab = sm + 2 * CC * FB;                       // N entries
+  // buffer b holds the m1 rows of an item's CC columns; a warp reads entries of
+  // one parity (rows 2 (t + G m) + h), so consecutive ones
   float* mrow = reinterpret_cast<float*>(wtab + N);
-  constexpr int MH = N / 2 + 1;  // even entries
+  constexpr int MH = FULL ? N : N / 2 + 1;  // even entries
   const int items = (ncols + CC - 1) / CC;
   const int total = items * mem.count;
   // every thread: its share of the m1 rows of item it2 into buffer b
@@ -490,15 +466,13 @@ __device__ __forceinline__ void col_main_body(int vb, int vg, Members mem, WsOff
     }
     cp_async_commit();
   };
-  if constexpr (TAB) {
-    for (int i = tid; i < N; i += GG::T_C) wtab[i] = twm(ay, i);
-    if (vb < total) fetch_mult(vb, 0);  // (a plan table: no wait needed)
-    __syncthreads();
-  }
+  for (int i = tid; i < N; i += GG::T_C) wtab[i] = twm(ay, i);
+  if (vb < total) fetch_mult(vb, 0);  // (a plan table: no wait needed)
+  __syncthreads();
   grid_dep_wait();
   // the next item's column values are loaded into registers before the
   // current item's inverse transform (PF), hiding their latency
-  constexpr bool PF = TAB && DSNU_COL_REGPF;
+  constexpr bool PF = DSNU_COL_REGPF;
   cpx<R> xn[PF ? 16 : 1];
   auto load_col = [&](int it2, cpx<R>(&x)[PF ? 16 : 1]) {
     const int mi2 = it2 / items;
@@ -534,12 +508,9 @@ __device__ __forceinline__ void col_main_body(int vb, int vg, Members mem, WsOff
     cpx<R>* __restrict__ A = ws_ptr<cpx<R>>(member_at(mem, mi), off.A);
     const int col = item * CC + cl;
     const bool valid = col < ncols;
-    const R wx2 = (!TAB && valid) ? mt.wx2[col] : R(0);
-    const R gx = (!TAB && valid) ? mt.gx[col] : R(0);
-    const R kxc = (GEN && valid) ? mt.kx[col] : R(0);
     // this thread's copies of the item's m1 rows have landed; the barriers of
     // the forward transform below make every thread's copies visible
-    if constexpr (TAB) cp_async_wait_all();
+    cp_async_wait_all();
     const float* mr = mrow + ((kk & 1) * CC + cl) * LDM;
     cpx<R> e[16], o[16];
 #pragma unroll
@@ -548,9 +519,7 @@ __device__ __forceinline__ void col_main_body(int vb, int vg, Members mem, WsOff
       cpx<R> x;
       if constexpr (PF) x = xn[m];
       else x = valid ? A[Tile<R>::at(n, col, ldqA)] : mk<R>(R(0), R(0));
-      cpx<R> w;
-      if constexpr (TAB) w = wtab[n];
-      else w = twm(ay, n);
+      cpx<R> w = wtab[n];
       w.y *= isg;
       e[m] = x;
       o[m] = cmul(x, w);
@@ -558,37 +527,24 @@ __device__ __forceinline__ void col_main_body(int vb, int vg, Members mem, WsOff
     block_fft2_regs<R, LOG2N>(e, o, buf_e, buf_o, t, stw, cj != 0);
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
-      const int q = 2 * (t + G * m);
-      if constexpr (TAB) {
-        // m1 at rows q and q + 1 (a = |qbar|, of the parity of q + h)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int qq = q + h;
-          const int a = (qq < N) ? qq : 2 * N - qq;
-          const R mv = valid ? mr[(h ? MH : 0) + (a >> 1)] : R(0);
-          if (h == 0) e[m] = e[m] * mv;
-          else o[m] = o[m] * mv;
-        }
-      } else {
-        e[m] = e[m] * (valid ? mult_high<GEN>(mt, wx2, kxc, gx, q) : R(0));
-        o[m] = o[m] * (valid ? mult_high<GEN>(mt, wx2, kxc, gx, q + 1) : R(0));
-      }
+      // m1 at the rows 2 k and 2 k + 1 (the entries of |qbar|, or of q itself)
+      const int k = t + G * m;
+      const int ke = (FULL || m < 8) ? k : N - k, ko = (FULL || m < 8) ? k : N - 1 - k;
+      e[m] = e[m] * (valid ? mr[ke] : R(0));
+      o[m] = o[m] * (valid ? mr[MH + ko] : R(0));
     }
     if (ctr && tid == 0) s_next[(kk + 1) & 1] = grabbed;
     if constexpr (PF)
       if (nxt < total) load_col(nxt, xn);
     // the next item's m1 rows into the other buffer (last read by the item
     // before this one, whose reads the barriers since then have completed)
-    if constexpr (TAB)
-      if (nxt < total) fetch_mult(nxt, (kk + 1) & 1);
+    if (nxt < total) fetch_mult(nxt, (kk + 1) & 1);
     block_fft2_regs<R, LOG2N>(e, o, buf_e, buf_o, t, stw, cj == 0);
     if (valid) {
 #pragma unroll
       for (int m = 0; m < 16; ++m) {
         const int n = t + G * m;
-        cpx<R> w;
-        if constexpr (TAB) w = wtab[n];
-        else w = twm(ay, n);
+        const cpx<R> w = wtab[n];
         A[Tile<R>::at(n, col, ldqA)] = cj ? e[m] + cmul(o[m], w) : e[m] + cmulc(o[m], w);
       }
     }
@@ -597,10 +553,10 @@ __device__ __forceinline__ void col_main_body(int vb, int vg, Members mem, WsOff
   }
 }
 
-template <typename R, int LOG2N, bool GEN>
+template <typename R, int LOG2N, bool FULL>
 __global__ void __launch_bounds__(Geo<R, LOG2N>::T_C, min_blocks<R>(DSNU_COLMAIN_MINB))
-k_col_main(Members mem, WsOff off, int ldqA, int ncols, AxisTabs<R> ay, MultTabs<R> mt, int cj) {
-  col_main_body<R, LOG2N, GEN>(blockIdx.x, gridDim.x, mem, off, ldqA, ncols, ay, mt, cj,
+k_col_main(Members mem, WsOff off, int ldqA, int ncols, AxisTabs<R> ay, MultRows<R> mt, int cj) {
+  col_main_body<R, LOG2N, FULL>(blockIdx.x, gridDim.x, mem, off, ldqA, ncols, ay, mt, cj,
                                ws_ptr<int>(member_at(mem, 0), off.sched));
 }
 
@@ -665,8 +621,10 @@ k_band_fwd(Members mem, WsOff off, int ldqB, int ncols, int ldq, int Q, AxisTabs
 
 // ---------------------------------------------------------------------------
 // Type-2 interpolation (eq. 2.2) and the polar weighting c_j = D_j rho_hat_j
-// (eq. I2PolarDisc, FP64 multiply), by tiles of stencil origins: the plan
-// groups the nodes by the kItile x kItile tile of the (q_x, q_y) plane that
+// (eq. I2PolarDisc, FP64 multiply), by tiles of stencil origins.  The nodes come
+// in pairs k and -k (n_half = n_theta/2 apart in a ring) whose values, the
+// density being real, are conjugates, with equal D: one of each pair (theta <
+// pi) is interpolated.  The plan groups those nodes by the kItile x kItile tile of the (q_x, q_y) plane that
 // holds their stencil origin, in work items of at most kItileNodes nodes of
 // one tile; one CTA per item copies the (kItile + w - 1)^2 band values its
 // stencils reach into shared memory (whole band columns' runs, read
@@ -685,7 +643,7 @@ __device__ __forceinline__ void interp_tile_body(int tile, int mi, Members mem, 
                                                  const int2* __restrict__ q0, const R* __restrict__ wts,
                                                  const double* __restrict__ D, const int* __restrict__ tile_ptr,
                                                  const int2* __restrict__ tile_org,
-                                                 const int* __restrict__ tile_nodes, int w, int cj) {
+                                                 const int* __restrict__ tile_nodes, int w, int n_half, int cj) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* reg = reinterpret_cast<cpx<R>*>(smem_raw);  // [dx][dy], S x S
   const int S = kItile + w - 1;
@@ -739,15 +697,20 @@ __device__ __forceinline__ void interp_tile_body(int tile, int mi, Members mem, 
   ax += __shfl_xor_sync(0xffffffffu, ax, 2);
   ay += __shfl_xor_sync(0xffffffffu, ay, 2);
   // the four partial sums of a node (lanes 4 s' .. 4 s' + 3 of the warp)
-  if (have && h == 0) c[j] = mk<R>(R(d * double(ax)), R(d * double(ay)));
+  if (have && h == 0) {
+    const cpx<R> v = mk<R>(R(d * double(ax)), R(d * double(ay)));
+    c[j] = v;
+    c[j + n_half] = conj(v);
+  }
 }
 
 template <typename R>
 __global__ void __launch_bounds__(256)
 k_interp_tile(Members mem, WsOff off, int ldq, int Q, const int2* __restrict__ q0, const R* __restrict__ wts,
               const double* __restrict__ D, const int* __restrict__ tile_ptr, const int2* __restrict__ tile_org,
-              const int* __restrict__ tile_nodes, int w, int cj) {
-  interp_tile_body<R>(blockIdx.x, blockIdx.y, mem, off, ldq, Q, q0, wts, D, tile_ptr, tile_org, tile_nodes, w, cj);
+              const int* __restrict__ tile_nodes, int w, int n_half, int cj) {
+  interp_tile_body<R>(blockIdx.x, blockIdx.y, mem, off, ldq, Q, q0, wts, D, tile_ptr, tile_org, tile_nodes, w, n_half,
+                      cj);
 }
 inline size_t interp_tile_smem(int w, size_t csz) { return size_t(kItile + w - 1) * size_t(kItile + w - 1) * csz; }
 

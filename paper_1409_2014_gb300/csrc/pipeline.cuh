@@ -1,6 +1,7 @@
 // pipeline.cuh -- launch sequence of one solve (included once per precision).
 #pragma once
 
+#include <algorithm>
 #include <cmath>
 
 #include "internal.h"
@@ -68,11 +69,11 @@ cudaError_t prepare_cols(PlanGeom& g) {
   cudaError_t e;
   const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if ((e = cudaFuncSetAttribute(k_col_main<R, L2, false>, A, int(GG::smem_col_main)))) return e;
-  if ((e = cudaFuncSetAttribute(k_col_main<R, L2, true>, A, int(GG::smem_col_main)))) return e;
+  if ((e = cudaFuncSetAttribute(k_col_main<R, L2, true>, A, int(GG::smem_col_full)))) return e;
   if ((e = cudaFuncSetAttribute(k_band_fwd<R, L2>, A, int(GG::smem_col)))) return e;
   if ((e = cudaFuncSetAttribute(k_band_inv<R, L2>, A, int(GG::smem_col)))) return e;
-  if ((e = g.m_generic ? resident_ctas(k_col_main<R, L2, true>, GG::T_C, GG::smem_col_main, &g.cap_col)
-                       : resident_ctas(k_col_main<R, L2, false>, GG::T_C, GG::smem_col_main, &g.cap_col)))
+  if ((e = g.m1_full ? resident_ctas(k_col_main<R, L2, true>, GG::T_C, GG::smem_col_full, &g.cap_col)
+                     : resident_ctas(k_col_main<R, L2, false>, GG::T_C, GG::smem_col_main, &g.cap_col)))
     return e;
   if ((e = resident_ctas(k_band_fwd<R, L2>, GG::T_C, GG::smem_col, &g.cap_bandf))) return e;
   return resident_ctas(k_band_inv<R, L2>, GG::T_C, GG::smem_col, &g.cap_bandi);
@@ -216,11 +217,7 @@ dsnu_status run_pipeline(const PlanGeom& g, const PlanTables& t, const WsLayout&
   const AxisTabs<R> ay{static_cast<const cpx<R>*>(t.stw_y), static_cast<const cpx<R>*>(t.twm_lo_y),
                        static_cast<const cpx<R>*>(t.twm_hi_y), g.log2lo_y, static_cast<const R*>(t.decon_y),
                        nullptr};
-  const MultTabs<R> mt{static_cast<const R*>(t.m_wx2), static_cast<const R*>(t.m_gx),
-                       R(-g.dky2 / (g.sigma * g.sigma) * 1.4426950408889634), R(g.dky2), g.ny, g.sharp,
-                       R(g.cut_radius * g.cut_radius), g.m_generic, g.m_alpha, R(g.m_a0), R(g.m_ac),
-                       R(2.0 * g.m_as), R(std::sqrt(g.dky2)), static_cast<const R*>(t.m_kx),
-                       static_cast<const R*>(t.m1tab), g.ny + 4};
+  const MultRows<R> mt{static_cast<const R*>(t.m1tab), g.m1_ld};
   const R* dcy = static_cast<const R*>(t.decon_y);
   const R* wts = static_cast<const R*>(t.node_w);
   const int ldqA = L.ldqA, ldqB = L.ldqB;
@@ -232,14 +229,14 @@ dsnu_status run_pipeline(const PlanGeom& g, const PlanTables& t, const WsLayout&
            dim3(Geo<R, L2>::T_RF), Geo<R, L2>::smem_row_fwd, st, mem, off, ldqA, ldqB, g.Q, g.ny, ax, dcy, cj, \
            t.status)
 #define DSNU_COLM(L2)                                                                               \
-  if (g.m_generic)                                                                                  \
+  if (g.m1_full)                                                                                    \
     launch_k(g.pdl != 0, k_col_main<R, L2, true>,                                                   \
              dim3(persistent_grid(nm * ((g.nx + 1 + Geo<R, L2>::CC - 1) / Geo<R, L2>::CC), capc)), \
-             dim3(Geo<R, L2>::T_C), Geo<R, L2>::smem_col_main, st, mem, off, ldqA, g.nx + 1, ay, mt, cj); \
+             dim3(Geo<R, L2>::T_C), Geo<R, L2>::smem_col_full, cst, mem, off, ldqA, g.nx + 1, ay, mt, cj); \
   else                                                                                              \
     launch_k(g.pdl != 0, k_col_main<R, L2, false>,                                                  \
              dim3(persistent_grid(nm * ((g.nx + 1 + Geo<R, L2>::CC - 1) / Geo<R, L2>::CC), capc)), \
-             dim3(Geo<R, L2>::T_C), Geo<R, L2>::smem_col_main, st, mem, off, ldqA, g.nx + 1, ay, mt, cj)
+             dim3(Geo<R, L2>::T_C), Geo<R, L2>::smem_col_main, cst, mem, off, ldqA, g.nx + 1, ay, mt, cj)
 #define DSNU_BANDF(L2)                                                                              \
   launch_k(g.pdl != 0, k_band_fwd<R, L2>,                                                           \
            dim3(persistent_grid(nm * ((g.Q + 1 + Geo<R, L2>::CC - 1) / Geo<R, L2>::CC), g.cap_bandf)), \
@@ -256,8 +253,8 @@ dsnu_status run_pipeline(const PlanGeom& g, const PlanTables& t, const WsLayout&
 #define DSNU_MARK(I) \
   if (ev) cudaEventRecord(ev[I], st)
   // the band chain (type-2 columns, interpolation, weighting, spreading,
-  // inverse band columns) on stream bst
-  cudaStream_t bst = st;
+  // inverse band columns) on stream bst, the column pass on cst
+  cudaStream_t bst = st, cst = st;
   int capc = g.cap_col;
   auto band_chain = [&](bool marks) -> dsnu_status {
     switch (g.log2ny) {
@@ -267,7 +264,7 @@ dsnu_status run_pipeline(const PlanGeom& g, const PlanTables& t, const WsLayout&
     if (marks) DSNU_MARK(2);
     launch_k(g.pdl != 0, k_interp_tile<R>, dim3(g.n_itiles, mem.count), dim3(256),
              interp_tile_smem(g.w, sizeof(cpx<R>)), bst, mem, off, L.ldq, g.Q, t.node_q0, wts, t.node_D, t.itile_ptr,
-             t.itile_org, t.itile_nodes, g.w, cj);
+             t.itile_org, t.itile_nodes, g.w, g.n_half, cj);
     if (marks) DSNU_MARK(3);
     launch_spread<R>(g.spread_cfg, mem, off, t, g, L.ldq, cj, bst, 0, g.pdl != 0);
     if (marks) DSNU_MARK(4);
@@ -279,24 +276,24 @@ dsnu_status run_pipeline(const PlanGeom& g, const PlanTables& t, const WsLayout&
     }
     return DSNU_OK;
   };
-  const bool overlap = ov && ov->reserve > 0 && !ev && g.cap_col > ov->reserve;
   DSNU_MARK(0);
   switch (g.log2nx) {
     DSNU_LOG2_CASES(DSNU_ROWF)
     default: return DSNU_EUNSUPPORTED;
   }
   DSNU_MARK(1);
-  if (overlap) {
-    // the column pass keeps all but `reserve` SMs; the band chain runs next
-    // to it on the plan's low-priority side stream; row_inv joins both
+  if (ov && !ev) {
+    // side by side, one of the two on the plan's low-priority side stream (see
+    // dsnu_plan_create), the column pass leaving `reserve` SMs free; row_inv
+    // joins both
     cudaEventRecord(ov->fork, st);
     cudaStreamWaitEvent(ov->side, ov->fork, 0);
-    capc = g.cap_col - ov->reserve;
+    capc = std::max(1, g.cap_col - ov->reserve * (g.cap_col / g.sms));
+    (ov->col_side ? cst : bst) = ov->side;
     switch (g.log2ny) {
       DSNU_LOG2_CASES(DSNU_COLM)
       default: return DSNU_EUNSUPPORTED;
     }
-    bst = ov->side;
     const dsnu_status sb = band_chain(false);
     if (sb != DSNU_OK) return sb;
     cudaEventRecord(ov->join, ov->side);
@@ -330,17 +327,18 @@ dsnu_status run_pipeline(const PlanGeom& g, const PlanTables& t, const WsLayout&
   return DSNU_OK;
 }
 
-template <typename R>
-cudaError_t time_spread(const PlanGeom& g, const PlanTables& t, const WsLayout& L, void* ws, int reps, float* ms) {
+// Average milliseconds of `reps` launches of the spreading pair, launch(members, offsets).
+template <typename F>
+cudaError_t time_spread(const WsLayout& L, void* ws, int reps, float* ms, F launch) {
   const WsOff off{L.off_A, L.off_B, L.off_Bband, L.off_Sband, L.off_c, L.off_partial, L.off_sched};
   const Members mem = single_member(nullptr, nullptr, ws);
   cudaEvent_t e0, e1;
   cudaError_t e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   if (e != cudaSuccess) return e;
-  launch_spread<R>(g.spread_cfg, mem, off, t, g, L.ldq, 0, 0, 2, false);  // warm-up
+  launch(mem, off);  // warm-up
   cudaEventRecord(e0, 0);
-  for (int i = 0; i < reps; ++i) launch_spread<R>(g.spread_cfg, mem, off, t, g, L.ldq, 0, 0, 2, false);
+  for (int i = 0; i < reps; ++i) launch(mem, off);
   cudaEventRecord(e1, 0);
   e = cudaEventSynchronize(e1);
   float total = 0.f;

@@ -1,8 +1,11 @@
 // FP64 (DSNU_FP64) plans: the FFT passes in 64-bit block fixed point
-// (kernels_fx.cuh, standard_fx.cuh), interpolation, weighting and spreading in
-// FP64.
+// (kernels_fx.cuh, standard_fx.cuh), interpolation and spreading sums too
+// (spread_fx.cuh), the polar weighting in FP64.
+#include <algorithm>
+
 #include "kernels_fx.cuh"
 #include "pipeline.cuh"
+#include "spread_fx.cuh"
 #include "standard_fx.cuh"
 
 namespace dsnu {
@@ -112,7 +115,9 @@ dsnu_status run_standard_fx(const PlanGeom& g, const PlanTables& t, const WsLayo
 }  // namespace
 
 cudaError_t prepare_kernels_f64(PlanGeom& g) {
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(k_fx_interp_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       int(interp_fx_smem(16)));
+  if (e != cudaSuccess) return e;
 #define DSNU_PREP_R(L2) e = g.standard ? prepare_fx_std_rows<L2>(g) : prepare_fx_rows<L2>(g)
 #define DSNU_PREP_C(L2) e = g.standard ? prepare_fx_std_cols<L2>(g) : prepare_fx_cols<L2>(g)
   switch (g.log2nx) {
@@ -134,7 +139,6 @@ dsnu_status run_pipeline_f64(const PlanGeom& g, const PlanTables& t, const WsLay
   // the conjugated pipeline of a real input is the conjugate of this one: the
   // same result (kernels_fx.cuh), so `cj` selects nothing
   (void)cj;
-  (void)ov;
   if (g.standard) return run_standard_fx(g, t, L, mem, st, ev);
   const WsOff off{L.off_A, L.off_B, L.off_Bband, L.off_Sband, L.off_c, L.off_partial, L.off_sched};
   const FxOff fo{L.off_A, L.off_B, L.off_Bband, L.off_Sband, L.off_rexp, L.off_rexpb, L.off_cexp, L.off_bexp};
@@ -145,24 +149,23 @@ dsnu_status run_pipeline_f64(const PlanGeom& g, const PlanTables& t, const WsLay
   const FxMult mt{static_cast<const fxr*>(t.m1tab), t.fx_mexp, g.m1_ld};
   const bool pdl = g.pdl != 0;
   const long nm = mem.count;
-  const double* wts = static_cast<const double*>(t.node_w);
   auto grid = [&](long n, int per, int cap) { return dim3(persistent_grid(nm * ((n + per - 1) / per), cap)); };
 #define DSNU_ROWF(L2)                                                                                       \
   launch_k(pdl, k_fx_row_fwd<L2>, grid(g.ny, FxGeo<L2>::PER, g.cap_rowf), dim3(FxGeo<L2>::T), FxGeo<L2>::smem, st, \
            mem, fo, L.ldqA, L.ldqB, g.Q, g.ny, ax, g.kdx)
 #define DSNU_BANDF(L2)                                                                                      \
   launch_k(pdl, k_fx_band_fwd<L2>, grid(g.Q + 1, FxGeo<L2>::PER, g.cap_bandf), dim3(FxGeo<L2>::T), FxGeo<L2>::smem, \
-           st, mem, fo, L.ldqB, g.Q + 1, L.ldq, g.Q, ay, g.kdy)
+           bst, mem, fo, L.ldqB, g.Q + 1, L.ldq, g.Q, ay, g.kdy)
 #define DSNU_BANDI(L2)                                                                                      \
   launch_k(pdl, k_fx_band_inv<L2>, grid(g.Q + 1, FxGeo<L2>::PER, g.cap_bandi), dim3(FxGeo<L2>::T), FxGeo<L2>::smem, \
-           st, mem, fo, L.ldq, g.Q, g.Q + 1, L.ldqB, ay, g.kdy)
+           bst, mem, fo, L.ldq, g.Q, g.Q + 1, L.ldqB, ay, g.kdy)
 #define DSNU_COLM(L2)                                                                                       \
   if (g.m1_full)                                                                                            \
-    launch_k(pdl, k_fx_col_main<L2, true>, grid(g.nx + 1, FxGeo<L2>::PER, g.cap_col), dim3(FxGeo<L2>::T),   \
-             FxGeo<L2>::smem, st, mem, fo, L.ldqA, g.nx + 1, ay, mt);                                       \
+    launch_k(pdl, k_fx_col_main<L2, true>, grid(g.nx + 1, FxGeo<L2>::PER, capc), dim3(FxGeo<L2>::T),   \
+             FxGeo<L2>::smem, cst, mem, fo, L.ldqA, g.nx + 1, ay, mt);                                       \
   else                                                                                                      \
-    launch_k(pdl, k_fx_col_main<L2, false>, grid(g.nx + 1, FxGeo<L2>::PER, g.cap_col), dim3(FxGeo<L2>::T),  \
-             FxGeo<L2>::smem, st, mem, fo, L.ldqA, g.nx + 1, ay, mt)
+    launch_k(pdl, k_fx_col_main<L2, false>, grid(g.nx + 1, FxGeo<L2>::PER, capc), dim3(FxGeo<L2>::T),  \
+             FxGeo<L2>::smem, cst, mem, fo, L.ldqA, g.nx + 1, ay, mt)
 #define DSNU_ROWI(L2)                                                                                       \
   launch_k(pdl, k_fx_row_inv<L2>, grid(g.ny, FxGeo<L2>::PER, g.cap_rowi), dim3(FxGeo<L2>::T), g.smem_rowi, st, \
            mem, fo, L.ldqA, L.ldqB, g.Q, g.ny, ax, g.kdx, -(ilogb(double(g.mx)) + ilogb(double(g.my))))
@@ -173,22 +176,44 @@ dsnu_status run_pipeline_f64(const PlanGeom& g, const PlanTables& t, const WsLay
   }
 #define DSNU_MARK(I) \
   if (ev) cudaEventRecord(ev[I], st)
+  // the band chain (stream bst) next to the column pass (cst), one of them on
+  // the plan's side stream and the column pass leaving `reserve` SMs free, or
+  // both in line (no `ov`, profiling)
+  cudaStream_t bst = st, cst = st;
+  int capc = g.cap_col;
+  auto band_chain = [&]() -> dsnu_status {
+    DSNU_STEP(g.log2ny, DSNU_BANDF)
+    DSNU_MARK(2);
+    launch_k(pdl, k_fx_interp_tile, dim3(g.n_itiles, mem.count), dim3(256), interp_fx_smem(g.w), bst, mem, off, L.ldq,
+             g.Q, t.node_q0, static_cast<const int2*>(t.node_w), t.node_D, t.itile_ptr, t.itile_org, t.itile_nodes, g.w,
+             g.n_half);
+    DSNU_MARK(3);
+    launch_spread_fx(g.spread_cfg, mem, off, t, g, L.ldq, bst, 0, pdl);
+    DSNU_MARK(4);
+    launch_spread_fx(g.spread_cfg, mem, off, t, g, L.ldq, bst, 1, pdl);
+    DSNU_MARK(5);
+    DSNU_STEP(g.log2ny, DSNU_BANDI)
+    DSNU_MARK(6);
+    return DSNU_OK;
+  };
   DSNU_MARK(0);
   DSNU_STEP(g.log2nx, DSNU_ROWF)
   DSNU_MARK(1);
-  DSNU_STEP(g.log2ny, DSNU_BANDF)
-  DSNU_MARK(2);
-  launch_k(pdl, k_interp_tile<double>, dim3(g.n_itiles, mem.count), dim3(256),
-           interp_tile_smem(g.w, sizeof(cpx<double>)), st, mem, off, L.ldq, g.Q, t.node_q0, wts, t.node_D, t.itile_ptr,
-           t.itile_org, t.itile_nodes, g.w, 0);
-  DSNU_MARK(3);
-  launch_spread<double>(g.spread_cfg, mem, off, t, g, L.ldq, 0, st, 0, pdl);
-  DSNU_MARK(4);
-  launch_spread<double>(g.spread_cfg, mem, off, t, g, L.ldq, 0, st, 1, pdl);
-  DSNU_MARK(5);
-  DSNU_STEP(g.log2ny, DSNU_BANDI)
-  DSNU_MARK(6);
-  DSNU_STEP(g.log2ny, DSNU_COLM)
+  if (ov && !ev) {
+    cudaEventRecord(ov->fork, st);
+    cudaStreamWaitEvent(ov->side, ov->fork, 0);
+    capc = std::max(1, g.cap_col - ov->reserve * (g.cap_col / g.sms));
+    (ov->col_side ? cst : bst) = ov->side;
+    DSNU_STEP(g.log2ny, DSNU_COLM)
+    const dsnu_status sb = band_chain();
+    if (sb != DSNU_OK) return sb;
+    cudaEventRecord(ov->join, ov->side);
+    cudaStreamWaitEvent(st, ov->join, 0);
+  } else {
+    const dsnu_status sb = band_chain();
+    if (sb != DSNU_OK) return sb;
+    DSNU_STEP(g.log2ny, DSNU_COLM)
+  }
   DSNU_MARK(7);
   DSNU_STEP(g.log2nx, DSNU_ROWI)
   DSNU_MARK(8);
@@ -209,7 +234,9 @@ dsnu_status run_pipeline_f64(const PlanGeom& g, const PlanTables& t, const WsLay
 
 cudaError_t time_spread_f64(const PlanGeom& g, const PlanTables& t, const WsLayout& L, void* ws, int reps,
                             float* ms) {
-  return time_spread<double>(g, t, L, ws, reps, ms);
+  return time_spread(L, ws, reps, ms, [&](const Members& mem, const WsOff& off) {
+    launch_spread_fx(g.spread_cfg, mem, off, t, g, L.ldq, 0, 2, false);
+  });
 }
 
 }  // namespace dsnu

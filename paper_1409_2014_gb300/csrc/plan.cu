@@ -167,6 +167,18 @@ static double es_kernel(double z, int w, double beta) {
   return std::exp(beta * (std::sqrt(u) - 1.0));
 }
 
+// A stencil weight as the kernels read it: FP32, or the two halves {wh, wl} of
+// w = wh 2^-28 + wl 2^-56 (spread_fx.cuh) in the eight bytes of an FP64 value.
+template <typename R>
+static R stencil_weight(double v) {
+  if constexpr (sizeof(R) == 4) return R(v);
+  const double s = v * 268435456.0, h = std::nearbyint(s);
+  const int halves[2] = {int(h), int(std::nearbyint((s - h) * 268435456.0))};
+  double out;
+  std::memcpy(&out, halves, sizeof(out));
+  return R(out);
+}
+
 // phi_hat(xi) = int_{-w/2}^{w/2} phi(z) e^{-i xi z} dz, by Gauss-Legendre in
 // t with z = (w/2) sin t (smooth integrand on [0, pi/2]).
 struct EsFourier {
@@ -198,7 +210,6 @@ template <typename R>
 struct HostTables {
   // complex tables interleaved (re, im)
   std::vector<R> stw_x, stwc_x, twm_lo_x, twm_hi_x, decon_x, stw_y, twm_lo_y, twm_hi_y, decon_y;
-  std::vector<R> m_wx2, m_gx, m_kx;
   std::vector<int2> node_q0;
   std::vector<int> itile_ptr, itile_nodes;
   std::vector<int2> itile_org;
@@ -506,63 +517,54 @@ static dsnu_status setup_spread(dsnu_plan_s* P, const std::vector<int2>& q0, con
 
 // The column multiplier of I1 (eq. SubInt1) on the padded grid,
 //   m1(q_x, a) = -(q_x dk_x)^2 / s * (1 - p),  s = (q_x dk_x)^2 + (a dk_y)^2,
-// with p = e^{-s/sigma^2} (Gaussian partition) or the indicator of s <= P^2
-// (sharp), m1 = 0 at s = 0; computed in FP64 with one rounding to FP32 (mixed
-// plans).  Row q_x holds a = 2 j at j <= ny/2 and
-// a = 2 j' + 1 at ny/2 + 1 + j', then zeros up to its ldm = ny + 4 entries.
-__global__ void k_fill_m1(float* tab, int nx1, int ny, int ldm, double dkx, double dky, double inv_sigma2, int sharp,
-                          double cut2) {
-  const long long n = (long long)nx1 * ldm;
-  const int mh = ny / 2 + 1;
+// (or another multiplier of the family) with p = e^{-s/sigma^2} (Gaussian
+// partition) or the indicator of s <= P^2 (sharp), m1 = 0 at s = 0; computed in
+// FP64.  Row q_x holds the even frequencies first: |qbar| = 2 j at j, 2 j' + 1 at
+// ny/2 + 1 + j' (full: the natural frequency q = 2 j at j, 2 j' + 1 at ny + j'),
+// then zeros up to its ld entries.
+struct MultSpec {
+  int nx, ny, ld, full, sharp, generic, alpha;
+  double dkx, dky, inv_sigma2, cut2, a0, ac, as;
+};
+__device__ __forceinline__ double mult_at(const MultSpec& p, int col, int j) {
+  const int mh = p.full ? p.ny : p.ny / 2 + 1, last = p.full ? 2 * p.ny : p.ny + 1;
+  if (j >= last) return 0.0;
+  const int q = (j < mh) ? 2 * j : 2 * (j - mh) + 1;
+  const int qs = (q < p.ny) ? q : (q == p.ny ? 0 : q - 2 * p.ny);  // signed, 0 at the Nyquist row (sin 2theta term)
+  const int a = (q <= p.ny) ? q : 2 * p.ny - q;
+  const double wx = col * p.dkx, wy = a * p.dky;
+  const double wx2 = wx * wx, wy2 = wy * wy, s = wx2 + wy2;
+  if (!(s > 0.0)) return 0.0;
+  double m = -wx2 / s;
+  if (p.generic) {
+    const double kx = col < p.nx ? wx : 0.0;  // (and at the Nyquist column)
+    m = p.a0 + (p.ac * (wx2 - wy2) + 2.0 * p.as * kx * (qs * p.dky)) / s;
+    if (p.alpha == 1) m *= sqrt(s);
+    if (p.alpha == -1) m /= sqrt(s);
+  }
+  return m * (p.sharp ? (s > p.cut2 ? 1.0 : 0.0) : -expm1(-s * p.inv_sigma2));
+}
+// Mixed plans: one rounding to FP32.
+__global__ void k_fill_m1(float* tab, MultSpec p) {
+  const long long n = (long long)(p.nx + 1) * p.ld;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int col = int(i / ldm), j = int(i - (long long)col * ldm);
-    float v = 0.f;
-    if (j <= ny) {
-      const int a = (j < mh) ? 2 * j : 2 * (j - mh) + 1;
-      const double wx = col * dkx, wy = a * dky;
-      const double wx2 = wx * wx, s = wx2 + wy * wy;
-      if (s > 0.0) {
-        const double part = sharp ? (s > cut2 ? 1.0 : 0.0) : -expm1(-s * inv_sigma2);
-        v = float(-wx2 / s * part);
-      }
-    }
-    tab[i] = v;
+    const int col = int(i / p.ld);
+    tab[i] = float(mult_at(p, col, int(i - (long long)col * p.ld)));
   }
 }
-
-// The multiplier table of the FP64 plans (FxMult): m1 2^-mexp[q_x] in
-// fixed-point halves, for any multiplier of the family.  Row q_x holds the
-// even frequencies first: |qbar| = 2 j at j, 2 j' + 1 at ny/2 + 1 + j' (full:
-// the natural frequency q = 2 j at j, 2 j' + 1 at ny + j').
-__global__ void k_fill_m1_fx(int2* tab, int nx, int ny, int ld, int full, double dkx, double dky, double inv_sigma2,
-                             int sharp, double cut2, int generic, int alpha, double a0, double ac, double as,
-                             const int* mexp) {
-  const long long n = (long long)(nx + 1) * ld;
-  const int mh = full ? ny : ny / 2 + 1, last = full ? 2 * ny : ny + 1;
+// FP64 plans (FxMult): m1 2^-mexp[q_x] in fixed-point halves.
+__device__ __forceinline__ int2 fx_mult_halves(double m, int e) {
+  const long long w = __double2ll_rn(ldexp(m, kFxMultBits + 32 - e));
+  int2 v;
+  v.y = int(w);
+  v.x = int((w - v.y) >> 32);
+  return v;
+}
+__global__ void k_fill_m1_fx(int2* tab, MultSpec p, const int* mexp) {
+  const long long n = (long long)(p.nx + 1) * p.ld;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int col = int(i / ld), j = int(i - (long long)col * ld);
-    int2 v = make_int2(0, 0);
-    if (j < last) {
-      const int q = (j < mh) ? 2 * j : 2 * (j - mh) + 1;
-      const int qs = (q < ny) ? q : (q == ny ? 0 : q - 2 * ny);  // signed, 0 at the Nyquist row (sin 2theta term)
-      const int a = (q <= ny) ? q : 2 * ny - q;
-      const double wx = col * dkx, wy = a * dky;
-      const double wx2 = wx * wx, wy2 = wy * wy, s = wx2 + wy2;
-      if (s > 0.0) {
-        double m = -wx2 / s;
-        if (generic) {
-          const double kx = col < nx ? wx : 0.0;  // (and at the Nyquist column)
-          m = a0 + (ac * (wx2 - wy2) + 2.0 * as * kx * (qs * dky)) / s;
-          if (alpha == 1) m *= sqrt(s);
-          if (alpha == -1) m /= sqrt(s);
-        }
-        m *= sharp ? (s > cut2 ? 1.0 : 0.0) : -expm1(-s * inv_sigma2);
-        const long long w = __double2ll_rn(ldexp(m, kFxMultBits + 32 - (mexp ? mexp[col] : 0)));
-        v.y = int(w);
-        v.x = int((w - v.y) >> 32);
-      }
-    }
-    tab[i] = v;
+    const int col = int(i / p.ld);
+    tab[i] = fx_mult_halves(mult_at(p, col, int(i - (long long)col * p.ld)), mexp ? mexp[col] : 0);
   }
 }
 
@@ -586,9 +588,7 @@ __global__ void k_fill_std_fx(int2* tab, int nx, int ny, int ld, int full, doubl
         if (alpha == 1) m *= sqrt(s);
         if (alpha == -1) m /= sqrt(s);
       }
-      const long long w = __double2ll_rn(ldexp(m, kFxMultBits + 32 - (mexp ? mexp[col] : 0)));
-      v.y = int(w);
-      v.x = int((w - v.y) >> 32);
+      v = fx_mult_halves(m, mexp ? mexp[col] : 0);
     }
     tab[i] = v;
   }
@@ -611,18 +611,14 @@ static std::vector<int> fx_mult_exponents(const PlanGeom& g, int ncols, double d
 template <typename R>
 static dsnu_status build_m1_table(dsnu_plan_s* P, double dkx, double dky, cudaStream_t st) {
   const PlanGeom& g = P->geom;
-  const int ldm = (sizeof(R) == 8) ? g.m1_ld : g.ny + 4;
-  const size_t bytes = size_t(g.nx + 1) * ldm * sizeof(R);
+  const MultSpec p{g.nx, g.ny, g.m1_ld, g.m1_full, g.sharp, g.m_generic, g.m_alpha, dkx, dky,
+                   1.0 / (g.sigma * g.sigma), g.cut_radius * g.cut_radius, g.m_a0, g.m_ac, g.m_as};
+  const size_t bytes = size_t(g.nx + 1) * g.m1_ld * sizeof(R);
   void* m = nullptr;
   cudaError_t e = cudaMalloc(&m, bytes);
   if (e != cudaSuccess) return fail(DSNU_ENOMEM, std::string("cudaMalloc(multiplier table): ") + cudaGetErrorString(e));
-  if constexpr (sizeof(R) == 8)
-    k_fill_m1_fx<<<1024, 256, 0, st>>>(static_cast<int2*>(m), g.nx, g.ny, ldm, g.m1_full, dkx, dky,
-                                       1.0 / (g.sigma * g.sigma), g.sharp, g.cut_radius * g.cut_radius, g.m_generic,
-                                       g.m_alpha, g.m_a0, g.m_ac, g.m_as, P->tab.fx_mexp);
-  else
-    k_fill_m1<<<1024, 256, 0, st>>>(static_cast<float*>(m), g.nx + 1, g.ny, ldm, dkx, dky, 1.0 / (g.sigma * g.sigma),
-                                       g.sharp, g.cut_radius * g.cut_radius);
+  if constexpr (sizeof(R) == 8) k_fill_m1_fx<<<1024, 256, 0, st>>>(static_cast<int2*>(m), p, P->tab.fx_mexp);
+  else k_fill_m1<<<1024, 256, 0, st>>>(static_cast<float*>(m), p);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
@@ -652,8 +648,10 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
     const double r = rn[i];
     const double pr = g.sharp ? 1.0 : std::exp(-r * r / (sigma * sigma));
     for (int j = 0; j < p.n_theta; ++j) {
-      const double th = 2.0 * M_PI * j / p.n_theta;
-      const double c = std::cos(th), s = std::sin(th);
+      // the second half of a ring is the first one's mirror, exactly
+      const double sg = (2 * j < p.n_theta) ? 1.0 : -1.0;
+      const double th = 2.0 * M_PI * (2 * j < p.n_theta ? j : j - p.n_theta / 2) / p.n_theta;
+      const double c = sg * std::cos(th), s = sg * std::sin(th);
       kx[i * p.n_theta + j] = r * c;
       ky[i * p.n_theta + j] = r * s;
       if (g.m_generic)  // r^alpha (a0 + ac cos 2theta + as sin 2theta) in place of -cos^2 theta
@@ -673,6 +671,8 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   std::vector<double> dcx(nx), dcy(ny);
   for (int n = 0; n < nx; ++n) dcx[n] = ph0 / fh(2.0 * M_PI * (n - nx / 2) / Mx);
   for (int n = 0; n < ny; ++n) dcy[n] = ph0 / fh(2.0 * M_PI * (n - ny / 2) / My);
+  g.m1_full = (g.m_generic && g.m_as != 0.0) ? 1 : 0;
+  g.m1_ld = g.m1_full ? My : ny + 4;
   if constexpr (sizeof(R) == 8) {
     fft_stage_twiddles(g.log2nx, tmp); T.fx_stw_x = fx_table(tmp, kFxTwBits);
     fft_stage_twiddles(g.log2ny, tmp); T.fx_stw_y = fx_table(tmp, kFxTwBits);
@@ -680,8 +680,6 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
     twiddles(ny / 2, My, tmp); T.fx_wm_y = fx_table(tmp, kFxTwBits);
     g.kdx = fx_decon(dcx, T.fx_dec_x);
     g.kdy = fx_decon(dcy, T.fx_dec_y);
-    g.m1_full = (g.m_generic && g.m_as != 0.0) ? 1 : 0;
-    g.m1_ld = g.m1_full ? My : ny + 4;
     if (g.m_generic) T.fx_mexp = fx_mult_exponents(g, nx + 1, dkx, dky, ny * dky);
   } else {
     fft_stage_twiddles(g.log2nx, tmp); T.stw_x = cast<R>(tmp);
@@ -695,19 +693,7 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
     g.log2lo_y = half_angle_tables(ny, tmp, tmp2); T.twm_lo_y = cast<R>(tmp); T.twm_hi_y = cast<R>(tmp2);
     T.decon_x = cast<R>(dcx);
     T.decon_y = cast<R>(dcy);
-    // multiplier axis tables: per column q_x
-    T.m_wx2.resize(nx + 1);
-    T.m_gx.resize(nx + 1);
-    T.m_kx.resize(nx + 1);
-    for (int q = 0; q <= nx; ++q) {
-      const double a = q * dkx;
-      T.m_wx2[q] = R(a * a);
-      T.m_gx[q] = R(-std::expm1(-(a * a) / (sigma * sigma)));
-      T.m_kx[q] = R(q < nx ? a : 0.0);  // Nyquist column: +-K averaged, the sin 2theta term vanishes
-    }
   }
-
-  g.dky2 = dky * dky;
 
   // per-node stencils
   T.node_q0.resize(nn);
@@ -720,8 +706,8 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
     const int q0y = int(std::ceil(uy - 0.5 * w));
     T.node_q0[j] = make_int2(q0x, q0y);
     for (int a = 0; a < w; ++a) {
-      T.node_w[size_t(j) * 2 * w + a] = R(es_kernel(ux - (q0x + a), w, beta));
-      T.node_w[size_t(j) * 2 * w + w + a] = R(es_kernel(uy - (q0y + a), w, beta));
+      T.node_w[size_t(j) * 2 * w + a] = stencil_weight<R>(es_kernel(ux - (q0x + a), w, beta));
+      T.node_w[size_t(j) * 2 * w + w + a] = stencil_weight<R>(es_kernel(uy - (q0y + a), w, beta));
     }
     Q = std::max({Q, std::abs(q0x), std::abs(q0x + w - 1), std::abs(q0y), std::abs(q0y + w - 1)});
     // rho_hat = hx hy / phi_hat(0)^2 * (stencil sum), then the type-1 scale
@@ -733,7 +719,8 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
     return fail(DSNU_EINVAL, "disk plus ES stencil does not fit the padded grid: need P*h + w*pi/M < pi");
   g.Q = Q;
 
-  // interpolation items: nodes grouped by the kItile x kItile tile of the
+  // interpolation items: the nodes with theta < pi (the others' values are their
+  // mirrors' conjugates) grouped by the kItile x kItile tile of the
   // plane of stencil origins q0 in [-Q, Q]^2 that holds theirs (node order
   // kept within a tile), each tile's nodes cut into items of at most
   // kItileNodes (the polar nodes crowd near the origin: a whole ring of small
@@ -741,8 +728,9 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   {
     const int nt = (2 * Q + 1 + kItile - 1) / kItile;
     std::vector<int> cnt(size_t(nt) * nt, 0);
-    std::vector<int> tix(nn);
+    std::vector<int> tix(nn, -1);
     for (int j = 0; j < nn; ++j) {
+      if (j % p.n_theta >= g.n_half) continue;  // the mirror of node j - n_half
       const int tx = (T.node_q0[j].x + Q) / kItile, ty = (T.node_q0[j].y + Q) / kItile;
       tix[j] = tx * nt + ty;
       ++cnt[tix[j]];
@@ -758,8 +746,9 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
           T.itile_org.push_back(make_int2(-Q + (t / nt) * kItile, -Q + (t % nt) * kItile));
         }
       }
-    T.itile_nodes.assign(nn, 0);
-    for (int j = 0; j < nn; ++j) T.itile_nodes[first[tix[j]]++] = j;
+    T.itile_nodes.assign(nn / 2, 0);
+    for (int j = 0; j < nn; ++j)
+      if (tix[j] >= 0) T.itile_nodes[first[tix[j]]++] = j;
     g.n_itiles = int(T.itile_org.size());
   }
 
@@ -769,7 +758,6 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   const size_t o_dx = b.add(T.decon_x), o_scx = b.add(T.stwc_x);
   const size_t o_sty = b.add(T.stw_y), o_tly = b.add(T.twm_lo_y), o_thy = b.add(T.twm_hi_y);
   const size_t o_dy = b.add(T.decon_y);
-  const size_t o_wx2 = b.add(T.m_wx2), o_gx = b.add(T.m_gx), o_kx = b.add(T.m_kx);
   const size_t o_q0 = b.add(T.node_q0), o_w = b.add(T.node_w), o_D = b.add(T.node_D);
   const size_t o_fsx = b.add(T.fx_stw_x), o_fwx = b.add(T.fx_wm_x), o_fdx = b.add(T.fx_dec_x);
   const size_t o_fsy = b.add(T.fx_stw_y), o_fwy = b.add(T.fx_wm_y), o_fdy = b.add(T.fx_dec_y);
@@ -784,7 +772,6 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   t.stw_x = d + o_stx; t.twm_lo_x = d + o_tlx; t.twm_hi_x = d + o_thx; t.decon_x = d + o_dx;
   t.stwc_x = d + o_scx;
   t.stw_y = d + o_sty; t.twm_lo_y = d + o_tly; t.twm_hi_y = d + o_thy; t.decon_y = d + o_dy;
-  t.m_wx2 = d + o_wx2; t.m_gx = d + o_gx; t.m_kx = d + o_kx;
   t.node_q0 = reinterpret_cast<int2*>(d + o_q0);
   t.itile_ptr = reinterpret_cast<int*>(d + o_itp);
   t.itile_org = reinterpret_cast<int2*>(d + o_ito);
@@ -795,10 +782,8 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   t.fx_stw_x = d + o_fsx; t.fx_wm_x = d + o_fwx; t.fx_dec_x = d + o_fdx;
   t.fx_stw_y = d + o_fsy; t.fx_wm_y = d + o_fwy; t.fx_dec_y = d + o_fdy;
   t.fx_mexp = (sizeof(R) == 8 && g.m_generic) ? reinterpret_cast<int*>(d + o_fme) : nullptr;
-  if (sizeof(R) == 8 || !g.m_generic) {
-    const dsnu_status sm = build_m1_table<R>(P, dkx, dky, st);
-    if (sm != DSNU_OK) return sm;
-  }
+  const dsnu_status sm = build_m1_table<R>(P, dkx, dky, st);
+  if (sm != DSNU_OK) return sm;
   return setup_spread<R>(P, T.node_q0, T.node_w, st);
 }
 
@@ -1003,6 +988,7 @@ dsnu_status dsnu_plan_create_multiplier(const dsnu_params* params, const dsnu_mu
   g.sigma = p.sigma;
   g.cut_radius = p.cut_radius;
   g.n_nodes = p.n_r * p.n_theta;
+  g.n_half = p.n_theta / 2;
   g.precision = p.precision;
   g.acc64 = (p.precision == DSNU_MIXED && p.accumulation == DSNU_ACCUM_FP64) ? 1 : 0;
   g.sharp = (p.partition == DSNU_PARTITION_SHARP);
@@ -1029,30 +1015,39 @@ dsnu_status dsnu_plan_create_multiplier(const dsnu_params* params, const dsnu_mu
     return fail(DSNU_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(e));
   }
   layout_workspace(P);
-  // mixed plans on large grids: the band chain runs next to the column pass
-  // on a low-priority side stream, the column pass leaving it 16 of every 152
-  // SMs at 4096^2 and a share growing as 1/sqrt(nx ny) for smaller grids,
-  // whose band chain (its node work is the same) is larger next to their
-  // column pass: measured best on GB300 16 SMs at 4096^2 (0.5137 ms against
-  // 0.5226 with 12 and 0.534 with the band chain in line) and 32 at 2048^2
-  // (0.131-0.134 ms against 0.139 with 16 and 0.150 in line);
-  // DSNU_BAND_SMS=<n> sets the number of SMs, 0 turns it off
-  if (p.precision == DSNU_MIXED && !standard) {
-    int dev = 0, sms = 0;
+  // The band chain and the column pass run side by side.  On large grids the
+  // column pass is the longer one: the band chain runs on the low-priority side
+  // stream, the column pass leaving it 16 of every 152 SMs at 4096^2 and a
+  // share growing as 1/sqrt(nx ny) below, since the band chain's node work is the
+  // same on every grid (mixed 4096^2 507 us with 16 SMs, 526 with 32, 524 in
+  // line; 2048^2 131 with 32, 139 with 16, 152 in line; FP64 4096^2 2208 us, in
+  // line 2234; 2048^2 530, in line 548).  Below 2048^2 the band chain is the
+  // longer one: it stays on the caller's stream, where its launches overlap, and
+  // the column pass fills the rest of the GPU from the side stream (FP64 512^2
+  // 92 us against 105 in line; 1024^2 164 against 187; mixed 256^2 44 against 48).
+  // There the share is capped: mixed 48 SMs (1024^2 57.7 us with 48, 65.5 with
+  // 16; 2048 x 512 53.6 and 59.7), FP64, whose column pass is heavier, 16 (1024^2
+  // 164 us with 16, 171 with 64).
+  // DSNU_BAND_SMS=<n> sets the number of SMs left free, 0 runs both in line.
+  {
+    int dev = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int reserve = 0;
-    if (p.nx >= 2048 && p.ny >= 2048)
-      reserve = std::max(1, int(std::lround(sms * (16.0 / 152.0) * 4096.0 / std::sqrt(double(p.nx) * p.ny))));
+    cudaDeviceGetAttribute(&g.sms, cudaDevAttrMultiProcessorCount, dev);
+  }
+  if (!standard) {
+    const double share = 16.0 / 152.0 * 4096.0 / std::sqrt(double(p.nx) * p.ny);
+    Overlap& ov = P->overlap;
+    ov.col_side = (p.nx < 2048 || p.ny < 2048) ? 1 : 0;
+    ov.reserve = std::max(1, int(std::lround(g.sms * (ov.col_side ? std::min(share, g.precision == DSNU_MIXED ? 48.0 / 152.0 : 16.0 / 152.0) : share))));
     const char* env = std::getenv("DSNU_BAND_SMS");
-    if (env) reserve = std::atoi(env);
-    if (reserve > 0) {
+    if (env) ov.reserve = std::atoi(env);
+    if (ov.reserve > 0) {
       int lo = 0, hi = 0;
       cudaError_t ce = cudaDeviceGetStreamPriorityRange(&lo, &hi);
-      if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(&P->overlap.side, cudaStreamNonBlocking, lo);
-      if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&P->overlap.fork, cudaEventDisableTiming);
-      if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&P->overlap.join, cudaEventDisableTiming);
-      if (ce == cudaSuccess) P->overlap.reserve = reserve;
+      if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(&ov.side, cudaStreamNonBlocking, lo);
+      if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&ov.fork, cudaEventDisableTiming);
+      if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&ov.join, cudaEventDisableTiming);
+      ov.on = (ce == cudaSuccess);
     }
   }
   *out = P;
@@ -1086,9 +1081,9 @@ static dsnu_status run(dsnu_plan plan, const double* in, double* out, void* stre
     ev = plan->prof_events + size_t(plan->prof_used++) * kProfEvents;
   if (plan->geom.precision == DSNU_MIXED)
     return run_pipeline_f32(plan->geom, plan->tab, plan->ws_layout, single_member(in, out, plan->ws), st,
-                            cj, ev, plan->overlap.reserve > 0 ? &plan->overlap : nullptr);
+                            cj, ev, plan->overlap.on ? &plan->overlap : nullptr);
   return run_pipeline_f64(plan->geom, plan->tab, plan->ws_layout, single_member(in, out, plan->ws), st, cj,
-                          ev);
+                          ev, plan->overlap.on ? &plan->overlap : nullptr);
 }
 
 static void free_profile(dsnu_plan plan) {
@@ -1121,7 +1116,7 @@ dsnu_status dsnu_status_poll(dsnu_plan plan, void* stream) {
 dsnu_status dsnu_plan_destroy(dsnu_plan plan) {
   if (!plan) return DSNU_OK;
   free_profile(plan);
-  if (plan->overlap.reserve > 0) {
+  if (plan->overlap.on) {
     cudaStreamSynchronize(plan->overlap.side);
     cudaStreamDestroy(plan->overlap.side);
     cudaEventDestroy(plan->overlap.fork);
