@@ -321,6 +321,10 @@ dsnu_status dsnu_ds_set_linear_step(dsnu_ds_plan plan, double tau, double alpha,
  * loaded), DSNU_ECUDA. */
 dsnu_status dsnu_ds_linear(dsnu_ds_plan plan, void* u_dev, int32_t adjoint, void* stream);
 
+/* The same with the result in out_dev (which may be u_dev; u_dev is otherwise
+ * only read). */
+dsnu_status dsnu_ds_linear_to(dsnu_ds_plan plan, const void* u_dev, void* out_dev, int32_t adjoint, void* stream);
+
 /* rho <- |u|^2 (FP64 [ny][nx], device), the density of eq. DSII_exact_pot. */
 dsnu_status dsnu_ds_abs2(dsnu_ds_plan plan, const void* u_dev, double* rho_dev, void* stream);
 
@@ -337,6 +341,11 @@ dsnu_status dsnu_ds_abs2_vjp(dsnu_ds_plan plan, const void* u_dev, const double*
  * phi_dev: FP64 [ny][nx] potential of the current density. */
 dsnu_status dsnu_ds_nonlinear(dsnu_ds_plan plan, void* u_dev, const double* phi_dev, double tau,
                               double beta, void* stream);
+
+/* The same with the result in out_dev (which may be u_dev; u_dev is otherwise
+ * only read). */
+dsnu_status dsnu_ds_nonlinear_to(dsnu_ds_plan plan, const void* u_dev, const double* phi_dev, void* out_dev,
+                                 double tau, double beta, void* stream);
 
 /* Vector-Jacobian product of the nonlinear flow u' = u e^{i theta}, theta =
  * tau (2 beta |u|^2 + 4 beta Phi(|u|^2)), for a real loss with gradients in

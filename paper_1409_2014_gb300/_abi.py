@@ -156,6 +156,8 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.dsnu_ds_plan_create.argtypes = [ctypes.POINTER(dsnu_ds_params), vp, ctypes.POINTER(vp)]
     lib.dsnu_ds_set_linear_step.argtypes = [vp, d, d, vp]
     lib.dsnu_ds_linear.argtypes = [vp, vp, ctypes.c_int32, vp]
+    lib.dsnu_ds_linear_to.argtypes = [vp, vp, vp, ctypes.c_int32, vp]
+    lib.dsnu_ds_nonlinear_to.argtypes = [vp, vp, vp, vp, d, d, vp]
     lib.dsnu_ds_abs2.argtypes = [vp, vp, vp, vp]
     lib.dsnu_ds_nonlinear.argtypes = [vp, vp, vp, d, d, vp]
     lib.dsnu_ds_nonlinear_vjp.argtypes = [vp, vp, vp, vp, d, d, vp, vp, vp]
@@ -163,7 +165,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.dsnu_ds_plan_destroy.argtypes = [vp]
     for name in ("dsnu_ds_plan_create", "dsnu_ds_set_linear_step", "dsnu_ds_linear", "dsnu_ds_abs2",
                  "dsnu_ds_nonlinear", "dsnu_ds_nonlinear_vjp", "dsnu_ds_nonlinear_vjp_finish",
-                 "dsnu_ds_plan_destroy"):
+                 "dsnu_ds_linear_to", "dsnu_ds_nonlinear_to", "dsnu_ds_plan_destroy"):
         getattr(lib, name).restype = st
     lib.dsnu_batch_create.argtypes = [ctypes.c_int32, ctypes.POINTER(vp), ctypes.POINTER(vp)]
     lib.dsnu_batch_workspace_bytes.argtypes = [vp]
@@ -340,6 +342,10 @@ def dsnu_ds_linear(plan: int, u: int, adjoint: int, stream: int = 0) -> None:
     _check(load().dsnu_ds_linear(_vp(plan), _vp(u), int(adjoint), _vp(stream)), "dsnu_ds_linear")
 
 
+def dsnu_ds_linear_to(plan: int, u: int, out: int, adjoint: int, stream: int = 0) -> None:
+    _check(load().dsnu_ds_linear_to(_vp(plan), _vp(u), _vp(out), int(adjoint), _vp(stream)), "dsnu_ds_linear_to")
+
+
 def dsnu_ds_abs2(plan: int, u: int, rho: int, stream: int = 0) -> None:
     _check(load().dsnu_ds_abs2(_vp(plan), _vp(u), _vp(rho), _vp(stream)), "dsnu_ds_abs2")
 
@@ -351,6 +357,11 @@ def dsnu_ds_abs2_vjp(plan: int, u: int, g_rho: int, grad: int, stream: int = 0) 
 def dsnu_ds_nonlinear(plan: int, u: int, phi: int, tau: float, beta: float, stream: int = 0) -> None:
     _check(load().dsnu_ds_nonlinear(_vp(plan), _vp(u), _vp(phi), float(tau), float(beta), _vp(stream)),
            "dsnu_ds_nonlinear")
+
+
+def dsnu_ds_nonlinear_to(plan: int, u: int, phi: int, out: int, tau: float, beta: float, stream: int = 0) -> None:
+    _check(load().dsnu_ds_nonlinear_to(_vp(plan), _vp(u), _vp(phi), _vp(out), float(tau), float(beta),
+                                       _vp(stream)), "dsnu_ds_nonlinear_to")
 
 
 def dsnu_ds_nonlinear_vjp(plan, u, phi, g, tau, beta, s, part, stream=0) -> None:

@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 #include <string>
@@ -30,17 +31,25 @@ struct GeoC2C {
   static constexpr int N = 1 << LOG2N;
   static constexpr int G = N / 16;
   static constexpr int FB = fft_buf_elems(N);
-  static constexpr int PER = (G >= 256) ? 1 : 256 / G;  // rows or columns per CTA
+  static constexpr int PER = (G >= 256) ? 1 : 256 / G;  // rows per CTA
   static constexpr int T = PER * G;
   static constexpr int STW = fft_stage_tw_elems(LOG2N) > 0 ? fft_stage_tw_elems(LOG2N) : 1;
   static constexpr int STWP = (STW + 1) & ~1;
   static constexpr size_t smem = size_t(STWP + PER * FB) * sizeof(cpx<R>);
+  // column pass: C adjacent columns, their threads interleaved (see the kernel),
+  // SETS such sets per CTA; buffers 16/C elements apart modulo 16
+  static constexpr int C = (G >= 256) ? 2 : 4;
+  static constexpr int SETS = (C * G >= 256) ? 1 : 256 / (C * G);
+  static constexpr int TC = SETS * C * G;
+  static constexpr int RS = ((FB + 15) & ~15) + 16 / C;
+  static constexpr size_t smem_cols = size_t(STWP + SETS * C * RS) * sizeof(cpx<R>);
 };
 
-// In-place length-nx DFT of every row (inv: unnormalised inverse).
+// Length-nx DFT of every row of src into dst (which may be src; inv:
+// unnormalised inverse).
 template <typename R, int LOG2N>
 __global__ void __launch_bounds__(GeoC2C<R, LOG2N>::T)
-k_c2c_rows(cpx<R>* __restrict__ u, int ny, const cpx<R>* __restrict__ stw_g, int inv) {
+k_c2c_rows(const cpx<R>* src, cpx<R>* dst, int ny, const cpx<R>* __restrict__ stw_g, int inv) {
   using GG = GeoC2C<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, PER = GG::PER;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -51,41 +60,49 @@ k_c2c_rows(cpx<R>* __restrict__ u, int ny, const cpx<R>* __restrict__ stw_g, int
   const int rr = tid / G, t = tid - rr * G;
   cpx<R>* buf = sm + rr * GG::FB;
   const int items = (ny + PER - 1) / PER;
+  grid_dep_wait();
 #pragma unroll 1
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
+    if (item + int(gridDim.x) >= items) grid_dep_trigger();  // last item of this CTA
     const int row = item * PER + rr;
     const bool valid = row < ny;
     cpx<R> v[16];
 #pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = valid ? u[size_t(row) * N + t + G * m] : mk<R>(R(0), R(0));
+    for (int m = 0; m < 16; ++m) v[m] = valid ? src[size_t(row) * N + t + G * m] : mk<R>(R(0), R(0));
     block_fft_regs<R, LOG2N>(v, buf, t, stw, inv != 0);
     if (valid) {
 #pragma unroll
-      for (int m = 0; m < 16; ++m) u[size_t(row) * N + t + G * m] = v[m];
+      for (int m = 0; m < 16; ++m) dst[size_t(row) * N + t + G * m] = v[m];
     }
   }
 }
 
 // Per column: DFT along y, multiply by px[col] py[k] * scale (conjugated when
 // adj), inverse DFT along y; in place.  px, py: the separable linear-flow
-// phases e^{-i tau k_x^2} and e^{+i tau alpha k_y^2} in FFT order.
+// phases e^{-i tau k_x^2} and e^{+i tau alpha k_y^2} in FFT order.  Four adjacent
+// columns (two at ny = 4096) go together with their threads interleaved lane by
+// lane: every access moves whole 32-byte sectors (one column per group of
+// threads moved 8 of each 32 bytes; linear flow of a 1024^2 complex64 field 33.9
+// -> 20.7 us, 2048^2 90 -> 59, with the launches overlapped).
 template <typename R, int LOG2N>
-__global__ void __launch_bounds__(GeoC2C<R, LOG2N>::T)
+__global__ void __launch_bounds__(GeoC2C<R, LOG2N>::TC)
 k_c2c_cols_phase(cpx<R>* __restrict__ u, int nx, const cpx<R>* __restrict__ stw_g,
                  const cpx<R>* __restrict__ px, const cpx<R>* __restrict__ py, R scale, int adj) {
   using GG = GeoC2C<R, LOG2N>;
-  constexpr int G = GG::G, PER = GG::PER;
+  constexpr int G = GG::G, C = GG::C, SETS = GG::SETS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* stw = reinterpret_cast<cpx<R>*>(smem_raw);
   cpx<R>* sm = stw + GG::STWP;
   copy_to_smem(stw, stw_g, GG::STW);
-  const int tid = threadIdx.x;
-  const int cl = tid / G, t = tid - cl * G;
-  cpx<R>* buf = sm + cl * GG::FB;
-  const int items = (nx + PER - 1) / PER;
+  const int set = threadIdx.x / (C * G), r = threadIdx.x - set * (C * G);
+  const int cl = r % C, t = r / C;
+  cpx<R>* buf = sm + (set * C + cl) * GG::RS;
+  const int items = (nx / C + SETS - 1) / SETS;
+  grid_dep_wait();
 #pragma unroll 1
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
-    const int col = item * PER + cl;
+    if (item + int(gridDim.x) >= items) grid_dep_trigger();  // last item of this CTA
+    const int col = (item * SETS + set) * C + cl;
     const bool valid = col < nx;
     cpx<R> v[16];
 #pragma unroll
@@ -118,7 +135,7 @@ k_c2c_cols_phase(cpx<R>* __restrict__ u, int nx, const cpx<R>* __restrict__ stw_
 // u[row][t + G m] of group threads t: the values' bits, and their largest
 // exponent (fx_top).
 template <int G, int P>
-__device__ __forceinline__ unsigned fx_load(fxc (&v)[16], const double2* __restrict__ u, size_t stride, bool valid,
+__device__ __forceinline__ unsigned fx_load(fxc (&v)[16], const double2* u, size_t stride, bool valid,
                                             unsigned* red) {
   unsigned mx = 0;
 #pragma unroll
@@ -143,7 +160,7 @@ __device__ __forceinline__ double2 fx_store(fxc v, int ex, unsigned mx) {
 
 template <int LOG2N>
 __global__ void __launch_bounds__(FxOne<LOG2N>::T, FxOne<LOG2N>::MINB)
-k_fx_c2c_rows(double2* __restrict__ u, int ny, const fxw* __restrict__ stw_g, int inv) {
+k_fx_c2c_rows(const double2* src, double2* dst, int ny, const fxw* __restrict__ stw_g, int inv) {
   using GG = FxOne<LOG2N>;
   constexpr int N = GG::N, G = GG::G, PER = GG::PER, W = GG::W;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -155,13 +172,15 @@ k_fx_c2c_rows(double2* __restrict__ u, int ny, const fxw* __restrict__ stw_g, in
   fxc* buf = sm + pr * GG::FB;
   __syncthreads();
   const int items = (ny + PER - 1) / PER;
+  grid_dep_wait();
 #pragma unroll 1
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
+    if (item + int(gridDim.x) >= items) grid_dep_trigger();  // last item of this CTA
     const int row = item * PER + pr;
     const bool valid = row < ny;
-    double2* ur = u + size_t(valid ? row : 0) * N + t;
+    const size_t at = size_t(valid ? row : 0) * N + t;
     fxc v[16];
-    const unsigned mx = fx_load<G, G>(v, ur, G, valid, red + 2 * W);
+    const unsigned mx = fx_load<G, G>(v, src + at, G, valid, red + 2 * W);
     if (inv) {
 #pragma unroll
       for (int m = 0; m < 16; ++m) v[m] = fx_swap(v[m]);
@@ -169,7 +188,7 @@ k_fx_c2c_rows(double2* __restrict__ u, int ny, const fxw* __restrict__ stw_g, in
     const int ex = fx_efm(mx) - kFxBias + 5 + fx_fft<LOG2N, G>(v, buf, t, stw, red);
     if (valid) {
 #pragma unroll
-      for (int m = 0; m < 16; ++m) ur[G * m] = fx_store(inv ? fx_swap(v[m]) : v[m], ex, mx);
+      for (int m = 0; m < 16; ++m) dst[at + G * m] = fx_store(inv ? fx_swap(v[m]) : v[m], ex, mx);
     }
   }
 }
@@ -203,8 +222,10 @@ k_fx_c2c_cols_phase(double2* __restrict__ u, int nx, const fxw* __restrict__ stw
   fxc* buf = sm + (2 * pr + h) * GG::FBS;
   __syncthreads();
   const int items = (nx / 2 + PER - 1) / PER;
+  grid_dep_wait();
 #pragma unroll 1
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
+    if (item + int(gridDim.x) >= items) grid_dep_trigger();  // last item of this CTA
     const int col = 2 * (item * PER + pr) + h;
     const bool valid = col < nx;
     double2* uc = u + size_t(t) * nx + (valid ? col : h);
@@ -240,6 +261,7 @@ k_fx_c2c_cols_phase(double2* __restrict__ u, int nx, const fxw* __restrict__ stw
 // rho = |u|^2 (FP64 out).
 template <typename R>
 __global__ void k_abs2(const cpx<R>* __restrict__ u, double* __restrict__ rho, size_t n) {
+  grid_dep_wait();
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
     const cpx<R> a = u[i];
     rho[i] = to_f64<R>(a.x * a.x + a.y * a.y);
@@ -251,6 +273,7 @@ __global__ void k_abs2(const cpx<R>* __restrict__ u, double* __restrict__ rho, s
 template <typename R>
 __global__ void k_abs2_vjp(const cpx<R>* __restrict__ u, const double* __restrict__ g_rho,
                            cpx<R>* __restrict__ grad, size_t n) {
+  grid_dep_wait();
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
     const cpx<R> a = u[i];
     const R g2 = R(2) * from_f64<R>(g_rho[i]);
@@ -270,15 +293,16 @@ __device__ __forceinline__ R nl_angle(cpx<R> a, double phi, R tau, R beta) {
   return tau * (R(2) * beta * (a.x * a.x + a.y * a.y) + R(4) * beta * from_f64<R>(phi));
 }
 
-// u <- u e^{i theta}.
+// out = u e^{i theta} (out may be u).
 template <typename R>
-__global__ void k_nonlinear(cpx<R>* __restrict__ u, const double* __restrict__ phi, size_t n, R tau,
+__global__ void k_nonlinear(const cpx<R>* u, cpx<R>* out, const double* __restrict__ phi, size_t n, R tau,
                             R beta) {
+  grid_dep_wait();
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
     const cpx<R> a = u[i];
     R s, c;
     sincos_r(nl_angle(a, phi[i], tau, beta), &s, &c);
-    u[i] = cmul(a, mk<R>(c, s));
+    out[i] = cmul(a, mk<R>(c, s));
   }
 }
 
@@ -290,6 +314,7 @@ template <typename R>
 __global__ void k_nonlinear_vjp(const cpx<R>* __restrict__ u, const double* __restrict__ phi,
                                 const cpx<R>* __restrict__ g, size_t n, R tau, R beta,
                                 double* __restrict__ sfld, cpx<R>* __restrict__ part) {
+  grid_dep_wait();
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
     const cpx<R> a = u[i];
     R s, c;
@@ -307,6 +332,7 @@ template <typename R>
 __global__ void k_nonlinear_vjp_finish(const cpx<R>* __restrict__ u, const double* __restrict__ sfld,
                                        const double* __restrict__ ats, size_t n, R tau, R beta,
                                        cpx<R>* __restrict__ part) {
+  grid_dep_wait();
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
     const R grho = tau * (R(2) * beta * from_f64<R>(sfld[i]) + R(4) * beta * from_f64<R>(ats[i]));
     const cpx<R> a = u[i];
@@ -381,6 +407,7 @@ struct dsnu_ds_plan_s {
   double tau, alpha; // phases currently loaded
   bool has_phase;
   int grid_rows, grid_cols;
+  bool pdl;          // launches with programmatic stream serialization
 };
 
 namespace {
@@ -446,10 +473,10 @@ cudaError_t prepare_f32(dsnu_ds_plan_s* P) {
     P->grid_rows = grid_for(k_c2c_rows<R, L2>, GeoC2C<R, L2>::T, GeoC2C<R, L2>::smem,            \
                                (P->prm.ny + GeoC2C<R, L2>::PER - 1) / GeoC2C<R, L2>::PER)
 #define DSNU_PC(L2)                                                                                 \
-  e = cudaFuncSetAttribute(k_c2c_cols_phase<R, L2>, A, int(GeoC2C<R, L2>::smem));                  \
+  e = cudaFuncSetAttribute(k_c2c_cols_phase<R, L2>, A, int(GeoC2C<R, L2>::smem_cols));             \
   if (e == cudaSuccess)                                                                             \
-    P->grid_cols = grid_for(k_c2c_cols_phase<R, L2>, GeoC2C<R, L2>::T, GeoC2C<R, L2>::smem,      \
-                               (P->prm.nx + GeoC2C<R, L2>::PER - 1) / GeoC2C<R, L2>::PER)
+    P->grid_cols = grid_for(k_c2c_cols_phase<R, L2>, GeoC2C<R, L2>::TC, GeoC2C<R, L2>::smem_cols, \
+                            (P->prm.nx / GeoC2C<R, L2>::C + GeoC2C<R, L2>::SETS - 1) / GeoC2C<R, L2>::SETS)
   switch (P->log2nx) {
     DSNU_C2C_CASES(DSNU_PR)
     default: return cudaErrorInvalidValue;
@@ -491,21 +518,23 @@ cudaError_t prepare_f64(dsnu_ds_plan_s* P) {
   return e;
 }
 
-dsnu_status linear_f32(dsnu_ds_plan_s* P, void* uv, int adjoint, cudaStream_t st) {
+dsnu_status linear_f32(dsnu_ds_plan_s* P, const void* uv, void* ov, int adjoint, cudaStream_t st) {
   using R = float;
-  cpx<R>* u = static_cast<cpx<R>*>(uv);
+  const cpx<R>* in = static_cast<const cpx<R>*>(uv);
+  cpx<R>* u = static_cast<cpx<R>*>(ov);
   const R scale = R(1.0 / (double(P->prm.nx) * double(P->prm.ny)));
   const cpx<R>* sx = static_cast<const cpx<R>*>(P->stw_x);
   const cpx<R>* sy = static_cast<const cpx<R>*>(P->stw_y);
   const cpx<R>* px = static_cast<const cpx<R>*>(P->px);
   const cpx<R>* py = static_cast<const cpx<R>*>(P->py);
-#define DSNU_ROWS(L2, INV)                                                                   \
-  k_c2c_rows<R, L2><<<P->grid_rows, GeoC2C<R, L2>::T, GeoC2C<R, L2>::smem, st>>>(u, P->prm.ny, sx, INV)
-#define DSNU_RF(L2) DSNU_ROWS(L2, 0)
-#define DSNU_RI(L2) DSNU_ROWS(L2, 1)
-#define DSNU_CP(L2)                                                                          \
-  k_c2c_cols_phase<R, L2><<<P->grid_cols, GeoC2C<R, L2>::T, GeoC2C<R, L2>::smem, st>>>(     \
-      u, P->prm.nx, sy, px, py, scale, adjoint)
+#define DSNU_ROWS(L2, SRC, INV)                                                                       \
+  launch_k(P->pdl, k_c2c_rows<R, L2>, dim3(P->grid_rows), dim3(GeoC2C<R, L2>::T), GeoC2C<R, L2>::smem, st, SRC, u, \
+           P->prm.ny, sx, INV)
+#define DSNU_RF(L2) DSNU_ROWS(L2, in, 0)
+#define DSNU_RI(L2) DSNU_ROWS(L2, static_cast<const cpx<R>*>(u), 1)
+#define DSNU_CP(L2)                                                                                   \
+  launch_k(P->pdl, k_c2c_cols_phase<R, L2>, dim3(P->grid_cols), dim3(GeoC2C<R, L2>::TC), GeoC2C<R, L2>::smem_cols, st, \
+           u, P->prm.nx, sy, px, py, scale, adjoint)
   switch (P->log2nx) {
     DSNU_C2C_CASES(DSNU_RF)
     default: return DSNU_EUNSUPPORTED;
@@ -526,20 +555,22 @@ dsnu_status linear_f32(dsnu_ds_plan_s* P, void* uv, int adjoint, cudaStream_t st
   return e == cudaSuccess ? DSNU_OK : ds_fail(DSNU_ECUDA, std::string("launch: ") + cudaGetErrorString(e));
 }
 
-dsnu_status linear_f64(dsnu_ds_plan_s* P, void* uv, int adjoint, cudaStream_t st) {
-  double2* u = static_cast<double2*>(uv);
+dsnu_status linear_f64(dsnu_ds_plan_s* P, const void* uv, void* ov, int adjoint, cudaStream_t st) {
+  const double2* in = static_cast<const double2*>(uv);
+  double2* u = static_cast<double2*>(ov);
   const int lscale = -(P->log2nx + P->log2ny);
   const fxw* sx = static_cast<const fxw*>(P->stw_x);
   const fxw* sy = static_cast<const fxw*>(P->stw_y);
   const fxw* px = static_cast<const fxw*>(P->px);
   const fxw* py = static_cast<const fxw*>(P->py);
-#define DSNU_ROWS(L2, INV) \
-  k_fx_c2c_rows<L2><<<P->grid_rows, FxOne<L2>::T, FxOne<L2>::smem, st>>>(u, P->prm.ny, sx, INV)
-#define DSNU_RF(L2) DSNU_ROWS(L2, 0)
-#define DSNU_RI(L2) DSNU_ROWS(L2, 1)
-#define DSNU_CP(L2)                                                                               \
-  k_fx_c2c_cols_phase<L2><<<P->grid_cols, FxCols<L2>::T, FxCols<L2>::smem, st>>>(u, P->prm.nx, sy, px, py, lscale, \
-                                                                                adjoint)
+#define DSNU_ROWS(L2, SRC, INV)                                                                        \
+  launch_k(P->pdl, k_fx_c2c_rows<L2>, dim3(P->grid_rows), dim3(FxOne<L2>::T), FxOne<L2>::smem, st, SRC, u, P->prm.ny, \
+           sx, INV)
+#define DSNU_RF(L2) DSNU_ROWS(L2, in, 0)
+#define DSNU_RI(L2) DSNU_ROWS(L2, static_cast<const double2*>(u), 1)
+#define DSNU_CP(L2)                                                                                    \
+  launch_k(P->pdl, k_fx_c2c_cols_phase<L2>, dim3(P->grid_cols), dim3(FxCols<L2>::T), FxCols<L2>::smem, st, u, P->prm.nx, \
+           sy, px, py, lscale, adjoint)
   switch (P->log2nx) {
     DSNU_C2C_CASES(DSNU_RF)
     default: return DSNU_EUNSUPPORTED;
@@ -636,6 +667,8 @@ dsnu_status dsnu_ds_plan_create(const dsnu_ds_params* params, void* stream, dsnu
     return ds_fail(DSNU_ECUDA, std::string("DS plan set-up: ") + cudaGetErrorString(e));
   }
   P->has_phase = false;
+  const char* env = std::getenv("DSNU_PDL");  // DSNU_PDL=0: plain stream-ordered launches
+  P->pdl = !(env && env[0] == '0');
   *out = P;
   return DSNU_OK;
 }
@@ -663,12 +696,16 @@ dsnu_status dsnu_ds_set_linear_step(dsnu_ds_plan plan, double tau, double alpha,
   return DSNU_OK;
 }
 
-dsnu_status dsnu_ds_linear(dsnu_ds_plan plan, void* u_dev, int32_t adjoint, void* stream) {
-  if (!plan || !u_dev) return ds_fail(DSNU_EINVAL, "NULL plan or field");
+dsnu_status dsnu_ds_linear_to(dsnu_ds_plan plan, const void* u_dev, void* out_dev, int32_t adjoint, void* stream) {
+  if (!plan || !u_dev || !out_dev) return ds_fail(DSNU_EINVAL, "NULL plan or field");
   if (!plan->has_phase) return ds_fail(DSNU_EINVAL, "no linear step set (dsnu_ds_set_linear_step)");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  return plan->prm.precision == DSNU_MIXED ? linear_f32(plan, u_dev, adjoint, st)
-                                           : linear_f64(plan, u_dev, adjoint, st);
+  return plan->prm.precision == DSNU_MIXED ? linear_f32(plan, u_dev, out_dev, adjoint, st)
+                                           : linear_f64(plan, u_dev, out_dev, adjoint, st);
+}
+
+dsnu_status dsnu_ds_linear(dsnu_ds_plan plan, void* u_dev, int32_t adjoint, void* stream) {
+  return dsnu_ds_linear_to(plan, u_dev, u_dev, adjoint, stream);
 }
 
 dsnu_status dsnu_ds_abs2(dsnu_ds_plan plan, const void* u_dev, double* rho_dev, void* stream) {
@@ -676,9 +713,9 @@ dsnu_status dsnu_ds_abs2(dsnu_ds_plan plan, const void* u_dev, double* rho_dev, 
   const size_t n = size_t(plan->prm.nx) * plan->prm.ny;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (plan->prm.precision == DSNU_MIXED)
-    k_abs2<float><<<grid_1d(n), 256, 0, st>>>(static_cast<const cpx<float>*>(u_dev), rho_dev, n);
+    launch_k(plan->pdl, k_abs2<float>, dim3(grid_1d(n)), dim3(256), 0, st, static_cast<const cpx<float>*>(u_dev), rho_dev, n);
   else
-    k_abs2<double><<<grid_1d(n), 256, 0, st>>>(static_cast<const cpx<double>*>(u_dev), rho_dev, n);
+    launch_k(plan->pdl, k_abs2<double>, dim3(grid_1d(n)), dim3(256), 0, st, static_cast<const cpx<double>*>(u_dev), rho_dev, n);
   return check_launch();
 }
 
@@ -688,25 +725,31 @@ dsnu_status dsnu_ds_abs2_vjp(dsnu_ds_plan plan, const void* u_dev, const double*
   const size_t n = size_t(plan->prm.nx) * plan->prm.ny;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (plan->prm.precision == DSNU_MIXED)
-    k_abs2_vjp<float><<<grid_1d(n), 256, 0, st>>>(static_cast<const cpx<float>*>(u_dev), g_rho_dev,
+    launch_k(plan->pdl, k_abs2_vjp<float>, dim3(grid_1d(n)), dim3(256), 0, st, static_cast<const cpx<float>*>(u_dev), g_rho_dev,
                                                  static_cast<cpx<float>*>(grad_dev), n);
   else
-    k_abs2_vjp<double><<<grid_1d(n), 256, 0, st>>>(static_cast<const cpx<double>*>(u_dev), g_rho_dev,
+    launch_k(plan->pdl, k_abs2_vjp<double>, dim3(grid_1d(n)), dim3(256), 0, st, static_cast<const cpx<double>*>(u_dev), g_rho_dev,
                                                   static_cast<cpx<double>*>(grad_dev), n);
+  return check_launch();
+}
+
+dsnu_status dsnu_ds_nonlinear_to(dsnu_ds_plan plan, const void* u_dev, const double* phi_dev, void* out_dev, double tau,
+                                 double beta, void* stream) {
+  if (!plan || !u_dev || !phi_dev || !out_dev) return ds_fail(DSNU_EINVAL, "NULL argument");
+  const size_t n = size_t(plan->prm.nx) * plan->prm.ny;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (plan->prm.precision == DSNU_MIXED)
+    launch_k(plan->pdl, k_nonlinear<float>, dim3(grid_1d(n)), dim3(256), 0, st, static_cast<const cpx<float>*>(u_dev),
+             static_cast<cpx<float>*>(out_dev), phi_dev, n, float(tau), float(beta));
+  else
+    launch_k(plan->pdl, k_nonlinear<double>, dim3(grid_1d(n)), dim3(256), 0, st,
+             static_cast<const cpx<double>*>(u_dev), static_cast<cpx<double>*>(out_dev), phi_dev, n, tau, beta);
   return check_launch();
 }
 
 dsnu_status dsnu_ds_nonlinear(dsnu_ds_plan plan, void* u_dev, const double* phi_dev, double tau, double beta,
                               void* stream) {
-  if (!plan || !u_dev || !phi_dev) return ds_fail(DSNU_EINVAL, "NULL argument");
-  const size_t n = size_t(plan->prm.nx) * plan->prm.ny;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (plan->prm.precision == DSNU_MIXED)
-    k_nonlinear<float><<<grid_1d(n), 256, 0, st>>>(static_cast<cpx<float>*>(u_dev), phi_dev, n, float(tau),
-                                                  float(beta));
-  else
-    k_nonlinear<double><<<grid_1d(n), 256, 0, st>>>(static_cast<cpx<double>*>(u_dev), phi_dev, n, tau, beta);
-  return check_launch();
+  return dsnu_ds_nonlinear_to(plan, u_dev, phi_dev, u_dev, tau, beta, stream);
 }
 
 dsnu_status dsnu_ds_nonlinear_vjp(dsnu_ds_plan plan, const void* u_dev, const double* phi_dev, const void* g_dev,
@@ -715,11 +758,11 @@ dsnu_status dsnu_ds_nonlinear_vjp(dsnu_ds_plan plan, const void* u_dev, const do
   const size_t n = size_t(plan->prm.nx) * plan->prm.ny;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (plan->prm.precision == DSNU_MIXED)
-    k_nonlinear_vjp<float><<<grid_1d(n), 256, 0, st>>>(
+    launch_k(plan->pdl, k_nonlinear_vjp<float>, dim3(grid_1d(n)), dim3(256), 0, st, 
         static_cast<const cpx<float>*>(u_dev), phi_dev, static_cast<const cpx<float>*>(g_dev), n, float(tau),
         float(beta), s_dev, static_cast<cpx<float>*>(part_dev));
   else
-    k_nonlinear_vjp<double><<<grid_1d(n), 256, 0, st>>>(
+    launch_k(plan->pdl, k_nonlinear_vjp<double>, dim3(grid_1d(n)), dim3(256), 0, st, 
         static_cast<const cpx<double>*>(u_dev), phi_dev, static_cast<const cpx<double>*>(g_dev), n, tau, beta,
         s_dev, static_cast<cpx<double>*>(part_dev));
   return check_launch();
@@ -732,11 +775,11 @@ dsnu_status dsnu_ds_nonlinear_vjp_finish(dsnu_ds_plan plan, const void* u_dev, c
   const size_t n = size_t(plan->prm.nx) * plan->prm.ny;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (plan->prm.precision == DSNU_MIXED)
-    k_nonlinear_vjp_finish<float><<<grid_1d(n), 256, 0, st>>>(
+    launch_k(plan->pdl, k_nonlinear_vjp_finish<float>, dim3(grid_1d(n)), dim3(256), 0, st, 
         static_cast<const cpx<float>*>(u_dev), s_dev, ats_dev, n, float(tau), float(beta),
         static_cast<cpx<float>*>(grad_dev));
   else
-    k_nonlinear_vjp_finish<double><<<grid_1d(n), 256, 0, st>>>(
+    launch_k(plan->pdl, k_nonlinear_vjp_finish<double>, dim3(grid_1d(n)), dim3(256), 0, st, 
         static_cast<const cpx<double>*>(u_dev), s_dev, ats_dev, n, tau, beta, static_cast<cpx<double>*>(grad_dev));
   return check_launch();
 }
