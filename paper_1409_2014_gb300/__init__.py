@@ -24,6 +24,14 @@ _RADIAL = {"legendre": _abi.DSNU_RADIAL_LEGENDRE, "jacobi": _abi.DSNU_RADIAL_JAC
 _ACCUM = {"fp64": _abi.DSNU_ACCUM_FP64, "working": _abi.DSNU_ACCUM_WORKING}
 
 
+def _raw_stream(device) -> int:
+    """The current stream's handle on a CUDA device with an index (the public
+    torch.cuda.current_stream builds a Stream object: 10 us on a Grace host)."""
+    import torch
+
+    return torch._C._cuda_getCurrentRawStream(device.index)
+
+
 def make_params(nx, ny, lx, ly, cut_radius, n_r, n_theta, sigma=0.0, kernel_width=0,
                 precision="fp64", partition="gauss", radial="legendre", accumulation="fp64") -> dsnu_params:
     """partition "none" selects the standard periodic FFT solver (no split, no
@@ -58,6 +66,7 @@ class Plan:
         dev = torch.device(device if device is not None else "cuda")
         if dev.type != "cuda":
             raise ValueError("the solver runs on CUDA devices only")
+        torch.cuda.init()
         if dev.index is None:
             dev = torch.device("cuda", torch.cuda.current_device())
         self.device = dev
@@ -67,7 +76,7 @@ class Plan:
         self.shape = (int(ny), int(nx))
         self._handle = None
         with torch.cuda.device(self.device):
-            stream = torch.cuda.current_stream(self.device).cuda_stream
+            stream = _raw_stream(self.device)
             if multiplier is None:
                 self._handle = dsnu_plan_create(self.params, stream)
             else:
@@ -114,7 +123,7 @@ class Plan:
             out = torch.empty_like(x)
         else:
             self._check_input(out)
-        stream = torch.cuda.current_stream(self.device).cuda_stream
+        stream = _raw_stream(self.device)
         fn(self._handle, x.data_ptr(), out.data_ptr(), stream)
         return out
 
@@ -136,7 +145,7 @@ class Plan:
                 raise ValueError("host buffers must be contiguous float64 CPU tensors of the grid shape")
         self._check_input(rho_dev)
         self._check_input(phi_dev)
-        stream = torch.cuda.current_stream(self.device).cuda_stream
+        stream = _raw_stream(self.device)
         dsnu_solve_host(self._handle, rho_host.data_ptr(), phi_host.data_ptr(), rho_dev.data_ptr(),
                         phi_dev.data_ptr(), stream)
         return phi_host
@@ -159,7 +168,7 @@ class Plan:
         nbytes = _abi.dsnu_stream_staging_bytes(self._handle)
         if getattr(self, "_staging", None) is None or self._staging.numel() < nbytes:
             self._staging = torch.empty(nbytes, dtype=torch.uint8, device=self.device)
-        stream = torch.cuda.current_stream(self.device).cuda_stream
+        stream = _raw_stream(self.device)
         _abi.dsnu_solve_host_stream(self._handle, [t.data_ptr() for t in rho_hosts],
                                     [t.data_ptr() for t in phi_hosts], self._staging.data_ptr(),
                                     self._staging.numel(), stream)
@@ -176,7 +185,7 @@ class Plan:
     def status_poll(self) -> int:
         import torch
 
-        return dsnu_status_poll(self._handle, torch.cuda.current_stream(self.device).cuda_stream)
+        return dsnu_status_poll(self._handle, _raw_stream(self.device))
 
     def close(self):
         if self._handle is not None:
@@ -223,7 +232,7 @@ class Batch:
         self.workspace = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=self.device)
         _abi.dsnu_batch_bind(self._h, [r.data_ptr() for r in rhos], [f.data_ptr() for f in phis],
                              self.workspace.data_ptr(), self.workspace.numel(),
-                             torch.cuda.current_stream(self.device).cuda_stream)
+                             _raw_stream(self.device))
 
     @property
     def schedule_in_use(self) -> str:
@@ -246,7 +255,7 @@ class Batch:
     def solve(self):
         import torch
 
-        _abi.dsnu_batch_solve(self._h, torch.cuda.current_stream(self.device).cuda_stream)
+        _abi.dsnu_batch_solve(self._h, _raw_stream(self.device))
         return self.phis
 
     def close(self):

@@ -25,13 +25,9 @@ import torch
 import torch.utils.checkpoint as _ckpt
 
 from . import _abi
-from . import Plan
+from . import Plan, _raw_stream as _stream
 
 _PREC = {"fp64": _abi.DSNU_FP64, "mixed": _abi.DSNU_MIXED}
-
-
-def _stream(dev):
-    return torch.cuda.current_stream(dev).cuda_stream
 
 
 class DSPlan:
@@ -43,6 +39,7 @@ class DSPlan:
         ny = nx if ny is None else ny
         ly = lx if ly is None else ly
         dev = torch.device(device if device is not None else "cuda")
+        torch.cuda.init()
         if dev.index is None:
             dev = torch.device("cuda", torch.cuda.current_device())
         self.device = dev
@@ -68,6 +65,13 @@ class DSPlan:
         _abi.dsnu_ds_linear(self._h, u.data_ptr(), 1 if adjoint else 0, _stream(self.device))
         return u
 
+    def linear(self, u, adjoint=False):
+        """The linear flow of u in a new tensor (u is only read)."""
+        self._chk(u)
+        out = torch.empty_like(u)
+        _abi.dsnu_ds_linear_to(self._h, u.data_ptr(), out.data_ptr(), 1 if adjoint else 0, _stream(self.device))
+        return out
+
     def abs2(self, u):
         self._chk(u)
         rho = torch.empty(self.shape, dtype=torch.float64, device=self.device)
@@ -86,6 +90,14 @@ class DSPlan:
         self._chk(u)
         _abi.dsnu_ds_nonlinear(self._h, u.data_ptr(), phi.data_ptr(), tau, beta, _stream(self.device))
         return u
+
+    def nonlinear(self, u, phi, tau, beta):
+        """The nonlinear flow of u in a new tensor (u is only read)."""
+        self._chk(u)
+        out = torch.empty_like(u)
+        _abi.dsnu_ds_nonlinear_to(self._h, u.data_ptr(), phi.data_ptr(), out.data_ptr(), tau, beta,
+                                  _stream(self.device))
+        return out
 
     def nonlinear_vjp(self, u, phi, g, tau, beta):
         self._chk(u)
@@ -162,12 +174,12 @@ class LinearFlow(torch.autograd.Function):
     def forward(ctx, u, ds: DSPlan, tau, alpha):
         ctx.ds, ctx.tau, ctx.alpha = ds, tau, alpha
         ds.set_linear_step(tau, alpha)
-        return ds.linear_(u.contiguous().clone())
+        return ds.linear(u.contiguous())
 
     @staticmethod
     def backward(ctx, g):
         ctx.ds.set_linear_step(ctx.tau, ctx.alpha)
-        return ctx.ds.linear_(g.contiguous().clone(), adjoint=True), None, None, None
+        return ctx.ds.linear(g.contiguous(), adjoint=True), None, None, None
 
 
 class NonlinearFlow(torch.autograd.Function):
@@ -179,7 +191,7 @@ class NonlinearFlow(torch.autograd.Function):
         phi = solver.solve(ds.abs2(u))
         ctx.save_for_backward(u, phi)
         ctx.ds, ctx.solver, ctx.tau, ctx.beta = ds, solver, tau, beta
-        return ds.nonlinear_(u.clone(), phi, tau, beta)
+        return ds.nonlinear(u, phi, tau, beta)
 
     @staticmethod
     def backward(ctx, g):
@@ -216,18 +228,30 @@ def yoshida_step(u, ds: DSPlan, solver: Plan, tau, alpha, beta):
     return u
 
 
-_SCHEMES = {"strang": strang_step, "yoshida": yoshida_step}
+# strang_step and yoshida_step as (linear sub-steps, nonlinear sub-steps) in the order they act
+_SUBSTEPS = {"strang": ((0.5, 0.5), (1.0,)), "yoshida": (YOSHIDA_A[::-1], YOSHIDA_B[::-1])}
 
 
 def evolve(u0, steps, ds: DSPlan, solver: Plan, tau, alpha, beta, checkpoint_every=0, scheme="strang"):
     """``steps`` steps of ``scheme`` ("strang" or "yoshida"); with
     checkpoint_every > 0 only the input of every segment of that many steps is
-    kept for the backward pass, and each segment is recomputed during backward."""
-    step = _SCHEMES[scheme]
+    kept for the backward pass, and each segment is recomputed during backward.
+
+    The last linear flow of a step and the first one of the next are one flow
+    over the sum of their steps (the linear flow is exact): a segment of n Strang
+    steps runs n + 1 linear flows instead of 2 n."""
+    lin, non = _SUBSTEPS[scheme]
 
     def segment(u, n):
-        for _ in range(n):
-            u = step(u, ds, solver, tau, alpha, beta)
+        if n:
+            u = LinearFlow.apply(u, ds, lin[0] * tau, alpha)
+        for k in range(n):
+            for j, b in enumerate(non):
+                u = NonlinearFlow.apply(u, ds, solver, b * tau, beta)
+                a = lin[j + 1]
+                if j + 1 == len(non) and k + 1 < n:
+                    a += lin[0]
+                u = LinearFlow.apply(u, ds, a * tau, alpha)
         return u
 
     u = u0
@@ -235,7 +259,8 @@ def evolve(u0, steps, ds: DSPlan, solver: Plan, tau, alpha, beta, checkpoint_eve
         done = 0
         while done < steps:
             n = min(checkpoint_every, steps - done)
-            u = _ckpt.checkpoint(segment, u, n, use_reentrant=False)
+            # (nothing in a segment draws random numbers)
+            u = _ckpt.checkpoint(segment, u, n, use_reentrant=False, preserve_rng_state=False)
             done += n
         return u
     return segment(u, steps)
