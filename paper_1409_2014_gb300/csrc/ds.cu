@@ -134,12 +134,12 @@ k_c2c_cols_phase(cpx<R>* __restrict__ u, int nx, const cpx<R>* __restrict__ stw_
 
 // u[row][t + G m] of group threads t: the values' bits, and their largest
 // exponent (fx_top).
-template <int G, int P>
-__device__ __forceinline__ unsigned fx_load(fxc (&v)[16], const double2* u, size_t stride, bool valid,
+template <int P, int E>
+__device__ __forceinline__ unsigned fx_load(fxc (&v)[E], const double2* u, size_t stride, bool valid,
                                             unsigned* red) {
   unsigned mx = 0;
 #pragma unroll
-  for (int m = 0; m < 16; ++m) {
+  for (int m = 0; m < E; ++m) {
     const double2 a = valid ? u[stride * m] : make_double2(0.0, 0.0);
     mx = fx_top(fx_top(mx, a.x), a.y);
     v[m] = fx_mk(__double_as_longlong(a.x), __double_as_longlong(a.y));
@@ -149,7 +149,7 @@ __device__ __forceinline__ unsigned fx_load(fxc (&v)[16], const double2* u, size
   mx = fx_read<P, true>(mx, red);
   const int efm = fx_efm(mx);
 #pragma unroll
-  for (int m = 0; m < 16; ++m)
+  for (int m = 0; m < E; ++m)
     v[m] = fx_shr<5>(fx_mk(fx_from_f64(__longlong_as_double(v[m].x), efm), fx_from_f64(__longlong_as_double(v[m].y), efm)));
   return mx;
 }
@@ -162,12 +162,12 @@ template <int LOG2N>
 __global__ void __launch_bounds__(FxOne<LOG2N>::T, FxOne<LOG2N>::MINB)
 k_fx_c2c_rows(const double2* src, double2* dst, int ny, const fxw* __restrict__ stw_g, int inv) {
   using GG = FxOne<LOG2N>;
-  constexpr int N = GG::N, G = GG::G, PER = GG::PER, W = GG::W;
+  constexpr int N = GG::N, E = GG::E, G = GG::G, PER = GG::PER, W = GG::W;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fxw* stw = reinterpret_cast<fxw*>(smem_raw);
   fxc* sm = reinterpret_cast<fxc*>(stw + GG::STW);
   unsigned* red = reinterpret_cast<unsigned*>(sm + PER * GG::FB);
-  fx_copy(stw, stw_g, fft_stage_tw_elems(LOG2N));
+  fx_copy(stw, stw_g, FxRad<LOG2N>::stw());
   const int pr = threadIdx.x / G, t = threadIdx.x - pr * G;
   fxc* buf = sm + pr * GG::FB;
   __syncthreads();
@@ -179,16 +179,16 @@ k_fx_c2c_rows(const double2* src, double2* dst, int ny, const fxw* __restrict__ 
     const int row = item * PER + pr;
     const bool valid = row < ny;
     const size_t at = size_t(valid ? row : 0) * N + t;
-    fxc v[16];
-    const unsigned mx = fx_load<G, G>(v, src + at, G, valid, red + 2 * W);
+    fxc v[E];
+    const unsigned mx = fx_load<G, E>(v, src + at, G, valid, red + 2 * W);
     if (inv) {
 #pragma unroll
-      for (int m = 0; m < 16; ++m) v[m] = fx_swap(v[m]);
+      for (int m = 0; m < E; ++m) v[m] = fx_swap(v[m]);
     }
     const int ex = fx_efm(mx) - kFxBias + 5 + fx_fft<LOG2N, G>(v, buf, t, stw, red);
     if (valid) {
 #pragma unroll
-      for (int m = 0; m < 16; ++m) dst[at + G * m] = fx_store(inv ? fx_swap(v[m]) : v[m], ex, mx);
+      for (int m = 0; m < E; ++m) dst[at + G * m] = fx_store(inv ? fx_swap(v[m]) : v[m], ex, mx);
     }
   }
 }
@@ -211,12 +211,12 @@ __global__ void __launch_bounds__(FxCols<LOG2N>::T, FxCols<LOG2N>::MINB)
 k_fx_c2c_cols_phase(double2* __restrict__ u, int nx, const fxw* __restrict__ stw_g, const fxw* __restrict__ px,
                     const fxw* __restrict__ py, int lscale, int adj) {
   using GG = FxCols<LOG2N>;
-  constexpr int G = GG::G, P = GG::P, PER = GG::PER, W = GG::W;
+  constexpr int E = GG::E, G = GG::G, P = GG::P, PER = GG::PER, W = GG::W;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fxw* stw = reinterpret_cast<fxw*>(smem_raw);
   fxc* sm = reinterpret_cast<fxc*>(stw + GG::STW);
   unsigned* red = reinterpret_cast<unsigned*>(sm + PER * 2 * GG::FBS);
-  fx_copy(stw, stw_g, fft_stage_tw_elems(LOG2N));
+  fx_copy(stw, stw_g, FxRad<LOG2N>::stw());
   const int pr = threadIdx.x / P, tp = threadIdx.x - pr * P;
   const int h = tp & 1, t = tp >> 1;
   fxc* buf = sm + (2 * pr + h) * GG::FBS;
@@ -229,8 +229,8 @@ k_fx_c2c_cols_phase(double2* __restrict__ u, int nx, const fxw* __restrict__ stw
     const int col = 2 * (item * PER + pr) + h;
     const bool valid = col < nx;
     double2* uc = u + size_t(t) * nx + (valid ? col : h);
-    fxc v[16];
-    const unsigned mx = fx_load<G, P>(v, uc, size_t(G) * nx, valid, red + 2 * W);
+    fxc v[E];
+    const unsigned mx = fx_load<P, E>(v, uc, size_t(G) * nx, valid, red + 2 * W);
     int ex = fx_efm(mx) - kFxBias + 5 + lscale;
 #pragma unroll 1
     for (int inv = 0;; ++inv) {  // forward, then inverse (one copy of the transform's code)
@@ -243,7 +243,7 @@ k_fx_c2c_cols_phase(double2* __restrict__ u, int nx, const fxw* __restrict__ stw
       fxw wx = fx_ldw(px + (valid ? col : 0));
       if (adj) wx = fx_conj(wx);
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         fxw wy = fx_ldw(py + t + G * m);
         if (adj) wy = fx_conj(wy);
         // /16 by each phase (magnitudes < 2^62.5), 2^3 between them; components
@@ -253,7 +253,7 @@ k_fx_c2c_cols_phase(double2* __restrict__ u, int nx, const fxw* __restrict__ stw
     }
     if (valid) {
 #pragma unroll
-      for (int m = 0; m < 16; ++m) uc[size_t(G) * m * nx] = fx_store(fx_swap(v[m]), ex, mx);
+      for (int m = 0; m < E; ++m) uc[size_t(G) * m * nx] = fx_store(fx_swap(v[m]), ex, mx);
     }
   }
 }
@@ -417,13 +417,11 @@ dsnu_status ds_fail(dsnu_status s, const std::string& m) {
   return s;
 }
 
-void stage_twiddles(int log2n, std::vector<double>& out) {
+// Stage twiddles for stages of radix 2^lr (the last one what is left).
+void stage_twiddles(int log2n, int lr, std::vector<double>& out) {
   out.clear();
-  const int full = log2n / 4;
-  const int nst = (log2n + 3) / 4;
-  for (int s = 1; s < nst; ++s) {
-    const int lr = (s < full) ? 4 : (log2n - 4 * full);
-    const int rad = 1 << lr, ns = 1 << (4 * s);
+  for (int s = 1; s * lr < log2n; ++s) {
+    const int rad = 1 << std::min(lr, log2n - s * lr), ns = 1 << (s * lr);
     for (int r = 1; r < rad; ++r)
       for (int k = 0; k < ns; ++k) {
         const double a = -2.0 * M_PI * double(r) * double(k) / double(ns * rad);
@@ -626,8 +624,9 @@ dsnu_status dsnu_ds_plan_create(const dsnu_ds_params* params, void* stream, dsnu
   P->log2ny = ilog2i(p.ny);
   const size_t rsz = p.precision == DSNU_MIXED ? 4 : 8;
   std::vector<double> sx, sy;
-  stage_twiddles(P->log2nx, sx);
-  stage_twiddles(P->log2ny, sy);
+  const bool fx = p.precision == DSNU_FP64;
+  stage_twiddles(P->log2nx, fx ? fx_log2_radix(P->log2nx) : 4, sx);
+  stage_twiddles(P->log2ny, fx ? fx_log2_radix(P->log2ny) : 4, sy);
   auto al = [](size_t v) { return (v + 255) & ~size_t(255); };
   const size_t o_sx = 0, o_sy = al(sx.size() * rsz), o_px = o_sy + al(sy.size() * rsz);
   const size_t o_py = o_px + al(2 * size_t(p.nx) * rsz), total = o_py + al(2 * size_t(p.ny) * rsz);

@@ -29,6 +29,10 @@
 
 #include "common.cuh"
 
+#ifndef FX_E8_MAX
+#define FX_E8_MAX 10
+#endif
+
 namespace dsnu {
 
 using i64 = long long;
@@ -172,10 +176,11 @@ __device__ __forceinline__ unsigned fx_mag(unsigned m, i64 v) {
   return m | unsigned(h ^ (h >> 31));
 }
 __device__ __forceinline__ unsigned fx_mag(unsigned m, fxc a) { return fx_mag(fx_mag(m, a.x), a.y); }
-__device__ __forceinline__ unsigned fx_mag(const fxc (&a)[16]) {
+template <int E>
+__device__ __forceinline__ unsigned fx_mag(const fxc (&a)[E]) {
   unsigned m = 0;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) m = fx_mag(m, a[i]);
+  for (int i = 0; i < E; ++i) m = fx_mag(m, a[i]);
   return m;
 }
 
@@ -214,8 +219,26 @@ template <int T>
 __device__ __forceinline__ int fx_norm_shift(unsigned m) { return max(__clz(int(m)) - (64 - T), 0); }
 
 // ---------------------------------------------------------------------------
-// Length-N DFT by a group of G = N/16 threads, 16 values per thread (the index
-// order and buffer layout of block_fft_regs).  P threads share one scale: G, or
+// Values per thread, the radix of the stages: 16, or 8 for the short transforms,
+// whose passes do not fill the GPU: twice the threads, each with less than half
+// the instructions in a row (FP64 solves with 8 against 16 values: 128^2 66 -> 49
+// us, 512^2 92 -> 86, 1024 x 256 88 -> 76, 1024^2 equal, 2048^2 534 -> 639).
+template <int LOG2N>
+struct FxRad {
+  static constexpr int LE = (LOG2N <= FX_E8_MAX) ? 3 : 4, E = 1 << LE;
+  static constexpr int FULL = LOG2N / LE, LR = LOG2N - LE * FULL;  // radix-E stages, log2 of the last one's radix
+  // stage twiddles (e^{-2 pi i r k/(NS RAD)}, r = 1 .. RAD - 1, k < NS, stage by stage)
+  __host__ __device__ static constexpr int stw() {
+    int n = 0;
+    for (int s = 1; s < FULL; ++s) n += (E - 1) << (LE * s);
+    return n + (LR > 0 ? ((1 << LR) - 1) << (LE * FULL) : 0);
+  }
+  static constexpr int STW = stw() > 0 ? stw() : 1;
+};
+inline int fx_log2_radix(int log2n) { return log2n <= FX_E8_MAX ? 3 : 4; }
+
+// Length-N DFT by a group of G = N/E threads, E values per thread (the index
+// order and buffer layout of block_fft_regs with E for 16).  P threads share one scale: G, or
 // 2 G where two groups work together (the even and the odd chain of one row or
 // column, two adjacent columns).  One transform per thread keeps it at 128 registers and one
 // copy of the radix-16 code for all stages (the loop below): two transforms per
@@ -223,18 +246,26 @@ __device__ __forceinline__ int fx_norm_shift(unsigned m) { return max(__clz(int(
 // twice as long (column pass at 4096^2 1405 us).
 // Returns the exponent that the result gained.  red: 2 words per warp.
 template <int LOG2N, int P>
-__device__ __forceinline__ int fx_fft(fxc (&v)[16], fxc* buf, int t, const fxw* __restrict__ stw, unsigned* red) {
-  constexpr int N = 1 << LOG2N, G = N / 16, FULL = LOG2N / 4, LR = LOG2N - 4 * FULL;
+__device__ __forceinline__ int fx_fft(fxc (&v)[FxRad<LOG2N>::E], fxc* buf, int t, const fxw* __restrict__ stw,
+                                      unsigned* red) {
+  using FR = FxRad<LOG2N>;
+  constexpr int N = 1 << LOG2N, LE = FR::LE, E = FR::E, G = N / E, FULL = FR::FULL, LR = FR::LR;
   int ex = 0;
-  // leave stage s (radix 16, NS = 16^s): exchange, and scale for the next one
+  // leave stage s (radix E, NS = E^s): exchange, and scale for the next one
   auto exchange = [&](int s) {
-    const int ns = 1 << (4 * s), k = t & (ns - 1);
-    const int base = pad16((t - k) * 16 + k), st = (s == 0) ? 1 : ns + (ns >> 4);
+    const int ns = 1 << (LE * s), k = t & (ns - 1);
+    const int base = (t - k) * E + k;
     unsigned* rd = red + (s & 1) * (blockDim.x >> 5);
     const unsigned m0 = fx_post<P>(fx_mag(v), rd);
     __syncthreads();  // every load of this buffer done (in place)
+    if constexpr (E == 16) {  // (pad16 is linear over the stride)
+      const int b0 = pad16(base), st = (s == 0) ? 1 : ns + (ns >> 4);
 #pragma unroll
-    for (int r = 0; r < 16; ++r) buf[base + r * st] = v[r];
+      for (int r = 0; r < E; ++r) buf[b0 + r * st] = v[r];
+    } else {
+#pragma unroll
+      for (int r = 0; r < E; ++r) buf[pad16(base + r * ns)] = v[r];
+    }
     __syncthreads();
     const int sh = fx_norm_shift<61>(fx_read<P>(m0, rd));
     ex += 4 - sh;
@@ -242,23 +273,23 @@ __device__ __forceinline__ int fx_fft(fxc (&v)[16], fxc* buf, int t, const fxw* 
   };
 #pragma unroll 1
   for (int s = 0;; ++s) {
-    fx_dft<16>(v);
+    fx_dft<E>(v);
     if (s == FULL - 1) break;
     const int sh = exchange(s);
-    const int ns = 16 << (4 * s);
-    const fxw* tw = stw + (ns - 16) + (t & (ns - 1));  // 15 (16 + .. + ns/16) = ns - 16 entries before
+    const int ns = E << (LE * s);
+    const fxw* tw = stw + (ns - E) + (t & (ns - 1));  // (E - 1)(E + .. + ns/E) = ns - E entries before
     v[0] = fx_shr<4>(fx_shl(buf[pad16(t)], sh));
 #pragma unroll
-    for (int r = 1; r < 16; ++r) v[r] = fx_mul(fx_shl(buf[pad16(t + r * G)], sh), tw[(r - 1) * ns]);
+    for (int r = 1; r < E; ++r) v[r] = fx_mul(fx_shl(buf[pad16(t + r * G)], sh), tw[(r - 1) * ns]);
   }
   if constexpr (LR > 0) {
-    constexpr int RAD = 1 << LR, NS = 1 << (4 * FULL), PER = 16 / RAD, NB = N / RAD;
+    constexpr int RAD = 1 << LR, NS = 1 << (LE * FULL), PER = E / RAD, NB = N / RAD;
     const int sh = exchange(FULL - 1);
-    fxc o[16];
+    fxc o[E];
 #pragma unroll
     for (int b = 0; b < PER; ++b) {
       const int j = t + b * G;
-      const fxw* tw = stw + (NS - 16) + (j & (NS - 1));
+      const fxw* tw = stw + (NS - E) + (j & (NS - 1));
       fxc u[RAD];
       u[0] = fx_shr<4>(fx_shl(buf[pad16(j)], sh));
 #pragma unroll
@@ -268,19 +299,20 @@ __device__ __forceinline__ int fx_fft(fxc (&v)[16], fxc* buf, int t, const fxw* 
       for (int r = 0; r < RAD; ++r) o[b + r * PER] = u[r];
     }
 #pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = o[m];
+    for (int m = 0; m < E; ++m) v[m] = o[m];
   }
   return ex;
 }
 // The unnormalised inverse e^{+2 pi i nk/N}: real and imaginary parts
 // exchanged before and after (register renaming).
 template <int LOG2N, int P>
-__device__ __forceinline__ int fx_ifft(fxc (&v)[16], fxc* buf, int t, const fxw* __restrict__ stw, unsigned* red) {
+__device__ __forceinline__ int fx_ifft(fxc (&v)[FxRad<LOG2N>::E], fxc* buf, int t, const fxw* __restrict__ stw,
+                                       unsigned* red) {
 #pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = fx_swap(v[m]);
+  for (int m = 0; m < FxRad<LOG2N>::E; ++m) v[m] = fx_swap(v[m]);
   const int ex = fx_fft<LOG2N, P>(v, buf, t, stw, red);
 #pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = fx_swap(v[m]);
+  for (int m = 0; m < FxRad<LOG2N>::E; ++m) v[m] = fx_swap(v[m]);
   return ex;
 }
 
@@ -317,13 +349,13 @@ __device__ __forceinline__ double fx_to_f64(i64 v, int e) { return fx_scale(__ll
 // one warp's worth for the short ones (a small grid spreads over the SMs).
 template <int LOG2N>
 struct FxOne {
-  static constexpr int N = 1 << LOG2N;
-  static constexpr int G = N / 16;
+  static constexpr int N = 1 << LOG2N, E = FxRad<LOG2N>::E;
+  static constexpr int G = N / E;
   static constexpr int PER = (G >= 64) ? 2 : (G >= 32) ? 1 : 32 / G;
   static constexpr int T = PER * G;
-  static constexpr int MINB = 512 / T;
+  static constexpr int MINB = (E == 16 ? 512 : 768) / T;
   static constexpr int FB = fft_buf_elems(N);
-  static constexpr int STW = fft_stage_tw_elems(LOG2N) > 0 ? fft_stage_tw_elems(LOG2N) : 1;
+  static constexpr int STW = FxRad<LOG2N>::STW;
   static constexpr int W = T / 32, RED = 5 * W;
   static constexpr size_t smem = size_t(STW + PER * FB) * 16 + ((RED * 4 + 15) & ~15);
 };
@@ -382,5 +414,16 @@ __device__ __forceinline__ fxc fx_sra(fxc a, int s) { return fx_mk(fx_sra(a.x, s
 // are stored below 2^63 and become smaller than 2^(63 - HEAD)).
 template <int HEAD>
 __device__ __forceinline__ int fx_align(int emax, int e) { return min(emax - e + HEAD, 63); }
+
+// Alignment shifts, a byte each, packed by four.
+template <int E>
+__device__ __forceinline__ void fx_pack(unsigned (&pk)[(E + 3) / 4], int i, int s) {
+  if ((i & 3) == 0) pk[i >> 2] = 0;
+  pk[i >> 2] |= unsigned(s) << (8 * (i & 3));
+}
+template <int W>
+__device__ __forceinline__ int fx_byte(const unsigned (&pk)[W], int i) {
+  return int((pk[i >> 2] >> (8 * (i & 3))) & 0xFFu);
+}
 
 }  // namespace dsnu

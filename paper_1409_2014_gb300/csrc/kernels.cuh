@@ -630,14 +630,17 @@ k_band_fwd(Members mem, WsOff off, int ldqB, int ncols, int ldq, int Q, AxisTabs
 // stencils reach into shared memory (whole band columns' runs, read
 // coalesced once; the Hermitian fold for q_x < 0 and the centring phase
 // applied on the way; zero outside the band) and then runs every node's
-// stencil sum from there, four threads per node.  The band values are read
+// stencil sum from there.  The band values are read
 // once per item instead of once per stencil that covers them, in runs rather
 // than in scattered 8-byte loads (one warp per node gathering them from the
 // band array took 79 us on 12 SMs, against 19 us on 6 for this form), and a CTA
 // starts all its nodes at once, which is what makes the stage fast on the few
 // SMs it gets next to the column pass.
-constexpr int kItile = 32;       // tile edge (stencil origins)
-constexpr int kItileNodes = 64;  // nodes per work item at most (four threads each: 256)
+// Small tiles with eight threads per node keep an item short: 32 x 32 tiles of up
+// to 64 nodes with four threads each took 10.2 us, these 8.6 (mixed, 16384 nodes,
+// event times); in FP64 plans (spread_fx.cuh) 14.9 and 10.8 at 2048 nodes.
+constexpr int kItile = 16;       // tile edge (stencil origins)
+constexpr int kItileNodes = 32;  // nodes per work item at most (eight threads each: 256)
 template <typename R>
 __device__ __forceinline__ void interp_tile_body(int tile, int mi, Members mem, WsOff off, int ldq, int Q,
                                                  const int2* __restrict__ q0, const R* __restrict__ wts,
@@ -649,10 +652,9 @@ __device__ __forceinline__ void interp_tile_body(int tile, int mi, Members mem, 
   const int S = kItile + w - 1;
   const int2 org = tile_org[tile];
   const int n0 = tile_ptr[tile], n1 = tile_ptr[tile + 1];
-  // four threads per node (an item holds at most 64), thread h of a node
-  // taking the stencil rows b = h, h + 4, ...; the node's plan data are
-  // fetched before the wait for the band values
-  const int s = threadIdx.x >> 2, h = threadIdx.x & 3;
+  // eight threads per node, thread h of a node taking the stencil rows b = h and
+  // h + 8; the node's plan data are fetched before the wait for the band values
+  const int s = threadIdx.x >> 3, h = threadIdx.x & 7;
   const bool have = n0 + s < n1;
   const int j = have ? tile_nodes[n0 + s] : 0;
   const int2 b0 = have ? q0[j] : make_int2(0, 0);
@@ -682,7 +684,7 @@ __device__ __forceinline__ void interp_tile_body(int tile, int mi, Members mem, 
     const R* wx = wts + size_t(j) * 2 * w;
     const R* wy = wx + w;
     const cpx<R>* rb = reg + (b0.x - org.x) * S + (b0.y - org.y);
-    for (int b = h; b < w; b += 4) {
+    for (int b = h; b < w; b += 8) {
       const R fy = wy[b];
       for (int a = 0; a < w; ++a) {
         const cpx<R> v = rb[a * S + b];
@@ -692,11 +694,12 @@ __device__ __forceinline__ void interp_tile_body(int tile, int mi, Members mem, 
       }
     }
   }
-  ax += __shfl_xor_sync(0xffffffffu, ax, 1);
-  ay += __shfl_xor_sync(0xffffffffu, ay, 1);
-  ax += __shfl_xor_sync(0xffffffffu, ax, 2);
-  ay += __shfl_xor_sync(0xffffffffu, ay, 2);
-  // the four partial sums of a node (lanes 4 s' .. 4 s' + 3 of the warp)
+  // the eight partial sums of a node (adjacent lanes)
+#pragma unroll
+  for (int i = 1; i < 8; i <<= 1) {
+    ax += __shfl_xor_sync(0xffffffffu, ax, i);
+    ay += __shfl_xor_sync(0xffffffffu, ay, i);
+  }
   if (have && h == 0) {
     const cpx<R> v = mk<R>(R(d * double(ax)), R(d * double(ay)));
     c[j] = v;

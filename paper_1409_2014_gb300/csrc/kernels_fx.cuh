@@ -17,10 +17,10 @@
 //   * for real input the transposed pipeline (every complex constant
 //     conjugated) computes the complex conjugate of each intermediate and the
 //     same real result, so dsnu_solve_adjoint runs these same kernels.
-// A pair of groups of G = N/16 threads works on one row or column: group h = 0
-// runs the even, h = 1 the odd chain (even and odd frequencies, or output
+// A pair of groups of G = N/E threads (E values per thread, 16 or 8) works on one
+// row or column: group h = 0 runs the even, h = 1 the odd chain (even and odd frequencies, or output
 // points).  Inputs are loaded, converted and aligned once, each thread taking
-// N/(2 G) of them, and handed to both chains through shared memory.  A CTA
+// E/2 of them, and handed to both chains through shared memory.  A CTA
 // holds one pair, or as many as fill a warp, so that a small grid spreads over
 // as many SMs as it has rows.
 #pragma once
@@ -32,13 +32,13 @@ namespace dsnu {
 
 template <int LOG2N>
 struct FxGeo {
-  static constexpr int N = 1 << LOG2N, M = 2 * N;
-  static constexpr int G = N / 16, P = 2 * G;         // threads per chain, per pair
+  static constexpr int N = 1 << LOG2N, M = 2 * N, E = FxRad<LOG2N>::E;
+  static constexpr int G = N / E, P = 2 * G;          // threads per chain, per pair
   static constexpr int PER = (P >= 32) ? 1 : 32 / P;  // pairs per CTA
   static constexpr int T = PER * P;
-  static constexpr int MINB = 512 / T;                // 16 warps per SM
+  static constexpr int MINB = (E == 16 ? 512 : 768) / T;  // 16 warps per SM, 24 with 8 values per thread
   static constexpr int FB = fft_buf_elems(N);
-  static constexpr int STW = fft_stage_tw_elems(LOG2N) > 0 ? fft_stage_tw_elems(LOG2N) : 1;
+  static constexpr int STW = FxRad<LOG2N>::STW;
   static constexpr int W = T / 32, RED = 5 * W;       // words of the reductions: two for the FFT, three more
   static constexpr size_t smem = size_t(STW + PER * 2 * FB) * 16 + ((RED * 4 + 15) & ~15);
   // inverse rows: a byte of alignment shift per column of A, and one of B
@@ -62,10 +62,11 @@ struct FxMult {
   int ldm;
 };
 
-// e^{-2 pi i n/M} at n = t + G m
+// e^{-2 pi i n/M} at n = t + G m, m < E
+template <int E>
 __device__ __forceinline__ fxw fx_wm(const fxw* __restrict__ wm, int t, int m, int G) {
-  fxw w = fx_ldw(wm + t + G * (m & 7));
-  if (m >= 8) {  // e^{-2 pi i (n' + N/2)/M} = -i e^{-2 pi i n'/M}
+  fxw w = fx_ldw(wm + t + G * (m & (E / 2 - 1)));
+  if (m >= E / 2) {  // e^{-2 pi i (n' + N/2)/M} = -i e^{-2 pi i n'/M}
     const fxw v = w;
     w.rh = v.ih;
     w.rl = v.il;
@@ -76,40 +77,40 @@ __device__ __forceinline__ fxw fx_wm(const fxw* __restrict__ wm, int t, int m, i
 }
 // The chains' inputs from the staged values z (|component| < 2^61 after the
 // shift s): z/16 for the even one, z e^{-2 pi i n/M}/16 for the odd one.
-template <int G>
-__device__ __forceinline__ void fx_chain_in(fxc (&v)[16], const fxc* st, int s, int h, int t, const fxw* wm) {
+template <int G, int E>
+__device__ __forceinline__ void fx_chain_in(fxc (&v)[E], const fxc* st, int s, int h, int t, const fxw* wm) {
   if (h == 0) {
 #pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = fx_shr<4>(fx_shl(st[pad16(t + G * m)], s));
+    for (int m = 0; m < E; ++m) v[m] = fx_shr<4>(fx_shl(st[pad16(t + G * m)], s));
   } else {
 #pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = fx_mul(fx_shl(st[pad16(t + G * m)], s), fx_wm(wm, t, m, G));
+    for (int m = 0; m < E; ++m) v[m] = fx_mul(fx_shl(st[pad16(t + G * m)], s), fx_wm<E>(wm, t, m, G));
   }
 }
 // The column sum e(n)/16 + e^{+2 pi i n/M} o(n)/16 of the two chains' results at
-// n = t + G (m + 8 h), m < 8: each chain hands the other half of its values over
+// n = t + G (m + h E/2), m < E/2: each chain hands the other half of its values over
 // (in its own buffer) and multiplies half of the odd ones.
-template <int G>
-__device__ __forceinline__ void fx_chain_out(fxc (&v)[16], fxc* buf_e, fxc* buf_o, int s, int h, int t,
+template <int G, int E>
+__device__ __forceinline__ void fx_chain_out(fxc (&v)[E], fxc* buf_e, fxc* buf_o, int s, int h, int t,
                                              const fxw* wm) {
   __syncthreads();  // the last stage's loads of the buffers are done
   if (h == 0) {
 #pragma unroll
-    for (int m = 8; m < 16; ++m) buf_e[pad16(t + G * m)] = v[m];
+    for (int m = E / 2; m < E; ++m) buf_e[pad16(t + G * m)] = v[m];
   } else {
 #pragma unroll
-    for (int m = 0; m < 8; ++m) buf_o[pad16(t + G * m)] = v[m];
+    for (int m = 0; m < E / 2; ++m) buf_o[pad16(t + G * m)] = v[m];
   }
   __syncthreads();
   if (h == 0) {
 #pragma unroll
-    for (int m = 0; m < 8; ++m)
-      v[m] = fx_shr<4>(fx_shl(v[m], s)) + fx_mul(fx_shl(buf_o[pad16(t + G * m)], s), fx_conj(fx_wm(wm, t, m, G)));
+    for (int m = 0; m < E / 2; ++m)
+      v[m] = fx_shr<4>(fx_shl(v[m], s)) + fx_mul(fx_shl(buf_o[pad16(t + G * m)], s), fx_conj(fx_wm<E>(wm, t, m, G)));
   } else {
 #pragma unroll
-    for (int m = 0; m < 8; ++m)
-      v[m] = fx_shr<4>(fx_shl(buf_e[pad16(t + G * (m + 8))], s)) +
-             fx_mul(fx_shl(v[m + 8], s), fx_conj(fx_wm(wm, t, m + 8, G)));
+    for (int m = 0; m < E / 2; ++m)
+      v[m] = fx_shr<4>(fx_shl(buf_e[pad16(t + G * (m + E / 2))], s)) +
+             fx_mul(fx_shl(v[m + E / 2], s), fx_conj(fx_wm<E>(wm, t, m + E / 2, G)));
   }
 }
 
@@ -117,12 +118,13 @@ __device__ __forceinline__ void fx_chain_out(fxc (&v)[16], fxc* buf_e, fxc* buf_
 #define DSNU_FX_SETUP(AX)                                                  \
   using GG = FxGeo<LOG2N>;                                                 \
   using TL = Tile<double>;                                                 \
-  constexpr int N = GG::N, G = GG::G, P = GG::P, PER = GG::PER, W = GG::W; \
+  constexpr int N = GG::N, E = GG::E, H = E / 2, G = GG::G, P = GG::P;     \
+  constexpr int PER = GG::PER, W = GG::W;                                  \
   extern __shared__ __align__(16) unsigned char smem_raw[];                \
   fxw* stw = reinterpret_cast<fxw*>(smem_raw);                             \
   fxc* sm = reinterpret_cast<fxc*>(stw + GG::STW);                         \
   unsigned* red = reinterpret_cast<unsigned*>(sm + PER * 2 * GG::FB);      \
-  fx_copy(stw, (AX).stw, fft_stage_tw_elems(LOG2N));                       \
+  fx_copy(stw, (AX).stw, FxRad<LOG2N>::stw());                             \
   const int pr = threadIdx.x / P, tp = threadIdx.x - pr * P;               \
   const int h = tp / G, t = tp - h * G;                                    \
   fxc* buf_e = sm + (2 * pr) * GG::FB;                                     \
@@ -144,11 +146,11 @@ k_fx_row_fwd(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
     const int mi = it / items, row = (it - mi * items) * PER + pr;
     const Member mb = member_at(mem, mi);
     const bool valid = row < ny;
-    double x[8];
-    fxr d[8];
+    double x[H];
+    fxr d[H];
     unsigned mx = 0, md = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < H; ++i) {
       x[i] = valid ? __ldg(mb.rho + size_t(row) * N + tp + P * i) : 0.0;
       d[i] = fx_ldr(ax.dec + tp + P * i);
       mx = fx_top(mx, x[i]);
@@ -164,19 +166,19 @@ k_fx_row_fwd(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
     // 2^(ef + 1), d_x/2^kd < 2^(1 - clz h)): z = rho + i rho d_x/2^k
     const int kr = min(max(int(md) - 32 + kd + 1 - efm, 0), kd);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < H; ++i) {
       const i64 v = fx_from_f64(x[i], efm);
       buf_e[pad16(tp + P * i)] = fx_mk(fx_shr<1>(v), fx_mulr(v, d[i]) << (kd - kr));  // <= 2^61
     }
     __syncthreads();
-    fxc v[16];
-    fx_chain_in<G>(v, buf_e, 0, h, t, ax.wm);
+    fxc v[E];
+    fx_chain_in<G, E>(v, buf_e, 0, h, t, ax.wm);
     const int ef = fx_fft<LOG2N, P>(v, buf, t, stw, red);
     const unsigned mag = fx_post<P>(fx_mag(v), red + 4 * W);
     __syncthreads();  // (and the last stage's loads are done)
     const int s1 = fx_norm_shift<62>(fx_read<P>(mag, red + 4 * W));  // sums of two: below 2^63
 #pragma unroll
-    for (int m = 0; m < 16; ++m) buf[pad16(t + G * m)] = v[m];
+    for (int m = 0; m < E; ++m) buf[pad16(t + G * m)] = v[m];
     __syncthreads();
     // exponent of Z: from_f64 (efm - kFxBias), the five bits, the stages;
     // A = (Z(q) + conj Z(M - q))/2 and B = (Z(q) - conj Z(M - q))/2i as sums, times 2^s1
@@ -189,9 +191,9 @@ k_fx_row_fwd(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
       fxc* Ar = ws_ptr<fxc>(mb, off.A) + TL::at(row, 0, ldqA);
       fxc* Br = ws_ptr<fxc>(mb, off.B) + TL::at(row, 0, ldqB);
 #pragma unroll
-      for (int i = 0; i < 9; ++i) {
+      for (int i = 0; i < H + 1; ++i) {
         const int q = tp + P * i;
-        if (i == 8 && q > N) break;
+        if (i == H && q > N) break;
         const int k = q >> 1;
         const fxc zq = (q & 1) ? buf_o[pad16(k)] : buf_e[pad16(k & (N - 1))];
         const fxc zm = (q & 1) ? buf_o[pad16(N - 1 - k)] : buf_e[pad16((N - k) & (N - 1))];
@@ -202,17 +204,16 @@ k_fx_row_fwd(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
   }
 }
 
-// Alignment shifts, a byte each, of the rows tp + P i that a thread stages.
-// Returns the rows' largest exponent.
-template <int P>
-__device__ __forceinline__ int fx_row_shifts(const int* rexp, int ny, int tp, unsigned* red, unsigned (&pk)[2]) {
+// Alignment shifts of the rows tp + P i that a thread stages.  Returns the rows'
+// largest exponent.
+template <int P, int H>
+__device__ __forceinline__ int fx_row_shifts(const int* rexp, int ny, int tp, unsigned* red,
+                                             unsigned (&pk)[(H + 3) / 4]) {
   const int emax = fx_cta_max(rexp, ny, red);
-  pk[0] = pk[1] = 0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) pk[i >> 2] |= unsigned(fx_align<2>(emax, rexp[tp + P * i])) << (8 * (i & 3));
+  for (int i = 0; i < H; ++i) fx_pack<H>(pk, i, fx_align<2>(emax, rexp[tp + P * i]));
   return emax;
 }
-__device__ __forceinline__ int fx_byte(const unsigned (&pk)[2], int i) { return int((pk[i >> 2] >> (8 * (i & 3))) & 0xFFu); }
 
 // ---------------------------------------------------------------------------
 // Column pass of I1 (k_col_main in fixed point).  FULL: the multiplier row has
@@ -225,34 +226,34 @@ k_fx_col_main(Members mem, FxOff off, int ldqA, int ncols, FxAxis ay, FxMult mt)
   constexpr int MH = FULL ? N : N / 2 + 1;  // even entries
   const int items = (ncols + PER - 1) / PER;
   int cur = -1, emax = 0;
-  unsigned pk[2] = {0, 0};
+  unsigned pk[(H + 3) / 4] = {};
 #pragma unroll 1
   for (int it = blockIdx.x; it < items * mem.count; it += gridDim.x) {
     if (it + int(gridDim.x) >= items * mem.count) grid_dep_trigger();  // last item of this CTA
     const int mi = it / items, col = (it - mi * items) * PER + pr;
     const Member mb = member_at(mem, mi);
     if (mi != cur) {
-      emax = fx_row_shifts<P>(ws_ptr<int>(mb, off.rexp), N, tp, red + 4 * W, pk);
+      emax = fx_row_shifts<P, H>(ws_ptr<int>(mb, off.rexp), N, tp, red + 4 * W, pk);
       cur = mi;
     }
     fxc* __restrict__ A = ws_ptr<fxc>(mb, off.A);
     const bool valid = col < ncols;
-    fxc v[16];
+    fxc v[E];
     unsigned mag = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = valid ? A[TL::at(tp + P * i, col, ldqA)] : fx_mk(0, 0);
+    for (int i = 0; i < H; ++i) v[i] = valid ? A[TL::at(tp + P * i, col, ldqA)] : fx_mk(0, 0);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < H; ++i) {
       v[i] = fx_sra(v[i], fx_byte(pk, i));
       mag = fx_mag(mag, v[i]);
     }
     mag = fx_post<P>(mag, red + 2 * W);
     __syncthreads();  // (and the previous item's reads of the buffers are done)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) buf_e[pad16(tp + P * i)] = v[i];
+    for (int i = 0; i < H; ++i) buf_e[pad16(tp + P * i)] = v[i];
     __syncthreads();
     const int s0 = fx_norm_shift<61>(fx_read<P>(mag, red + 2 * W));
-    fx_chain_in<G>(v, buf_e, s0, h, t, ay.wm);
+    fx_chain_in<G, E>(v, buf_e, s0, h, t, ay.wm);
     // exponent: the rows', s0, /16, stages, s1, multiplier (its own and /32), stages, s2, /16, the last 3 bits
     int ex = emax + 2 - s0 + 4 + (mt.mexp && valid ? mt.mexp[col] : 0) + 5 + 4 - 3;
 #pragma unroll 1
@@ -264,22 +265,22 @@ k_fx_col_main(Members mem, FxOff off, int ldqA, int ncols, FxAxis ay, FxMult mt)
       ex -= s;
       if (inv) {
 #pragma unroll
-        for (int m = 0; m < 16; ++m) v[m] = fx_swap(v[m]);
-        fx_chain_out<G>(v, buf_e, buf_o, s, h, t, ay.wm);
+        for (int m = 0; m < E; ++m) v[m] = fx_swap(v[m]);
+        fx_chain_out<G, E>(v, buf_e, buf_o, s, h, t, ay.wm);
         break;
       }
       const fxr* mg = mt.m1 + size_t(valid ? col : 0) * mt.ldm + (h ? MH : 0);
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         const int k = t + G * m;  // row q = 2 k + h: |qbar| / 2 rounded down
-        const fxr c = fx_ldr(mg + (FULL ? k : (m < 8 ? k : N - h - k)));
+        const fxr c = fx_ldr(mg + (FULL ? k : (m < H ? k : N - h - k)));
         const fxc x = fx_shl(v[m], s);
         v[m] = fx_mk(fx_mulr(x.y, c), fx_mulr(x.x, c));  // (components exchanged: the inverse transform)
       }
     }
     if (valid) {
 #pragma unroll
-      for (int m = 0; m < 8; ++m) A[TL::at(t + G * (m + 8 * h), col, ldqA)] = fx_shl(v[m], 3);  // < 2^59.5 before
+      for (int m = 0; m < H; ++m) A[TL::at(t + G * (m + H * h), col, ldqA)] = fx_shl(v[m], 3);  // < 2^59.5 before
       if (tp == 0) ws_ptr<int>(mb, off.cexp)[col] = (emax >= kFxBad) ? kFxBad : (emax <= kFxZero) ? kFxZero : ex;
     }
   }
@@ -295,25 +296,25 @@ k_fx_band_fwd(Members mem, FxOff off, int ldqB, int ncols, int ldq, int Q, FxAxi
   constexpr int M = GG::M;
   const int items = (ncols + PER - 1) / PER;
   int cur = -1, emax = 0;
-  unsigned pk[2] = {0, 0};
+  unsigned pk[(H + 3) / 4] = {};
 #pragma unroll 1
   for (int it = blockIdx.x; it < items * mem.count; it += gridDim.x) {
     if (it + int(gridDim.x) >= items * mem.count) grid_dep_trigger();  // last item of this CTA
     const int mi = it / items, col = (it - mi * items) * PER + pr;
     const Member mb = member_at(mem, mi);
     if (mi != cur) {
-      emax = fx_row_shifts<P>(ws_ptr<int>(mb, off.rexpb), N, tp, red + 4 * W, pk);
+      emax = fx_row_shifts<P, H>(ws_ptr<int>(mb, off.rexpb), N, tp, red + 4 * W, pk);
       cur = mi;
     }
     const fxc* __restrict__ B = ws_ptr<fxc>(mb, off.B);
     double2* __restrict__ Bband = ws_ptr<double2>(mb, off.Bband);
     const bool valid = col < ncols;
-    fxc v[16];
+    fxc v[E];
     unsigned mag = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = valid ? B[TL::at(tp + P * i, col, ldqB)] : fx_mk(0, 0);
+    for (int i = 0; i < H; ++i) v[i] = valid ? B[TL::at(tp + P * i, col, ldqB)] : fx_mk(0, 0);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < H; ++i) {
       v[i] = fx_sra(v[i], fx_byte(pk, i));
       mag = fx_mag(mag, v[i]);
     }
@@ -321,19 +322,19 @@ k_fx_band_fwd(Members mem, FxOff off, int ldqB, int ncols, int ldq, int Q, FxAxi
     __syncthreads();
     const int s0 = fx_norm_shift<61>(fx_read<P>(mag, red + 2 * W));
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < H; ++i) {
       const fxr d = fx_ldr(ay.dec + tp + P * i);  // d_y/2^kdy, and /2
       const fxc x = fx_shl(v[i], s0);
       buf_e[pad16(tp + P * i)] = fx_mk(fx_mulr(x.x, d), fx_mulr(x.y, d));
     }
     __syncthreads();
-    fx_chain_in<G>(v, buf_e, 1, h, t, ay.wm);
+    fx_chain_in<G, E>(v, buf_e, 1, h, t, ay.wm);
     const int ex = emax + 2 - s0 + kdy + 4 + fx_fft<LOG2N, P>(v, buf, t, stw, red);
     if (valid) {
       const bool bad = emax >= kFxBad;
       const double nan = __longlong_as_double(0x7FF8000000000000ll);
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         const int q = 2 * (t + G * m) + h, sq = q < N ? q : q - M;
         if (sq >= -Q && sq <= Q)
           Bband[size_t(col) * ldq + sq + Q] =
@@ -359,10 +360,10 @@ k_fx_band_inv(Members mem, FxOff off, int ldq, int Q, int ncols, int ldqB, FxAxi
     const double2* __restrict__ Sband = ws_ptr<double2>(mb, off.Sband);
     fxc* __restrict__ St = ws_ptr<fxc>(mb, off.B);
     const bool valid = col < ncols;
-    fxc v[16];
+    fxc v[E];
     unsigned mx = 0;
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
+    for (int m = 0; m < E; ++m) {
       const int q = 2 * (t + G * m) + h, sq = q < N ? q : q - M;
       double2 a = make_double2(0.0, 0.0);
       if (valid && sq >= -Q && sq <= Q) a = Sband[size_t(col) * ldq + sq + Q];
@@ -374,17 +375,17 @@ k_fx_band_inv(Members mem, FxOff off, int ldq, int Q, int ncols, int ldqB, FxAxi
     mx = fx_read<P, true>(mx, red + 2 * W);
     const int efm = fx_efm(mx);
 #pragma unroll
-    for (int m = 0; m < 16; ++m)
+    for (int m = 0; m < E; ++m)
       v[m] = fx_shr<5>(fx_mk(fx_from_f64(__longlong_as_double(v[m].x), efm), fx_from_f64(__longlong_as_double(v[m].y), efm)));
     const int ef = fx_ifft<LOG2N, P>(v, buf, t, stw, red);
     const unsigned mag = fx_post<P>(fx_mag(v), red + 3 * W);
     __syncthreads();
     const int s1 = fx_norm_shift<62>(fx_read<P>(mag, red + 3 * W));
-    fx_chain_out<G>(v, buf_e, buf_o, s1, h, t, ay.wm);
+    fx_chain_out<G, E>(v, buf_e, buf_o, s1, h, t, ay.wm);
     if (valid) {
 #pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        const int n = t + G * (m + 8 * h);
+      for (int m = 0; m < H; ++m) {
+        const int n = t + G * (m + H * h);
         const fxr d = fx_ldr(ay.dec + n);
         St[TL::at(n, col, ldqB)] = fx_shl(fx_mk(fx_mulr(v[m].x, d), fx_mulr(v[m].y, d)), 4);  // < 2^58.5 before
       }
@@ -425,19 +426,19 @@ k_fx_row_inv(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
     const fxc* __restrict__ Ar = ws_ptr<fxc>(mb, off.A) + TL::at(valid ? row : 0, 0, ldqA);
     const fxc* __restrict__ Br = ws_ptr<fxc>(mb, off.B) + TL::at(valid ? row : 0, 0, ldqB);
     const fxc z = fx_mk(0, 0);
-    fxc v[16];  // X in the first, R in the second half
+    fxc v[E];  // X in the first, R in the second half
     unsigned mag = 0;
     fxc yn = z;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = valid ? Ar[(tp + P * i) * TL::TR] : z;
+    for (int i = 0; i < H; ++i) v[i] = valid ? Ar[(tp + P * i) * TL::TR] : z;
     if (valid && tp == 0) yn = Ar[N * TL::TR];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < H; ++i) {
       const int q = tp + P * i;
       const fxc y = fx_sra(v[i], sh_a[q]);
       const fxc s = (valid && q <= Q) ? fx_sra(Br[q * TL::TR], sh_b[q]) : z;
       v[i] = fx_mk(y.x - s.y, y.y + s.x);
-      v[i + 8] = fx_mk(y.x + s.y, y.y - s.x);
+      v[i + H] = fx_mk(y.x + s.y, y.y - s.x);
     }
     mag = fx_mag(v);
     if (tp == 0) {  // conj X(N) (Q < N: no band value) in the place of conj R(N - 0)
@@ -448,25 +449,25 @@ k_fx_row_inv(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
     mag = fx_post<P>(mag, red + 2 * W);
     __syncthreads();  // (and the previous item's reads of the buffers are done)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < H; ++i) {
       const int q = tp + P * i;
       buf_e[pad16(q)] = v[i];
-      if (q != 0) buf_o[pad16(N - q)] = v[i + 8];  // R(N - q) at q
+      if (q != 0) buf_o[pad16(N - q)] = v[i + H];  // R(N - q) at q
     }
     if (tp == 0) buf_o[0] = yn;
     __syncthreads();
     const int s0 = fx_norm_shift<60>(fx_read<P>(mag, red + 2 * W));
     if (h == 0) {
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         const fxc x = buf_e[pad16(t + G * m)], r = buf_o[pad16(t + G * m)];
         v[m] = fx_shr<4>(fx_shl(fx_mk(x.x + r.x, x.y - r.y), s0));
       }
     } else {
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         const fxc x = buf_e[pad16(t + G * m)], r = buf_o[pad16(t + G * m)];
-        v[m] = fx_mul(fx_shl(fx_mk(x.x - r.x, x.y + r.y), s0), fx_conj(fx_wm(ax.wm, t, m, G)));
+        v[m] = fx_mul(fx_shl(fx_mk(x.x - r.x, x.y + r.y), s0), fx_conj(fx_wm<E>(ax.wm, t, m, G)));
       }
     }
     const int ex = emax + 4 - s0 + 4 + kd + 1 + lscale + fx_ifft<LOG2N, P>(v, buf, t, stw, red);
@@ -475,7 +476,7 @@ k_fx_row_inv(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
       const bool bad = emax >= kFxBad;
       const i64 half = i64(1) << kd;
 #pragma unroll
-      for (int m = 0; m < 8; ++m) {
+      for (int m = 0; m < H; ++m) {
         const int n = 2 * (t + G * m);
         // Re T 2^-(kd + 1) + Im T d_x/2^kd /2
         const i64 f = ((v[m].x + half) >> (kd + 1)) + fx_mulr(v[m].y, fx_ldr(ax.dec + n + h));

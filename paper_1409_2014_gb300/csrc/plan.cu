@@ -310,13 +310,11 @@ static void twiddles(int n, int m, std::vector<double>& out) {
 // FFT stage twiddles of a length-2^log2n transform in the order the device
 // FFT reads them: stage s >= 1 (radix RAD, NS = product of the earlier
 // radices), r = 1..RAD-1, k = 0..NS-1: e^{-2 pi i r k / (NS RAD)}.
-static void fft_stage_twiddles(int log2n, std::vector<double>& out) {
+// (lr: log2 of the full stages' radix)
+static void fft_stage_twiddles(int log2n, std::vector<double>& out, int lr = 4) {
   out.clear();
-  const int full = log2n / 4;
-  const int nst = (log2n + 3) / 4;
-  for (int s = 1; s < nst; ++s) {
-    const int lr = (s < full) ? 4 : (log2n - 4 * full);
-    const int rad = 1 << lr, ns = 1 << (4 * s);
+  for (int s = 1; s * lr < log2n; ++s) {
+    const int rad = 1 << std::min(lr, log2n - s * lr), ns = 1 << (s * lr);
     for (int r = 1; r < rad; ++r)
       for (int k = 0; k < ns; ++k) {
         const double a = -2.0 * M_PI * double(r) * double(k) / double(ns * rad);
@@ -674,8 +672,8 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   g.m1_full = (g.m_generic && g.m_as != 0.0) ? 1 : 0;
   g.m1_ld = g.m1_full ? My : ny + 4;
   if constexpr (sizeof(R) == 8) {
-    fft_stage_twiddles(g.log2nx, tmp); T.fx_stw_x = fx_table(tmp, kFxTwBits);
-    fft_stage_twiddles(g.log2ny, tmp); T.fx_stw_y = fx_table(tmp, kFxTwBits);
+    fft_stage_twiddles(g.log2nx, tmp, fx_log2_radix(g.log2nx)); T.fx_stw_x = fx_table(tmp, kFxTwBits);
+    fft_stage_twiddles(g.log2ny, tmp, fx_log2_radix(g.log2ny)); T.fx_stw_y = fx_table(tmp, kFxTwBits);
     twiddles(nx / 2, Mx, tmp); T.fx_wm_x = fx_table(tmp, kFxTwBits);
     twiddles(ny / 2, My, tmp); T.fx_wm_y = fx_table(tmp, kFxTwBits);
     g.kdx = fx_decon(dcx, T.fx_dec_x);
@@ -829,9 +827,9 @@ static dsnu_status build_tables_standard_fx(dsnu_plan_s* P, cudaStream_t st) {
   const dsnu_params& p = P->prm;
   PlanGeom& g = P->geom;
   std::vector<double> tmp;
-  fft_stage_twiddles(g.log2nx, tmp);
+  fft_stage_twiddles(g.log2nx, tmp, fx_log2_radix(g.log2nx));
   const std::vector<int> stw_x = fx_table(tmp, kFxTwBits);
-  fft_stage_twiddles(g.log2ny, tmp);
+  fft_stage_twiddles(g.log2ny, tmp, fx_log2_radix(g.log2ny));
   const std::vector<int> stw_y = fx_table(tmp, kFxTwBits);
   const double dkx = M_PI / p.lx, dky = M_PI / p.ly;
   std::vector<int> mexp;

@@ -64,8 +64,8 @@ k_fx_interp_tile(Members mem, WsOff off, int ldq, int Q, const int2* __restrict_
   int2* sw = reinterpret_cast<int2*>(reg + S * S);          // [node of the item][2 w]
   const int2 org = tile_org[blockIdx.x];
   const int n0 = tile_ptr[blockIdx.x], cnt = tile_ptr[blockIdx.x + 1] - n0;
-  // four threads per node, thread h of a node taking the stencil rows b = h, h + 4, ...
-  const int s = threadIdx.x >> 2, h = threadIdx.x & 3;
+  // eight threads per node, thread h of a node taking the stencil rows b = h and h + 8
+  const int s = threadIdx.x >> 3, h = threadIdx.x & 7;
   const bool have = s < cnt;
   const int j = have ? tile_nodes[n0 + s] : 0;
   const int2 b0 = have ? q0[j] : org;
@@ -107,7 +107,7 @@ k_fx_interp_tile(Members mem, WsOff off, int ldq, int Q, const int2* __restrict_
   if (have) {
     const int2* wx = sw + s * w2;
     const int4* rb = reg + (b0.x - org.x) * S + (b0.y - org.y);
-    for (int b = h; b < w; b += 4) {
+    for (int b = h; b < w; b += 8) {
       i64 p = 0, q = 0, r = 0, u = 0;
 #pragma unroll 4
       for (int a = 0; a < w; ++a) {
@@ -128,10 +128,11 @@ k_fx_interp_tile(Members mem, WsOff off, int ldq, int Q, const int2* __restrict_
     }
   }
   i64 sx = fx_sum28(px, qx), sy = fx_sum28(py, qy);
-  sx += __shfl_xor_sync(0xffffffffu, sx, 1);
-  sy += __shfl_xor_sync(0xffffffffu, sy, 1);
-  sx += __shfl_xor_sync(0xffffffffu, sx, 2);
-  sy += __shfl_xor_sync(0xffffffffu, sy, 2);
+#pragma unroll
+  for (int i = 1; i < 8; i <<= 1) {
+    sx += __shfl_xor_sync(0xffffffffu, sx, i);
+    sy += __shfl_xor_sync(0xffffffffu, sy, i);
+  }
   if (have && h == 0) {
     const int ex = efm - kFxBias54 + 4;
     double2 r = make_double2(d * fx_to_f64(sx, ex), d * fx_to_f64(sy, ex));

@@ -15,12 +15,13 @@ namespace dsnu {
 #define DSNU_FX_SETUP1(STWG)                                               \
   using GG = FxOne<LOG2N>;                                                 \
   using TL = Tile<double>;                                                 \
-  constexpr int N = GG::N, G = GG::G, P = G, PER = GG::PER, W = GG::W;     \
+  constexpr int N = GG::N, E = GG::E, H = E / 2, G = GG::G, P = G;         \
+  constexpr int PER = GG::PER, W = GG::W;                                  \
   extern __shared__ __align__(16) unsigned char smem_raw[];                \
   fxw* stw = reinterpret_cast<fxw*>(smem_raw);                             \
   fxc* sm = reinterpret_cast<fxc*>(stw + GG::STW);                         \
   unsigned* red = reinterpret_cast<unsigned*>(sm + PER * GG::FB);          \
-  fx_copy(stw, STWG, fft_stage_tw_elems(LOG2N));                           \
+  fx_copy(stw, STWG, FxRad<LOG2N>::stw());                                 \
   const int pr = threadIdx.x / G, t = threadIdx.x - pr * G;                \
   fxc* buf = sm + pr * GG::FB;                                             \
   __syncthreads();                                                         \
@@ -38,10 +39,10 @@ k_fx_std_row_fwd(Members mem, size_t offH, size_t offE, int ldq, int ny, const f
     const Member mb = member_at(mem, mi);
     const bool valid = pi < pairs;
     const double* ra = mb.rho + size_t(valid ? 2 * pi : 0) * N;
-    fxc v[16];
+    fxc v[E];
     unsigned mx = 0;
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
+    for (int m = 0; m < E; ++m) {
       const double a = valid ? __ldg(ra + t + G * m) : 0.0, b = valid ? __ldg(ra + N + t + G * m) : 0.0;
       mx = fx_top(fx_top(mx, a), b);
       v[m] = fx_mk(__double_as_longlong(a), __double_as_longlong(b));
@@ -51,25 +52,25 @@ k_fx_std_row_fwd(Members mem, size_t offH, size_t offE, int ldq, int ny, const f
     mx = fx_read<P, true>(mx, red + 2 * W);
     const int efm = fx_efm(mx);
 #pragma unroll
-    for (int m = 0; m < 16; ++m)
+    for (int m = 0; m < E; ++m)
       v[m] = fx_shr<5>(fx_mk(fx_from_f64(__longlong_as_double(v[m].x), efm), fx_from_f64(__longlong_as_double(v[m].y), efm)));
     const int ef = fx_fft<LOG2N, P>(v, buf, t, stw, red);
     const unsigned mag = fx_post<P>(fx_mag(v), red + 3 * W);
     __syncthreads();
     const int s1 = fx_norm_shift<62>(fx_read<P>(mag, red + 3 * W));  // sums of two: below 2^63
 #pragma unroll
-    for (int m = 0; m < 16; ++m) buf[pad16(t + G * m)] = v[m];
+    for (int m = 0; m < E; ++m) buf[pad16(t + G * m)] = v[m];
     __syncthreads();
     if (valid) {
-      fxc* H = ws_ptr<fxc>(mb, offH) + TL::at(2 * pi, 0, ldq);
+      fxc* hs = ws_ptr<fxc>(mb, offH) + TL::at(2 * pi, 0, ldq);
 #pragma unroll
-      for (int i = 0; i < 9; ++i) {
+      for (int i = 0; i < H + 1; ++i) {
         const int q = t + G * i;
-        if (i == 8 && q > N / 2) break;
+        if (i == H && q > N / 2) break;
         const fxc zq = buf[pad16(q)], zm = buf[pad16((N - q) & (N - 1))];
         // X_a = (Z(q) + conj Z(N - q)) / 2,  X_b = (Z(q) - conj Z(N - q)) / (2i), as sums
-        H[q * TL::TR] = fx_shl(fx_mk(zq.x + zm.x, zq.y - zm.y), s1);
-        H[q * TL::TR + 1] = fx_shl(fx_mk(zq.y + zm.y, zm.x - zq.x), s1);
+        hs[q * TL::TR] = fx_shl(fx_mk(zq.x + zm.x, zq.y - zm.y), s1);
+        hs[q * TL::TR + 1] = fx_shl(fx_mk(zq.y + zm.y, zm.x - zq.x), s1);
       }
       if (t == 0) ws_ptr<int>(mb, offE)[pi] = fx_exp(mx, efm - kFxBias + 5 + ef - 1 - s1);
     }
@@ -85,7 +86,7 @@ k_fx_std_col(Members mem, size_t offH, size_t offE, size_t offC, int ldq, int nc
   DSNU_FX_SETUP1(stw_g)
   const int items = (ncols + PER - 1) / PER;
   int cur = -1, emax = 0;
-  unsigned pk[4] = {0, 0, 0, 0};  // alignment shifts of the rows t + G m
+  unsigned pk[(E + 3) / 4] = {};  // alignment shifts of the rows t + G m
 #pragma unroll 1
   for (int it = blockIdx.x; it < items * mem.count; it += gridDim.x) {
     if (it + int(gridDim.x) >= items * mem.count) grid_dep_trigger();  // last item of this CTA
@@ -95,28 +96,25 @@ k_fx_std_col(Members mem, size_t offH, size_t offE, size_t offC, int ldq, int nc
       const int* re = ws_ptr<int>(mb, offE);
       emax = fx_cta_max(re, N / 2, red + 4 * W);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) pk[i] = 0;
-#pragma unroll
-      for (int m = 0; m < 16; ++m)
-        pk[m >> 2] |= unsigned(fx_align<2>(emax, re[(t + G * m) >> 1])) << (8 * (m & 3));
+      for (int m = 0; m < E; ++m) fx_pack<E>(pk, m, fx_align<2>(emax, re[(t + G * m) >> 1]));
       cur = mi;
     }
-    fxc* __restrict__ H = ws_ptr<fxc>(mb, offH);
+    fxc* __restrict__ hs = ws_ptr<fxc>(mb, offH);
     const bool valid = col < ncols;
-    fxc v[16];
+    fxc v[E];
     unsigned mag = 0;
 #pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = valid ? H[TL::at(t + G * m, col, ldq)] : fx_mk(0, 0);
+    for (int m = 0; m < E; ++m) v[m] = valid ? hs[TL::at(t + G * m, col, ldq)] : fx_mk(0, 0);
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      v[m] = fx_sra(v[m], int((pk[m >> 2] >> (8 * (m & 3))) & 0xFFu));
+    for (int m = 0; m < E; ++m) {
+      v[m] = fx_sra(v[m], fx_byte(pk, m));
       mag = fx_mag(mag, v[m]);
     }
     mag = fx_post<P>(mag, red + 2 * W);
     __syncthreads();
     const int s0 = fx_norm_shift<61>(fx_read<P>(mag, red + 2 * W));
 #pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = fx_shr<4>(fx_shl(v[m], s0));
+    for (int m = 0; m < E; ++m) v[m] = fx_shr<4>(fx_shl(v[m], s0));
     int ex = emax + 2 - s0 + 4 + (mt.mexp && valid ? mt.mexp[col] : 0) + 5;
 #pragma unroll 1
     for (int inv = 0;; ++inv) {  // forward, then inverse (one copy of the transform's code)
@@ -128,16 +126,16 @@ k_fx_std_col(Members mem, size_t offH, size_t offE, size_t offC, int ldq, int nc
       if (inv) {
         if (valid) {
 #pragma unroll
-          for (int m = 0; m < 16; ++m) H[TL::at(t + G * m, col, ldq)] = fx_shl(fx_swap(v[m]), s);
+          for (int m = 0; m < E; ++m) hs[TL::at(t + G * m, col, ldq)] = fx_shl(fx_swap(v[m]), s);
           if (t == 0) ws_ptr<int>(mb, offC)[col] = (emax >= kFxBad) ? kFxBad : (emax <= kFxZero) ? kFxZero : ex;
         }
         break;
       }
       const fxr* mg = mt.m1 + size_t(valid ? col : 0) * mt.ldm;
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         const int q = t + G * m;
-        const fxr c = fx_ldr(mg + (FULL || m < 8 ? q : N - q));
+        const fxr c = fx_ldr(mg + (FULL || m < H ? q : N - q));
         const fxc x = fx_shl(v[m], s);
         v[m] = fx_mk(fx_mulr(x.y, c), fx_mulr(x.x, c));  // (components exchanged: the inverse transform)
       }
@@ -151,7 +149,7 @@ k_fx_std_row_inv(Members mem, size_t offH, size_t offC, int ldq, int ny, const f
   DSNU_FX_SETUP1(stw_g)
   const int pairs = ny / 2, items = (pairs + PER - 1) / PER;
   int cur = -1, emax = 0;
-  unsigned pk[4] = {0, 0, 0, 0};  // alignment shifts of the columns |qbar| of q = t + G m
+  unsigned pk[(E + 3) / 4] = {};  // alignment shifts of the columns |qbar| of q = t + G m
 #pragma unroll 1
   for (int it = blockIdx.x; it < items * mem.count; it += gridDim.x) {
     if (it + int(gridDim.x) >= items * mem.count) grid_dep_trigger();  // last item of this CTA
@@ -161,26 +159,24 @@ k_fx_std_row_inv(Members mem, size_t offH, size_t offC, int ldq, int ny, const f
       const int* ce = ws_ptr<int>(mb, offC);
       emax = fx_cta_max(ce, N / 2 + 1, red + 4 * W);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) pk[i] = 0;
-#pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         const int q = t + G * m;
-        pk[m >> 2] |= unsigned(fx_align<3>(emax, ce[q > N / 2 ? N - q : q])) << (8 * (m & 3));
+        fx_pack<E>(pk, m, fx_align<3>(emax, ce[q > N / 2 ? N - q : q]));
       }
       cur = mi;
     }
     const bool valid = pi < pairs;
-    const fxc* __restrict__ H = ws_ptr<fxc>(mb, offH) + TL::at(valid ? 2 * pi : 0, 0, ldq);
-    fxc v[16];
+    const fxc* __restrict__ hs = ws_ptr<fxc>(mb, offH) + TL::at(valid ? 2 * pi : 0, 0, ldq);
+    fxc v[E];
     unsigned mag = 0;
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
+    for (int m = 0; m < E; ++m) {
       const int q = t + G * m, qq = q > N / 2 ? N - q : q;
-      const int s = int((pk[m >> 2] >> (8 * (m & 3))) & 0xFFu);
+      const int s = fx_byte(pk, m);
       fxc ya = fx_mk(0, 0), yb = ya;
       if (valid) {
-        ya = fx_sra(H[qq * TL::TR], s);
-        yb = fx_sra(H[qq * TL::TR + 1], s);
+        ya = fx_sra(hs[qq * TL::TR], s);
+        yb = fx_sra(hs[qq * TL::TR + 1], s);
       }
       if (q > N / 2) {
         ya.y = -ya.y;
@@ -193,14 +189,14 @@ k_fx_std_row_inv(Members mem, size_t offH, size_t offC, int ldq, int ny, const f
     __syncthreads();
     const int s0 = fx_norm_shift<61>(fx_read<P>(mag, red + 2 * W));
 #pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = fx_shr<4>(fx_shl(v[m], s0));
+    for (int m = 0; m < E; ++m) v[m] = fx_shr<4>(fx_shl(v[m], s0));
     const int ex = emax + 3 - s0 + 4 + lscale + fx_ifft<LOG2N, P>(v, buf, t, stw, red);
     if (valid) {
       const bool bad = emax >= kFxBad;
       const double nan = __longlong_as_double(0x7FF8000000000000ll);
       double* phi = mb.phi + size_t(2 * pi) * N;
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         phi[t + G * m] = bad ? nan : fx_to_f64(v[m].x, ex);
         phi[N + t + G * m] = bad ? nan : fx_to_f64(v[m].y, ex);
       }
