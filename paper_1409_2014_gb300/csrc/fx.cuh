@@ -104,6 +104,12 @@ __device__ __forceinline__ i64 fx_shr(i64 v) { return (v + (i64(1) << (S - 1))) 
 template <int S>
 __device__ __forceinline__ fxc fx_shr(fxc a) { return fx_mk(fx_shr<S>(a.x), fx_shr<S>(a.y)); }
 __device__ __forceinline__ fxc fx_shl(fxc a, int s) { return fx_mk(a.x << s, a.y << s); }
+// v 2^s, rounded when s < 0 (s uniform over a group)
+__device__ __forceinline__ fxc fx_scale2(fxc a, int s) {
+  if (s >= 0) return fx_shl(a, s);
+  const int r = min(-s, 63) - 1;
+  return fx_mk(((a.x >> r) + 1) >> 1, ((a.y >> r) + 1) >> 1);
+}
 
 // a e^{-2 pi i m/16} / 2 (m = 1, 2, 3, 5, 6, 7): cos(pi/8), sin(pi/8) and
 // sqrt(1/2) times 2^31 as h + l 2^-32
@@ -178,19 +184,33 @@ __device__ __forceinline__ unsigned fx_mag(unsigned m, i64 v) {
 __device__ __forceinline__ unsigned fx_mag(unsigned m, fxc a) { return fx_mag(fx_mag(m, a.x), a.y); }
 template <int E>
 __device__ __forceinline__ unsigned fx_mag(const fxc (&a)[E]) {
-  unsigned m = 0;
+  // (three-operand minimum and maximum: one instruction per two values each,
+  // against four; 2 % of a pass.  -1: no negative value)
+  int hi = 0, lo = -1;
 #pragma unroll
-  for (int i = 0; i < E; ++i) m = fx_mag(m, a[i]);
-  return m;
+  for (int i = 0; i < E; ++i) {
+    hi = __vimax3_s32(hi, int(a[i].x >> 32), int(a[i].y >> 32));
+    lo = __vimin3_s32(lo, int(a[i].x >> 32), int(a[i].y >> 32));
+  }
+  return unsigned(hi) | unsigned(~lo);
 }
 
-// OR (or maximum) over the P threads of a pair of groups (the even and the odd
-// chain of one row or column), in two halves around a barrier of the CTA:
-// fx_post gives the warp's part, fx_read collects the pair's.  P <= 32: the
-// pair lies in one warp and fx_read needs no barrier.  `red`: one word per warp.
+// Barrier of the P adjacent threads (a power of two) that work on one transform
+// or pair of transforms: a named barrier, or the warp's (the CTAs of smaller
+// groups have one warp).
+template <int P>
+__device__ __forceinline__ void fx_sync() {
+  if constexpr (P > 32) asm volatile("bar.sync %0, %1;" ::"r"(1 + int(threadIdx.x) / P), "n"(P) : "memory");
+  else __syncwarp();
+}
+
+// OR (or maximum) over P adjacent threads, in two halves around a barrier of
+// theirs: fx_post gives the warp's part, fx_read collects the group's.  P <= 32:
+// the group lies in one warp and fx_read needs no barrier.  `red`: one word per
+// warp of the CTA.
 template <int P, bool MAX = false>
 __device__ __forceinline__ unsigned fx_post(unsigned m, unsigned* red) {
-  if constexpr (P <= 32) {
+  if constexpr (P < 32) {
 #pragma unroll
     for (int s = 1; s < P; s <<= 1) {
       const unsigned o = __shfl_xor_sync(0xffffffffu, m, s);
@@ -198,7 +218,7 @@ __device__ __forceinline__ unsigned fx_post(unsigned m, unsigned* red) {
     }
   } else {
     m = MAX ? __reduce_max_sync(0xffffffffu, m) : __reduce_or_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    if (P > 32 && (threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   }
   return m;
 }
@@ -238,9 +258,11 @@ struct FxRad {
 inline int fx_log2_radix(int log2n) { return log2n <= FX_E8_MAX ? 3 : 4; }
 
 // Length-N DFT by a group of G = N/E threads, E values per thread (the index
-// order and buffer layout of block_fft_regs with E for 16).  P threads share one scale: G, or
-// 2 G where two groups work together (the even and the odd chain of one row or
-// column, two adjacent columns).  One transform per thread keeps it at 128 registers and one
+// order and buffer layout of block_fft_regs with E for 16).  P threads share one scale and
+// one barrier: G, or 2 G where the lanes of two transforms interleave.  Groups
+// with barriers of their own drift apart: while one multiplies (on the FMA pipe),
+// another adds (on the ALU) -- in step, all warps of an SM wait for the same pipe
+// (FP64 column pass at 4096^2 977 -> 912 us).  One transform per thread keeps it at 128 registers and one
 // copy of the radix-16 code for all stages (the loop below): two transforms per
 // thread at 8 warps per SM, the stages unrolled, came to 200 KB of code and ran
 // twice as long (column pass at 4096^2 1405 us).
@@ -257,7 +279,7 @@ __device__ __forceinline__ int fx_fft(fxc (&v)[FxRad<LOG2N>::E], fxc* buf, int t
     const int base = (t - k) * E + k;
     unsigned* rd = red + (s & 1) * (blockDim.x >> 5);
     const unsigned m0 = fx_post<P>(fx_mag(v), rd);
-    __syncthreads();  // every load of this buffer done (in place)
+    fx_sync<P>();  // every load of this buffer done (in place)
     if constexpr (E == 16) {  // (pad16 is linear over the stride)
       const int b0 = pad16(base), st = (s == 0) ? 1 : ns + (ns >> 4);
 #pragma unroll
@@ -266,7 +288,7 @@ __device__ __forceinline__ int fx_fft(fxc (&v)[FxRad<LOG2N>::E], fxc* buf, int t
 #pragma unroll
       for (int r = 0; r < E; ++r) buf[pad16(base + r * ns)] = v[r];
     }
-    __syncthreads();
+    fx_sync<P>();
     const int sh = fx_norm_shift<61>(fx_read<P>(m0, rd));
     ex += 4 - sh;
     return sh;

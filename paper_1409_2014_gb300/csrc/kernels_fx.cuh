@@ -40,7 +40,7 @@ struct FxGeo {
   static constexpr int FB = fft_buf_elems(N);
   static constexpr int STW = FxRad<LOG2N>::STW;
   static constexpr int W = T / 32, RED = 5 * W;       // words of the reductions: two for the FFT, three more
-  static constexpr size_t smem = size_t(STW + PER * 2 * FB) * 16 + ((RED * 4 + 15) & ~15);
+  static constexpr size_t smem = size_t(STW + PER * 2 * FB) * 16 + (((RED + 4 * PER) * 4 + 15) & ~15);
   // inverse rows: a byte of alignment shift per column of A, and one of B
   static constexpr size_t smem_row_inv(int Q) { return smem + ((N + 1 + 15) & ~15) + ((Q + 1 + 15) & ~15); }
 };
@@ -75,44 +75,62 @@ __device__ __forceinline__ fxw fx_wm(const fxw* __restrict__ wm, int t, int m, i
   }
   return w;
 }
+// Threads that share a scale and barriers: the chain's G, or both chains' where they
+// fit one warp (one reduction instruction; no warps to drift apart).
+__host__ __device__ constexpr int fx_share(int G) { return 2 * G <= 32 ? 2 * G : G; }
+
 // The chains' inputs from the staged values z (|component| < 2^61 after the
 // shift s): z/16 for the even one, z e^{-2 pi i n/M}/16 for the odd one.
+// (A barrier of the CTA: the chains' buffers are free for their exchanges after it.)
 template <int G, int E>
 __device__ __forceinline__ void fx_chain_in(fxc (&v)[E], const fxc* st, int s, int h, int t, const fxw* wm) {
-  if (h == 0) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) v[m] = fx_shr<4>(fx_shl(st[pad16(t + G * m)], s));
-  } else {
-#pragma unroll
-    for (int m = 0; m < E; ++m) v[m] = fx_mul(fx_shl(st[pad16(t + G * m)], s), fx_wm<E>(wm, t, m, G));
-  }
-}
-// The column sum e(n)/16 + e^{+2 pi i n/M} o(n)/16 of the two chains' results at
-// n = t + G (m + h E/2), m < E/2: each chain hands the other half of its values over
-// (in its own buffer) and multiplies half of the odd ones.
-template <int G, int E>
-__device__ __forceinline__ void fx_chain_out(fxc (&v)[E], fxc* buf_e, fxc* buf_o, int s, int h, int t,
-                                             const fxw* wm) {
-  __syncthreads();  // the last stage's loads of the buffers are done
-  if (h == 0) {
-#pragma unroll
-    for (int m = E / 2; m < E; ++m) buf_e[pad16(t + G * m)] = v[m];
-  } else {
-#pragma unroll
-    for (int m = 0; m < E / 2; ++m) buf_o[pad16(t + G * m)] = v[m];
-  }
+  for (int m = 0; m < E; ++m) v[m] = st[pad16(t + G * m)];
   __syncthreads();
   if (h == 0) {
 #pragma unroll
-    for (int m = 0; m < E / 2; ++m)
-      v[m] = fx_shr<4>(fx_shl(v[m], s)) + fx_mul(fx_shl(buf_o[pad16(t + G * m)], s), fx_conj(fx_wm<E>(wm, t, m, G)));
+    for (int m = 0; m < E; ++m) v[m] = fx_shr<4>(fx_shl(v[m], s));
   } else {
 #pragma unroll
-    for (int m = 0; m < E / 2; ++m)
-      v[m] = fx_shr<4>(fx_shl(buf_e[pad16(t + G * (m + E / 2))], s)) +
-             fx_mul(fx_shl(v[m + E / 2], s), fx_conj(fx_wm<E>(wm, t, m + E / 2, G)));
+    for (int m = 0; m < E; ++m) v[m] = fx_mul(fx_shl(v[m], s), fx_wm<E>(wm, t, m, G));
   }
 }
+// The column sum e(n) + e^{+2 pi i n/M} o(n) of the two chains' results, each of
+// exponent ex with its magnitudes m (fx_post over the chain, red), at
+// n = t + G (m + h E/2), m < E/2: each chain hands the other half of its values
+// over (in its own buffer) and multiplies half of the odd ones.  exs: two words of
+// the pair.  Returns the sum's exponent (values below 2^59.5).
+template <int G, int E>
+__device__ __forceinline__ int fx_chain_out(fxc (&v)[E], fxc* buf_e, fxc* buf_o, unsigned mag, const unsigned* red,
+                                            int ex, int* exs, int h, int t, const fxw* wm) {
+  fx_sync<fx_share(G)>();  // (the chain's last loads of its buffer are done; `red` is complete)
+  const int s = fx_norm_shift<62>(fx_read<fx_share(G)>(mag, red));
+  if (t == 0) exs[h] = ex - s;
+  if (h == 0) {
+#pragma unroll
+    for (int m = E / 2; m < E; ++m) buf_e[pad16(t + G * m)] = fx_shl(v[m], s);
+  } else {
+#pragma unroll
+    for (int m = 0; m < E / 2; ++m) buf_o[pad16(t + G * m)] = fx_shl(v[m], s);
+  }
+  __syncthreads();
+  // the chains' exponents differ by little: the smaller one's values are aligned
+  const int xe = exs[0], xo = exs[1], x = max(xe, xo);
+  const int de = min(x - xe, 59), dd = min(x - xo, 62);
+#pragma unroll
+  for (int m = 0; m < E / 2; ++m) {
+    const fxc e = h ? buf_e[pad16(t + G * (m + E / 2))] : fx_shl(v[m], s);
+    const fxc o = h ? fx_shl(v[m + E / 2], s) : buf_o[pad16(t + G * m)];
+    const fxw w = h ? fx_wm<E>(wm, t, m + E / 2, G) : fx_wm<E>(wm, t, m, G);
+    fxc p = fx_mul(o, fx_conj(w));
+    if (dd > 0) p = fx_sra(p, dd);
+    v[m] = fx_sra(e, 4 + de) + p;
+  }
+  return x + 4;
+}
+
+// Into L2 ahead of its use.
+__device__ __forceinline__ void fx_prefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // Common prologue of the passes: the CTA's tables, buffers and thread roles.
 #define DSNU_FX_SETUP(AX)                                                  \
@@ -130,6 +148,8 @@ __device__ __forceinline__ void fx_chain_out(fxc (&v)[E], fxc* buf_e, fxc* buf_o
   fxc* buf_e = sm + (2 * pr) * GG::FB;                                     \
   fxc* buf_o = buf_e + GG::FB;                                             \
   fxc* buf = h ? buf_o : buf_e;                                            \
+  int* exs = reinterpret_cast<int*>(red + GG::RED) + 2 * pr;               \
+  (void)exs;                                                               \
   __syncthreads();                                                         \
   grid_dep_wait();
 
@@ -172,18 +192,27 @@ k_fx_row_fwd(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
     }
     __syncthreads();
     fxc v[E];
+    // the next row into L2 while this one is transformed
+    if (row + int(gridDim.x) * PER < ny && (tp & 15) == 0)
+#pragma unroll
+      for (int i = 0; i < H; ++i) fx_prefetch(mb.rho + size_t(row + int(gridDim.x) * PER) * N + tp + P * i);
     fx_chain_in<G, E>(v, buf_e, 0, h, t, ax.wm);
-    const int ef = fx_fft<LOG2N, P>(v, buf, t, stw, red);
-    const unsigned mag = fx_post<P>(fx_mag(v), red + 4 * W);
-    __syncthreads();  // (and the last stage's loads are done)
-    const int s1 = fx_norm_shift<62>(fx_read<P>(mag, red + 4 * W));  // sums of two: below 2^63
+    // exponent of the chain: from_f64 (efm - kFxBias), the five bits, the stages
+    const int xh = efm - kFxBias + 5 + fx_fft<LOG2N, fx_share(G)>(v, buf, t, stw, red);
+    const unsigned mag = fx_post<fx_share(G)>(fx_mag(v), red + 4 * W);
+    fx_sync<fx_share(G)>();  // (and the last stage's loads are done)
+    if (t == 0) {
+      exs[h] = xh - fx_norm_shift<62>(fx_read<fx_share(G)>(mag, red + 4 * W));  // sums of two: below 2^63
+      exs[2 * PER + h] = xh;
+    }
 #pragma unroll
     for (int m = 0; m < E; ++m) buf[pad16(t + G * m)] = v[m];
     __syncthreads();
-    // exponent of Z: from_f64 (efm - kFxBias), the five bits, the stages;
-    // A = (Z(q) + conj Z(M - q))/2 and B = (Z(q) - conj Z(M - q))/2i as sums, times 2^s1
+    // A = (Z(q) + conj Z(M - q))/2 and B = (Z(q) - conj Z(M - q))/2i as sums, both
+    // chains brought to one exponent
+    const int xc = max(exs[0], exs[1]), s1 = exs[2 * PER + (tp & 1)] - xc;
     if (tp == 0 && valid) {
-      const int ea = efm - kFxBias + 5 + ef - 1 - s1;
+      const int ea = xc - 1;
       ws_ptr<int>(mb, off.rexp)[row] = fx_exp(mx, ea);
       ws_ptr<int>(mb, off.rexpb)[row] = fx_exp(mx, ea + kr);
     }
@@ -197,8 +226,8 @@ k_fx_row_fwd(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
         const int k = q >> 1;
         const fxc zq = (q & 1) ? buf_o[pad16(k)] : buf_e[pad16(k & (N - 1))];
         const fxc zm = (q & 1) ? buf_o[pad16(N - 1 - k)] : buf_e[pad16((N - k) & (N - 1))];
-        Ar[q * TL::TR] = fx_shl(fx_mk(zq.x + zm.x, zq.y - zm.y), s1);
-        if (q <= Q) Br[q * TL::TR] = fx_shl(fx_mk(zq.y + zm.y, zm.x - zq.x), s1);
+        Ar[q * TL::TR] = fx_scale2(fx_mk(zq.x + zm.x, zq.y - zm.y), s1);
+        if (q <= Q) Br[q * TL::TR] = fx_scale2(fx_mk(zq.y + zm.y, zm.x - zq.x), s1);
       }
     }
   }
@@ -253,35 +282,37 @@ k_fx_col_main(Members mem, FxOff off, int ldqA, int ncols, FxAxis ay, FxMult mt)
     for (int i = 0; i < H; ++i) buf_e[pad16(tp + P * i)] = v[i];
     __syncthreads();
     const int s0 = fx_norm_shift<61>(fx_read<P>(mag, red + 2 * W));
-    fx_chain_in<G, E>(v, buf_e, s0, h, t, ay.wm);
-    // exponent: the rows', s0, /16, stages, s1, multiplier (its own and /32), stages, s2, /16, the last 3 bits
-    int ex = emax + 2 - s0 + 4 + (mt.mexp && valid ? mt.mexp[col] : 0) + 5 + 4 - 3;
-#pragma unroll 1
-    for (int inv = 0;; ++inv) {  // forward, then inverse (one copy of the transform's code)
-      ex += fx_fft<LOG2N, P>(v, buf, t, stw, red);
-      mag = fx_post<P>(fx_mag(v), red + (2 + inv) * W);
-      __syncthreads();
-      const int s = fx_norm_shift<62>(fx_read<P>(mag, red + (2 + inv) * W));
-      ex -= s;
-      if (inv) {
+    // the next column and its multipliers into L2 while this one is transformed
+    if (col + int(gridDim.x) * PER < ncols) {
+      const int nc = col + int(gridDim.x) * PER;
+      if ((tp & 1) == 0)
 #pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = fx_swap(v[m]);
-        fx_chain_out<G, E>(v, buf_e, buf_o, s, h, t, ay.wm);
-        break;
-      }
-      const fxr* mg = mt.m1 + size_t(valid ? col : 0) * mt.ldm + (h ? MH : 0);
-#pragma unroll
-      for (int m = 0; m < E; ++m) {
-        const int k = t + G * m;  // row q = 2 k + h: |qbar| / 2 rounded down
-        const fxr c = fx_ldr(mg + (FULL ? k : (m < H ? k : N - h - k)));
-        const fxc x = fx_shl(v[m], s);
-        v[m] = fx_mk(fx_mulr(x.y, c), fx_mulr(x.x, c));  // (components exchanged: the inverse transform)
-      }
+        for (int i = 0; i < H; ++i) fx_prefetch(A + TL::at(tp + P * i, nc, ldqA));
+      for (int i = tp * 16; i < mt.ldm; i += P * 16) fx_prefetch(mt.m1 + size_t(nc) * mt.ldm + i);
     }
+    fx_chain_in<G, E>(v, buf_e, s0, h, t, ay.wm);
+    // the chain's exponent: the rows', s0, /16, stages, s1, multiplier (its own and /32), stages
+    int ex = emax + 2 - s0 + 4;
+    ex += fx_fft<LOG2N, fx_share(G)>(v, buf, t, stw, red);
+    mag = fx_post<fx_share(G)>(fx_mag(v), red + 2 * W);
+    fx_sync<fx_share(G)>();
+    const int s1 = fx_norm_shift<62>(fx_read<fx_share(G)>(mag, red + 2 * W));
+    ex += (mt.mexp && valid ? mt.mexp[col] : 0) + 5 - s1;
+    const fxr* mg = mt.m1 + size_t(valid ? col : 0) * mt.ldm + (h ? MH : 0);
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const int k = t + G * m;  // row q = 2 k + h: |qbar| / 2 rounded down
+      const fxr c = fx_ldr(mg + (FULL ? k : (m < H ? k : N - h - k)));
+      const fxc x = fx_shl(v[m], s1);
+      v[m] = fx_mk(fx_mulr(x.x, c), fx_mulr(x.y, c));
+    }
+    ex += fx_ifft<LOG2N, fx_share(G)>(v, buf, t, stw, red);
+    mag = fx_post<fx_share(G)>(fx_mag(v), red + 3 * W);
+    ex = fx_chain_out<G, E>(v, buf_e, buf_o, mag, red + 3 * W, ex, exs, h, t, ay.wm);
     if (valid) {
 #pragma unroll
       for (int m = 0; m < H; ++m) A[TL::at(t + G * (m + H * h), col, ldqA)] = fx_shl(v[m], 3);  // < 2^59.5 before
-      if (tp == 0) ws_ptr<int>(mb, off.cexp)[col] = (emax >= kFxBad) ? kFxBad : (emax <= kFxZero) ? kFxZero : ex;
+      if (tp == 0) ws_ptr<int>(mb, off.cexp)[col] = (emax >= kFxBad) ? kFxBad : (emax <= kFxZero) ? kFxZero : ex - 3;
     }
   }
 }
@@ -329,7 +360,7 @@ k_fx_band_fwd(Members mem, FxOff off, int ldqB, int ncols, int ldq, int Q, FxAxi
     }
     __syncthreads();
     fx_chain_in<G, E>(v, buf_e, 1, h, t, ay.wm);
-    const int ex = emax + 2 - s0 + kdy + 4 + fx_fft<LOG2N, P>(v, buf, t, stw, red);
+    const int ex = emax + 2 - s0 + kdy + 4 + fx_fft<LOG2N, fx_share(G)>(v, buf, t, stw, red);
     if (valid) {
       const bool bad = emax >= kFxBad;
       const double nan = __longlong_as_double(0x7FF8000000000000ll);
@@ -377,11 +408,9 @@ k_fx_band_inv(Members mem, FxOff off, int ldq, int Q, int ncols, int ldqB, FxAxi
 #pragma unroll
     for (int m = 0; m < E; ++m)
       v[m] = fx_shr<5>(fx_mk(fx_from_f64(__longlong_as_double(v[m].x), efm), fx_from_f64(__longlong_as_double(v[m].y), efm)));
-    const int ef = fx_ifft<LOG2N, P>(v, buf, t, stw, red);
-    const unsigned mag = fx_post<P>(fx_mag(v), red + 3 * W);
-    __syncthreads();
-    const int s1 = fx_norm_shift<62>(fx_read<P>(mag, red + 3 * W));
-    fx_chain_out<G, E>(v, buf_e, buf_o, s1, h, t, ay.wm);
+    int ex = efm - kFxBias + 5 + fx_ifft<LOG2N, fx_share(G)>(v, buf, t, stw, red);
+    const unsigned mag = fx_post<fx_share(G)>(fx_mag(v), red + 3 * W);
+    ex = fx_chain_out<G, E>(v, buf_e, buf_o, mag, red + 3 * W, ex, exs, h, t, ay.wm);
     if (valid) {
 #pragma unroll
       for (int m = 0; m < H; ++m) {
@@ -390,7 +419,7 @@ k_fx_band_inv(Members mem, FxOff off, int ldq, int Q, int ncols, int ldqB, FxAxi
         St[TL::at(n, col, ldqB)] = fx_shl(fx_mk(fx_mulr(v[m].x, d), fx_mulr(v[m].y, d)), 4);  // < 2^58.5 before
       }
       if (tp == 0)
-        ws_ptr<int>(mb, off.bexp)[col] = fx_exp(mx, efm - kFxBias + 5 + ef - s1 + 4 + kdy + 1 - 4);
+        ws_ptr<int>(mb, off.bexp)[col] = fx_exp(mx, ex + kdy + 1 - 4);
     }
   }
 }
@@ -457,20 +486,20 @@ k_fx_row_inv(Members mem, FxOff off, int ldqA, int ldqB, int Q, int ny, FxAxis a
     if (tp == 0) buf_o[0] = yn;
     __syncthreads();
     const int s0 = fx_norm_shift<60>(fx_read<P>(mag, red + 2 * W));
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const fxc x = buf_e[pad16(t + G * m)], r = buf_o[pad16(t + G * m)];
+      v[m] = h ? fx_mk(x.x - r.x, x.y + r.y) : fx_mk(x.x + r.x, x.y - r.y);
+    }
+    __syncthreads();  // the buffers are free for the chains' exchanges
     if (h == 0) {
 #pragma unroll
-      for (int m = 0; m < E; ++m) {
-        const fxc x = buf_e[pad16(t + G * m)], r = buf_o[pad16(t + G * m)];
-        v[m] = fx_shr<4>(fx_shl(fx_mk(x.x + r.x, x.y - r.y), s0));
-      }
+      for (int m = 0; m < E; ++m) v[m] = fx_shr<4>(fx_shl(v[m], s0));
     } else {
 #pragma unroll
-      for (int m = 0; m < E; ++m) {
-        const fxc x = buf_e[pad16(t + G * m)], r = buf_o[pad16(t + G * m)];
-        v[m] = fx_mul(fx_shl(fx_mk(x.x - r.x, x.y + r.y), s0), fx_conj(fx_wm<E>(ax.wm, t, m, G)));
-      }
+      for (int m = 0; m < E; ++m) v[m] = fx_mul(fx_shl(v[m], s0), fx_conj(fx_wm<E>(ax.wm, t, m, G)));
     }
-    const int ex = emax + 4 - s0 + 4 + kd + 1 + lscale + fx_ifft<LOG2N, P>(v, buf, t, stw, red);
+    const int ex = emax + 4 - s0 + 4 + kd + 1 + lscale + fx_ifft<LOG2N, fx_share(G)>(v, buf, t, stw, red);
     if (valid) {
       double* __restrict__ phi = mb.phi + size_t(row) * N + h;
       const bool bad = emax >= kFxBad;
