@@ -1015,17 +1015,17 @@ dsnu_status dsnu_plan_create_multiplier(const dsnu_params* params, const dsnu_mu
   layout_workspace(P);
   // The band chain and the column pass run side by side.  On large grids the
   // column pass is the longer one: the band chain runs on the low-priority side
-  // stream, the column pass leaving it 16 of every 152 SMs at 4096^2 and a
-  // share growing as 1/sqrt(nx ny) below, since the band chain's node work is the
-  // same on every grid (mixed 4096^2 507 us with 16 SMs, 526 with 32, 524 in
-  // line; 2048^2 131 with 32, 139 with 16, 152 in line; FP64 4096^2 2208 us, in
-  // line 2234; 2048^2 530, in line 548).  Below 2048^2 the band chain is the
+  // stream, the column pass leaving it 16 of every 152 SMs, in mixed plans a share
+  // growing as 1/sqrt(nx ny) below 4096^2, since the band chain's node work is the
+  // same on every grid (mixed 4096^2 507 us with 16 SMs, 525 with 32, 521 in
+  // line; 2048^2 131 with 32, 139 with 16, 150 in line; FP64, whose column pass is
+  // heavier, 4096^2 2041 us, with 24 SMs 2093, in line 2057; 2048^2 499, with 32
+  // SMs 516, in line 541).  Below 2048^2 the band chain is the
   // longer one: it stays on the caller's stream, where its launches overlap, and
   // the column pass fills the rest of the GPU from the side stream (FP64 512^2
-  // 92 us against 105 in line; 1024^2 164 against 187; mixed 256^2 44 against 48).
-  // There the share is capped: mixed 48 SMs (1024^2 57.7 us with 48, 65.5 with
-  // 16; 2048 x 512 53.6 and 59.7), FP64, whose column pass is heavier, 16 (1024^2
-  // 164 us with 16, 171 with 64).
+  // 74 us; 1024^2 156, in line 166; mixed 256^2 41 against 47).
+  // There the mixed share is capped at 48 SMs (1024^2 55.6 us with 48, 63.3 with
+  // 16; 2048 x 512 53.6 and 59.7).
   // DSNU_BAND_SMS=<n> sets the number of SMs left free, 0 runs both in line.
   {
     int dev = 0;
@@ -1033,10 +1033,11 @@ dsnu_status dsnu_plan_create_multiplier(const dsnu_params* params, const dsnu_mu
     cudaDeviceGetAttribute(&g.sms, cudaDevAttrMultiProcessorCount, dev);
   }
   if (!standard) {
-    const double share = 16.0 / 152.0 * 4096.0 / std::sqrt(double(p.nx) * p.ny);
+    double share = 16.0 / 152.0;
+    if (g.precision == DSNU_MIXED) share *= 4096.0 / std::sqrt(double(p.nx) * p.ny);
     Overlap& ov = P->overlap;
     ov.col_side = (p.nx < 2048 || p.ny < 2048) ? 1 : 0;
-    ov.reserve = std::max(1, int(std::lround(g.sms * (ov.col_side ? std::min(share, g.precision == DSNU_MIXED ? 48.0 / 152.0 : 16.0 / 152.0) : share))));
+    ov.reserve = std::max(1, int(std::lround(g.sms * (ov.col_side ? std::min(share, 48.0 / 152.0) : share))));
     const char* env = std::getenv("DSNU_BAND_SMS");
     if (env) ov.reserve = std::atoi(env);
     if (ov.reserve > 0) {
