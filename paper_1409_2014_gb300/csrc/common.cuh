@@ -571,6 +571,16 @@ __device__ __forceinline__ float f32_of_f64_int(double d, bool& odd) {
 }
 static __device__ __noinline__ float f32_of_f64_hw(double d) { return __double2float_rn(d); }
 
+// FP32 -> FP64 by integer instructions, exact: the exponent rebiased and the
+// fraction extended.  `odd` is set for zeros, subnormals, infinities and NaNs,
+// which the caller converts with the hardware instruction, out of line.
+__device__ __forceinline__ double f64_of_f32_int(float x, bool& odd) {
+  const unsigned u = __float_as_uint(x);
+  odd = ((u + 0x00800000u) & 0x7F000000u) == 0u;  // exponent field 0 or 255
+  return __hiloint2double(int(((u & 0x7FFFFFFFu) >> 3) + 0x38000000u | (u & 0x80000000u)), int(u << 29));
+}
+static __device__ __noinline__ double f64_of_f32_hw(float x) { return double(x); }
+
 // 1/b in FP64 by Newton-Raphson: the hardware's approximate reciprocal
 // (rcp.approx.ftz.f64, about 2^-20 relative) refined twice by
 // r <- r + r (1 - b r), which squares the relative error each step, so the

@@ -37,8 +37,11 @@ struct GeoStd {
   static constexpr int N = 1 << LOG2N;
   static constexpr int G = N / 16;                       // threads per transform
   static constexpr int FB = fft_buf_elems(N);
-  static constexpr int PER = (G >= 256) ? 1 : 256 / G;   // row pairs or columns per CTA
-  static constexpr int T = PER * G;
+  // row pairs or columns per CTA: CTAs of 128 threads where that holds one, whose
+  // barriers do not keep all of an SM's warps in step (2048^2: the row passes
+  // 23.4 -> 21.0 and 21.8 -> 20.5 us against CTAs of 256)
+  static constexpr int PER = (G >= 128) ? 1 : 128 / G;
+  static constexpr int T = PER * G, MINB = 512 / T;
   static constexpr int STW = fft_stage_tw_elems(LOG2N) > 0 ? fft_stage_tw_elems(LOG2N) : 1;
   static constexpr int STWP = (STW + 1) & ~1;
   static constexpr size_t smem = size_t(STWP + PER * FB) * sizeof(cpx<R>);
@@ -54,7 +57,7 @@ struct GeoStd {
 };
 
 template <typename R, int LOG2N>
-__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, 2)
+__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, GeoStd<R, LOG2N>::MINB)
 k_std_row_fwd(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restrict__ stw_g, int cj, int* status) {
   using GG = GeoStd<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, PER = GG::PER;
@@ -128,7 +131,7 @@ k_std_row_fwd(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restric
 }
 
 template <typename R, int LOG2N>
-__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, 2)
+__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, GeoStd<R, LOG2N>::MINB)
 k_std_col(Members mem, size_t offH, int ldq, int ncols, const cpx<R>* __restrict__ stw_g,
           MultTabs<R> mt, R scale, int cj) {
   using GG = GeoStd<R, LOG2N>;
@@ -197,7 +200,7 @@ k_std_col(Members mem, size_t offH, int ldq, int ncols, const cpx<R>* __restrict
 }
 
 template <typename R, int LOG2N>
-__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, 2)
+__global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, GeoStd<R, LOG2N>::MINB)
 k_std_row_inv(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restrict__ stw_g, int cj) {
   using GG = GeoStd<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, PER = GG::PER, T = GG::T;
@@ -259,11 +262,24 @@ k_std_row_inv(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restric
     if (it + int(gridDim.x) < total) prefetch(it + gridDim.x);
     block_fft_regs<R, LOG2N, true>(v, buf, t, stw, cj == 0);
     if (valid) {
+      // three of four values widened by integer instructions, one on the narrow
+      // FP64 pipe (2048^2: 16.9 us; all on the FP64 pipe 20.5, all by integers 17.6)
+      double* dst = mb.phi + size_t(row) * N + t;
 #pragma unroll
       for (int m = 0; m < 16; ++m) {
-        const int n = t + G * m;
-        mb.phi[size_t(row) * N + n] = to_f64<R>(v[m].x);
-        mb.phi[size_t(row + 1) * N + n] = to_f64<R>(v[m].y);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float x = h ? v[m].y : v[m].x;
+          bool odd = false;
+          double d;
+          if ((2 * m + h) % 4 < 3) {
+            d = f64_of_f32_int(x, odd);
+            if (odd) d = f64_of_f32_hw(x);
+          } else {
+            d = double(x);
+          }
+          dst[h * N + G * m] = d;
+        }
       }
     }
   }
