@@ -45,6 +45,9 @@ namespace {
 
 constexpr int kLog2Min = 8, kLog2Max = 11;  // grid sizes of the one-launch-per-stage schedule
 constexpr int kRagThreads = 256;
+// one block size for every grid size of the schedule
+template <int L>
+using RagGeo = Geo<float, L, kRagThreads>;
 
 enum RagStage { RS_ROWF = 0, RS_BANDF, RS_INTERP, RS_SPREAD, RS_REDUCE, RS_BANDI, RS_COL, RS_ROWI, RS_N };
 
@@ -110,14 +113,14 @@ __device__ __forceinline__ int rag_group(const RagTable& T, int s, int b) {
   }
 
 #define DSNU_RAG_ROWF(L) \
-  row_fwd_body<float, L>(vb, vg, a.mem, a.off, a.ldqA, a.ldqB, a.Q, a.ny, a.ax, a.decon_y, 0, a.status)
-#define DSNU_RAG_BANDF(L) band_fwd_body<float, L>(vb, vg, a.mem, a.off, a.ldqB, a.Q + 1, a.ldq, a.Q, a.ay, 0)
+  row_fwd_body<float, L, RagGeo<L>>(vb, vg, a.mem, a.off, a.ldqA, a.ldqB, a.Q, a.ny, a.ax, a.decon_y, 0, a.status)
+#define DSNU_RAG_BANDF(L) band_fwd_body<float, L, RagGeo<L>>(vb, vg, a.mem, a.off, a.ldqB, a.Q + 1, a.ldq, a.Q, a.ay, 0)
 #define DSNU_RAG_COL(L)                                                                  \
-  col_main_body<float, L, false>(vb, vg, a.mem, a.off, a.ldqA, a.nx + 1, a.ay, a.mt, 0, \
+  col_main_body<float, L, false, RagGeo<L>>(vb, vg, a.mem, a.off, a.ldqA, a.nx + 1, a.ay, a.mt, 0, \
                                  ws_ptr<int>(member_at(a.mem, 0), a.off.sched))
-#define DSNU_RAG_BANDI(L) band_inv_body<float, L>(vb, vg, a.mem, a.off, a.ldq, a.Q, a.Q + 1, a.ldqB, a.ay, 0)
+#define DSNU_RAG_BANDI(L) band_inv_body<float, L, RagGeo<L>>(vb, vg, a.mem, a.off, a.ldq, a.Q, a.Q + 1, a.ldqB, a.ay, 0)
 #define DSNU_RAG_ROWI(L)                                                                                       \
-  row_inv_body<float, L>(vb, vg, a.mem, a.off, a.ldqA, a.ldqB, a.Q, a.ny, a.ax, a.decon_y, a.scale, 0, a.bpf, \
+  row_inv_body<float, L, RagGeo<L>>(vb, vg, a.mem, a.off, a.ldqA, a.ldqB, a.Q, a.ny, a.ax, a.decon_y, a.scale, 0, a.bpf, \
                          a.acc64)
 
 // (minimum resident CTAs as in the single-plan launches, but one for the band
@@ -125,7 +128,7 @@ __device__ __forceinline__ int rag_group(const RagTable& T, int s, int b) {
 // registers that the single-plan launch reads from the constant bank)
 DSNU_RAG_PERSISTENT(k_rag_row_fwd, RS_ROWF, 2, log2nx, DSNU_RAG_ROWF)
 DSNU_RAG_PERSISTENT(k_rag_band_fwd, RS_BANDF, 1, log2ny, DSNU_RAG_BANDF)
-DSNU_RAG_PERSISTENT(k_rag_col_main, RS_COL, DSNU_COLMAIN_MINB, log2ny, DSNU_RAG_COL)
+DSNU_RAG_PERSISTENT(k_rag_col_main, RS_COL, 1, log2ny, DSNU_RAG_COL)
 DSNU_RAG_PERSISTENT(k_rag_band_inv, RS_BANDI, 1, log2ny, DSNU_RAG_BANDI)
 DSNU_RAG_PERSISTENT(k_rag_row_inv, RS_ROWI, 2, log2nx, DSNU_RAG_ROWI)
 
@@ -167,15 +170,18 @@ __global__ void __launch_bounds__(TILE * TILE) k_rag_spread_reduce(const __grid_
 // Per-size launch constants of the bodies (host side).
 struct SizeInfo {
   int rows_f, rows_i, cols;                        // rows per item of the row passes, columns per item
-  size_t smem_rowf, smem_col, smem_col_main;
+  size_t smem_rowf, smem_rowi, smem_col, smem_col_main;
+  bool rowi_pf;
 };
 
 template <int L>
 SizeInfo size_info_of() {
-  using GG = Geo<float, L>;
-  static_assert(GG::T_RF == kRagThreads && GG::T_RI == kRagThreads && GG::T_C == kRagThreads,
+  using GG = RagGeo<L>;
+  static_assert(GG::T_RF == kRagThreads && GG::T_RI == kRagThreads && GG::T_C == kRagThreads &&
+                    GG::T_B == kRagThreads,
                 "one block size for every grid size of the schedule");
-  return SizeInfo{GG::RB_F, GG::RB_I, GG::CC, GG::smem_row_fwd, GG::smem_col, GG::smem_col_main};
+  return SizeInfo{GG::RB_F, GG::RB_I, GG::CC, GG::smem_row_fwd, GG::smem_row_inv, GG::smem_band,
+                  GG::smem_col_main, GG::ROWI_PF};
 }
 
 SizeInfo size_info(int log2n) {
@@ -356,7 +362,8 @@ dsnu_status ragged_create(const RaggedGroupIn* groups, int n, Ragged** out) {
     T.per[RS_SPREAD][i] = std::max(g.n_items, 1);
     T.per[RS_REDUCE][i] = std::max(g.n_tiles, 1);
     R->smem[RS_ROWF] = std::max(R->smem[RS_ROWF], sx.smem_rowf);
-    R->smem[RS_ROWI] = std::max(R->smem[RS_ROWI], g.smem_rowi);
+    // (with the prefetch the geometry is the single launch's, and so is the room for the band values)
+    R->smem[RS_ROWI] = std::max(R->smem[RS_ROWI], sx.rowi_pf ? g.smem_rowi : sx.smem_rowi);
     R->smem[RS_COL] = std::max(R->smem[RS_COL], sy.smem_col_main);
     R->smem[RS_BANDF] = std::max(R->smem[RS_BANDF], sy.smem_col);
     R->smem[RS_BANDI] = R->smem[RS_BANDF];

@@ -46,12 +46,6 @@
 
 // Occupancy targets (minimum resident CTAs per SM) and rows per CTA of the
 // FP32 row passes; overridable at compile time for tuning sweeps.
-#ifndef DSNU_ROW_MINB
-#define DSNU_ROW_MINB 2
-#endif
-#ifndef DSNU_COL_MINB
-#define DSNU_COL_MINB 2
-#endif
 #ifndef DSNU_ROWF_RB32
 #define DSNU_ROWF_RB32 2
 #endif
@@ -81,9 +75,6 @@
 #endif
 #ifndef DSNU_TILE_LT32
 #define DSNU_TILE_LT32 2
-#endif
-#ifndef DSNU_COLMAIN_MINB
-#define DSNU_COLMAIN_MINB 1
 #endif
 
 namespace dsnu {
@@ -170,9 +161,18 @@ struct Tile {
 template <typename R>
 constexpr int min_blocks(int fp32_target) { return sizeof(R) == 4 ? fp32_target : 1; }
 
-// Launch geometry shared by the kernels and their launchers.
-template <typename R, int LOG2N>
+// Launch geometry shared by the kernels and their launchers.  The row and band
+// kernels' CTAs have at least TM threads: 64 for the short transforms, so that a
+// small grid's rows and band columns spread over the SMs (mixed 256^2 41.6 us with
+// 256, 37.8 with 128, 37.1 with 64, 39.9 with 32; 512^2 45.4, 43.3, 41.7, 43.9),
+// 256 from length 1024, where smaller ones only copy their tables more often
+// (1024^2 55.5 us, with 64 59.6; 2048^2 130 and 134).  TMIN fixes it for launches
+// of several sizes.
+template <typename R, int LOG2N, int TMIN = 0>
 struct Geo {
+  static constexpr int TM = TMIN ? TMIN : (LOG2N <= 9 ? 64 : 256);
+  // resident CTAs per SM asked of the compiler
+  __host__ __device__ static constexpr int ctas(int t) { return t >= 512 ? 1 : t >= 256 ? 2 : 448 / t; }
   static constexpr int N = 1 << LOG2N;
   static constexpr int M = 2 * N;
   static constexpr int G = N / 16;                   // threads per length-N FFT
@@ -183,14 +183,16 @@ struct Geo {
   // (more rows for short rows), two transform buffers per row
   static constexpr int RMAX = (sizeof(R) == 4) ? 64 : 32;
   static constexpr int RB_F0 = (sizeof(R) == 4) ? DSNU_ROWF_RB32 : 1;
-  static constexpr int RB_F = (RB_F0 * G >= 256) ? RB_F0 : ((256 / G < RMAX) ? 256 / G : RMAX);
+  static constexpr int RB_F = (RB_F0 * G >= TM) ? RB_F0 : ((TM / G < RMAX) ? TM / G : RMAX);
   static constexpr int T_RF = RB_F * G;
   static constexpr int RB_I0 = (sizeof(R) == 4) ? DSNU_ROWI_RB32 : 1;
-  static constexpr int RB_I = (RB_I0 * G >= 256) ? RB_I0 : ((256 / G < RMAX) ? 256 / G : RMAX);
+  static constexpr int RB_I = (RB_I0 * G >= TM) ? RB_I0 : ((TM / G < RMAX) ? TM / G : RMAX);
   static constexpr int T_RI = RB_I * G;
   // column passes: CC columns per CTA
   static constexpr int CC = (G >= 256) ? 1 : 256 / G;
   static constexpr int T_C = CC * G;
+  static constexpr int CB = (G >= TM) ? 1 : TM / G;  // and of the band kernels
+  static constexpr int T_B = CB * G, MINB_B = 512 / T_B;
   static constexpr int STW = fft_stage_tw_elems(LOG2N) > 0 ? fft_stage_tw_elems(LOG2N) : 1;
   static constexpr int STWP = (STW + 1) & ~1;  // keep the buffers 16-byte aligned
   // FP32 row passes keep e^{-2 pi i n/M} (n < N) in a shared table after the buffers
@@ -207,7 +209,7 @@ struct Geo {
   static constexpr int LS = N + DSNU_ROWF_LPAD;
   static constexpr size_t smem_row_fwd_pf =
       size_t(STWCP + 2 * RB_F * RS + N / 2 + RB_F * LS * 8 / int(sizeof(cpx<R>)) + 2) * sizeof(cpx<R>);
-  static constexpr int MINB_F0 = (T_RF >= 512) ? 1 : DSNU_ROW_MINB;
+  static constexpr int MINB_F0 = ctas(T_RF);
   static constexpr bool ROW_PF =
       sizeof(R) == 4 && DSNU_ROWF_PF && MINB_F0 * (smem_row_fwd_pf + 1024) <= size_t(233472);
   static constexpr size_t smem_row_fwd =
@@ -217,7 +219,7 @@ struct Geo {
   // asynchronous copies into a landing buffer [q][2], with the same compact
   // stage table and half twiddle table as the forward pass.
   static constexpr size_t smem_row_inv_pf = size_t(STWCP + 2 * RB_I * RS + N / 2 + 2 * (N + 1)) * sizeof(cpx<R>);
-  static constexpr int MINB_I0 = (T_RI >= 512) ? 1 : DSNU_ROW_MINB;
+  static constexpr int MINB_I0 = ctas(T_RI);
   static constexpr bool ROWI_PF = sizeof(R) == 4 && DSNU_ROWI_PF && RB_I == 2 && TR == 4 &&
                                   MINB_I0 * (smem_row_inv_pf + 1024) <= size_t(233472);
   static constexpr size_t smem_row_inv =
@@ -230,16 +232,18 @@ struct Geo {
   // the two rows' elements of a 32-byte row tile are touched by adjacent lanes
   static constexpr bool ILV_F = (RB_F == 2);
   static constexpr bool ILV_I = (RB_I == 2);
-  static constexpr int MINB_F = (T_RF >= 512) ? 1 : DSNU_ROW_MINB;
-  static constexpr int MINB_I = (T_RI >= 512) ? 1 : DSNU_ROW_MINB;
-  static constexpr size_t smem_col = size_t(STWP + 2 * CC * FB) * sizeof(cpx<R>);  // two chains
+  static constexpr int MINB_F = MINB_F0;
+  static constexpr int MINB_I = MINB_I0;
+  static constexpr size_t smem_band = size_t(STWP + 2 * CB * FB) * sizeof(cpx<R>);  // two chains
   // FP32 column pass of I1: on top the table e^{-2 pi i n/M} (n < N)
   static constexpr bool COL_TAB = sizeof(R) == 4;
   // and two buffers of CC multiplier rows (N + 4 floats each, M for FULL ones),
   // the current item's and the next one's
   static constexpr int LDM = N + 4;
-  static constexpr size_t smem_col_main = smem_col + (COL_TAB ? size_t(N) * 8 + size_t(2 * CC * LDM) * 4 : 0);
-  static constexpr size_t smem_col_full = smem_col + (COL_TAB ? size_t(N) * 8 + size_t(2 * CC * M) * 4 : 0);
+  static constexpr size_t smem_col_main =
+      size_t(STWP + 2 * CC * FB) * sizeof(cpx<R>) + (COL_TAB ? size_t(N) * 8 + size_t(2 * CC * LDM) * 4 : 0);
+  static constexpr size_t smem_col_full =
+      size_t(STWP + 2 * CC * FB) * sizeof(cpx<R>) + (COL_TAB ? size_t(N) * 8 + size_t(2 * CC * M) * 4 : 0);
   static_assert(LOG2N >= 4 && LOG2N <= 12, "grid size 16..4096");
 };
 
@@ -255,11 +259,10 @@ struct Geo {
 // zero-padded length-M DFT of z = rho + i b are computed together (two
 // interleaved length-N transforms of z and z w_M^n), then the two real-signal
 // spectra are separated at every q in [0, N].
-template <typename R, int LOG2N>
+template <typename R, int LOG2N, typename GG = Geo<R, LOG2N>>
 __device__ __forceinline__ void row_fwd_body(int vb, int vg, Members mem, WsOff off, int ldqA, int ldqB, int Q,
                                              int ny, AxisTabs<R> ax, const R* __restrict__ decon_y, int cj,
                                              int* status) {
-  using GG = Geo<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, RB = GG::RB_F, T = GG::T_RF, RS = GG::RS;
   constexpr bool PF = GG::ROW_PF;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -429,10 +432,9 @@ k_row_fwd(Members mem, WsOff off, int ldqA, int ldqB, int Q, int ny, AxisTabs<R>
 // padded column DFT) go forward together, are multiplied by m1 and come back
 // together; their sum is the column of I1's inverse.  All loads of a column
 // precede the first barrier, so the in-place update is safe.
-template <typename R, int LOG2N, bool FULL>
+template <typename R, int LOG2N, bool FULL, typename GG = Geo<R, LOG2N>>
 __device__ __forceinline__ void col_main_body(int vb, int vg, Members mem, WsOff off, int ldqA, int ncols,
                                               AxisTabs<R> ay, MultRows<R> mt, int cj, int* ctr) {
-  using GG = Geo<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, CC = GG::CC, FB = GG::FB;
   // the e^{-2 pi i n/M} factors of the odd chain come from a shared table filled
   // once per CTA with the arithmetic of twm(), and m1 of the item's columns from
@@ -554,7 +556,7 @@ __device__ __forceinline__ void col_main_body(int vb, int vg, Members mem, WsOff
 }
 
 template <typename R, int LOG2N, bool FULL>
-__global__ void __launch_bounds__(Geo<R, LOG2N>::T_C, min_blocks<R>(DSNU_COLMAIN_MINB))
+__global__ void __launch_bounds__(Geo<R, LOG2N>::T_C, min_blocks<R>(1))
 k_col_main(Members mem, WsOff off, int ldqA, int ncols, AxisTabs<R> ay, MultRows<R> mt, int cj) {
   col_main_body<R, LOG2N, FULL>(blockIdx.x, gridDim.x, mem, off, ldqA, ncols, ay, mt, cj,
                                ws_ptr<int>(member_at(mem, 0), off.sched));
@@ -564,11 +566,10 @@ k_col_main(Members mem, WsOff off, int ldqA, int ncols, AxisTabs<R> ay, MultRows
 // ---------------------------------------------------------------------------
 // Band columns of the type-2 spectrum: per column of B, both output parities
 // of the padded column DFT in one paired transform; rows |qbar| <= Q kept.
-template <typename R, int LOG2N>
+template <typename R, int LOG2N, typename GG = Geo<R, LOG2N>>
 __device__ __forceinline__ void band_fwd_body(int vb, int vg, Members mem, WsOff off, int ldqB, int ncols, int ldq,
                                               int Q, AxisTabs<R> ay, int cj) {
-  using GG = Geo<R, LOG2N>;
-  constexpr int N = GG::N, M = GG::M, G = GG::G, CC = GG::CC, FB = GG::FB;
+  constexpr int N = GG::N, M = GG::M, G = GG::G, CC = GG::CB, FB = GG::FB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* stw = reinterpret_cast<cpx<R>*>(smem_raw);
   cpx<R>* sm = stw + GG::STWP;
@@ -614,7 +615,7 @@ __device__ __forceinline__ void band_fwd_body(int vb, int vg, Members mem, WsOff
 }
 
 template <typename R, int LOG2N>
-__global__ void __launch_bounds__(Geo<R, LOG2N>::T_C, min_blocks<R>(DSNU_COL_MINB))
+__global__ void __launch_bounds__(Geo<R, LOG2N>::T_B, min_blocks<R>(Geo<R, LOG2N>::MINB_B))
 k_band_fwd(Members mem, WsOff off, int ldqB, int ncols, int ldq, int Q, AxisTabs<R> ay, int cj) {
   band_fwd_body<R, LOG2N>(blockIdx.x, gridDim.x, mem, off, ldqB, ncols, ldq, Q, ay, cj);
 }
@@ -874,11 +875,10 @@ void launch_spread(int cfg, const Members& mem, const WsOff& off, const PlanTabl
 // ---------------------------------------------------------------------------
 // Inverse band columns: the even and odd rows of each band column of S go
 // through one paired inverse transform; T = even + e^{+2 pi i n/M} odd, n < N.
-template <typename R, int LOG2N>
+template <typename R, int LOG2N, typename GG = Geo<R, LOG2N>>
 __device__ __forceinline__ void band_inv_body(int vb, int vg, Members mem, WsOff off, int ldq, int Q, int ncols,
                                               int ldqB, AxisTabs<R> ay, int cj) {
-  using GG = Geo<R, LOG2N>;
-  constexpr int N = GG::N, M = GG::M, G = GG::G, CC = GG::CC, FB = GG::FB;
+  constexpr int N = GG::N, M = GG::M, G = GG::G, CC = GG::CB, FB = GG::FB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* stw = reinterpret_cast<cpx<R>*>(smem_raw);
   cpx<R>* sm = stw + GG::STWP;
@@ -921,7 +921,7 @@ __device__ __forceinline__ void band_inv_body(int vb, int vg, Members mem, WsOff
 }
 
 template <typename R, int LOG2N>
-__global__ void __launch_bounds__(Geo<R, LOG2N>::T_C, min_blocks<R>(DSNU_COL_MINB))
+__global__ void __launch_bounds__(Geo<R, LOG2N>::T_B, min_blocks<R>(Geo<R, LOG2N>::MINB_B))
 k_band_inv(Members mem, WsOff off, int ldq, int Q, int ncols, int ldqB, AxisTabs<R> ay, int cj) {
   band_inv_body<R, LOG2N>(blockIdx.x, gridDim.x, mem, off, ldq, Q, ncols, ldqB, ay, cj);
 }
@@ -937,11 +937,10 @@ k_band_inv(Members mem, WsOff off, int ldq, int Q, int ncols, int ldqB, AxisTabs
 // (Mx My) are each formed in FP32 (1/(Mx My) is a power of two, so the
 // scaling is exact), and their FP64 sum is formed by add_f32_f64 (bitwise
 // the FP64 addition of the two widened terms).
-template <typename R, int LOG2N>
+template <typename R, int LOG2N, typename GG = Geo<R, LOG2N>>
 __device__ __forceinline__ void row_inv_body(int vb, int vg, Members mem, WsOff off, int ldqA, int ldqB, int Q,
                                              int ny, AxisTabs<R> ax, const R* __restrict__ decon_y, R scale, int cj,
                                              int bpf, int acc64) {
-  using GG = Geo<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, RB = GG::RB_I, RS = GG::RS, T = GG::T_RI;
   constexpr bool PF = GG::ROWI_PF;
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -39,8 +39,10 @@ struct GeoStd {
   static constexpr int FB = fft_buf_elems(N);
   // row pairs or columns per CTA: CTAs of 128 threads where that holds one, whose
   // barriers do not keep all of an SM's warps in step (2048^2: the row passes
-  // 23.4 -> 21.0 and 21.8 -> 20.5 us against CTAs of 256)
-  static constexpr int PER = (G >= 128) ? 1 : 128 / G;
+  // 23.4 -> 21.0 and 21.8 -> 20.5 us against CTAs of 256), and of 64 for the short
+  // transforms, which then reach more SMs (256^2 solve 11.4 -> 10.8 us)
+  static constexpr int TM = LOG2N <= 9 ? 64 : 128;
+  static constexpr int PER = (G >= TM) ? 1 : TM / G;
   static constexpr int T = PER * G, MINB = 512 / T;
   static constexpr int STW = fft_stage_tw_elems(LOG2N) > 0 ? fft_stage_tw_elems(LOG2N) : 1;
   static constexpr int STWP = (STW + 1) & ~1;

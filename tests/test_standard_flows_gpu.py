@@ -72,3 +72,24 @@ def test_complex64_flows_match_numpy(nx, ny):
     # a few roundings of the angle (relative) and of the product
     assert np.abs(out.cpu().numpy() - ref).max() <= 4 * EPS * (np.abs(th).max() + 2) * np.abs(u).max()
     assert torch.equal(torch.view_as_real(ds.nonlinear_(t.clone(), phi, tau, beta)), torch.view_as_real(out))
+
+
+@pytest.mark.parametrize("multiplier", [None, (0, 0.3, -0.2, 0.4)], ids=["ds", "generic"])
+@pytest.mark.parametrize("nx,ny", [(16, 16), (32, 16), (16, 64), (128, 32), (256, 512), (512, 256), (512, 1024), (1024, 64)])
+def test_mixed_short_lengths_match_fp64(nx, ny, multiplier):
+    """Every CTA shape of the mixed passes, several members of one plan among
+    them: within the mixed plans' 2e-5 of the FP64 result."""
+    from paper_1409_2014_gb300 import Batch, Plan
+
+    prm = dict(nx=nx, ny=ny, lx=4.0, ly=4.0, cut_radius=2.0, n_r=12, n_theta=24, multiplier=multiplier)
+    rho = torch.from_numpy(np.random.default_rng(nx * ny).standard_normal((3, ny, nx))).cuda()
+    mixed, full = Plan(precision="mixed", **prm), Plan(precision="fp64", **prm)
+    phi = torch.stack([mixed.solve(r) for r in rho])
+    ref = torch.stack([full.solve(r) for r in rho])
+    assert float((phi - ref).abs().max() / ref.abs().max()) <= 2e-5
+    ref = full.solve_adjoint(rho[0])
+    assert float((mixed.solve_adjoint(rho[0]) - ref).abs().max() / ref.abs().max()) <= 2e-5
+    out = [torch.empty_like(r) for r in rho]
+    Batch([mixed] * 3, list(rho), out).solve()
+    torch.cuda.synchronize()
+    assert torch.equal(torch.stack(out), phi)
