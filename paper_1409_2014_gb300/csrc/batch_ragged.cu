@@ -180,7 +180,7 @@ SizeInfo size_info_of() {
   static_assert(GG::T_RF == kRagThreads && GG::T_RI == kRagThreads && GG::T_C == kRagThreads &&
                     GG::T_B == kRagThreads,
                 "one block size for every grid size of the schedule");
-  return SizeInfo{GG::RB_F, GG::RB_I, GG::CC, GG::smem_row_fwd, GG::smem_row_inv, GG::smem_band,
+  return SizeInfo{GG::RB_F, GG::RB_I, GG::CC, GG::smem_row_fwd, GG::smem_row_inv, GG::smem_col,
                   GG::smem_col_main, GG::ROWI_PF};
 }
 

@@ -234,7 +234,7 @@ struct Geo {
   static constexpr bool ILV_I = (RB_I == 2);
   static constexpr int MINB_F = MINB_F0;
   static constexpr int MINB_I = MINB_I0;
-  static constexpr size_t smem_band = size_t(STWP + 2 * CB * FB) * sizeof(cpx<R>);  // two chains
+  static constexpr size_t smem_col = size_t(STWP + 2 * CB * FB) * sizeof(cpx<R>);  // two chains
   // FP32 column pass of I1: on top the table e^{-2 pi i n/M} (n < N)
   static constexpr bool COL_TAB = sizeof(R) == 4;
   // and two buffers of CC multiplier rows (N + 4 floats each, M for FULL ones),

@@ -70,13 +70,13 @@ cudaError_t prepare_cols(PlanGeom& g) {
   const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if ((e = cudaFuncSetAttribute(k_col_main<R, L2, false>, A, int(GG::smem_col_main)))) return e;
   if ((e = cudaFuncSetAttribute(k_col_main<R, L2, true>, A, int(GG::smem_col_full)))) return e;
-  if ((e = cudaFuncSetAttribute(k_band_fwd<R, L2>, A, int(GG::smem_band)))) return e;
-  if ((e = cudaFuncSetAttribute(k_band_inv<R, L2>, A, int(GG::smem_band)))) return e;
+  if ((e = cudaFuncSetAttribute(k_band_fwd<R, L2>, A, int(GG::smem_col)))) return e;
+  if ((e = cudaFuncSetAttribute(k_band_inv<R, L2>, A, int(GG::smem_col)))) return e;
   if ((e = g.m1_full ? resident_ctas(k_col_main<R, L2, true>, GG::T_C, GG::smem_col_full, &g.cap_col)
                      : resident_ctas(k_col_main<R, L2, false>, GG::T_C, GG::smem_col_main, &g.cap_col)))
     return e;
-  if ((e = resident_ctas(k_band_fwd<R, L2>, GG::T_B, GG::smem_band, &g.cap_bandf))) return e;
-  return resident_ctas(k_band_inv<R, L2>, GG::T_B, GG::smem_band, &g.cap_bandi);
+  if ((e = resident_ctas(k_band_fwd<R, L2>, GG::T_B, GG::smem_col, &g.cap_bandf))) return e;
+  return resident_ctas(k_band_inv<R, L2>, GG::T_B, GG::smem_col, &g.cap_bandi);
 }
 
 template <typename R, int L2>
@@ -240,11 +240,11 @@ dsnu_status run_pipeline(const PlanGeom& g, const PlanTables& t, const WsLayout&
 #define DSNU_BANDF(L2)                                                                              \
   launch_k(g.pdl != 0, k_band_fwd<R, L2>,                                                           \
            dim3(persistent_grid(nm * ((g.Q + 1 + Geo<R, L2>::CB - 1) / Geo<R, L2>::CB), g.cap_bandf)), \
-           dim3(Geo<R, L2>::T_B), Geo<R, L2>::smem_band, bst, mem, off, ldqB, g.Q + 1, L.ldq, g.Q, ay, cj)
+           dim3(Geo<R, L2>::T_B), Geo<R, L2>::smem_col, bst, mem, off, ldqB, g.Q + 1, L.ldq, g.Q, ay, cj)
 #define DSNU_BANDI(L2)                                                                              \
   launch_k(g.pdl != 0, k_band_inv<R, L2>,                                                           \
            dim3(persistent_grid(nm * ((g.Q + 1 + Geo<R, L2>::CB - 1) / Geo<R, L2>::CB), g.cap_bandi)), \
-           dim3(Geo<R, L2>::T_B), Geo<R, L2>::smem_band, bst, mem, off, L.ldq, g.Q, g.Q + 1, ldqB, ay, cj)
+           dim3(Geo<R, L2>::T_B), Geo<R, L2>::smem_col, bst, mem, off, L.ldq, g.Q, g.Q + 1, ldqB, ay, cj)
 #define DSNU_ROWI(L2)                                                                               \
   launch_k(g.pdl != 0, k_row_inv<R, L2>,                                                            \
            dim3(persistent_grid(nm * ((g.ny + Geo<R, L2>::RB_I - 1) / Geo<R, L2>::RB_I), g.cap_rowi)), \
