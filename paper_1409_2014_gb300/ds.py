@@ -30,6 +30,15 @@ from . import Plan, _raw_stream as _stream
 _PREC = {"fp64": _abi.DSNU_FP64, "mixed": _abi.DSNU_MIXED}
 
 
+def _mem(t):
+    """t with its values in contiguous memory (t itself where they are).  The
+    library reads pointers: torch's lazy conjugate and negative bits, which
+    contiguous() passes on, have to be resolved first."""
+    if t.is_conj() or t.is_neg():
+        t = t.resolve_conj().resolve_neg()
+    return t.contiguous()
+
+
 class DSPlan:
     """Unpadded periodic transform and pointwise kernels for u on [-lx,lx) x [-ly,ly).
 
@@ -52,7 +61,7 @@ class DSPlan:
             self._h = _abi.dsnu_ds_plan_create(prm, _stream(dev))
 
     def _chk(self, u):
-        if u.dtype != self.cdtype or tuple(u.shape) != self.shape or not u.is_contiguous() \
+        if u.dtype != self.cdtype or u.shape != self.shape or not u.is_contiguous() \
                 or u.device != self.device:
             raise ValueError(f"expected a contiguous {self.cdtype} tensor of shape {self.shape} on "
                              f"{self.device}")
@@ -62,18 +71,21 @@ class DSPlan:
 
     def linear_(self, u, adjoint=False):
         self._chk(u)
-        _abi.dsnu_ds_linear(self._h, u.data_ptr(), 1 if adjoint else 0, _stream(self.device))
-        return u
+        v = _mem(u)
+        _abi.dsnu_ds_linear(self._h, v.data_ptr(), 1 if adjoint else 0, _stream(self.device))
+        return u if v is u else u.copy_(v)
 
     def linear(self, u, adjoint=False):
         """The linear flow of u in a new tensor (u is only read)."""
         self._chk(u)
+        u = _mem(u)
         out = torch.empty_like(u)
         _abi.dsnu_ds_linear_to(self._h, u.data_ptr(), out.data_ptr(), 1 if adjoint else 0, _stream(self.device))
         return out
 
     def abs2(self, u):
         self._chk(u)
+        u = _mem(u)
         rho = torch.empty(self.shape, dtype=torch.float64, device=self.device)
         _abi.dsnu_ds_abs2(self._h, u.data_ptr(), rho.data_ptr(), _stream(self.device))
         return rho
@@ -81,19 +93,21 @@ class DSPlan:
     def abs2_vjp(self, u, g_rho):
         """2 g_rho u: the gradient with respect to u through rho = |u|^2."""
         self._chk(u)
+        u, g_rho = _mem(u), _mem(g_rho)
         grad = torch.empty_like(u)
-        _abi.dsnu_ds_abs2_vjp(self._h, u.data_ptr(), g_rho.contiguous().data_ptr(), grad.data_ptr(),
-                              _stream(self.device))
+        _abi.dsnu_ds_abs2_vjp(self._h, u.data_ptr(), g_rho.data_ptr(), grad.data_ptr(), _stream(self.device))
         return grad
 
     def nonlinear_(self, u, phi, tau, beta):
         self._chk(u)
-        _abi.dsnu_ds_nonlinear(self._h, u.data_ptr(), phi.data_ptr(), tau, beta, _stream(self.device))
-        return u
+        v, phi = _mem(u), _mem(phi)
+        _abi.dsnu_ds_nonlinear(self._h, v.data_ptr(), phi.data_ptr(), tau, beta, _stream(self.device))
+        return u if v is u else u.copy_(v)
 
     def nonlinear(self, u, phi, tau, beta):
         """The nonlinear flow of u in a new tensor (u is only read)."""
         self._chk(u)
+        u, phi = _mem(u), _mem(phi)
         out = torch.empty_like(u)
         _abi.dsnu_ds_nonlinear_to(self._h, u.data_ptr(), phi.data_ptr(), out.data_ptr(), tau, beta,
                                   _stream(self.device))
@@ -102,6 +116,7 @@ class DSPlan:
     def nonlinear_vjp(self, u, phi, g, tau, beta):
         self._chk(u)
         self._chk(g)
+        u, phi, g = _mem(u), _mem(phi), _mem(g)
         s = torch.empty(self.shape, dtype=torch.float64, device=self.device)
         part = torch.empty_like(u)
         _abi.dsnu_ds_nonlinear_vjp(self._h, u.data_ptr(), phi.data_ptr(), g.data_ptr(), tau, beta,
@@ -109,9 +124,10 @@ class DSPlan:
         return s, part
 
     def nonlinear_vjp_finish_(self, u, s, ats, tau, beta, part):
+        u, s, ats, v = _mem(u), _mem(s), _mem(ats), _mem(part)
         _abi.dsnu_ds_nonlinear_vjp_finish(self._h, u.data_ptr(), s.data_ptr(), ats.data_ptr(), tau, beta,
-                                          part.data_ptr(), _stream(self.device))
-        return part
+                                          v.data_ptr(), _stream(self.device))
+        return part if v is part else part.copy_(v)
 
     def close(self):
         if getattr(self, "_h", None):
@@ -134,11 +150,11 @@ class PotentialFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, rho, plan: Plan):
         ctx.plan = plan
-        return plan.solve(rho.contiguous())
+        return plan.solve(_mem(rho))
 
     @staticmethod
     def backward(ctx, g):
-        return ctx.plan.solve_adjoint(g.contiguous()), None
+        return ctx.plan.solve_adjoint(_mem(g)), None
 
 
 def potential(rho, plan: Plan):
@@ -150,7 +166,7 @@ class PotentialOfWaveFn(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, u, ds: DSPlan, plan: Plan):
-        u = u.contiguous()
+        u = _mem(u)
         ctx.save_for_backward(u)
         ctx.ds, ctx.plan = ds, plan
         return plan.solve(ds.abs2(u))
@@ -158,7 +174,7 @@ class PotentialOfWaveFn(torch.autograd.Function):
     @staticmethod
     def backward(ctx, g):
         (u,) = ctx.saved_tensors
-        return ctx.ds.abs2_vjp(u, ctx.plan.solve_adjoint(g.contiguous())), None, None
+        return ctx.ds.abs2_vjp(u, ctx.plan.solve_adjoint(_mem(g))), None, None
 
 
 def potential_of_wave(u, ds: DSPlan, plan: Plan):
@@ -187,7 +203,7 @@ class NonlinearFlow(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, u, ds: DSPlan, solver: Plan, tau, beta):
-        u = u.contiguous()
+        u = _mem(u)
         phi = solver.solve(ds.abs2(u))
         ctx.save_for_backward(u, phi)
         ctx.ds, ctx.solver, ctx.tau, ctx.beta = ds, solver, tau, beta
