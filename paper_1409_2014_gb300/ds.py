@@ -259,7 +259,7 @@ def evolve(u0, steps, ds: DSPlan, solver: Plan, tau, alpha, beta, checkpoint_eve
     lin, non = _SUBSTEPS[scheme]
 
     def segment(u, n):
-        if n:
+        if n > 0:
             u = LinearFlow.apply(u, ds, lin[0] * tau, alpha)
         for k in range(n):
             for j, b in enumerate(non):

@@ -162,3 +162,13 @@ def test_plan_methods_take_lazy_views(loop):
                lambda a: ds.nonlinear_vjp_finish_(_lazy(g), s, _lazy(s), 0.1, 1.0, a)):
         v, want = _lazy(u), fn(u.clone())
         assert fn(v) is v and v.is_conj() and torch.equal(v, want)
+
+
+@pytest.mark.parametrize("scheme", ["strang", "yoshida"])
+@pytest.mark.parametrize("steps", [0, -1, -5])
+def test_no_steps_return_the_field(loop, steps, scheme):
+    ds, solver, log = loop
+    u = _field(11)
+    for every in (0, 2):
+        assert D.evolve(u, steps, ds, solver, 0.02, 1.0, -1.0, checkpoint_every=every, scheme=scheme) is u
+    assert not log
