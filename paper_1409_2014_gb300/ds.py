@@ -218,68 +218,63 @@ class NonlinearFlow(torch.autograd.Function):
         return ds.nonlinear_vjp_finish_(u, s, ats, ctx.tau, ctx.beta, part), None, None, None, None
 
 
-def strang_step(u, ds: DSPlan, solver: Plan, tau, alpha, beta):
-    """One Strang step: L(tau/2) N(tau) L(tau/2) (Sec. 2.3)."""
-    u = LinearFlow.apply(u, ds, 0.5 * tau, alpha)
-    u = NonlinearFlow.apply(u, ds, solver, tau, beta)
-    return LinearFlow.apply(u, ds, 0.5 * tau, alpha)
-
-
 _CBRT2 = 2.0 ** (1.0 / 3.0)
 # Sec. 2.3: b1 = b3 = 1/(2 - 2^(1/3)), b2 = -2^(1/3) b3, a1 = a4 = b3/2,
 # a2 = a3 = (b3 + b2)/2
 YOSHIDA_B = (1.0 / (2.0 - _CBRT2), -_CBRT2 / (2.0 - _CBRT2), 1.0 / (2.0 - _CBRT2))
 YOSHIDA_A = (0.5 * YOSHIDA_B[0], 0.5 * (YOSHIDA_B[0] + YOSHIDA_B[1]),
              0.5 * (YOSHIDA_B[0] + YOSHIDA_B[1]), 0.5 * YOSHIDA_B[0])
+# one step as (linear sub-steps, nonlinear sub-steps) in the order they act
+_SUBSTEPS = {"strang": ((0.5, 0.5), (1.0,)), "yoshida": (YOSHIDA_A[::-1], YOSHIDA_B[::-1])}
+
+
+def _advance(u, n, scheme, first, last, ds: DSPlan, solver: Plan, tau, alpha, beta):
+    """n neighbouring steps of a loop.  The linear flow is exact, so the last one of a step and the first
+    one of the next are one flow over the sum of their steps; the step before runs it.  first, last:
+    whether the loop begins and ends with these steps (no step before them, none after)."""
+    lin, non = _SUBSTEPS[scheme]
+    if first:
+        u = LinearFlow.apply(u, ds, lin[0] * tau, alpha)
+    for k in range(n):
+        for j, b in enumerate(non):
+            u = NonlinearFlow.apply(u, ds, solver, b * tau, beta)
+            a = lin[j + 1]
+            if j + 1 == len(non) and not (last and k + 1 == n):
+                a += lin[0]
+            u = LinearFlow.apply(u, ds, a * tau, alpha)
+    return u
+
+
+def strang_step(u, ds: DSPlan, solver: Plan, tau, alpha, beta):
+    """One Strang step: L(tau/2) N(tau) L(tau/2) (Sec. 2.3)."""
+    return _advance(u, 1, "strang", True, True, ds, solver, tau, alpha, beta)
 
 
 def yoshida_step(u, ds: DSPlan, solver: Plan, tau, alpha, beta):
     """u <- A(a1 tau) B(b1 tau) A(a2 tau) B(b2 tau) A(a3 tau) B(b3 tau) A(a4 tau) u
     (Sec. 2.3; the rightmost sub-flow acts first).  Each nonlinear sub-flow
     freezes Phi of the field it starts from."""
-    u = LinearFlow.apply(u, ds, YOSHIDA_A[3] * tau, alpha)
-    for j in (2, 1, 0):
-        u = NonlinearFlow.apply(u, ds, solver, YOSHIDA_B[j] * tau, beta)
-        u = LinearFlow.apply(u, ds, YOSHIDA_A[j] * tau, alpha)
-    return u
-
-
-# strang_step and yoshida_step as (linear sub-steps, nonlinear sub-steps) in the order they act
-_SUBSTEPS = {"strang": ((0.5, 0.5), (1.0,)), "yoshida": (YOSHIDA_A[::-1], YOSHIDA_B[::-1])}
+    return _advance(u, 1, "yoshida", True, True, ds, solver, tau, alpha, beta)
 
 
 def evolve(u0, steps, ds: DSPlan, solver: Plan, tau, alpha, beta, checkpoint_every=0, scheme="strang"):
     """``steps`` steps of ``scheme`` ("strang" or "yoshida"); with
     checkpoint_every > 0 only the input of every segment of that many steps is
     kept for the backward pass, and each segment is recomputed during backward.
-
-    The last linear flow of a step and the first one of the next are one flow
-    over the sum of their steps (the linear flow is exact): a segment of n Strang
-    steps runs n + 1 linear flows instead of 2 n."""
-    lin, non = _SUBSTEPS[scheme]
-
-    def segment(u, n):
-        if n > 0:
-            u = LinearFlow.apply(u, ds, lin[0] * tau, alpha)
-        for k in range(n):
-            for j, b in enumerate(non):
-                u = NonlinearFlow.apply(u, ds, solver, b * tau, beta)
-                a = lin[j + 1]
-                if j + 1 == len(non) and k + 1 < n:
-                    a += lin[0]
-                u = LinearFlow.apply(u, ds, a * tau, alpha)
-        return u
-
-    u = u0
-    if checkpoint_every and checkpoint_every > 0:
-        done = 0
-        while done < steps:
-            n = min(checkpoint_every, steps - done)
-            # (nothing in a segment draws random numbers)
-            u = _ckpt.checkpoint(segment, u, n, use_reentrant=False, preserve_rng_state=False)
-            done += n
-        return u
-    return segment(u, steps)
+    n Strang steps run n + 1 linear flows (see _advance), the same ones whatever
+    checkpoint_every is: checkpoints do not change a bit of the result."""
+    if scheme not in _SUBSTEPS:
+        raise KeyError(scheme)
+    every = checkpoint_every if checkpoint_every and checkpoint_every > 0 else 0
+    u, done = u0, 0
+    while done < steps:
+        n = min(every, steps - done) if every else steps
+        args = (u, n, scheme, done == 0, done + n == steps, ds, solver, tau, alpha, beta)
+        # (nothing in a segment draws random numbers)
+        u = _ckpt.checkpoint(_advance, *args, use_reentrant=False, preserve_rng_state=False) if every \
+            else _advance(*args)
+        done += n
+    return u
 
 
 def mass(u, lx, ly):

@@ -172,3 +172,28 @@ def test_no_steps_return_the_field(loop, steps, scheme):
     for every in (0, 2):
         assert D.evolve(u, steps, ds, solver, 0.02, 1.0, -1.0, checkpoint_every=every, scheme=scheme) is u
     assert not log
+
+
+@pytest.mark.parametrize("scheme,single", [("strang", D.strang_step), ("yoshida", D.yoshida_step)])
+def test_flows_do_not_depend_on_checkpoints(loop, scheme, single):
+    """One sequence of flows for every checkpoint_every (so one result, bit for bit), equal to single steps up to
+    the merged linear flows' rounding."""
+    ds, solver, log = loop
+    a, steps = (ds, solver, 0.02, 1.0, -1.0), 5
+    out, grads, flows = [], [], []
+    for every in (0, 1, 2, 3, 5, 7):
+        x = _field(12).requires_grad_(True)
+        del log[:]
+        v = D.evolve(x, steps, *a, checkpoint_every=every, scheme=scheme)
+        flows.append(list(log))
+        out.append(v.detach())
+        grads.append(torch.autograd.grad(v, x, _field(13))[0])
+    assert all(f == flows[0] for f in flows) and len(flows[0]) == steps * (2 if scheme == "strang" else 6) + 1
+    assert all(torch.equal(v, out[0]) for v in out) and all(torch.equal(g, grads[0]) for g in grads)
+    x = _field(12).requires_grad_(True)
+    v = x
+    for _ in range(steps):
+        v = single(v, *a)
+    g, = torch.autograd.grad(v, x, _field(13))
+    assert float((v.detach() - out[0]).abs().max()) <= 1e-13 and float((g - grads[0]).abs().max()) <= 1e-12
+    assert torch.equal(single(_field(12), *a), D.evolve(_field(12), 1, *a, scheme=scheme))

@@ -1,5 +1,5 @@
 """The DS time loop on the GPU: lazily conjugated fields and cotangents give
-the bits of the resolved ones."""
+the bits of the resolved ones, checkpoints those of the loop without them."""
 
 import pytest
 
@@ -76,3 +76,19 @@ def test_overlap_loss_equals_its_real_form(loop):
     got, ref = grad(lambda v: (v.conj() * w).sum().abs()), grad(real_form)
     # sums of N^2 terms in another order: sqrt(N^2) roundings of their norm against |<v, w>| of that size
     assert float((got - ref).norm()) <= 16 * N * eps * float(ref.norm())
+
+
+@pytest.mark.parametrize("scheme", ["strang", "yoshida"])
+def test_checkpoints_do_not_change_a_bit(loop, scheme):
+    from paper_1409_2014_gb300.ds import evolve
+
+    field, a = loop
+
+    def run(every):
+        x = field(5).requires_grad_(True)
+        v = evolve(x, 5, *a, checkpoint_every=every, scheme=scheme)
+        return v.detach(), torch.autograd.grad(v, x, field(6))[0]
+
+    ref = run(0)
+    for every in (1, 2, 3, 5):
+        assert all(torch.equal(p, q) for p, q in zip(run(every), ref))
