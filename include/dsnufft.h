@@ -322,7 +322,7 @@ dsnu_status dsnu_ds_set_linear_step(dsnu_ds_plan plan, double tau, double alpha,
 dsnu_status dsnu_ds_linear(dsnu_ds_plan plan, void* u_dev, int32_t adjoint, void* stream);
 
 /* The same with the result in out_dev (which may be u_dev; u_dev is otherwise
- * only read). */
+ * only read).  DSNU_EINVAL, nothing launched, when the two overlap in part. */
 dsnu_status dsnu_ds_linear_to(dsnu_ds_plan plan, const void* u_dev, void* out_dev, int32_t adjoint, void* stream);
 
 /* rho <- |u|^2 (FP64 [ny][nx], device), the density of eq. DSII_exact_pot. */
@@ -343,7 +343,8 @@ dsnu_status dsnu_ds_nonlinear(dsnu_ds_plan plan, void* u_dev, const double* phi_
                               double beta, void* stream);
 
 /* The same with the result in out_dev (which may be u_dev; u_dev is otherwise
- * only read). */
+ * only read).  DSNU_EINVAL, nothing launched, when out_dev overlaps u_dev in part
+ * or phi_dev. */
 dsnu_status dsnu_ds_nonlinear_to(dsnu_ds_plan plan, const void* u_dev, const double* phi_dev, void* out_dev,
                                  double tau, double beta, void* stream);
 

@@ -599,6 +599,32 @@ dsnu_status check_launch() {
   return e == cudaSuccess ? DSNU_OK : ds_fail(DSNU_ECUDA, std::string("launch: ") + cudaGetErrorString(e));
 }
 
+// Bytes of a field, and whether two ranges share any.
+size_t field_bytes(const dsnu_ds_plan_s* P) {
+  return size_t(P->prm.nx) * P->prm.ny * (P->prm.precision == DSNU_MIXED ? sizeof(float2) : sizeof(double2));
+}
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const char *p = static_cast<const char*>(a), *q = static_cast<const char*>(b);
+  return p < q + nb && q < p + na;
+}
+
+dsnu_status linear(dsnu_ds_plan_s* P, const void* u, void* out, int adjoint, cudaStream_t st) {
+  if (!P->has_phase) return ds_fail(DSNU_EINVAL, "no linear step set (dsnu_ds_set_linear_step)");
+  return P->prm.precision == DSNU_MIXED ? linear_f32(P, u, out, adjoint, st) : linear_f64(P, u, out, adjoint, st);
+}
+
+dsnu_status nonlinear(dsnu_ds_plan_s* P, const void* u, const double* phi, void* out, double tau, double beta,
+                      cudaStream_t st) {
+  const size_t n = size_t(P->prm.nx) * P->prm.ny;
+  if (P->prm.precision == DSNU_MIXED)
+    launch_k(P->pdl, k_nonlinear<float>, dim3(grid_1d(n)), dim3(256), 0, st, static_cast<const cpx<float>*>(u),
+             static_cast<cpx<float>*>(out), phi, n, float(tau), float(beta));
+  else
+    launch_k(P->pdl, k_nonlinear<double>, dim3(grid_1d(n)), dim3(256), 0, st, static_cast<const cpx<double>*>(u),
+             static_cast<cpx<double>*>(out), phi, n, tau, beta);
+  return check_launch();
+}
+
 int ilog2i(int v) {
   int l = 0;
   while ((1 << l) < v) ++l;
@@ -697,14 +723,15 @@ dsnu_status dsnu_ds_set_linear_step(dsnu_ds_plan plan, double tau, double alpha,
 
 dsnu_status dsnu_ds_linear_to(dsnu_ds_plan plan, const void* u_dev, void* out_dev, int32_t adjoint, void* stream) {
   if (!plan || !u_dev || !out_dev) return ds_fail(DSNU_EINVAL, "NULL plan or field");
-  if (!plan->has_phase) return ds_fail(DSNU_EINVAL, "no linear step set (dsnu_ds_set_linear_step)");
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  return plan->prm.precision == DSNU_MIXED ? linear_f32(plan, u_dev, out_dev, adjoint, st)
-                                           : linear_f64(plan, u_dev, out_dev, adjoint, st);
+  const size_t nb = field_bytes(plan);
+  if (out_dev != u_dev && overlap(u_dev, nb, out_dev, nb))
+    return ds_fail(DSNU_EINVAL, "input and output overlap in part");
+  return linear(plan, u_dev, out_dev, adjoint, static_cast<cudaStream_t>(stream));
 }
 
 dsnu_status dsnu_ds_linear(dsnu_ds_plan plan, void* u_dev, int32_t adjoint, void* stream) {
-  return dsnu_ds_linear_to(plan, u_dev, u_dev, adjoint, stream);
+  if (!plan || !u_dev) return ds_fail(DSNU_EINVAL, "NULL plan or field");
+  return linear(plan, u_dev, u_dev, adjoint, static_cast<cudaStream_t>(stream));
 }
 
 dsnu_status dsnu_ds_abs2(dsnu_ds_plan plan, const void* u_dev, double* rho_dev, void* stream) {
@@ -735,20 +762,17 @@ dsnu_status dsnu_ds_abs2_vjp(dsnu_ds_plan plan, const void* u_dev, const double*
 dsnu_status dsnu_ds_nonlinear_to(dsnu_ds_plan plan, const void* u_dev, const double* phi_dev, void* out_dev, double tau,
                                  double beta, void* stream) {
   if (!plan || !u_dev || !phi_dev || !out_dev) return ds_fail(DSNU_EINVAL, "NULL argument");
-  const size_t n = size_t(plan->prm.nx) * plan->prm.ny;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (plan->prm.precision == DSNU_MIXED)
-    launch_k(plan->pdl, k_nonlinear<float>, dim3(grid_1d(n)), dim3(256), 0, st, static_cast<const cpx<float>*>(u_dev),
-             static_cast<cpx<float>*>(out_dev), phi_dev, n, float(tau), float(beta));
-  else
-    launch_k(plan->pdl, k_nonlinear<double>, dim3(grid_1d(n)), dim3(256), 0, st,
-             static_cast<const cpx<double>*>(u_dev), static_cast<cpx<double>*>(out_dev), phi_dev, n, tau, beta);
-  return check_launch();
+  const size_t nb = field_bytes(plan);
+  if ((out_dev != u_dev && overlap(u_dev, nb, out_dev, nb)) ||
+      overlap(phi_dev, size_t(plan->prm.nx) * plan->prm.ny * sizeof(double), out_dev, nb))
+    return ds_fail(DSNU_EINVAL, "the output overlaps phi, or the input in part");
+  return nonlinear(plan, u_dev, phi_dev, out_dev, tau, beta, static_cast<cudaStream_t>(stream));
 }
 
 dsnu_status dsnu_ds_nonlinear(dsnu_ds_plan plan, void* u_dev, const double* phi_dev, double tau, double beta,
                               void* stream) {
-  return dsnu_ds_nonlinear_to(plan, u_dev, phi_dev, u_dev, tau, beta, stream);
+  if (!plan || !u_dev || !phi_dev) return ds_fail(DSNU_EINVAL, "NULL argument");
+  return nonlinear(plan, u_dev, phi_dev, u_dev, tau, beta, static_cast<cudaStream_t>(stream));
 }
 
 dsnu_status dsnu_ds_nonlinear_vjp(dsnu_ds_plan plan, const void* u_dev, const double* phi_dev, const void* g_dev,

@@ -92,3 +92,42 @@ def test_checkpoints_do_not_change_a_bit(loop, scheme):
     ref = run(0)
     for every in (1, 2, 3, 5):
         assert all(torch.equal(p, q) for p, q in zip(run(every), ref))
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_partly_overlapping_outputs_are_refused(prec):
+    """The flows into another buffer take the input's own or a disjoint one, down to neighbouring bytes; what
+    overlaps in part (a race between rows) is refused before anything is launched."""
+    from paper_1409_2014_gb300 import _abi
+    from paper_1409_2014_gb300.ds import DSPlan
+
+    ds = DSPlan(32, 16, 4.0, 4.0, precision=prec)
+    ds.set_linear_step(1e-2, 1.0)
+    n = 32 * 16
+    pool = torch.zeros(4 * n, dtype=ds.cdtype, device="cuda")
+    pool[:n] = torch.randn(n, dtype=ds.cdtype, device="cuda")
+    before, size = pool.clone(), pool.element_size()
+    base, stream = pool.data_ptr(), torch.cuda.current_stream().cuda_stream
+    phi = torch.ones(16, 32, dtype=torch.float64, device="cuda")
+
+    def flows(out, phi_ptr=phi.data_ptr()):
+        return (lambda: _abi.dsnu_ds_linear_to(ds._h, base, out, 0, stream),
+                lambda: _abi.dsnu_ds_nonlinear_to(ds._h, base, phi_ptr, out, 0.1, 1.0, stream))
+
+    refused = [f for e in (1, 32, n - 1) for f in flows(base + e * size)]
+    refused.append(flows(base + n * size, base + (2 * n - 2) * size)[1])  # phi's first bytes
+    refused.append(flows(base + 3 * n * size, base + 3 * n * size)[1])
+    for f in refused:
+        with pytest.raises(_abi.DsnuError) as e:
+            f()
+        assert e.value.status == _abi.DSNU_EINVAL and "overlap" in str(e.value)
+    torch.cuda.synchronize()
+    assert torch.equal(pool, before)
+    for i in (0, 1):
+        for out in (base + n * size, base):
+            pool.copy_(before)
+            flows(out)[i]()
+            want = ds.linear(before[:n].view(16, 32)) if i == 0 else ds.nonlinear(before[:n].view(16, 32), phi, 0.1, 1.0)
+            at = 0 if out == base else n
+            assert torch.equal(pool[at:at + n].view(16, 32), want)
+    ds.close()
