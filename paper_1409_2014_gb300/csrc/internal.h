@@ -8,6 +8,7 @@
 #include <string>
 
 #include "dsnufft.h"
+#include "overlap.h"
 
 namespace dsnu {
 
@@ -104,17 +105,6 @@ struct PlanGeom {
 constexpr int kStages = 8;       // kernels per solve
 constexpr int kProfEvents = kStages + 1;  // events per profiled solve (see run_pipeline)
 
-// Concurrency of the band chain with the column pass: one of the two runs on
-// `side` (a low-priority stream owned by the plan): the band chain, or with
-// col_side the column pass, whose persistent grid leaves `reserve` SMs free.
-struct Overlap {
-  cudaStream_t side;
-  cudaEvent_t fork, join;
-  int reserve;
-  int col_side;
-  bool on;
-};
-
 // Launchers (one translation unit per precision).  `ev`, when not NULL,
 // holds kProfEvents events recorded around the kernels (the kernels then run
 // one after the other on `st`); `ov`, when not NULL, runs the band chain
@@ -186,5 +176,5 @@ struct dsnu_plan_s {
   bool has_copy_streams;
   cudaStream_t copy_in, copy_out;
   cudaEvent_t ev_start, ev_in[2], ev_solved[2], ev_out[2];
-  dsnu::Overlap overlap;    // band chain next to the column pass (reserve 0: off)
+  dsnu::Overlap overlap;    // band chain next to the column pass
 };

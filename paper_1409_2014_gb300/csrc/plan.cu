@@ -1040,14 +1040,7 @@ dsnu_status dsnu_plan_create_multiplier(const dsnu_params* params, const dsnu_mu
     ov.reserve = std::max(1, int(std::lround(g.sms * (ov.col_side ? std::min(share, 48.0 / 152.0) : share))));
     const char* env = std::getenv("DSNU_BAND_SMS");
     if (env) ov.reserve = std::atoi(env);
-    if (ov.reserve > 0) {
-      int lo = 0, hi = 0;
-      cudaError_t ce = cudaDeviceGetStreamPriorityRange(&lo, &hi);
-      if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(&ov.side, cudaStreamNonBlocking, lo);
-      if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&ov.fork, cudaEventDisableTiming);
-      if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&ov.join, cudaEventDisableTiming);
-      ov.on = (ce == cudaSuccess);
-    }
+    if (ov.reserve > 0) overlap_open(ov);
   }
   *out = P;
   return DSNU_OK;
@@ -1115,12 +1108,7 @@ dsnu_status dsnu_status_poll(dsnu_plan plan, void* stream) {
 dsnu_status dsnu_plan_destroy(dsnu_plan plan) {
   if (!plan) return DSNU_OK;
   free_profile(plan);
-  if (plan->overlap.on) {
-    cudaStreamSynchronize(plan->overlap.side);
-    cudaStreamDestroy(plan->overlap.side);
-    cudaEventDestroy(plan->overlap.fork);
-    cudaEventDestroy(plan->overlap.join);
-  }
+  overlap_close(plan->overlap);
   if (plan->has_copy_streams) {
     cudaStreamSynchronize(plan->copy_in);
     cudaStreamSynchronize(plan->copy_out);
