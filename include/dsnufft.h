@@ -163,7 +163,8 @@ dsnu_status dsnu_set_workspace(dsnu_plan plan, void* workspace_dev, size_t bytes
  * one of them on a low-priority stream owned by the plan (the band chain on
  * grids of at least 2048 x 2048, the column pass on smaller ones), the column
  * pass leaving a number of SMs free (DSNU_BAND_SMS=<n> in the environment at
- * plan creation sets it, 0 runs everything on `stream`); the plan orders that
+ * plan creation sets it; 0, or as many as the device has, runs everything on
+ * `stream`); the plan orders that
  * stream after `stream`'s earlier work and `stream` after it, so the call
  * behaves as if everything ran on `stream`.
  * rho_dev: [ny][nx] FP64 density (device, read only).

@@ -1013,33 +1013,15 @@ dsnu_status dsnu_plan_create_multiplier(const dsnu_params* params, const dsnu_mu
     return fail(DSNU_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(e));
   }
   layout_workspace(P);
-  // The band chain and the column pass run side by side.  On large grids the
-  // column pass is the longer one: the band chain runs on the low-priority side
-  // stream, the column pass leaving it 16 of every 152 SMs, in mixed plans a share
-  // growing as 1/sqrt(nx ny) below 4096^2, since the band chain's node work is the
-  // same on every grid (mixed 4096^2 507 us with 16 SMs, 525 with 32, 521 in
-  // line; 2048^2 131 with 32, 139 with 16, 150 in line; FP64, whose column pass is
-  // heavier, 4096^2 2041 us, with 24 SMs 2093, in line 2057; 2048^2 499, with 32
-  // SMs 516, in line 541).  Below 2048^2 the band chain is the
-  // longer one: it stays on the caller's stream, where its launches overlap, and
-  // the column pass fills the rest of the GPU from the side stream (FP64 512^2
-  // 74 us; 1024^2 156, in line 166; mixed 256^2 41 against 47).
-  // There the mixed share is capped at 48 SMs (1024^2 55.6 us with 48, 63.3 with
-  // 16; 2048 x 512 53.6 and 59.7).
-  // DSNU_BAND_SMS=<n> sets the number of SMs left free, 0 runs both in line.
   {
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&g.sms, cudaDevAttrMultiProcessorCount, dev);
   }
-  if (!standard) {
-    double share = 16.0 / 152.0;
-    if (g.precision == DSNU_MIXED) share *= 4096.0 / std::sqrt(double(p.nx) * p.ny);
+  if (!standard) {  // band chain and column pass side by side (overlap.h)
     Overlap& ov = P->overlap;
-    ov.col_side = (p.nx < 2048 || p.ny < 2048) ? 1 : 0;
-    ov.reserve = std::max(1, int(std::lround(g.sms * (ov.col_side ? std::min(share, 48.0 / 152.0) : share))));
-    const char* env = std::getenv("DSNU_BAND_SMS");
-    if (env) ov.reserve = std::atoi(env);
+    ov.col_side = overlap_col_side(p.nx, p.ny) ? 1 : 0;
+    ov.reserve = overlap_reserve(p.nx, p.ny, g.precision == DSNU_MIXED, g.sms, std::getenv("DSNU_BAND_SMS"));
     if (ov.reserve > 0) overlap_open(ov);
   }
   *out = P;

@@ -1,7 +1,7 @@
 // Host-only check of overlap.h with a fake of the runtime's calls: whichever
 // creation fails, nothing of the stream and the events is left, the error is
 // cleared and the plan is told to run in line; on success everything is
-// dropped once by the close.  Prints "OK" or the failing checks.
+// dropped once by the close.  And the rule for the SMs left free.  Prints "OK" or the failing checks.
 #include <cstdio>
 
 #include "overlap.h"
@@ -56,6 +56,17 @@ int main() {
     dsnu::overlap_close<Fake>(ov);
     expect(live == 0, "closed twice", fail_at);
   }
+  // the reserve: the measured shares of 152 SMs, scaled to other devices; a wish
+  // that leaves the column pass no SM, or none, runs in line
+  struct { int nx, ny, mixed, sms; const char* env; int want; } rule[] = {
+      {4096, 4096, 1, 152, nullptr, 16}, {2048, 2048, 1, 152, nullptr, 32}, {4096, 2048, 1, 152, nullptr, 23},
+      {1024, 1024, 1, 152, nullptr, 48}, {128, 16, 1, 152, nullptr, 48},    {2048, 512, 1, 152, nullptr, 48},
+      {4096, 4096, 0, 152, nullptr, 16}, {64, 64, 0, 152, nullptr, 16},     {64, 64, 0, 4, nullptr, 1},
+      {64, 64, 0, 1, nullptr, 0},        {512, 512, 1, 152, "24", 24},      {512, 512, 1, 152, "151", 151},
+      {512, 512, 1, 152, "152", 0},      {512, 512, 0, 152, "1000", 0},     {4096, 4096, 1, 152, "0", 0},
+      {4096, 4096, 0, 152, "-3", 0},     {4096, 4096, 0, 152, "", 0}};
+  for (auto& r : rule)
+    expect(dsnu::overlap_reserve(r.nx, r.ny, r.mixed != 0, r.sms, r.env) == r.want, "reserve", r.nx * 10000 + r.ny);
   if (failures == 0) std::printf("OK\n");
   return failures == 0 ? 0 : 1;
 }
