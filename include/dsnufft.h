@@ -274,7 +274,8 @@ const char* dsnu_stage_name(int32_t stage);
  * library, held until the process exits) instead of the plan's workspace; no
  * workspace needs to be attached.  Enough for grids up to 1024 x 1024 in
  * either precision; a plan needing more scratch gets DSNU_EINVAL with a
- * message naming both sizes.
+ * message naming both sizes (the exponents at the end of an FP64 plan's
+ * workspace, at most 67 KB, do not count: the library has room for them apart).
  * The first call on a device looks up the array's device address
  * (cudaGetSymbolAddress, with that device current); make that first call
  * before any stream capture.  Every call on a device shares the one array,

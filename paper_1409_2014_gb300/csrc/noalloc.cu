@@ -22,8 +22,13 @@
 namespace {
 
 constexpr size_t kStaticScratchBytes = size_t(32) << 20;  // 32 MiB per device
+// and room for the exponents of an FP64 plan's rows and columns (the end of its
+// workspace), so that they do not count against the 32 MiB: two ints per row,
+// one per column of A and B, each array rounded up to 256 bytes
+constexpr size_t kExponentBytes = size_t(72) << 10;
+static_assert(4 * (2 * 4096 + 4097 + 4096) + 4 * 255 <= kExponentBytes, "the exponents of the largest grid");
 
-__device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
+__device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes + kExponentBytes];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_scratch_mutex;
@@ -76,7 +81,8 @@ dsnu_status dsnu_solve_noalloc(dsnu_plan plan, const double* rho, double* phi, v
     dsnu::set_last_error("input and output must be 16-byte aligned");
     return DSNU_EINVAL;
   }
-  const size_t need = plan->ws_layout.total;
+  const dsnu::WsLayout& L = plan->ws_layout;
+  const size_t need = plan->geom.precision == DSNU_FP64 ? L.off_rexp : L.total;  // (without the exponents)
   if (need > kStaticScratchBytes) {
     dsnu::set_last_error("dsnu_solve_noalloc: this plan needs " + std::to_string(need) +
                          " bytes of scratch but the library's static scratch holds " +

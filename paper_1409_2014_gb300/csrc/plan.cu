@@ -894,7 +894,7 @@ static void layout_workspace(dsnu_plan_s* P) {  // defined after the autotuner, 
   L.off_c = take(size_t(g.n_nodes) * csz);
   L.off_partial = take(size_t(std::max(g.n_items, 1)) * g.spread_tile * g.spread_tile * csz);
   L.off_sched = take(sizeof(int));
-  if (g.precision == DSNU_FP64) {
+  if (g.precision == DSNU_FP64) {  // (last: dsnu_solve_noalloc does not count them)
     L.off_rexp = take(size_t(g.ny) * sizeof(int));
     L.off_rexpb = take(size_t(g.ny) * sizeof(int));
     L.off_cexp = take(size_t(g.nx + 1) * sizeof(int));
