@@ -53,6 +53,9 @@ constexpr int kFxTwBits = 28, kFxMultBits = 27, kFxDeconBits = 31;
 
 // Exponents of all-zero transforms, and of ones with an infinity or a NaN.
 constexpr int kFxZero = -(1 << 20), kFxBad = 1 << 20;
+// The exponent of a multiplier's column whose entries are not all finite: added to
+// those of any transform it gives one above kFxBad.
+constexpr int kFxMultBad = 2 * kFxBad;
 
 __device__ __forceinline__ fxc fx_mk(i64 x, i64 y) { fxc c; c.x = x; c.y = y; return c; }
 __device__ __forceinline__ fxc operator+(fxc a, fxc b) { return fx_mk(a.x + b.x, a.y + b.y); }

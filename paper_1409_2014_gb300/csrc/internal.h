@@ -45,7 +45,7 @@ struct PlanTables {
   int* status;    // one int
   void* m1tab;    // split plans: the multiplier rows (MultRows), in fixed point in FP64 plans (FxMult, both solvers)
   // FP64 plans: the fixed-point tables of both axes (fx.cuh, FxAxis) and the
-  // multiplier's exponent per column (generic multipliers, else NULL)
+  // multiplier's exponent per column (fx_mult_exponents; NULL: all 0)
   void *fx_stw_x, *fx_wm_x, *fx_dec_x, *fx_stw_y, *fx_wm_y, *fx_dec_y;
   int* fx_mexp;
 };

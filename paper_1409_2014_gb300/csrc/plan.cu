@@ -593,15 +593,22 @@ __global__ void k_fill_std_fx(int2* tab, int nx, int ny, int ld, int full, doubl
 }
 
 // Exponents of the columns of a generic multiplier's fixed-point table:
-// |m| <= (|a0| + |a_cos| + |a_sin|) |k|^alpha < 2^(mexp - 1) on column q.
+// |m| <= (|a0| + |a_cos| + |a_sin|) |k|^alpha < 2^(mexp - 1) on column q, and
+// kFxMultBad where that bound, or |k|^2 of the grid's corner, is beyond the FP64
+// range (an entry then is infinite or a NaN).  Empty for the DS multiplier on a
+// grid within the range: its |m| <= 1 needs none.
 static std::vector<int> fx_mult_exponents(const PlanGeom& g, int ncols, double dkx, double dky, double kymax) {
   std::vector<int> out;
+  const double kxmax = (ncols - 1) * dkx;
+  const bool over = !std::isfinite(kxmax * kxmax + kymax * kymax);
+  if (!g.m_generic && !over) return out;
   const double amp = std::fabs(g.m_a0) + std::fabs(g.m_ac) + std::fabs(g.m_as);
   for (int q = 0; q < ncols; ++q) {
     const double k1 = q * dkx;
     const double b = (g.m_alpha == 1) ? amp * std::sqrt(k1 * k1 + kymax * kymax)
                      : (g.m_alpha == -1) ? amp / (q == 0 ? dky : k1) : amp;
-    out.push_back(b > 0.0 ? std::min(std::max(std::ilogb(b) + 2, -1200), 1100) : 0);
+    out.push_back(over || !std::isfinite(b) ? kFxMultBad
+                  : b > 0.0 ? std::min(std::max(std::ilogb(b) + 2, -1200), 1100) : 0);
   }
   return out;
 }
@@ -678,7 +685,7 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
     twiddles(ny / 2, My, tmp); T.fx_wm_y = fx_table(tmp, kFxTwBits);
     g.kdx = fx_decon(dcx, T.fx_dec_x);
     g.kdy = fx_decon(dcy, T.fx_dec_y);
-    if (g.m_generic) T.fx_mexp = fx_mult_exponents(g, nx + 1, dkx, dky, ny * dky);
+    T.fx_mexp = fx_mult_exponents(g, nx + 1, dkx, dky, ny * dky);
   } else {
     fft_stage_twiddles(g.log2nx, tmp); T.stw_x = cast<R>(tmp);
     fft_stage_twiddles(g.log2ny, tmp); T.stw_y = cast<R>(tmp);
@@ -779,7 +786,7 @@ static dsnu_status build_tables(dsnu_plan_s* P, cudaStream_t st) {
   t.status = reinterpret_cast<int*>(d + o_st);
   t.fx_stw_x = d + o_fsx; t.fx_wm_x = d + o_fwx; t.fx_dec_x = d + o_fdx;
   t.fx_stw_y = d + o_fsy; t.fx_wm_y = d + o_fwy; t.fx_dec_y = d + o_fdy;
-  t.fx_mexp = (sizeof(R) == 8 && g.m_generic) ? reinterpret_cast<int*>(d + o_fme) : nullptr;
+  t.fx_mexp = T.fx_mexp.empty() ? nullptr : reinterpret_cast<int*>(d + o_fme);
   const dsnu_status sm = build_m1_table<R>(P, dkx, dky, st);
   if (sm != DSNU_OK) return sm;
   return setup_spread<R>(P, T.node_q0, T.node_w, st);
@@ -832,8 +839,7 @@ static dsnu_status build_tables_standard_fx(dsnu_plan_s* P, cudaStream_t st) {
   fft_stage_twiddles(g.log2ny, tmp, fx_log2_radix(g.log2ny));
   const std::vector<int> stw_y = fx_table(tmp, kFxTwBits);
   const double dkx = M_PI / p.lx, dky = M_PI / p.ly;
-  std::vector<int> mexp;
-  if (g.m_generic) mexp = fx_mult_exponents(g, g.nx / 2 + 1, dkx, dky, 0.5 * g.ny * dky);
+  const std::vector<int> mexp = fx_mult_exponents(g, g.nx / 2 + 1, dkx, dky, 0.5 * g.ny * dky);
   g.m1_full = (g.m_generic && g.m_as != 0.0) ? 1 : 0;
   g.m1_ld = g.m1_full ? g.ny : g.ny / 2 + 1;
   Builder b;
@@ -846,7 +852,7 @@ static dsnu_status build_tables_standard_fx(dsnu_plan_s* P, cudaStream_t st) {
   PlanTables& t = P->tab;
   t.fx_stw_x = d + o_stx;
   t.fx_stw_y = d + o_sty;
-  t.fx_mexp = g.m_generic ? reinterpret_cast<int*>(d + o_me) : nullptr;
+  t.fx_mexp = mexp.empty() ? nullptr : reinterpret_cast<int*>(d + o_me);
   t.status = reinterpret_cast<int*>(d + o_st);
   const size_t bytes = size_t(g.nx / 2 + 1) * g.m1_ld * sizeof(int2);
   cudaError_t e = cudaMalloc(&P->m1_block, bytes);
