@@ -47,9 +47,9 @@ struct alignas(8) fxr {  // real constant in the same form
   int h, l;
 };
 
-// k of the tables: the twiddles carry 1/16, the multiplier 1/32, the
-// deconvolution factors 1/2
-constexpr int kFxTwBits = 28, kFxMultBits = 27, kFxDeconBits = 31;
+// k of the tables: the twiddles carry 1/16, the multiplier and the deconvolution
+// factors 1/2
+constexpr int kFxTwBits = 28, kFxMultBits = 31, kFxDeconBits = 31;
 
 // Exponents of all-zero transforms, and of ones with an infinity or a NaN.
 constexpr int kFxZero = -(1 << 20), kFxBad = 1 << 20;
@@ -240,6 +240,10 @@ __device__ __forceinline__ unsigned fx_read(unsigned m, const unsigned* red) {
 // above: a component of a complex value whose magnitude is below 2^(T + 1/2)).
 template <int T>
 __device__ __forceinline__ int fx_norm_shift(unsigned m) { return max(__clz(int(m)) - (64 - T), 0); }
+
+// Right shift that brings magnitudes OR-ed to m below 2^T.
+template <int T>
+__device__ __forceinline__ int fx_excess(unsigned m) { return max(64 - T - __clz(int(m)), 0); }
 
 // ---------------------------------------------------------------------------
 // Values per thread, the radix of the stages: 16, or 8 for the short transforms,

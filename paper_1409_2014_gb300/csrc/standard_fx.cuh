@@ -115,15 +115,15 @@ k_fx_std_col(Members mem, size_t offH, size_t offE, size_t offC, int ldq, int nc
     const int s0 = fx_norm_shift<61>(fx_read<P>(mag, red + 2 * W));
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = fx_shr<4>(fx_shl(v[m], s0));
-    int ex = emax + 2 - s0 + 4 + (mt.mexp && valid ? mt.mexp[col] : 0) + 5;
+    int ex = emax + 2 - s0 + 4 + (mt.mexp && valid ? mt.mexp[col] : 0) + 1;
 #pragma unroll 1
     for (int inv = 0;; ++inv) {  // forward, then inverse (one copy of the transform's code)
       ex += fx_fft<LOG2N, P>(v, buf, t, stw, red);
-      mag = fx_post<P>(fx_mag(v), red + (2 + inv) * W);
-      __syncthreads();
-      const int s = fx_norm_shift<62>(fx_read<P>(mag, red + (2 + inv) * W));
-      ex -= s;
       if (inv) {
+        mag = fx_post<P>(fx_mag(v), red + 3 * W);
+        __syncthreads();
+        const int s = fx_norm_shift<62>(fx_read<P>(mag, red + 3 * W));
+        ex -= s;
         if (valid) {
 #pragma unroll
           for (int m = 0; m < E; ++m) hs[TL::at(t + G * m, col, ldq)] = fx_shl(fx_swap(v[m]), s);
@@ -136,9 +136,16 @@ k_fx_std_col(Members mem, size_t offH, size_t offE, size_t offC, int ldq, int nc
       for (int m = 0; m < E; ++m) {
         const int q = t + G * m;
         const fxr c = fx_ldr(mg + (FULL || m < H ? q : N - q));
-        const fxc x = fx_shl(v[m], s);
-        v[m] = fx_mk(fx_mulr(x.y, c), fx_mulr(x.x, c));  // (components exchanged: the inverse transform)
+        v[m] = fx_mk(fx_mulr(v[m].y, c), fx_mulr(v[m].x, c));  // (components exchanged: the inverse transform)
       }
+      // room for the inverse's first stage (as in k_fx_col_main)
+      mag = fx_post<P>(fx_mag(v), red + 2 * W);
+      __syncthreads();
+      const int d = fx_excess<57>(fx_read<P>(mag, red + 2 * W));
+      ex += d;
+      if (d > 0)
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = fx_sra(v[m], d);
     }
   }
 }
