@@ -29,10 +29,6 @@
 
 #include "common.cuh"
 
-#ifndef FX_E8_MAX
-#define FX_E8_MAX 10
-#endif
-
 namespace dsnu {
 
 using i64 = long long;
@@ -250,9 +246,10 @@ __device__ __forceinline__ int fx_excess(unsigned m) { return max(64 - T - __clz
 // whose passes do not fill the GPU: twice the threads, each with less than half
 // the instructions in a row (FP64 solves with 8 against 16 values: 128^2 66 -> 49
 // us, 512^2 92 -> 86, 1024 x 256 88 -> 76, 1024^2 equal, 2048^2 534 -> 639).
+constexpr int kFxE8Max = 10;  // log2 of the longest transform with 8 values per thread
 template <int LOG2N>
 struct FxRad {
-  static constexpr int LE = (LOG2N <= FX_E8_MAX) ? 3 : 4, E = 1 << LE;
+  static constexpr int LE = (LOG2N <= kFxE8Max) ? 3 : 4, E = 1 << LE;
   static constexpr int FULL = LOG2N / LE, LR = LOG2N - LE * FULL;  // radix-E stages, log2 of the last one's radix
   // stage twiddles (e^{-2 pi i r k/(NS RAD)}, r = 1 .. RAD - 1, k < NS, stage by stage)
   __host__ __device__ static constexpr int stw() {
@@ -262,7 +259,7 @@ struct FxRad {
   }
   static constexpr int STW = stw() > 0 ? stw() : 1;
 };
-inline int fx_log2_radix(int log2n) { return log2n <= FX_E8_MAX ? 3 : 4; }
+inline int fx_log2_radix(int log2n) { return log2n <= kFxE8Max ? 3 : 4; }
 
 // Length-N DFT by a group of G = N/E threads, E values per thread (the index
 // order and buffer layout of block_fft_regs with E for 16).  P threads share one scale and

@@ -263,6 +263,7 @@ template <typename R, int LOG2N, typename GG = Geo<R, LOG2N>>
 __device__ __forceinline__ void row_fwd_body(int vb, int vg, Members mem, WsOff off, int ldqA, int ldqB, int Q,
                                              int ny, AxisTabs<R> ax, const R* __restrict__ decon_y, int cj,
                                              int* status) {
+  static_assert(sizeof(R) == 4, "the mixed plans' passes (tables and copies in FP32)");
   constexpr int N = GG::N, G = GG::G, RB = GG::RB_F, T = GG::T_RF, RS = GG::RS;
   constexpr bool PF = GG::ROW_PF;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -435,6 +436,7 @@ k_row_fwd(Members mem, WsOff off, int ldqA, int ldqB, int Q, int ny, AxisTabs<R>
 template <typename R, int LOG2N, bool FULL, typename GG = Geo<R, LOG2N>>
 __device__ __forceinline__ void col_main_body(int vb, int vg, Members mem, WsOff off, int ldqA, int ncols,
                                               AxisTabs<R> ay, MultRows<R> mt, int cj, int* ctr) {
+  static_assert(sizeof(R) == 4, "the mixed plans' passes (tables and copies in FP32)");
   constexpr int N = GG::N, G = GG::G, CC = GG::CC, FB = GG::FB;
   // the e^{-2 pi i n/M} factors of the odd chain come from a shared table filled
   // once per CTA with the arithmetic of twm(), and m1 of the item's columns from
@@ -569,6 +571,7 @@ k_col_main(Members mem, WsOff off, int ldqA, int ncols, AxisTabs<R> ay, MultRows
 template <typename R, int LOG2N, typename GG = Geo<R, LOG2N>>
 __device__ __forceinline__ void band_fwd_body(int vb, int vg, Members mem, WsOff off, int ldqB, int ncols, int ldq,
                                               int Q, AxisTabs<R> ay, int cj) {
+  static_assert(sizeof(R) == 4, "the mixed plans' passes (tables and copies in FP32)");
   constexpr int N = GG::N, M = GG::M, G = GG::G, CC = GG::CB, FB = GG::FB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* stw = reinterpret_cast<cpx<R>*>(smem_raw);
@@ -878,6 +881,7 @@ void launch_spread(int cfg, const Members& mem, const WsOff& off, const PlanTabl
 template <typename R, int LOG2N, typename GG = Geo<R, LOG2N>>
 __device__ __forceinline__ void band_inv_body(int vb, int vg, Members mem, WsOff off, int ldq, int Q, int ncols,
                                               int ldqB, AxisTabs<R> ay, int cj) {
+  static_assert(sizeof(R) == 4, "the mixed plans' passes (tables and copies in FP32)");
   constexpr int N = GG::N, M = GG::M, G = GG::G, CC = GG::CB, FB = GG::FB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* stw = reinterpret_cast<cpx<R>*>(smem_raw);
@@ -941,6 +945,7 @@ template <typename R, int LOG2N, typename GG = Geo<R, LOG2N>>
 __device__ __forceinline__ void row_inv_body(int vb, int vg, Members mem, WsOff off, int ldqA, int ldqB, int Q,
                                              int ny, AxisTabs<R> ax, const R* __restrict__ decon_y, R scale, int cj,
                                              int bpf, int acc64) {
+  static_assert(sizeof(R) == 4, "the mixed plans' passes (tables and copies in FP32)");
   constexpr int N = GG::N, G = GG::G, RB = GG::RB_I, RS = GG::RS, T = GG::T_RI;
   constexpr bool PF = GG::ROWI_PF;
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -61,6 +61,7 @@ struct GeoStd {
 template <typename R, int LOG2N>
 __global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, GeoStd<R, LOG2N>::MINB)
 k_std_row_fwd(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restrict__ stw_g, int cj, int* status) {
+  static_assert(sizeof(R) == 4, "the mixed plans' passes (tables and copies in FP32)");
   using GG = GeoStd<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, PER = GG::PER;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -136,6 +137,7 @@ template <typename R, int LOG2N>
 __global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, GeoStd<R, LOG2N>::MINB)
 k_std_col(Members mem, size_t offH, int ldq, int ncols, const cpx<R>* __restrict__ stw_g,
           MultTabs<R> mt, R scale, int cj) {
+  static_assert(sizeof(R) == 4, "the mixed plans' passes (tables and copies in FP32)");
   using GG = GeoStd<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, PER = GG::PER;
   constexpr bool PF = LOG2N >= 9;  // (below, the registers for it are not there)
@@ -204,6 +206,7 @@ k_std_col(Members mem, size_t offH, int ldq, int ncols, const cpx<R>* __restrict
 template <typename R, int LOG2N>
 __global__ void __launch_bounds__(GeoStd<R, LOG2N>::T, GeoStd<R, LOG2N>::MINB)
 k_std_row_inv(Members mem, size_t offH, int ldq, int ny, const cpx<R>* __restrict__ stw_g, int cj) {
+  static_assert(sizeof(R) == 4, "the mixed plans' passes (tables and copies in FP32)");
   using GG = GeoStd<R, LOG2N>;
   constexpr int N = GG::N, G = GG::G, PER = GG::PER, T = GG::T;
   constexpr int HS = N / 2 + 1;  // segments per row pair
