@@ -22,6 +22,7 @@
 
 #include "internal.h"
 #include "kernels_fx.cuh"
+#include "tables.h"
 
 namespace dsnu {
 
@@ -417,21 +418,6 @@ dsnu_status ds_fail(dsnu_status s, const std::string& m) {
   return s;
 }
 
-// Stage twiddles for stages of radix 2^lr (the last one what is left).
-void stage_twiddles(int log2n, int lr, std::vector<double>& out) {
-  out.clear();
-  for (int s = 1; s * lr < log2n; ++s) {
-    const int rad = 1 << std::min(lr, log2n - s * lr), ns = 1 << (s * lr);
-    for (int r = 1; r < rad; ++r)
-      for (int k = 0; k < ns; ++k) {
-        const double a = -2.0 * M_PI * double(r) * double(k) / double(ns * rad);
-        out.push_back(std::cos(a));
-        out.push_back(std::sin(a));
-      }
-  }
-  if (out.empty()) out.assign(2, 0.0);
-}
-
 template <typename R, typename V>
 void upload(void* dst, const V& v, cudaStream_t st, cudaError_t* e) {
   std::vector<R> tmp(v.begin(), v.end());
@@ -651,8 +637,8 @@ dsnu_status dsnu_ds_plan_create(const dsnu_ds_params* params, void* stream, dsnu
   const size_t rsz = p.precision == DSNU_MIXED ? 4 : 8;
   std::vector<double> sx, sy;
   const bool fx = p.precision == DSNU_FP64;
-  stage_twiddles(P->log2nx, fx ? fx_log2_radix(P->log2nx) : 4, sx);
-  stage_twiddles(P->log2ny, fx ? fx_log2_radix(P->log2ny) : 4, sy);
+  fft_stage_twiddles(P->log2nx, sx, fx ? fx_log2_radix(P->log2nx) : 4);
+  fft_stage_twiddles(P->log2ny, sy, fx ? fx_log2_radix(P->log2ny) : 4);
   auto al = [](size_t v) { return (v + 255) & ~size_t(255); };
   const size_t o_sx = 0, o_sy = al(sx.size() * rsz), o_px = o_sy + al(sy.size() * rsz);
   const size_t o_py = o_px + al(2 * size_t(p.nx) * rsz), total = o_py + al(2 * size_t(p.ny) * rsz);
@@ -672,18 +658,8 @@ dsnu_status dsnu_ds_plan_create(const dsnu_ds_params* params, void* stream, dsnu
     upload<float>(P->stw_y, sy, st, &e);
     if (e == cudaSuccess) e = prepare_f32(P);
   } else {
-    auto fixed = [](const std::vector<double>& v) {  // fxw entries
-      std::vector<int> out;
-      for (double c : v) {
-        const double x = std::ldexp(c, kFxTwBits), h = std::nearbyint(x);
-        const double l = std::nearbyint((x - h) * 4294967296.0);
-        out.push_back(int(h));
-        out.push_back(int(std::min(std::max(l, -2147483647.0), 2147483647.0)));
-      }
-      return out;
-    };
-    upload<int>(P->stw_x, fixed(sx), st, &e);
-    upload<int>(P->stw_y, fixed(sy), st, &e);
+    upload<int>(P->stw_x, fx_table(sx, kFxTwBits), st, &e);
+    upload<int>(P->stw_y, fx_table(sy, kFxTwBits), st, &e);
     if (e == cudaSuccess) e = prepare_f64(P);
   }
   if (e != cudaSuccess) {

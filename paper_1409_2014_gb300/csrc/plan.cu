@@ -30,6 +30,7 @@
 #include "internal.h"
 #include "kernels.cuh"
 #include "kernels_fx.cuh"
+#include "tables.h"
 
 namespace dsnu {
 
@@ -219,19 +220,6 @@ struct HostTables {
   std::vector<int> fx_stw_x, fx_wm_x, fx_dec_x, fx_stw_y, fx_wm_y, fx_dec_y, fx_mexp;
 };
 
-// A constant |v| <= 1 as v 2^bits = h + l 2^-32, h and l signed 32-bit (|l| < 2^31).
-static void fx_put(std::vector<int>& out, double v, int bits) {
-  const double s = std::ldexp(v, bits), h = std::nearbyint(s);
-  const double l = std::nearbyint((s - h) * 4294967296.0);
-  out.push_back(int(h));
-  out.push_back(int(std::min(std::max(l, -2147483647.0), 2147483647.0)));
-}
-static std::vector<int> fx_table(const std::vector<double>& v, int bits) {
-  std::vector<int> out;
-  out.reserve(2 * v.size());
-  for (double x : v) fx_put(out, x, bits);
-  return out;
-}
 // The deconvolution factors d / 2^kd with 2^kd > max d; returns kd.
 static int fx_decon(const std::vector<double>& d, std::vector<int>& out) {
   const int kd = int(std::floor(std::log2(*std::max_element(d.begin(), d.end()) * (1.0 + 1e-6)))) + 1;
@@ -305,24 +293,6 @@ static void twiddles(int n, int m, std::vector<double>& out) {
     out[2 * i] = std::cos(a);
     out[2 * i + 1] = std::sin(a);
   }
-}
-
-// FFT stage twiddles of a length-2^log2n transform in the order the device
-// FFT reads them: stage s >= 1 (radix RAD, NS = product of the earlier
-// radices), r = 1..RAD-1, k = 0..NS-1: e^{-2 pi i r k / (NS RAD)}.
-// (lr: log2 of the full stages' radix)
-static void fft_stage_twiddles(int log2n, std::vector<double>& out, int lr = 4) {
-  out.clear();
-  for (int s = 1; s * lr < log2n; ++s) {
-    const int rad = 1 << std::min(lr, log2n - s * lr), ns = 1 << (s * lr);
-    for (int r = 1; r < rad; ++r)
-      for (int k = 0; k < ns; ++k) {
-        const double a = -2.0 * M_PI * double(r) * double(k) / double(ns * rad);
-        out.push_back(std::cos(a));
-        out.push_back(std::sin(a));
-      }
-  }
-  if (out.empty()) out.assign(2, 0.0);
 }
 
 // The compact form (fft_stage_tw_elems_ct): stage 1 as above, then the two
