@@ -27,7 +27,7 @@ _ACCUM = {"fp64": _abi.DSNU_ACCUM_FP64, "working": _abi.DSNU_ACCUM_WORKING}
 def _raw_stream(device) -> int:
     """The current stream's handle on a CUDA device with an index: by torch's
     direct accessor where it has one (the public torch.cuda.current_stream builds
-    a Stream object: 10 us on a Grace host, the accessor below 1 us)."""
+    a Stream object: 1.9 us on a Grace host, this function 0.2)."""
     import torch
 
     raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)

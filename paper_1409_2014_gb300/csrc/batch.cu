@@ -11,7 +11,7 @@
 //   * one launch sequence per group on forked streams, so that different grid
 //     sizes overlap (any plans).
 // DSNU_BATCH_AUTO takes the forked streams: on GB300 they solve the 64-member
-// batch of grids 256^2 .. 2048^2 in 2.85 ms against 3.42 ms for the stage
+// batch of grids 256^2 .. 2048^2 in 2.91 ms against 3.45 ms for the stage
 // launches, since the hardware interleaves the concurrent groups' stages
 // while a stage launch ends for all groups at once.  Either launch sequence
 // can be captured once into a CUDA graph and replayed.

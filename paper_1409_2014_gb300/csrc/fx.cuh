@@ -15,11 +15,19 @@
 // multiplication carries the factor 1/16: complex magnitudes enter a butterfly
 // below 2^57.5 and leave it below 2^61.5, with no overflow in any partial sum
 // (a partial sum of a DFT is a DFT of fewer terms).  The quantum is then at
-// most 2^-56 of the largest component at every stage, whatever the data: a
-// fixed 1/16 per stage would cost localised data, which do not grow in the
-// first stages, four bits each (measured: 5 times the FP64 transforms' error).
-// As in floating point, errors are relative to the norm of a transform's
-// input, not to single elements.
+// most 2^-56 of the block's largest component at every stage (the shift looks at
+// the high words and recovers up to 29 bits at a time): a fixed 1/16 per stage
+// would cost localised data, which do not grow in the first stages, four bits
+// each (measured: 5 times the FP64 transforms' error).
+//
+// As in floating point, errors are relative to the norm of a transform's input,
+// not to single elements; their constant grows with the ratio of a block's
+// largest component to its root mean square, 3-5 for noise, up to sqrt(N) for a
+// single wave.  Against the same passes in FP64 arithmetic (standard solver and
+// linear flow, lengths 32-4096, noise, smooth densities, single waves), relative
+// to max |m| ||rho||, the errors are 0.5-1.0 times as large and at most 1.1 times
+// on the blocks with the largest ratio; where a multiplier damps the whole input
+// (by 2^-8 and more) they can be three times as large relative to the small result.
 //
 // Multiplication: x = xh 2^32 + xl with both halves signed (xl in [-2^31,
 // 2^31)), the constant as w 2^k = h + l 2^-32 in two signed 32-bit halves;

@@ -33,7 +33,8 @@ struct Overlap {
 // 1024^2 156, in line 166; mixed 256^2 41 against 47).  There the mixed share is
 // capped at 48 SMs (1024^2 55.6 us with 48, 63.3 with 16; 2048 x 512 53.6 and
 // 59.7).  All measured with 16384 nodes of the default widths: node count and
-// width do not enter.
+// width do not enter.  With few nodes a smaller share would do (2048 x 1024 with
+// 288 nodes: 76 us, with 16 SMs 70, in line 84; with 16384 nodes 82, 84 and 94).
 //
 // `env` (DSNU_BAND_SMS) sets the number.  One that leaves the column pass no SM
 // runs both in line: its grid would be a single CTA.
